@@ -18,6 +18,8 @@ from paper_2505_21036_b200 import api, layer
 STEPS = 50            # sampling steps; the first tenth are dense, so step 0 is a dense call and step 25 a sparse one
 BANDWIDTHS = (0.125, 0.25, 0.5)   # candidates of the dynamic-bandwidth variant
 MOST_PAIRS = 1.7e11   # query-key pairs (times D / 128) of the largest listed case
+MOST_EXACT = 3e13     # B * H * N^2 * D up to which the 64-bit result takes less than about 20 seconds
+SPATIAL, TEMPORAL, TEXTURAL = api.RF_SPATIAL, api.RF_TEMPORAL, api.RF_TEXTURAL
 
 
 def _case(name, kind, B, H, D, T, fh, fw, L, omega, mode=0, amp=1.5, lse=False, permute=1, key_frame=False, window_2d=False,
@@ -186,3 +188,92 @@ def tolerance(case):
     # 2.2e-3 and max 5e-3 to 1.44e-2 (heads of the tiny, ragged, 8x1024 and CogVideoX shapes): four times that.  Head
     # classes and windows are exact: the planted structure leaves no recall near the threshold.
     return {"rel": 7e-3, "max": 6e-2}
+
+
+def _kept(c, kind, window, rows, cols):
+    """Which of the pairs (row token, key token) a head of this kind keeps, by the definitions of the patterns; `rows`
+    and `cols` are token indices in original order."""
+    S, W, Nv = c["fh"] * c["fw"], c["fw"], c["T"] * c["fh"] * c["fw"]
+    if kind == TEXTURAL:
+        p = cols % S
+        return ((cols >= Nv) | ((p // W) % 2 == (p % W) % 2)).expand(len(rows), -1)
+    r, u = rows[:, None], cols[None, :]
+    if kind == SPATIAL:
+        keep = (r // S - u // S).abs() <= window
+        if c["key_frame"]:
+            keep |= u < S
+    elif c["window_2d"]:
+        pr, pu = r % S, u % S
+        keep = ((pr // W - pu // W).abs() <= c["fh"] // 4) & ((pr % W - pu % W).abs() <= c["fw"] // 4)
+    else:
+        keep = (r % S - u % S).abs() <= window
+    return keep | (r >= Nv) | (u >= Nv)
+
+
+def _recalls(c, q, k, tokens, kind, windows):
+    """Mean share of the softmax mass that each window of a pattern keeps among the sampled tokens (64 bits)."""
+    got = torch.zeros(len(windows), dtype=torch.float64, device=q.device)
+    scaled, keys = q[tokens].double() / math.sqrt(c["D"]), k[tokens].double()
+    for r0 in range(0, len(tokens), 4096):
+        p = torch.softmax(scaled[r0:r0 + 4096] @ keys.T, dim=-1)
+        for i, w in enumerate(windows):
+            got[i] += (p * _kept(c, kind, w, tokens[r0:r0 + 4096], tokens)).sum()
+    return (got / len(tokens)).tolist()
+
+
+def _classify(c, q, k):
+    """(class, window) of one head by Algorithm 1, or by the smallest bandwidth that qualifies."""
+    T, S = c["T"], c["fh"] * c["fw"]
+    every = torch.arange(0, T * S, c["omega"], device=q.device)
+    first = torch.arange(S, device=q.device) if c["mode"] == 0 else every
+    wf, ws = _windows(c)
+    plus = c["kind"] == "plus"
+    wt = [int(b * S) for b in BANDWIDTHS] if plus else [ws]
+    wsp = [int(b * T) for b in BANDWIDTHS] if plus else [wf]
+    for kind, tokens, windows in ((TEMPORAL, first, wt), (SPATIAL, every, wsp)):
+        for w, recall in zip(windows, _recalls(c, q, k, tokens, kind, windows)):
+            if recall >= 0.9:
+                return kind, w
+    return TEXTURAL, -1
+
+
+def exact(case, seed):
+    """`run`'s outputs from the definitions in 64 bits: explicit masks, explicit softmax, a block of rows at a time."""
+    c = case
+    q, k, v = _inputs(c, seed)
+    B, H, N, D = q.shape
+    if B * H * float(N) * N * D > MOST_EXACT:
+        return None
+    dev = q.device
+    tokens = torch.arange(N, device=dev)
+    o = torch.empty(q.shape, dtype=torch.float64, device=dev)
+    lse = torch.empty(q.shape[:3], dtype=torch.float64, device=dev)
+    classes, windows = (torch.full((B, H), -1, dtype=torch.int32, device=dev) for _ in range(2))
+    for b in range(B):
+        for h in range(H):
+            keep_all, cols = c["kind"] == "dense", tokens
+            if not keep_all:
+                kind, window = _classify(c, q[b, h], k[b, h])
+                classes[b, h], windows[b, h] = kind, window
+                if kind == TEXTURAL:
+                    cols, keep_all = tokens[_kept(c, kind, 0, tokens[:1], tokens)[0]], True
+            keys, values = k[b, h][cols].double(), v[b, h][cols].double()
+            step = max(128, (1 << 28) // len(cols))
+            for r0 in range(0, N, step):
+                rows = tokens[r0:r0 + step]
+                s = (q[b, h][rows].double() / math.sqrt(D)) @ keys.T
+                if not keep_all:
+                    s.masked_fill_(~_kept(c, kind, window, rows, cols), -math.inf)
+                top = s.amax(dim=1, keepdim=True)
+                s.sub_(top).exp_()
+                total = s.sum(dim=1, keepdim=True)
+                o[b, h, r0:r0 + step] = (s @ values).div_(total)
+                lse[b, h, r0:r0 + step] = (top + total.log())[:, 0]
+    if c["kind"] == "host":
+        return {"o": o}
+    out = {"o": o, "lse": lse if c["lse"] else None}
+    if c["kind"] != "dense":
+        out["head_class"] = classes
+    if c["kind"] == "plus":
+        out["head_window"] = windows
+    return out
