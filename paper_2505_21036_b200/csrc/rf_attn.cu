@@ -12,7 +12,7 @@
 // Per listed tile and stream: S lands in TMEM, the softmax warps read their rows (tcgen05.ld), keep a
 // running maximum and sum in fp32, write P as packed bf16 back into TMEM (tcgen05.st: on top of the S
 // columns at D = 96 / 128, into spare columns at D = 64) and the MMA warp multiplies it with V straight
-// from TMEM.  The running maximum is raised lazily (see kSumLimit), in which case the softmax warp itself
+// from TMEM.  The running maximum is raised lazily (see kRaise), in which case the softmax warp itself
 // rescales its rows of O in TMEM; the final O / l and the log-sum-exp do not depend on it.
 // PARTIAL tiles apply the exact element mask of the head's pattern; FULL tiles skip it.
 #include "rf_attn_common.cuh"
@@ -24,13 +24,21 @@ using namespace rf_attn;
 
 constexpr int kThreads = kWsThreads;        // 3 warpgroups: softmax 0, softmax 1, {TMA, MMA, 2 idle warps}
 constexpr int kTmaWarp = 8, kMmaWarp = 9;
-// Lazy rescaling of the running maximum.  A tile's weights are taken as 2^(score - running maximum) and accepted
-// while their row sum stays within kSumLimit; beyond it the row's maximum is raised.  bf16 P and the fp32 sums
-// carry the same relative precision at every exponent and 2^32 times the longest row is far from overflow, so
-// O / l and the log-sum-exp do not depend on how stale the running maximum is.
-constexpr float kSumLimit = 4294967296.0f;  // 2^32
-constexpr float kRaiseMargin = 8.0f;        // log2 units: on the slow path, rows this far above their maximum raise it
-constexpr float kLazyRaise = 32.0f;         // log2 units: where the exact tile maximum is at hand (D = 64)
+// What bounds the loop: a stream is the chain scores -> softmax -> P V -> Q K^T, so what counts is how few dependent
+// operations stand between the scores' arrival and the hand-over of P.  At D = 96 / 128 the first kSpec weights are taken
+// while the tile's maximum is being found, the first half of P is stored under the second half's exponentials, and the
+// row sums (192 of 512 instructions) follow the hand-over.  24 heads, 8448 tokens, D = 128 (B200, one box): masked
+// 513 -> 490 us, dense 945 -> 928 us against checking the row sum before the store; without lse the exact sum is left out
+// (a template: dense D = 64, 17776 tokens, 48 heads 5.74 -> 5.59 ms).
+// At D = 64 the maximum comes first and the sums stay in the exponential loop: taking them after the hand-over made the
+// masked case slower (2.94 -> 3.14 ms), the two streams then meet at the exponential pipe.
+// Lazy rescaling of the running maximum: it is raised once a tile's maximum exceeds it by kRaise (log2 units; all rows
+// of the warp more than kRaiseMargin above theirs then raise it together).  A tile's weights thus sum to 2^32 at most;
+// bf16 P and the fp32 sums carry the same relative precision at every exponent and 2^32 times the longest row is far
+// from overflow, so O / l and the log-sum-exp do not depend on how stale the running maximum is.
+constexpr float kLazyRaise = 32.0f;         // D = 64: the maximum comes before the weights there
+constexpr float kRaise = 25.0f, kRaiseMargin = 8.0f;
+constexpr int kSpec = 32;                   // weights taken before the tile's maximum is known
 
 struct Maps { CUtensorMap m[8]; };
 
@@ -67,14 +75,47 @@ struct Cfg {
   static constexpr int B_Q = 0, B_K0 = 1, B_K0E = 2, B_F = 3, B_E = B_F + NP, B_SF = B_E + NP,
                        B_PF = B_SF + 2, B_OF = B_PF + 2, B_SE = B_OF + 2 /* S read, S_EARLY only */, B_COUNT = B_SE + 2;
   static constexpr uint32_t MISC = BAR + 8 * ((B_COUNT + 7) / 8 * 8);
-  static constexpr uint32_t TOTAL = MISC + 64;
+  static constexpr uint32_t KEEP = MISC + 64;         // 128-bit keep word per softmax thread
+  static constexpr uint32_t TOTAL = KEEP + 256 * 16;
   static constexpr uint32_t ALLOC = TOTAL + 1024;     // slack for manual 1024-byte alignment
   // TMEM columns
   static constexpr uint32_t S_COL0 = 0, S_COL1 = 128, O_COL0 = 256, O_COL1 = S_EARLY ? 320 : 384, TMEM_COLS = 512;
   static constexpr uint32_t P_COL0 = S_EARLY ? 384 : S_COL0, P_COL1 = S_EARLY ? 448 : S_COL1;   // packed bf16, 64 columns
 };
 
+// This thread's row of O times alpha (warp-collective).
 template <int D>
+__device__ __forceinline__ void rescale_o(uint32_t t_o, float alpha) {
+  tc_fence_after();
+#pragma unroll
+  for (int c = 0; c < D / 32; ++c) {
+    uint32_t v[32];
+    tmem_ld32(t_o + c * 32, v);
+    tc_wait_ld();
+#pragma unroll
+    for (int i = 0; i < 32; ++i) v[i] = __float_as_uint(__uint_as_float(v[i]) * alpha);
+    tmem_st32(t_o + c * 32, v);
+  }
+  tc_wait_st();
+  tc_fence_before();
+}
+
+// Weights of the key columns [C0, C1) of a tile: 2^(score * sc - m), packed to bf16; with LSE also their sum before rounding.
+template <int C0, int C1, bool LSE>
+__device__ __forceinline__ void take_weights(const uint32_t (&s)[BN], uint32_t (&pk)[BN / 2], float2& la, float2 sc2, float2 mneg) {
+#pragma unroll
+  for (int c = C0; c < C1; c += 4) {
+    float2 e0 = __ffma2_rn(make_float2(__uint_as_float(s[c]), __uint_as_float(s[c + 1])), sc2, mneg);
+    float2 e1 = __ffma2_rn(make_float2(__uint_as_float(s[c + 2]), __uint_as_float(s[c + 3])), sc2, mneg);
+    e0.x = ex2(e0.x); e0.y = ex2(e0.y);
+    e1.x = ex2(e1.x); e1.y = ex2(e1.y);
+    pk[c / 2] = pack_bf16(e0.x, e0.y);
+    pk[c / 2 + 1] = pack_bf16(e1.x, e1.y);
+    if (LSE) la = __fadd2_rn(la, __fadd2_rn(e0, e1));
+  }
+}
+
+template <int D, bool LSE>
 __global__ void __launch_bounds__(kThreads, 1) rf_attn_kernel(const __grid_constant__ Maps maps, const RfAttnArgs a) {
   using C = Cfg<D>;
   constexpr int KB = C::KB;
@@ -299,38 +340,48 @@ __global__ void __launch_bounds__(kThreads, 1) rf_attn_kernel(const __grid_const
     const float sc = a.scale_log2;
     float m_run = -INFINITY;   // running maximum, log2 domain (score * sc)
     float l_run = 0.f;         // sum of the weights as rounded to bf16, the ones P V multiplies: normalises O
-    float l_exact = 0.f;       // sum of the unrounded weights: the log-sum-exp
+    float l_exact = 0.f;       // sum of the unrounded weights: the log-sum-exp (LSE only)
+    uint4* keep = reinterpret_cast<uint4*>(base_ptr + C::KEEP) + tid;   // this row's keep words of a PARTIAL tile
 
     for (int it = 0; it < n; ++it) {
       const uint32_t entry = L.entry(j, it);
-      const bool partial = (entry & RF_PARTIAL_BIT) != 0;
-      const int u0 = (int)(entry & ~RF_PARTIAL_BIT) * BN;
+      // The keep words of a PARTIAL tile do not depend on its scores: they are worked out before the wait for the
+      // scores, where a stream spends a third of its time anyway, and wait in shared memory (four registers live
+      // through the exponentials cost every tile 3 %).
+      bool partial = (entry & RF_PARTIAL_BIT) != 0;
+      if (partial) {
+        uint32_t w[4];
+        rmask.tile_bits((int)(entry & ~RF_PARTIAL_BIT) * BN, w);
+        partial = __any_sync(0xffffffffu, (w[0] & w[1] & w[2] & w[3]) != 0xffffffffu);   // a warp's rows may keep it whole
+        *keep = make_uint4(w[0], w[1], w[2], w[3]);
+      }
       mbar_wait(bar(C::B_SF + j), it & 1, wc);
       tc_fence_after();
-      if constexpr (C::S_EARLY) {
-        // S into registers and the accumulator handed back at once; P goes to TMEM columns of its own.
-        uint32_t s[128];
-        {
-          uint32_t(&s0)[32] = *reinterpret_cast<uint32_t(*)[32]>(&s[0]);
-          uint32_t(&s1)[32] = *reinterpret_cast<uint32_t(*)[32]>(&s[32]);
-          uint32_t(&s2)[32] = *reinterpret_cast<uint32_t(*)[32]>(&s[64]);
-          uint32_t(&s3)[32] = *reinterpret_cast<uint32_t(*)[32]>(&s[96]);
-          tmem_ld32(t_s, s0);
-          tmem_ld32(t_s + 32, s1);
-          tmem_ld32(t_s + 64, s2);
-          tmem_ld32(t_s + 96, s3);
-          tc_wait_ld();
-        }
+      uint32_t s[128];
+      {
+        uint32_t(&s0)[32] = *reinterpret_cast<uint32_t(*)[32]>(&s[0]);
+        uint32_t(&s1)[32] = *reinterpret_cast<uint32_t(*)[32]>(&s[32]);
+        uint32_t(&s2)[32] = *reinterpret_cast<uint32_t(*)[32]>(&s[64]);
+        uint32_t(&s3)[32] = *reinterpret_cast<uint32_t(*)[32]>(&s[96]);
+        tmem_ld32(t_s, s0);
+        tmem_ld32(t_s + 32, s1);
+        tmem_ld32(t_s + 64, s2);
+        tmem_ld32(t_s + 96, s3);
+        tc_wait_ld();
+      }
+      if constexpr (C::S_EARLY) {   // the accumulator is handed back at once; P goes to TMEM columns of its own
         tc_fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive(bar(C::B_SE + j));
-        if (partial) {
-          uint32_t w[4];
-          rmask.tile_bits(u0, w);
+      }
+      if (partial) {
+        const uint4 kw = *keep;
+        const uint32_t w[4] = {kw.x, kw.y, kw.z, kw.w};
 #pragma unroll
-          for (int c = 0; c < 128; ++c)
-            if (!((w[c >> 5] >> (c & 31)) & 1u)) s[c] = 0xff800000u;  // -inf
-        }
+        for (int c = 0; c < 128; ++c)
+          if (!((w[c >> 5] >> (c & 31)) & 1u)) s[c] = 0xff800000u;  // -inf
+      }
+      if constexpr (C::S_EARLY) {
         // The scores are gone from TMEM, so the exact row maximum comes first and the exponentials are
         // taken once; the running maximum is raised only when the tile exceeds it by kLazyRaise.
         float mx0 = -INFINITY, mx1 = -INFINITY;
@@ -347,7 +398,7 @@ __global__ void __launch_bounds__(kThreads, 1) rf_attn_kernel(const __grid_const
           alpha = ex2(m_run - m_tile);   // 0 when m_run = -inf
           m_run = m_tile;
           l_run *= alpha;
-          l_exact *= alpha;
+          if (LSE) l_exact *= alpha;
         }
         // P V of the previous tile reads the P columns this tile is about to overwrite, and O may only be
         // rescaled once everything issued into it has landed.  The wait sits in front of the P store (the
@@ -357,20 +408,7 @@ __global__ void __launch_bounds__(kThreads, 1) rf_attn_kernel(const __grid_const
         if (it > 0 && any_raise) {
           mbar_wait(bar(C::B_OF + j), (it - 1) & 1, wc);
           o_landed = true;
-          {
-            tc_fence_after();
-#pragma unroll
-            for (int c = 0; c < D / 32; ++c) {
-              uint32_t v[32];
-              tmem_ld32(t_o + c * 32, v);
-              tc_wait_ld();
-#pragma unroll
-              for (int i = 0; i < 32; ++i) v[i] = __float_as_uint(__uint_as_float(v[i]) * alpha);
-              tmem_st32(t_o + c * 32, v);
-            }
-            tc_wait_st();
-            tc_fence_before();
-          }
+          rescale_o<D>(t_o, alpha);
         }
         const float m_use = m_run == -INFINITY ? 0.f : m_run;
         const float2 sc2 = make_float2(sc, sc), mneg = make_float2(-m_use, -m_use);
@@ -384,10 +422,10 @@ __global__ void __launch_bounds__(kThreads, 1) rf_attn_kernel(const __grid_const
           e1.x = ex2(e1.x); e1.y = ex2(e1.y);
           pk[c / 2] = pack_bf16(e0.x, e0.y);
           pk[c / 2 + 1] = pack_bf16(e1.x, e1.y);
-          la = __fadd2_rn(la, __fadd2_rn(e0, e1));
+          if (LSE) la = __fadd2_rn(la, __fadd2_rn(e0, e1));
           lb = __fadd2_rn(lb, __fadd2_rn(unpack_bf16(pk[c / 2]), unpack_bf16(pk[c / 2 + 1])));
         }
-        l_exact += la.x + la.y;
+        if (LSE) l_exact += la.x + la.y;
         l_run += lb.x + lb.y;
         if (!o_landed) mbar_wait(bar(C::B_OF + j), (it - 1) & 1, wc);
         {
@@ -403,92 +441,56 @@ __global__ void __launch_bounds__(kThreads, 1) rf_attn_kernel(const __grid_const
         if (lane == 0) mbar_arrive(bar(C::B_PF + j));
         continue;
       }
-      // Exponentials are taken against the running maximum of the previous tiles, without looking at the
-      // tile's own maximum: all weights are non-negative, so a row sum within kSumLimit proves that none
-      // of them left the safe range.  Only if some row's sum does not (its maximum grew by more than
-      // ~2^25; rare after a row's first tile) is the exact tile maximum taken from the scores, which are
-      // still in TMEM because P has not been stored yet, the running maximum raised, O rescaled and the
-      // pass repeated.
+      // The first kSpec weights are taken against the running maximum of the previous tiles while the tile's own
+      // maximum is being found; only if it exceeds the running one by kRaise (a row's first tile, rare after it) is
+      // the running maximum raised, O rescaled and the weights taken so far taken again.
       uint32_t pk[64];
-#pragma unroll 1
-      for (int pass = 0; pass < 2; ++pass) {
-        uint32_t s[128];
-        {
-          uint32_t(&s0)[32] = *reinterpret_cast<uint32_t(*)[32]>(&s[0]);
-          uint32_t(&s1)[32] = *reinterpret_cast<uint32_t(*)[32]>(&s[32]);
-          uint32_t(&s2)[32] = *reinterpret_cast<uint32_t(*)[32]>(&s[64]);
-          uint32_t(&s3)[32] = *reinterpret_cast<uint32_t(*)[32]>(&s[96]);
-          tmem_ld32(t_s, s0);
-          tmem_ld32(t_s + 32, s1);
-          tmem_ld32(t_s + 64, s2);
-          tmem_ld32(t_s + 96, s3);
-          tc_wait_ld();
-        }
-        if (partial) {
-          uint32_t w[4];
-          rmask.tile_bits(u0, w);
+      float2 la = make_float2(0.f, 0.f);
+      const float2 sc2 = make_float2(sc, sc);
+      float m_use = m_run == -INFINITY ? 0.f : m_run;
+      take_weights<0, kSpec, LSE>(s, pk, la, sc2, make_float2(-m_use, -m_use));
+      float mx0 = -INFINITY, mx1 = -INFINITY;
 #pragma unroll
-          for (int c = 0; c < 128; ++c)
-            if (!((w[c >> 5] >> (c & 31)) & 1u)) s[c] = 0xff800000u;  // -inf
-        }
-        const float m_use = m_run == -INFINITY ? 0.f : m_run;
-        const float2 sc2 = make_float2(sc, sc), mneg = make_float2(-m_use, -m_use);
-        // several partial sums, so that the chain of dependent additions left after the last exponential is
-        // short (the sum of the rounded weights gates the P store)
-        float2 la[2], lb[4];
-        la[0] = la[1] = lb[0] = lb[1] = lb[2] = lb[3] = make_float2(0.f, 0.f);
-#pragma unroll
-        for (int c = 0; c < 128; c += 4) {
-          float2 e0 = __ffma2_rn(make_float2(__uint_as_float(s[c]), __uint_as_float(s[c + 1])), sc2, mneg);
-          float2 e1 = __ffma2_rn(make_float2(__uint_as_float(s[c + 2]), __uint_as_float(s[c + 3])), sc2, mneg);
-          e0.x = ex2(e0.x); e0.y = ex2(e0.y);
-          e1.x = ex2(e1.x); e1.y = ex2(e1.y);
-          pk[c / 2] = pack_bf16(e0.x, e0.y);
-          pk[c / 2 + 1] = pack_bf16(e1.x, e1.y);
-          la[(c >> 2) & 1] = __fadd2_rn(la[(c >> 2) & 1], __fadd2_rn(e0, e1));
-          lb[(c >> 2) & 3] = __fadd2_rn(lb[(c >> 2) & 3], __fadd2_rn(unpack_bf16(pk[c / 2]), unpack_bf16(pk[c / 2 + 1])));
-        }
-        la[0] = __fadd2_rn(la[0], la[1]);
-        lb[0] = __fadd2_rn(__fadd2_rn(lb[0], lb[1]), __fadd2_rn(lb[2], lb[3]));
-        const float l_tile = lb[0].x + lb[0].y, l_tile_exact = la[0].x + la[0].y;
-        if (pass == 1) { l_run += l_tile; l_exact += l_tile_exact; break; }
-        const bool bad = !(l_tile <= kSumLimit) || m_run == -INFINITY;
-        if (!__any_sync(0xffffffffu, bad)) { l_run += l_tile; l_exact += l_tile_exact; break; }
-        const float m_tile = tile_row_max(t_s, partial, rmask, u0) * sc;
-        const bool raise = m_tile > m_run + kRaiseMargin || (m_run == -INFINITY && m_tile > -INFINITY);
+      for (int c = 0; c < 128; c += 4) {
+        mx0 = fmaxf(mx0, fmaxf(__uint_as_float(s[c]), __uint_as_float(s[c + 1])));
+        mx1 = fmaxf(mx1, fmaxf(__uint_as_float(s[c + 2]), __uint_as_float(s[c + 3])));
+      }
+      const float m_tile = fmaxf(mx0, mx1) * sc;
+      if (__any_sync(0xffffffffu, m_tile > m_run + kRaise)) {
         float alpha = 1.f;
-        if (raise) {
+        if (m_tile > m_run + kRaiseMargin) {
           alpha = ex2(m_run - m_tile);   // 0 when m_run = -inf
           m_run = m_tile;
           l_run *= alpha;
-          l_exact *= alpha;
+          if (LSE) l_exact *= alpha;
         }
         if (it > 0) {
           // O of the previous tiles must be complete before it is rescaled
           mbar_wait(bar(C::B_OF + j), (it - 1) & 1, wc);
-          tc_fence_after();
-#pragma unroll
-          for (int c = 0; c < D / 32; ++c) {
-            uint32_t v[32];
-            tmem_ld32(t_o + c * 32, v);
-            tc_wait_ld();
-#pragma unroll
-            for (int i = 0; i < 32; ++i) v[i] = __float_as_uint(__uint_as_float(v[i]) * alpha);
-            tmem_st32(t_o + c * 32, v);
-          }
-          tc_wait_st();
+          rescale_o<D>(t_o, alpha);
         }
+        m_use = m_run == -INFINITY ? 0.f : m_run;
+        la = make_float2(0.f, 0.f);
+        take_weights<0, kSpec, LSE>(s, pk, la, sc2, make_float2(-m_use, -m_use));
       }
-      {
-        uint32_t(&p0)[32] = *reinterpret_cast<uint32_t(*)[32]>(&pk[0]);
-        uint32_t(&p1)[32] = *reinterpret_cast<uint32_t(*)[32]>(&pk[32]);
-        tmem_st32(t_s, p0);
-        tmem_st32(t_s + 32, p1);
-        tc_wait_st();
-      }
+      const uint32_t t_p = tmem_base + lane_sel + (j ? C::P_COL1 : C::P_COL0);
+      take_weights<kSpec, 64, LSE>(s, pk, la, sc2, make_float2(-m_use, -m_use));
+      tmem_st32(t_p, *reinterpret_cast<uint32_t(*)[32]>(&pk[0]));
+      take_weights<64, BN, LSE>(s, pk, la, sc2, make_float2(-m_use, -m_use));
+      tmem_st32(t_p + 32, *reinterpret_cast<uint32_t(*)[32]>(&pk[32]));
+      tc_wait_st();
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(bar(C::B_PF + j));
+      // The row sums gate nothing: they are taken after P has been handed over, under the wait for the next scores.
+      float2 lb[4];
+      lb[0] = lb[1] = lb[2] = lb[3] = make_float2(0.f, 0.f);
+#pragma unroll
+      for (int c = 0; c < 64; c += 2)
+        lb[(c >> 1) & 3] = __fadd2_rn(lb[(c >> 1) & 3], __fadd2_rn(unpack_bf16(pk[c]), unpack_bf16(pk[c + 1])));
+      lb[0] = __fadd2_rn(__fadd2_rn(lb[0], lb[1]), __fadd2_rn(lb[2], lb[3]));
+      l_run += lb[0].x + lb[0].y;
+      if (LSE) l_exact += la.x + la.y;
     }
 
     if (n > 0) {
@@ -497,6 +499,8 @@ __global__ void __launch_bounds__(kThreads, 1) rf_attn_kernel(const __grid_const
       int tok = r;
       if (perm && r < g.Nv) tok = (r % g.T) * g.S + r / g.T;
       const float inv = l_run > 0.f ? 1.f / l_run : 0.f;
+      // a thread writes its row alone, so a warp's store touches 32 rows: whole 32-byte sectors where O allows it
+      const bool o32 = (reinterpret_cast<uintptr_t>(a.o) & 31u) == 0;
       uint4* dst = reinterpret_cast<uint4*>(a.o + ((size_t)bh * g.N + min(tok, g.N - 1)) * D);
 #pragma unroll
       for (int c = 0; c < D / 32; ++c) {
@@ -505,17 +509,17 @@ __global__ void __launch_bounds__(kThreads, 1) rf_attn_kernel(const __grid_const
         tc_wait_ld();
         if (r < g.N && rf_in_bounds(tok, g.N, a.dev_status)) {
 #pragma unroll
-          for (int i = 0; i < 32; i += 8) {
-            uint4 w;
-            w.x = pack_bf16(__uint_as_float(v[i]) * inv, __uint_as_float(v[i + 1]) * inv);
-            w.y = pack_bf16(__uint_as_float(v[i + 2]) * inv, __uint_as_float(v[i + 3]) * inv);
-            w.z = pack_bf16(__uint_as_float(v[i + 4]) * inv, __uint_as_float(v[i + 5]) * inv);
-            w.w = pack_bf16(__uint_as_float(v[i + 6]) * inv, __uint_as_float(v[i + 7]) * inv);
-            dst[(c * 32 + i) / 8] = w;
+          for (int i = 0; i < 16; ++i) v[i] = pack_bf16(__uint_as_float(v[2 * i]) * inv, __uint_as_float(v[2 * i + 1]) * inv);
+          if (o32) {
+            st_global_v8(dst + c * 4, v);
+            st_global_v8(dst + c * 4 + 2, v + 8);
+          } else {
+#pragma unroll
+            for (int i = 0; i < 4; ++i) dst[c * 4 + i] = make_uint4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
           }
         }
       }
-      if (r < g.N && a.lse != nullptr && rf_in_bounds(tok, g.N, a.dev_status)) a.lse[(size_t)bh * g.N + tok] = (m_run + log2f(l_exact)) * 0.6931471805599453f;
+      if (LSE && r < g.N && rf_in_bounds(tok, g.N, a.dev_status)) a.lse[(size_t)bh * g.N + tok] = (m_run + log2f(l_exact)) * 0.6931471805599453f;
     }
   }
 
@@ -528,22 +532,26 @@ __global__ void __launch_bounds__(kThreads, 1) rf_attn_kernel(const __grid_const
   }
 }
 
-template <int D>
+template <int D, bool LSE>
 rf_status launch(const RfAttnArgs& a, const CUtensorMap* maps, cudaStream_t st) {
   static bool configured[64] = {};
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return RF_ERR_CUDA;
   if (dev >= 0 && dev < 64 && !configured[dev]) {
-    if (!rf_regs_ok(rf_attn_kernel<D>)) return RF_ERR_UNSUPPORTED;   // setmaxnreg.inc could never be granted
-    if (cudaFuncSetAttribute(rf_attn_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg<D>::ALLOC) != cudaSuccess)
+    if (!rf_regs_ok(rf_attn_kernel<D, LSE>)) return RF_ERR_UNSUPPORTED;   // setmaxnreg.inc could never be granted
+    if (cudaFuncSetAttribute(rf_attn_kernel<D, LSE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg<D>::ALLOC) != cudaSuccess)
       return RF_ERR_CUDA;
     configured[dev] = true;
   }
   Maps m;
   for (int i = 0; i < 8; ++i) m.m[i] = maps[i];
   dim3 grid(rf_cdiv(a.g.nQ, 2), a.g.B * a.g.H);
-  rf_attn_kernel<D><<<grid, kThreads, Cfg<D>::ALLOC, st>>>(m, a);
+  rf_attn_kernel<D, LSE><<<grid, kThreads, Cfg<D>::ALLOC, st>>>(m, a);
   return cudaGetLastError() == cudaSuccess ? RF_OK : RF_ERR_CUDA;
+}
+template <int D>
+rf_status launch(const RfAttnArgs& a, const CUtensorMap* maps, cudaStream_t st) {
+  return a.lse != nullptr ? launch<D, true>(a, maps, st) : launch<D, false>(a, maps, st);
 }
 
 }  // namespace

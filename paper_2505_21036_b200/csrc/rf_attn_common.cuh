@@ -120,23 +120,6 @@ __device__ __forceinline__ RowMask make_row_mask(const RfGeom& g, int cls, int r
   return m;
 }
 
-// Exact maximum of this thread's row of the S tile at t_s (slow path of the softmax; warp-collective loads).
-static __device__ __noinline__ float tile_row_max(uint32_t t_s, bool partial, const RowMask& rmask, int u0) {
-  uint32_t w[4] = {0xffffffffu, 0xffffffffu, 0xffffffffu, 0xffffffffu};
-  if (partial) rmask.tile_bits(u0, w);
-  float mx = -INFINITY;
-#pragma unroll 1
-  for (int q = 0; q < 4; ++q) {
-    uint32_t v[32];
-    tmem_ld32(t_s + q * 32, v);
-    tc_wait_ld();
-#pragma unroll
-    for (int c = 0; c < 32; ++c)
-      if ((w[q] >> c) & 1u) mx = fmaxf(mx, __uint_as_float(v[c]));
-  }
-  return mx;
-}
-
 // The two streams' ascending tile lists and their merge (the order K/V tiles are fetched in).
 struct Lists {
   const int32_t* l0;
