@@ -1,20 +1,28 @@
 // Pattern-masked FlashAttention forward on tcgen05 / TMEM / TMA (Eq. 1-2 with the masks of Sec. 3.2).
 //
-// One CTA owns two adjacent 128-row query tiles of one head (two "streams") and walks the union of
+// An item of work is two adjacent 128-row query tiles of one head (two "streams"); a CTA walks the union of
 // their KV-tile lists, so every K/V tile fetched by TMA feeds up to two S = Q K^T and two O += P V
-// contractions.  Warp roles:
+// contractions.  A CTA works off one item after another: its own, then those of CTAs that have not started yet, which it
+// takes over through cluster launch control.  The TMA and MMA warps run on into the next item while the softmax
+// warps write out the last one: per item that hides what a CTA of its own pays for its start, its Q and first K, its first
+// scores and its end, 6 to 9 us (24 heads, 8448 tokens, D = 128: 83 us an item, 490 -> 480 us a call; 48 heads,
+// 17 776 tokens, D = 64: 130 us an item, 2930 -> 2700 us masked, 5590 -> 5210 dense, most of it from the issuing
+// thread's shorter code).  Warp roles:
 //   warps 0-3  softmax of stream 0   (one thread per query row, TMEM lane = row)
 //   warps 4-7  softmax of stream 1
 //   warp  8    TMA producer: Q once, then K and V tiles into two shared-memory rings (V of tile u and K of
 //              tile u + 1 as a pair under one full / one empty mbarrier)
 //   warp  9    MMA issuer: tcgen05.mma, accumulators in TMEM (S0, S1, O0, O1)
-//   (warps 10-11 only fill the third warpgroup, which hands its registers to the softmax warpgroups)
+//   warp  10   one thread fetches items and publishes them in shared memory
+//   (warp 11 only fills the third warpgroup, which hands its registers to the softmax warpgroups)
 // Per listed tile and stream: S lands in TMEM, the softmax warps read their rows (tcgen05.ld), keep a
 // running maximum and sum in fp32, write P as packed bf16 back into TMEM (tcgen05.st: on top of the S
 // columns at D = 96 / 128, into spare columns at D = 64) and the MMA warp multiplies it with V straight
 // from TMEM.  The running maximum is raised lazily (see kRaise), in which case the softmax warp itself
 // rescales its rows of O in TMEM; the final O / l and the log-sum-exp do not depend on it.
 // PARTIAL tiles apply the exact element mask of the head's pattern; FULL tiles skip it.
+#include <algorithm>
+
 #include "rf_attn_common.cuh"
 
 namespace {
@@ -23,7 +31,9 @@ using namespace sm100;
 using namespace rf_attn;
 
 constexpr int kThreads = kWsThreads;        // 3 warpgroups: softmax 0, softmax 1, {TMA, MMA, 2 idle warps}
-constexpr int kTmaWarp = 8, kMmaWarp = 9;
+constexpr int kTmaWarp = 8, kMmaWarp = 9, kItemWarp = 10;
+constexpr int kItemSlots = 2, kItemWords = 8, kItemReaders = 10;   // readers: eight softmax warps, the TMA and the MMA thread
+constexpr int kAskAhead = 4;   // tiles an item has left when the next one is asked for: about 8 us, an answer takes about one
 // What bounds the loop: a stream is the chain scores -> softmax -> P V -> Q K^T, so what counts is how few dependent
 // operations stand between the scores' arrival and the hand-over of P.  At D = 96 / 128 the first kSpec weights are taken
 // while the tile's maximum is being found, the first half of P is stored under the second half's exponentials, and the
@@ -39,6 +49,8 @@ constexpr int kTmaWarp = 8, kMmaWarp = 9;
 constexpr float kLazyRaise = 32.0f;         // D = 64: the maximum comes before the weights there
 constexpr float kRaise = 25.0f, kRaiseMargin = 8.0f;
 constexpr int kSpec = 32;                   // weights taken before the tile's maximum is known
+
+constexpr size_t kL2Bytes = 48u << 20;      // K and V of the heads worked on at the same time: well inside the 126 MB L2
 
 struct Maps { CUtensorMap m[8]; };
 
@@ -73,15 +85,33 @@ struct Cfg {
   static_assert(NK == NV, "K and V rings advance together");
   static constexpr int NP = NV;
   static constexpr int B_Q = 0, B_K0 = 1, B_K0E = 2, B_F = 3, B_E = B_F + NP, B_SF = B_E + NP,
-                       B_PF = B_SF + 2, B_OF = B_PF + 2, B_SE = B_OF + 2 /* S read, S_EARLY only */, B_COUNT = B_SE + 2;
+                       B_PF = B_SF + 2, B_OF = B_PF + 2, B_SE = B_OF + 2 /* S read, S_EARLY only */, B_QE = B_SE + 2 /* Q consumed */,
+                       B_REQ = B_QE + 1, B_CLC = B_REQ + 1, B_IF = B_CLC + 1, B_IE = B_IF + kItemSlots, B_COUNT = B_IE + kItemSlots;
   static constexpr uint32_t MISC = BAR + 8 * ((B_COUNT + 7) / 8 * 8);
   static constexpr uint32_t KEEP = MISC + 64;         // 128-bit keep word per softmax thread
-  static constexpr uint32_t TOTAL = KEEP + 256 * 16;
+  static constexpr uint32_t ITEM = KEEP + 256 * 16;   // kItemSlots items of kItemWords words, then the launch-control answer
+  static constexpr uint32_t ANSWER = ITEM + kItemSlots * kItemWords * 4;
+  static constexpr uint32_t TOTAL = ANSWER + 16;
   static constexpr uint32_t ALLOC = TOTAL + 1024;     // slack for manual 1024-byte alignment
   // TMEM columns
   static constexpr uint32_t S_COL0 = 0, S_COL1 = 128, O_COL0 = 256, O_COL1 = S_EARLY ? 320 : 384, TMEM_COLS = 512;
   static constexpr uint32_t P_COL0 = S_EARLY ? 384 : S_COL0, P_COL1 = S_EARLY ? 448 : S_COL1;   // packed bf16, 64 columns
 };
+
+// One item of work: two adjacent query tiles of one head.
+struct Item { int bh, qt0, cls, n0, n1, window; };
+
+// Which item the CTA of index `lin` of the grid stands for.  Heads are taken in groups whose K and V fit the L2 cache
+// together (one head at a time where they are long); inside a group the last pair of query tiles of every head comes
+// first: the text rows list every tile and are the longest items, while the first pairs list the fewest (the windows of
+// Spatial and Temporal heads are cut at the ends), so the SMs run out of work with short items.
+__device__ __forceinline__ void place_item(uint64_t lin, int group, int heads, int pairs, int& bh, int& pair) {
+  const uint64_t per = (uint64_t)group * pairs;
+  const int g0 = (int)(lin / per) * group;
+  const uint32_t r = (uint32_t)(lin % per), in = min(group, heads - g0);
+  bh = g0 + (int)(r % in);
+  pair = pairs - 1 - (int)(r / in);
+}
 
 // This thread's row of O times alpha (warp-collective).
 template <int D>
@@ -129,46 +159,9 @@ __global__ void __launch_bounds__(kThreads, 1) rf_attn_kernel(const __grid_const
   volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(base_ptr + C::MISC);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(base_ptr + C::MISC + 8);
 
-  RfGeom g = a.g;
+  const RfGeom& g = a.g;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int bh = blockIdx.y;
-  const int qt0 = 2 * blockIdx.x, qt1 = qt0 + 1;
-
-  int cls = RF_DENSE;
-  if (a.head_class != nullptr) {
-    cls = a.head_class[bh];
-    if (cls < 0 || cls > 3) {
-      if (tid == 0) rf_report(a.dev_status, RF_ERR_INVALID_ARG);
-      cls = RF_DENSE;
-    }
-  }
-  if (a.head_window != nullptr) {   // dynamic bandwidth: this head's own window
-    const int w = a.head_window[bh];
-    if (cls == RF_SPATIAL && w >= 0) g.wf = min(w, g.T);     // past the extent: same mask, no overflow
-    if (cls == RF_TEMPORAL && w >= 0) g.ws = min(w, g.S);
-  }
-  const bool perm = cls == RF_TEMPORAL && g.permute;
-  const bool tex = cls == RF_TEXTURAL;
-  const CUtensorMap* map_q = &maps.m[perm ? 3 : 0];
-  const CUtensorMap* map_k = &maps.m[perm ? 4 : (tex ? 6 : 1)];
-  const CUtensorMap* map_v = &maps.m[perm ? 5 : (tex ? 7 : 2)];
-
-  Lists L;
-  L.lkv = rf_kv_len(g, cls);
-  L.listed = a.head_class != nullptr;
-  if (L.listed) {
-    L.n0 = a.count[(size_t)bh * g.nQ + qt0];
-    L.n1 = qt1 < g.nQ ? a.count[(size_t)bh * g.nQ + qt1] : 0;
-    // a schedule that was not built for this shape could hold any count: the checking build refuses to walk past a row
-    if (!rf_in_bounds(L.n0, g.nKmax + 1, a.dev_status)) L.n0 = 0;
-    if (!rf_in_bounds(L.n1, g.nKmax + 1, a.dev_status)) L.n1 = 0;
-    L.l0 = a.kv_tile + ((size_t)bh * g.nQ + qt0) * g.nKmax;
-    L.l1 = a.kv_tile + ((size_t)bh * g.nQ + min(qt1, g.nQ - 1)) * g.nKmax;
-  } else {
-    L.n0 = rf_cdiv(L.lkv, BN);
-    L.n1 = qt1 < g.nQ ? L.n0 : 0;
-    L.l0 = L.l1 = nullptr;
-  }
+  int* items = reinterpret_cast<int*>(base_ptr + C::ITEM);
 
   if (tid == 0) {
     mbar_init(bar(C::B_Q), 1);
@@ -181,11 +174,15 @@ __global__ void __launch_bounds__(kThreads, 1) rf_attn_kernel(const __grid_const
       mbar_init(bar(C::B_OF + j), 1);
       mbar_init(bar(C::B_SE + j), 4);
     }
+    mbar_init(bar(C::B_QE), 1);
+    mbar_init(bar(C::B_REQ), 1);
+    mbar_init(bar(C::B_CLC), 1);
+    for (int i = 0; i < kItemSlots; ++i) { mbar_init(bar(C::B_IF + i), 1); mbar_init(bar(C::B_IE + i), kItemReaders); }
     *abort_flag = 0;
     mbar_init_fence();
   }
   if (warp == kTmaWarp) {
-    if (lane == 0) { prefetch_tmap(map_q); prefetch_tmap(map_k); prefetch_tmap(map_v); }
+    if (lane < 8) prefetch_tmap(&maps.m[lane]);
     __syncwarp();
     tmem_alloc(smem_u32(const_cast<uint32_t*>(tmem_slot)), C::TMEM_COLS);
   }
@@ -195,29 +192,128 @@ __global__ void __launch_bounds__(kThreads, 1) rf_attn_kernel(const __grid_const
   const uint32_t tmem_base = *tmem_slot;
   const WaitCtx wc{abort_flag, a.dev_status};
 
+  // The i-th item of this CTA.  False: there is none (or a wait was abandoned).
+  auto take = [&](int i, Item& im, int waited) -> bool {
+    const int slot = i % kItemSlots;
+    if (!mbar_wait_long(bar(C::B_IF + slot), (i / kItemSlots) & 1, wc, waited)) return false;
+    const int* w = items + slot * kItemWords;
+    im.bh = w[0]; im.qt0 = w[1]; im.cls = w[2]; im.n0 = w[3]; im.n1 = w[4]; im.window = w[5];
+    return im.bh >= 0;
+  };
+  auto lists = [&](const Item& im) -> Lists {
+    Lists L;
+    L.lkv = rf_kv_len(g, im.cls);
+    L.listed = a.head_class != nullptr;
+    L.n0 = im.n0;
+    L.n1 = im.n1;
+    L.l0 = L.listed ? a.kv_tile + ((size_t)im.bh * g.nQ + im.qt0) * g.nKmax : nullptr;
+    L.l1 = L.listed ? a.kv_tile + ((size_t)im.bh * g.nQ + min(im.qt0 + 1, g.nQ - 1)) * g.nKmax : nullptr;
+    return L;
+  };
+
   if (warp >= 8) {
   RF_SETMAXNREG_DEC();
-  if (warp == kTmaWarp) {
-    // ------------------------------------------------------------ TMA producer
+  if (warp == kItemWarp) {
+    // ------------------------------------------------------------ items: the own one, then those of CTAs not started yet
     if (lane == 0) {
-      mbar_expect_tx(bar(C::B_Q), 2 * C::TILE);
-#pragma unroll
-      for (int j = 0; j < 2; ++j)
-#pragma unroll
-        for (int kb = 0; kb < KB; ++kb)
-          tma_load_3d(base + C::Q + j * C::TILE + kb * C::BLK, map_q, kb * C::COL1, (qt0 + j) * BM, bh, bar(C::B_Q));
+      uint32_t x = blockIdx.x, y = blockIdx.y;
+      bool more = true;
+      for (int i = 0;; ++i) {
+        const int slot = i % kItemSlots;
+        int* w = items + slot * kItemWords;
+        if (i >= kItemSlots) mbar_wait(bar(C::B_IE + slot), ((i / kItemSlots) - 1) & 1, wc);
+        int n0 = 0, n1 = 0;
+        if (more) {
+          int bh, pair;
+          place_item((uint64_t)y * gridDim.x + x, a.heads_l2, g.B * g.H, gridDim.x, bh, pair);
+          const int qt0 = 2 * pair, qt1 = qt0 + 1;
+          int cls = RF_DENSE, window = -1;
+          if (a.head_class != nullptr) {
+            cls = a.head_class[bh];
+            if (cls < 0 || cls > 3) {
+              rf_report(a.dev_status, RF_ERR_INVALID_ARG);
+              cls = RF_DENSE;
+            }
+            if (a.head_window != nullptr) window = a.head_window[bh];
+            n0 = a.count[(size_t)bh * g.nQ + qt0];
+            n1 = qt1 < g.nQ ? a.count[(size_t)bh * g.nQ + qt1] : 0;
+            // a schedule that was not built for this shape could hold any count: the checking build refuses to walk past a row
+            if (!rf_in_bounds(n0, g.nKmax + 1, a.dev_status)) n0 = 0;
+            if (!rf_in_bounds(n1, g.nKmax + 1, a.dev_status)) n1 = 0;
+          } else {
+            n0 = rf_cdiv(rf_kv_len(g, cls), BN);
+            n1 = qt1 < g.nQ ? n0 : 0;
+          }
+          w[0] = bh; w[1] = qt0; w[2] = cls; w[3] = n0; w[4] = n1; w[5] = window;
+        } else {
+          w[0] = -1;
+        }
+        mbar_arrive(bar(C::B_IF + slot));
+        if (!more) break;
+        more = false;
+        // not before the TMA warp has nearly worked the item off: an item taken early would wait here while other SMs idle
+        if (mbar_wait_long(bar(C::B_REQ), i & 1, wc, n0 + n1)) {
+          fence_proxy_async_smem();
+          mbar_expect_tx(bar(C::B_CLC), 16);
+          clc_request(base + C::ANSWER, bar(C::B_CLC));
+          if (mbar_wait(bar(C::B_CLC), i & 1, wc)) more = clc_answer(base + C::ANSWER, x, y);
+        }
+      }
+    }
+  } else if (warp == kTmaWarp) {
+    // ------------------------------------------------------------ TMA producer
+    // The CTA's items are one sequence of tiles: the last tile's V of an item travels with the first K of the next one.
+    if (lane == 0) {
+      Item im;
+      Lists L;
       Merge mg;
-      mg.start(L);
-      int tile, uses, ntile = 0;
-      bool has = mg.next(L, tile, uses);
+      int item = -1, tile = 0, ntile = 0, uses, left = 0;
+      bool asked = true;
+      const CUtensorMap *map_k = nullptr, *map_v = nullptr;
+      // moves on to the next item that lists a tile; Q is fetched by the caller
+      auto advance = [&](int& t) -> bool {
+        for (;;) {
+          if (!asked) mbar_arrive(bar(C::B_REQ));
+          ++item;
+          if (!take(item, im, left)) return false;
+          mbar_arrive(bar(C::B_IE + item % kItemSlots));
+          asked = false;
+          L = lists(im);
+          mg.start(L);
+          left = mg.left(L);
+          const bool perm = im.cls == RF_TEMPORAL && g.permute, tex = im.cls == RF_TEXTURAL;
+          map_k = &maps.m[perm ? 4 : (tex ? 6 : 1)];
+          map_v = &maps.m[perm ? 5 : (tex ? 7 : 2)];
+          if (mg.next(L, t, uses)) return true;
+        }
+      };
+      auto load_q = [&]() {
+        const CUtensorMap* map_q = &maps.m[im.cls == RF_TEMPORAL && g.permute ? 3 : 0];
+        mbar_expect_tx(bar(C::B_Q), 2 * C::TILE);
+#pragma unroll
+        for (int j = 0; j < 2; ++j)
+#pragma unroll
+          for (int kb = 0; kb < KB; ++kb)
+            tma_load_3d(base + C::Q + j * C::TILE + kb * C::BLK, map_q, kb * C::COL1, (im.qt0 + j) * BM, im.bh, bar(C::B_Q));
+      };
+      bool has = advance(tile);
       if (has) {
+        load_q();
         mbar_expect_tx(bar(C::B_K0), C::TILE);
 #pragma unroll
         for (int kb = 0; kb < KB; ++kb)
-          tma_load_3d(base + C::K0 + kb * C::BLK, map_k, kb * C::COL1, tile * BN, bh, bar(C::B_K0));
+          tma_load_3d(base + C::K0 + kb * C::BLK, map_k, kb * C::COL1, tile * BN, im.bh, bar(C::B_K0));
       }
+      int nq = 1;      // Q tiles loaded
       for (int u = 0; has; ++u) {
-        const bool has_nxt = mg.next(L, ntile, uses);
+        if (!asked && mg.left(L) <= kAskAhead) {
+          mbar_arrive(bar(C::B_REQ));
+          asked = true;
+        }
+        const CUtensorMap* cur_v = map_v;
+        const int cur_bh = im.bh;
+        bool has_nxt = mg.next(L, ntile, uses), new_item = false;
+        if (!has_nxt) has_nxt = new_item = advance(ntile);
         const int ps = u % C::NP, ksn = (u + 1) % C::NK;
         // pair u reuses the V slot of pair u - NP and the K slot that pair filled; the first tile's K slot
         // comes round at u = NK - 1
@@ -226,11 +322,16 @@ __global__ void __launch_bounds__(kThreads, 1) rf_attn_kernel(const __grid_const
         mbar_expect_tx(bar(C::B_F + ps), has_nxt ? 2 * C::TILE : C::TILE);
 #pragma unroll
         for (int kb = 0; kb < KB; ++kb)
-          tma_load_3d(base + C::V0 + ps * C::TILE + kb * C::BLK, map_v, kb * C::COL1, tile * BN, bh, bar(C::B_F + ps));
+          tma_load_3d(base + C::V0 + ps * C::TILE + kb * C::BLK, cur_v, kb * C::COL1, tile * BN, cur_bh, bar(C::B_F + ps));
         if (has_nxt) {
 #pragma unroll
           for (int kb = 0; kb < KB; ++kb)
-            tma_load_3d(base + C::K0 + ksn * C::TILE + kb * C::BLK, map_k, kb * C::COL1, ntile * BN, bh, bar(C::B_F + ps));
+            tma_load_3d(base + C::K0 + ksn * C::TILE + kb * C::BLK, map_k, kb * C::COL1, ntile * BN, im.bh, bar(C::B_F + ps));
+        }
+        if (new_item) {
+          mbar_wait(bar(C::B_QE), (nq - 1) & 1, wc);   // the item before has taken its last scores
+          load_q();
+          ++nq;
         }
         has = has_nxt;
         tile = ntile;
@@ -248,7 +349,9 @@ __global__ void __launch_bounds__(kThreads, 1) rf_attn_kernel(const __grid_const
       const uint32_t q_lo = ((base + C::Q) >> 4) | LO_KMAJOR, k_lo = ((base + C::K0) >> 4) | LO_KMAJOR;
       const uint32_t v_lo = ((base + C::V0) >> 4) | LO_VMAJOR;
       auto issue_s = [&](int j, int ks) {
-        const uint32_t a0 = q_lo + j * (C::TILE >> 4), b0 = k_lo + ks * (C::TILE >> 4);
+        uint32_t a0 = q_lo + j * (C::TILE >> 4);
+        const uint32_t b0 = k_lo + ks * (C::TILE >> 4);
+        asm volatile("" : "+r"(a0));   // the descriptors of Q are added up here, not kept in (spilled) registers
         // the accumulate flag is a compile-time constant: the issuing thread blocks on every MMA, so each
         // instruction between two of them is idle tensor time
         const uint32_t t_d = tmem_base + (j ? C::S_COL1 : C::S_COL0);
@@ -258,32 +361,83 @@ __global__ void __launch_bounds__(kThreads, 1) rf_attn_kernel(const __grid_const
           mma_ss_c<true>(t_d, desc(a0 + (C::koff(k) >> 4)), desc(b0 + (C::koff(k) >> 4)), IDESC_S);
         tc_commit(bar(C::B_SF + j));
       };
-      auto issue_pv = [&](int j, int vs, bool first) {
+      auto issue_pv = [&](int j, int vs, uint32_t acc) {
         const uint32_t b0 = v_lo + vs * (C::TILE >> 4);
         const uint32_t t_p = tmem_base + (j ? C::P_COL1 : C::P_COL0), t_o = tmem_base + (j ? C::O_COL1 : C::O_COL0);
-        mma_ts(t_o, t_p, desc(b0), IDESC_PV, !first);
+        mma_ts(t_o, t_p, desc(b0), IDESC_PV, acc);
 #pragma unroll
         for (int k = 1; k < BN / 16; ++k)
           mma_ts_c<true>(t_o, t_p + k * 8, desc(b0 + k * (2048 >> 4)), IDESC_PV);
         tc_commit(bar(C::B_OF + j));
       };
+      Item im;
+      Lists L;
       Merge mg;
-      mg.start(L);
-      int cur_tile, cur_uses, nxt_tile = 0, nxt_uses = 0;
-      bool has_cur = mg.next(L, cur_tile, cur_uses);
-      int pv_cnt[2] = {0, 0};
-      int s_cnt[2] = {0, 0};   // S_EARLY: S tiles issued per stream
-      mbar_wait(bar(C::B_Q), 0, wc);
+      int item = -1, uses_c = 0, uses_n = 0, tile, left = 0;
+      auto advance = [&](int& uses) -> bool {
+        for (;;) {
+          ++item;
+          if (!take(item, im, left)) return false;
+          mbar_arrive(bar(C::B_IE + item % kItemSlots));
+          L = lists(im);
+          mg.start(L);
+          left = mg.left(L);
+          if (mg.next(L, tile, uses)) return true;
+        }
+      };
+      // one bit per stream
+      uint32_t pv_par = 0;               // parity of the P V bursts issued
+      uint32_t s_par = 3;                // S_EARLY: parity of the S tiles issued, less one
+      uint32_t acc = 0;                  // the stream's next P V adds to O (clear: it opens an item)
+      int nq = 0;                        // Q tiles taken
+      bool has_cur = advance(uses_c);
       if (has_cur) {
+        mbar_wait(bar(C::B_Q), 0, wc);
+        ++nq;
         mbar_wait(bar(C::B_K0), 0, wc);
         tc_fence_after();
-        if (cur_uses & 1) { issue_s(0, 0); ++s_cnt[0]; }
-        if (cur_uses & 2) { issue_s(1, 0); ++s_cnt[1]; }
+        if (uses_c & 1) { issue_s(0, 0); s_par ^= 1; }
+        if (uses_c & 2) { issue_s(1, 0); s_par ^= 2; }
         tc_commit(bar(C::B_K0E));
       }
       for (int u = 0; has_cur; ++u) {
-        const bool has_nxt = mg.next(L, nxt_tile, nxt_uses);
+        bool has_nxt = mg.next(L, tile, uses_n);
         const int vs = u % C::NV, ksn = (u + 1) % C::NK;
+        if (!has_nxt) {
+          // The item's last tile: its scores have all been issued, Q may be overwritten once they are done.  Both P V go
+          // first, then the next item's first scores (its O is not written before the softmax warps have read this
+          // item's: their P of the new item follows their reads).
+          tc_commit(bar(C::B_QE));
+          has_nxt = advance(uses_n);
+          mbar_wait(bar(C::B_F + vs), (u / C::NP) & 1, wc);
+#pragma unroll 1
+          for (int j = 0; j < 2; ++j) {
+            if (uses_c & (1 << j)) {
+              mbar_wait(bar(C::B_PF + j), (pv_par >> j) & 1, wc);
+              tc_fence_after();
+              issue_pv(j, vs, (acc >> j) & 1);
+              pv_par ^= 1u << j;
+            }
+          }
+          acc = 0;
+          if (has_nxt) {
+            mbar_wait(bar(C::B_Q), nq & 1, wc);
+            ++nq;
+#pragma unroll 1
+            for (int j = 0; j < 2; ++j) {
+              if (uses_n & (1 << j)) {
+                if (C::S_EARLY) mbar_wait(bar(C::B_SE + j), (s_par >> j) & 1, wc);
+                tc_fence_after();
+                issue_s(j, ksn);
+                s_par ^= 1u << j;
+              }
+            }
+          }
+          tc_commit(bar(C::B_E + vs));
+          has_cur = has_nxt;
+          uses_c = uses_n;
+          continue;
+        }
         // the TMA barrier first (V of this tile and K of the next): the data has normally landed long ago, and
         // checking here keeps it out of the gap between a stream's P arriving and its MMAs being issued
         mbar_wait(bar(C::B_F + vs), (u / C::NP) & 1, wc);
@@ -294,35 +448,36 @@ __global__ void __launch_bounds__(kThreads, 1) rf_attn_kernel(const __grid_const
           // instead of sitting in their exponentials at the same time.
 #pragma unroll
           for (int j = 0; j < 2; ++j) {
-            if (has_nxt && (nxt_uses & (1 << j))) {
-              mbar_wait(bar(C::B_SE + j), (s_cnt[j] - 1) & 1, wc);
+            if (uses_n & (1 << j)) {
+              mbar_wait(bar(C::B_SE + j), (s_par >> j) & 1, wc);
               tc_fence_after();
               issue_s(j, ksn);
-              ++s_cnt[j];
+              s_par ^= 1u << j;
             }
-            if (cur_uses & (1 << j)) {
-              mbar_wait(bar(C::B_PF + j), pv_cnt[j] & 1, wc);
+            if (uses_c & (1 << j)) {
+              mbar_wait(bar(C::B_PF + j), (pv_par >> j) & 1, wc);
               tc_fence_after();
-              issue_pv(j, vs, pv_cnt[j] == 0);
-              ++pv_cnt[j];
+              issue_pv(j, vs, (acc >> j) & 1);
+              acc |= 1u << j;
+              pv_par ^= 1u << j;
             }
           }
         } else {
 #pragma unroll
           for (int j = 0; j < 2; ++j) {
-            if (cur_uses & (1 << j)) {
-              mbar_wait(bar(C::B_PF + j), pv_cnt[j] & 1, wc);
+            if (uses_c & (1 << j)) {
+              mbar_wait(bar(C::B_PF + j), (pv_par >> j) & 1, wc);
               tc_fence_after();
-              issue_pv(j, vs, pv_cnt[j] == 0);
-              ++pv_cnt[j];
+              issue_pv(j, vs, (acc >> j) & 1);
+              acc |= 1u << j;
+              pv_par ^= 1u << j;
             }
-            if (has_nxt && (nxt_uses & (1 << j))) issue_s(j, ksn);
+            if (uses_n & (1 << j)) issue_s(j, ksn);
           }
         }
         tc_commit(bar(C::B_E + vs));
         has_cur = has_nxt;
-        cur_tile = nxt_tile;
-        cur_uses = nxt_uses;
+        uses_c = uses_n;
       }
     }
   }
@@ -331,20 +486,29 @@ __global__ void __launch_bounds__(kThreads, 1) rf_attn_kernel(const __grid_const
     // ------------------------------------------------------------ softmax + epilogue, one thread per query row
     const int j = warp >> 2;                       // stream
     const int row_in_tile = tid & 127;
-    const int r = (qt0 + j) * BM + row_in_tile;    // query slot in the head's coordinate space
-    const int n = j == 0 ? L.n0 : L.n1;
     const uint32_t lane_sel = (uint32_t)((warp & 3) * 32) << 16;
     const uint32_t t_s = tmem_base + lane_sel + (j ? C::S_COL1 : C::S_COL0);
     const uint32_t t_o = tmem_base + lane_sel + (j ? C::O_COL1 : C::O_COL0);
-    const RowMask rmask = make_row_mask(g, cls, min(r, g.N - 1));
     const float sc = a.scale_log2;
+    uint4* keep = reinterpret_cast<uint4*>(base_ptr + C::KEEP) + tid;   // this row's keep words of a PARTIAL tile
+    uint32_t done = 0;         // tiles of this stream in the items before: the barriers' phases run on
+    Item im;
+    im.n0 = im.n1 = 0;
+    // (a warp leaves as a whole: after an abandoned wait its lanes may differ in what they saw)
+    for (int item = 0; __all_sync(0xffffffffu, take(item, im, im.n0 + im.n1)); ++item) {
+    if (lane == 0) mbar_arrive(bar(C::B_IE + item % kItemSlots));
+    const int bh = im.bh, cls = im.cls;
+    const int r = (im.qt0 + j) * BM + row_in_tile;    // query slot in the head's coordinate space
+    const int n = j == 0 ? im.n0 : im.n1;
+    const int32_t* list = a.head_class != nullptr ? a.kv_tile + ((size_t)bh * g.nQ + min(im.qt0 + j, g.nQ - 1)) * g.nKmax : nullptr;
+    const bool perm = cls == RF_TEMPORAL && g.permute;
+    const RowMask rmask = make_row_mask(g, cls, im.window, min(r, g.N - 1));
     float m_run = -INFINITY;   // running maximum, log2 domain (score * sc)
     float l_run = 0.f;         // sum of the weights as rounded to bf16, the ones P V multiplies: normalises O
     float l_exact = 0.f;       // sum of the unrounded weights: the log-sum-exp (LSE only)
-    uint4* keep = reinterpret_cast<uint4*>(base_ptr + C::KEEP) + tid;   // this row's keep words of a PARTIAL tile
 
     for (int it = 0; it < n; ++it) {
-      const uint32_t entry = L.entry(j, it);
+      const uint32_t entry = list != nullptr ? (uint32_t)list[it] : dense_entry(it, g.N);
       // The keep words of a PARTIAL tile do not depend on its scores: they are worked out before the wait for the
       // scores, where a stream spends a third of its time anyway, and wait in shared memory (four registers live
       // through the exponentials cost every tile 3 %).
@@ -355,7 +519,7 @@ __global__ void __launch_bounds__(kThreads, 1) rf_attn_kernel(const __grid_const
         partial = __any_sync(0xffffffffu, (w[0] & w[1] & w[2] & w[3]) != 0xffffffffu);   // a warp's rows may keep it whole
         *keep = make_uint4(w[0], w[1], w[2], w[3]);
       }
-      mbar_wait(bar(C::B_SF + j), it & 1, wc);
+      mbar_wait(bar(C::B_SF + j), (done + it) & 1, wc);
       tc_fence_after();
       uint32_t s[128];
       {
@@ -406,7 +570,7 @@ __global__ void __launch_bounds__(kThreads, 1) rf_attn_kernel(const __grid_const
         // one tile ahead of the MMA warp, which tracks the P barrier by phase parity.
         bool o_landed = it == 0;
         if (it > 0 && any_raise) {
-          mbar_wait(bar(C::B_OF + j), (it - 1) & 1, wc);
+          mbar_wait(bar(C::B_OF + j), (done + it - 1) & 1, wc);
           o_landed = true;
           rescale_o<D>(t_o, alpha);
         }
@@ -427,7 +591,7 @@ __global__ void __launch_bounds__(kThreads, 1) rf_attn_kernel(const __grid_const
         }
         if (LSE) l_exact += la.x + la.y;
         l_run += lb.x + lb.y;
-        if (!o_landed) mbar_wait(bar(C::B_OF + j), (it - 1) & 1, wc);
+        if (!o_landed) mbar_wait(bar(C::B_OF + j), (done + it - 1) & 1, wc);
         {
           const uint32_t t_p = tmem_base + lane_sel + (j ? C::P_COL1 : C::P_COL0);
           uint32_t(&p0)[32] = *reinterpret_cast<uint32_t(*)[32]>(&pk[0]);
@@ -466,7 +630,7 @@ __global__ void __launch_bounds__(kThreads, 1) rf_attn_kernel(const __grid_const
         }
         if (it > 0) {
           // O of the previous tiles must be complete before it is rescaled
-          mbar_wait(bar(C::B_OF + j), (it - 1) & 1, wc);
+          mbar_wait(bar(C::B_OF + j), (done + it - 1) & 1, wc);
           rescale_o<D>(t_o, alpha);
         }
         m_use = m_run == -INFINITY ? 0.f : m_run;
@@ -494,7 +658,7 @@ __global__ void __launch_bounds__(kThreads, 1) rf_attn_kernel(const __grid_const
     }
 
     if (n > 0) {
-      mbar_wait(bar(C::B_OF + j), (n - 1) & 1, wc);
+      mbar_wait(bar(C::B_OF + j), (done + n - 1) & 1, wc);
       tc_fence_after();
       int tok = r;
       if (perm && r < g.Nv) tok = (r % g.T) * g.S + r / g.T;
@@ -520,6 +684,9 @@ __global__ void __launch_bounds__(kThreads, 1) rf_attn_kernel(const __grid_const
         }
       }
       if (LSE && r < g.N && rf_in_bounds(tok, g.N, a.dev_status)) a.lse[(size_t)bh * g.N + tok] = (m_run + log2f(l_exact)) * 0.6931471805599453f;
+      tc_fence_before();   // O has been read: the next P hand-over lets it be overwritten
+      done += n;
+    }
     }
   }
 
@@ -533,7 +700,7 @@ __global__ void __launch_bounds__(kThreads, 1) rf_attn_kernel(const __grid_const
 }
 
 template <int D, bool LSE>
-rf_status launch(const RfAttnArgs& a, const CUtensorMap* maps, cudaStream_t st) {
+rf_status launch(RfAttnArgs a, const CUtensorMap* maps, cudaStream_t st) {
   static bool configured[64] = {};
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return RF_ERR_CUDA;
@@ -545,7 +712,9 @@ rf_status launch(const RfAttnArgs& a, const CUtensorMap* maps, cudaStream_t st) 
   }
   Maps m;
   for (int i = 0; i < 8; ++i) m.m[i] = maps[i];
-  dim3 grid(rf_cdiv(a.g.nQ, 2), a.g.B * a.g.H);
+  const size_t kv_bytes = (size_t)a.g.N * D * 2 * sizeof(__nv_bfloat16);
+  a.heads_l2 = (int)std::min<size_t>(std::max<size_t>(kL2Bytes / kv_bytes, 1), (size_t)a.g.B * a.g.H);
+  dim3 grid(rf_cdiv(a.g.nQ, 2), a.g.B * a.g.H);   // one CTA an item; running CTAs take over what has not started
   rf_attn_kernel<D, LSE><<<grid, kThreads, Cfg<D>::ALLOC, st>>>(m, a);
   return cudaGetLastError() == cudaSuccess ? RF_OK : RF_ERR_CUDA;
 }

@@ -87,21 +87,24 @@ struct RowMask {
   }
 };
 
-__device__ __forceinline__ RowMask make_row_mask(const RfGeom& g, int cls, int r) {
+__device__ __forceinline__ RowMask make_row_mask(const RfGeom& g, int cls, int window, int r) {
+  // dynamic bandwidth: the head's own window; past the extent the mask is the same, and nothing overflows
+  const int wf = cls == RF_SPATIAL && window >= 0 ? min(window, g.T) : g.wf;
+  const int ws = cls == RF_TEMPORAL && window >= 0 ? min(window, g.S) : g.ws;
   RowMask m;
   m.lkv = rf_kv_len(g, cls);
   m.text0 = m.lkv;
   m.lo = 0;
   m.hi = m.lkv;
   m.first_end = 0;
-  m.p = 0; m.ws = g.ws; m.S = g.S; m.T = g.T;
+  m.p = 0; m.ws = ws; m.S = g.S; m.T = g.T;
   m.mode = RowMask::kRange;
   if ((cls == RF_SPATIAL || cls == RF_TEMPORAL) && r < g.Nv) {
     m.text0 = g.Nv;
     if (cls == RF_SPATIAL) {
       const int f = r / g.S;
-      m.lo = max(0, f - g.wf) * g.S;
-      m.hi = min(g.T, f + g.wf + 1) * g.S;
+      m.lo = max(0, f - wf) * g.S;
+      m.hi = min(g.T, f + wf + 1) * g.S;
       m.first_end = g.key_first ? g.S : 0;
     } else if (g.t2d) {
       m.mode = RowMask::kWindow2d;
@@ -110,8 +113,8 @@ __device__ __forceinline__ RowMask make_row_mask(const RfGeom& g, int cls, int r
       m.ws = g.permute;
     } else if (g.permute) {
       const int p = r / g.T;
-      m.lo = max(0, p - g.ws) * g.T;
-      m.hi = min(g.S, p + g.ws + 1) * g.T;
+      m.lo = max(0, p - ws) * g.T;
+      m.hi = min(g.S, p + ws + 1) * g.T;
     } else {
       m.mode = RowMask::kPeriodic;
       m.p = r % g.S;
@@ -119,6 +122,9 @@ __device__ __forceinline__ RowMask make_row_mask(const RfGeom& g, int cls, int r
   }
   return m;
 }
+
+// Entry i of the implicit list of a dense head: every tile, the last one PARTIAL where it reaches past the keys.
+__device__ __forceinline__ uint32_t dense_entry(int i, int lkv) { return (uint32_t)i | ((i + 1) * BN > lkv ? RF_PARTIAL_BIT : 0u); }
 
 // The two streams' ascending tile lists and their merge (the order K/V tiles are fetched in).
 struct Lists {
@@ -129,16 +135,18 @@ struct Lists {
   bool listed;
   __device__ __forceinline__ uint32_t entry(int j, int i) const {
     if (listed) return (uint32_t)(j == 0 ? l0[i] : l1[i]);
-    const bool tail = (i + 1) * BN > lkv;
-    return (uint32_t)i | (tail ? RF_PARTIAL_BIT : 0u);
+    return dense_entry(i, lkv);
   }
 };
 struct Merge {
   int i0 = 0, i1 = 0;
+  // tiles the union has left at most
+  __device__ __forceinline__ int left(const Lists& L) const { return max(L.n0 - i0, L.n1 - i1); }
   // Raw list entries at i0 / i1, loaded by the previous call and not touched until the next one, so
   // that the load latency never sits between two MMA bursts of the (in-order) issuing thread.
   uint32_t raw0 = 0, raw1 = 0;
   __device__ __forceinline__ void start(const Lists& L) {
+    i0 = i1 = 0;
     if (L.n0 > 0) raw0 = L.entry(0, 0);
     if (L.n1 > 0) raw1 = L.entry(1, 0);
   }

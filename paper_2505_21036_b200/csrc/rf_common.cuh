@@ -86,6 +86,7 @@ struct RfAttnArgs {
   float* lse;
   int32_t* dev_status;
   float scale_log2;           // log2(e) / sqrt(D)
+  int heads_l2 = 1;           // heads whose items are interleaved (filled by the launcher)
 };
 // Tensor maps: [0..2] Q/K/V in original order, [3..5] the workspace copies with N rows per head
 // (position-major Q/K/V of Temporal heads), [6..7] workspace K/V with LkvTex rows per head (Textural).

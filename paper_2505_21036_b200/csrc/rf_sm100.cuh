@@ -63,6 +63,44 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, const W
   return false;
 }
 
+// The same for waits that may rightly last as long as `tiles` key tiles take (a role that idles while the others work an
+// item off): 2 s plus 0.2 ms per tile.
+__device__ __forceinline__ bool mbar_wait_long(uint32_t bar, uint32_t parity, const WaitCtx& w, int tiles) {
+  if (mbar_try(bar, parity)) return true;
+  const uint64_t t0 = global_timer_ns(), limit = w.limit_ns + (uint64_t)tiles * 200000ull, most = (1ull << 26) + ((uint64_t)tiles << 13);
+  for (uint64_t it = 0; it < most; ++it) {
+    if (mbar_try(bar, parity)) return true;
+    if (*w.abort_flag) return false;
+    if (global_timer_ns() - t0 > limit) break;
+  }
+  *w.abort_flag = 1;
+  rf_report(w.dev_status, RF_ERR_TIMEOUT);
+  return false;
+}
+
+// ---------------------------------------------------------------- cluster launch control
+// A running CTA takes over the work of one that has not started yet: the request cancels the launch of some later CTA of
+// the grid and its index arrives in shared memory (16 bytes, counted on the barrier).  After a request that found none
+// no further one may be made.
+__device__ __forceinline__ void clc_request(uint32_t response, uint32_t bar) {
+  asm volatile("clusterlaunchcontrol.try_cancel.async.shared::cta.mbarrier::complete_tx::bytes.b128 [%0], [%1];" ::"r"(response), "r"(bar)
+               : "memory");
+}
+__device__ __forceinline__ bool clc_answer(uint32_t response, uint32_t& x, uint32_t& y) {
+  uint32_t ok;
+  x = y = 0;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t.reg .b128 r;\n\t"
+      "ld.shared.b128 r, [%3];\n\t"
+      "clusterlaunchcontrol.query_cancel.is_canceled.pred.b128 p, r;\n\t"
+      "selp.u32 %2, 1, 0, p;\n\t"
+      "@p clusterlaunchcontrol.query_cancel.get_first_ctaid.v4.b32.b128 {%0, %1, _, _}, r;\n\t}"
+      : "+r"(x), "+r"(y), "=r"(ok)
+      : "r"(response)
+      : "memory");
+  return ok != 0;
+}
+
 // ---------------------------------------------------------------- register budget of warp-specialised CTAs
 // The attention and ARM kernels run 384 threads: two softmax warpgroups that raise their register count with
 // setmaxnreg.inc and one warpgroup (TMA, MMA, two filler warps) that lowers its own first.  setmaxnreg.inc waits,
@@ -83,6 +121,13 @@ inline bool rf_regs_ok(K kernel) {
   cudaFuncAttributes fa;
   if (cudaFuncGetAttributes(&fa, kernel) != cudaSuccess) return false;
   return fa.numRegs * kWsThreads >= kWsRegsNeeded;
+}
+
+// True in one lane of a converged warp.  (Unlike `lane == 0` this tells the compiler that a single thread runs the branch.)
+__device__ __forceinline__ bool elect_one() {
+  uint32_t ok;
+  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(ok));
+  return ok != 0;
 }
 
 // ---------------------------------------------------------------- TMA
