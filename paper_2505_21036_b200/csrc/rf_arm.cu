@@ -135,6 +135,13 @@ __global__ void __launch_bounds__(ARM_THREADS, 1) rf_arm_kernel(const __grid_con
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
   const WaitCtx wc{abort_flag, arm_flag};
+  rf_grid_trigger();
+  rf_grid_wait();
+#ifndef RF_BOUNDS_CHECK
+  // The call's failure flag is cleared here and not by a launch of its own: the first wait that can raise it runs out
+  // two seconds from now.  (The bounds-checking build, whose reports come at once, clears it before the launch.)
+  if (blockIdx.x == 0 && blockIdx.y == 0 && tid == 0) *arm_flag = 0;
+#endif
 
   if (warp >= 8) {
     RF_SETMAXNREG_DEC();
@@ -380,6 +387,8 @@ __global__ void __launch_bounds__(256) rf_arm_decide_kernel(int nb, int nb_user,
                                                              float* __restrict__ recall_plus,
                                                              const int32_t* __restrict__ arm_flag, int32_t* dev_status) {
   __shared__ double red[2 * ARM_MAX_NB + 1][256];
+  rf_grid_trigger();
+  rf_grid_wait();
   const int bh = blockIdx.x, tid = threadIdx.x;
   const int nm = 2 * nb + 1;
   const int failed = *arm_flag;
@@ -443,7 +452,10 @@ __global__ void __launch_bounds__(256) rf_arm_decide_kernel(int nb, int nb_user,
 }
 
 // Self-test only: stands in for a score kernel whose wait ran out.
-__global__ void rf_arm_set_flag_kernel(int32_t* arm_flag, int code) { *arm_flag = code; }
+__global__ void rf_arm_set_flag_kernel(int32_t* arm_flag, int code) {
+  rf_grid_wait();
+  *arm_flag = code;
+}
 
 template <int D, int NB, bool TEX>
 cudaError_t launch_arm_t(const ArmMaps& maps, const RfGeom& g, const ArmSample& s0, const ArmSample& s1,
@@ -460,8 +472,7 @@ cudaError_t launch_arm_t(const ArmMaps& maps, const RfGeom& g, const ArmSample& 
   }
   dim3 grid(s0.pairs + s1.pairs, g.B * g.H);
   const float scale_log2 = 1.4426950408889634f / sqrtf((float)D);
-  rf_arm_kernel<D, NB, TEX><<<grid, ARM_THREADS, ArmCfg<D>::ALLOC, st>>>(maps, g, s0, s1, win, n_pad, scale_log2, arm_flag);
-  return cudaGetLastError();
+  return rf_launch(rf_arm_kernel<D, NB, TEX>, grid, ARM_THREADS, ArmCfg<D>::ALLOC, st, maps, g, s0, s1, win, n_pad, scale_log2, arm_flag);
 }
 
 template <int D>
@@ -517,11 +528,13 @@ cudaError_t rf_launch_arm(const RfGeom& g, int sample_mode, int omega, float alp
   s0.want_t = alg1 ? 0 : 1; s0.want_s = 1; s0.out = rows_glb;
   s1.n = n_loc; s1.stride = 1; s1.pairs = alg1 ? rf_cdiv(rf_cdiv(n_loc, ARM_TILE), 2) : 0;
   s1.want_t = 1; s1.want_s = 0; s1.out = rows_loc;
-  cudaError_t e = cudaMemsetAsync(arm_flag, 0, sizeof(int32_t), st);
+  cudaError_t e = cudaSuccess;
+#ifdef RF_BOUNDS_CHECK
+  e = cudaMemsetAsync(arm_flag, 0, sizeof(int32_t), st);
   if (e != cudaSuccess) return e;
+#endif
   if (selftest_abandon) {
-    rf_arm_set_flag_kernel<<<1, 1, 0, st>>>(arm_flag, RF_ERR_TIMEOUT);
-    e = cudaGetLastError();
+    e = rf_launch(rf_arm_set_flag_kernel, dim3(1), 1, 0, st, arm_flag, (int)RF_ERR_TIMEOUT);
   } else
   switch (g.D) {
     case 64: e = launch_arm_n<64>(plus, tex, maps, g, s0, s1, win, n_pad, arm_flag, st); break;
@@ -530,9 +543,8 @@ cudaError_t rf_launch_arm(const RfGeom& g, int sample_mode, int omega, float alp
     default: e = cudaErrorInvalidValue;
   }
   if (e != cudaSuccess) return e;
-  rf_arm_decide_kernel<<<heads, 256, 0, st>>>(NB, nb, n_loc, n_glb, n_pad, sample_mode, alpha, g.two_mask, win, tex ? 1 : 0, rows_loc,
-                                              rows_glb, head_class, head_window, recall, recall_plus, arm_flag, dev_status);
-  return cudaGetLastError();
+  return rf_launch(rf_arm_decide_kernel, dim3(heads), 256, 0, st, NB, nb, n_loc, n_glb, n_pad, sample_mode, alpha, g.two_mask, win,
+                   tex ? 1 : 0, rows_loc, rows_glb, head_class, head_window, recall, recall_plus, arm_flag, dev_status);
 }
 
 // ------------------------------------------------------------------------------------------------

@@ -191,6 +191,7 @@ __global__ void __launch_bounds__(kThreads, 1) rf_attn_kernel(const __grid_const
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
   const WaitCtx wc{abort_flag, a.dev_status};
+  rf_grid_wait();
 
   // The i-th item of this CTA.  False: there is none (or a wait was abandoned).
   auto take = [&](int i, Item& im, int waited) -> bool {
@@ -258,6 +259,7 @@ __global__ void __launch_bounds__(kThreads, 1) rf_attn_kernel(const __grid_const
           clc_request(base + C::ANSWER, bar(C::B_CLC));
           if (mbar_wait(bar(C::B_CLC), i & 1, wc)) more = clc_answer(base + C::ANSWER, x, y);
         }
+        if (!more) rf_grid_trigger();
       }
     }
   } else if (warp == kTmaWarp) {
@@ -715,8 +717,7 @@ rf_status launch(RfAttnArgs a, const CUtensorMap* maps, cudaStream_t st) {
   const size_t kv_bytes = (size_t)a.g.N * D * 2 * sizeof(__nv_bfloat16);
   a.heads_l2 = (int)std::min<size_t>(std::max<size_t>(kL2Bytes / kv_bytes, 1), (size_t)a.g.B * a.g.H);
   dim3 grid(rf_cdiv(a.g.nQ, 2), a.g.B * a.g.H);   // one CTA an item; running CTAs take over what has not started
-  rf_attn_kernel<D, LSE><<<grid, kThreads, Cfg<D>::ALLOC, st>>>(m, a);
-  return cudaGetLastError() == cudaSuccess ? RF_OK : RF_ERR_CUDA;
+  return rf_launch(rf_attn_kernel<D, LSE>, grid, kThreads, Cfg<D>::ALLOC, st, m, a) == cudaSuccess ? RF_OK : RF_ERR_CUDA;
 }
 template <int D>
 rf_status launch(const RfAttnArgs& a, const CUtensorMap* maps, cudaStream_t st) {

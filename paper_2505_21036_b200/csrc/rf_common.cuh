@@ -49,6 +49,27 @@ __host__ __device__ __forceinline__ int rf_kv_len(const RfGeom& g, int cls) {
   return cls == RF_TEXTURAL ? g.LkvTex : g.N;
 }
 
+// Programmatic dependent launch.  Every kernel of the path is launched so that its CTAs may become resident, and set up
+// what depends on no global memory, while the kernel before it in the stream drains; rf_grid_wait then waits until all of
+// that kernel's writes are visible.  All threads of a kernel call it before their first access to global memory.
+// rf_grid_trigger lets the next kernel's CTAs come in as soon as every CTA of this one has called it or ended.
+__device__ __forceinline__ void rf_grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void rf_grid_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+template <typename... P, typename... A>
+inline cudaError_t rf_launch(void (*kernel)(P...), dim3 grid, unsigned block, size_t smem, cudaStream_t st, const A&... args) {
+  cudaLaunchConfig_t c = {};
+  c.gridDim = grid;
+  c.blockDim = dim3(block);
+  c.dynamicSmemBytes = smem;
+  c.stream = st;
+  cudaLaunchAttribute at;
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  c.attrs = &at;
+  c.numAttrs = 1;
+  return cudaLaunchKernelEx(&c, kernel, static_cast<P>(args)...);
+}
+
 // Launchers implemented in the .cu files (host).
 // head_window (nullable): per-head window replacing g.wf (Spatial heads) / g.ws (Temporal heads)
 cudaError_t rf_launch_build_tiles(const RfGeom& g, const int32_t* head_class, const int32_t* head_window, int32_t* count,
