@@ -32,7 +32,8 @@ using namespace rf_attn;
 
 constexpr int kThreads = kWsThreads;        // 3 warpgroups: softmax 0, softmax 1, {TMA, MMA, 2 idle warps}
 constexpr int kTmaWarp = 8, kMmaWarp = 9, kItemWarp = 10;
-constexpr int kItemSlots = 2, kItemWords = 8, kItemReaders = 10;   // readers: eight softmax warps, the TMA and the MMA thread
+constexpr int kItemSlots = 2, kItemWords = 8, kItemReaders = 9;   // readers: eight softmax warps and the TMA thread
+constexpr uint32_t kMore = 4, kLast = 8;   // of a tile record, see the TMA producer
 constexpr int kAskAhead = 4;   // tiles an item has left when the next one is asked for: about 8 us, an answer takes about one
 // What bounds the loop: a stream is the chain scores -> softmax -> P V -> Q K^T, so what counts is how few dependent
 // operations stand between the scores' arrival and the hand-over of P.  At D = 96 / 128 the first kSpec weights are taken
@@ -91,7 +92,8 @@ struct Cfg {
   static constexpr uint32_t KEEP = MISC + 64;         // 128-bit keep word per softmax thread
   static constexpr uint32_t ITEM = KEEP + 256 * 16;   // kItemSlots items of kItemWords words, then the launch-control answer
   static constexpr uint32_t ANSWER = ITEM + kItemSlots * kItemWords * 4;
-  static constexpr uint32_t TOTAL = ANSWER + 16;
+  static constexpr uint32_t RECORD = ANSWER + 16;     // tile records: one per ring slot, then the first tile's
+  static constexpr uint32_t TOTAL = RECORD + 4 * (NP + 1);
   static constexpr uint32_t ALLOC = TOTAL + 1024;     // slack for manual 1024-byte alignment
   // TMEM columns
   static constexpr uint32_t S_COL0 = 0, S_COL1 = 128, O_COL0 = 256, O_COL1 = S_EARLY ? 320 : 384, TMEM_COLS = 512;
@@ -113,6 +115,37 @@ __device__ __forceinline__ void place_item(uint64_t lin, int group, int heads, i
   pair = pairs - 1 - (int)(r / in);
 }
 
+// 32 bf16 columns of an output row.
+__device__ __forceinline__ void store_columns(uint4* dst, const uint32_t* v, bool o32) {
+  if (o32) {
+    st_global_v8(dst, v);
+    st_global_v8(dst + 2, v + 8);
+  } else {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) dst[i] = make_uint4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
+  }
+}
+
+// Where this thread's row of an item goes.
+struct Row {
+  uint4* o;
+  size_t at;       // row of [B*H][N]
+  bool inside;     // false: past the sequence
+  bool o32;        // a thread writes its row alone, so a warp's store touches 32 rows: whole 32-byte sectors where O allows it
+};
+__device__ __forceinline__ Row output_row(const RfAttnArgs& a, const int* iw, int j, int row_in_tile) {
+  const RfGeom& g = a.g;
+  const int r = (iw[1] + j) * BM + row_in_tile;
+  int tok = r;
+  if (iw[2] == RF_TEMPORAL && g.permute && r < g.Nv) tok = (r % g.T) * g.S + r / g.T;
+  Row row;
+  row.inside = r < g.N && rf_in_bounds(tok, g.N, a.dev_status);
+  row.at = (size_t)iw[0] * g.N + min(tok, g.N - 1);
+  row.o = reinterpret_cast<uint4*>(a.o + row.at * g.D);
+  row.o32 = (reinterpret_cast<uintptr_t>(a.o) & 31u) == 0;
+  return row;
+}
+
 // This thread's row of O times alpha (warp-collective).
 template <int D>
 __device__ __forceinline__ void rescale_o(uint32_t t_o, float alpha) {
@@ -128,6 +161,22 @@ __device__ __forceinline__ void rescale_o(uint32_t t_o, float alpha) {
   }
   tc_wait_st();
   tc_fence_before();
+}
+
+// This thread's row of scores, and the masked ones of a PARTIAL tile set to -inf.
+__device__ __forceinline__ void load_scores(uint32_t t_s, uint32_t (&s)[BN]) {
+  tmem_ld32(t_s, *reinterpret_cast<uint32_t(*)[32]>(&s[0]));
+  tmem_ld32(t_s + 32, *reinterpret_cast<uint32_t(*)[32]>(&s[32]));
+  tmem_ld32(t_s + 64, *reinterpret_cast<uint32_t(*)[32]>(&s[64]));
+  tmem_ld32(t_s + 96, *reinterpret_cast<uint32_t(*)[32]>(&s[96]));
+  tc_wait_ld();
+}
+__device__ __forceinline__ void mask_scores(const uint4* keep, uint32_t (&s)[BN]) {
+  const uint4 kw = *keep;
+  const uint32_t w[4] = {kw.x, kw.y, kw.z, kw.w};
+#pragma unroll
+  for (int c = 0; c < BN; ++c)
+    if (!((w[c >> 5] >> (c & 31)) & 1u)) s[c] = 0xff800000u;  // -inf
 }
 
 // Weights of the key columns [C0, C1) of a tile: 2^(score * sc - m), packed to bf16; with LSE also their sum before rounding.
@@ -146,7 +195,7 @@ __device__ __forceinline__ void take_weights(const uint32_t (&s)[BN], uint32_t (
 }
 
 template <int D, bool LSE>
-__global__ void __launch_bounds__(kThreads, 1) rf_attn_kernel(const __grid_constant__ Maps maps, const RfAttnArgs a) {
+__global__ void __launch_bounds__(kThreads, 1) rf_attn_kernel(const __grid_constant__ Maps maps, const __grid_constant__ RfAttnArgs a) {
   using C = Cfg<D>;
   constexpr int KB = C::KB;
   constexpr uint32_t IDESC_S = idesc_bf16(BM, BN, 0);
@@ -162,6 +211,7 @@ __global__ void __launch_bounds__(kThreads, 1) rf_attn_kernel(const __grid_const
   const RfGeom& g = a.g;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   int* items = reinterpret_cast<int*>(base_ptr + C::ITEM);
+  volatile uint32_t* records = reinterpret_cast<volatile uint32_t*>(base_ptr + C::RECORD);
 
   if (tid == 0) {
     mbar_init(bar(C::B_Q), 1);
@@ -299,6 +349,11 @@ __global__ void __launch_bounds__(kThreads, 1) rf_attn_kernel(const __grid_const
             tma_load_3d(base + C::Q + j * C::TILE + kb * C::BLK, map_q, kb * C::COL1, (im.qt0 + j) * BM, im.bh, bar(C::B_Q));
       };
       bool has = advance(tile);
+      // A tile's record: which streams list it, whether it ends its item; 0 ends the sequence.  It is published with the
+      // barrier its K is counted on, so the MMA thread walks no lists.
+      auto record = [&](bool any) -> uint32_t { return any ? uses | kMore | (mg.left(L) == 0 ? kLast : 0u) : 0u; };
+      records[C::NP] = record(has);
+      if (!has) mbar_arrive(bar(C::B_K0));
       if (has) {
         load_q();
         mbar_expect_tx(bar(C::B_K0), C::TILE);
@@ -321,6 +376,7 @@ __global__ void __launch_bounds__(kThreads, 1) rf_attn_kernel(const __grid_const
         // comes round at u = NK - 1
         if (u >= C::NP) mbar_wait(bar(C::B_E + ps), ((u / C::NP) - 1) & 1, wc);
         else if (has_nxt && ksn == 0) mbar_wait(bar(C::B_K0E), 0, wc);
+        records[ps] = record(has_nxt);
         mbar_expect_tx(bar(C::B_F + ps), has_nxt ? 2 * C::TILE : C::TILE);
 #pragma unroll
         for (int kb = 0; kb < KB; ++kb)
@@ -341,7 +397,11 @@ __global__ void __launch_bounds__(kThreads, 1) rf_attn_kernel(const __grid_const
     }
   } else if (warp == kMmaWarp) {
     // ------------------------------------------------------------ MMA issuer
-    if (lane == 0) {
+    // elect.sync tells the compiler that one thread issues, which shortens what stands between two instructions: D = 96 /
+    // 128 2 to 3 % faster (24 heads, 32 896 tokens, dense 11.92 -> 11.69 and 10.81 -> 10.54 ms).  At D = 64, where the
+    // streams' distance from one another counts for more, the plain branch is the faster one (dense, 48 heads, 17 776
+    // tokens: 5.09 against 5.44 ms).
+    if (C::S_EARLY ? lane == 0 : elect_one()) {
       // Descriptors differ only in their 14-bit start-address field: keep the constant words in
       // registers and add the byte offset (>> 4) per k-step.
       constexpr uint32_t DESC_HI = (1024u >> 4) | (1u << 14) | (2u << 29);      // SBO 1024 B, version 1, 128B swizzle
@@ -372,49 +432,33 @@ __global__ void __launch_bounds__(kThreads, 1) rf_attn_kernel(const __grid_const
           mma_ts_c<true>(t_o, t_p + k * 8, desc(b0 + k * (2048 >> 4)), IDESC_PV);
         tc_commit(bar(C::B_OF + j));
       };
-      Item im;
-      Lists L;
-      Merge mg;
-      int item = -1, uses_c = 0, uses_n = 0, tile, left = 0;
-      auto advance = [&](int& uses) -> bool {
-        for (;;) {
-          ++item;
-          if (!take(item, im, left)) return false;
-          mbar_arrive(bar(C::B_IE + item % kItemSlots));
-          L = lists(im);
-          mg.start(L);
-          left = mg.left(L);
-          if (mg.next(L, tile, uses)) return true;
-        }
-      };
       // one bit per stream
       uint32_t pv_par = 0;               // parity of the P V bursts issued
       uint32_t s_par = 3;                // S_EARLY: parity of the S tiles issued, less one
       uint32_t acc = 0;                  // the stream's next P V adds to O (clear: it opens an item)
-      int nq = 0;                        // Q tiles taken
-      bool has_cur = advance(uses_c);
-      if (has_cur) {
+      uint32_t cur = 0, nq = 0;          // the current tile's record; Q tiles taken
+      if (mbar_wait(bar(C::B_K0), 0, wc)) cur = records[C::NP];
+      if (cur & kMore) {
         mbar_wait(bar(C::B_Q), 0, wc);
         ++nq;
-        mbar_wait(bar(C::B_K0), 0, wc);
         tc_fence_after();
-        if (uses_c & 1) { issue_s(0, 0); s_par ^= 1; }
-        if (uses_c & 2) { issue_s(1, 0); s_par ^= 2; }
+        if (cur & 1) { issue_s(0, 0); s_par ^= 1; }
+        if (cur & 2) { issue_s(1, 0); s_par ^= 2; }
         tc_commit(bar(C::B_K0E));
+        if (cur & kLast) tc_commit(bar(C::B_QE));
       }
-      for (int u = 0; has_cur; ++u) {
-        bool has_nxt = mg.next(L, tile, uses_n);
+      for (int u = 0; cur & kMore; ++u) {
         const int vs = u % C::NV, ksn = (u + 1) % C::NK;
-        if (!has_nxt) {
-          // The item's last tile: its scores have all been issued, Q may be overwritten once they are done.  Both P V go
-          // first, then the next item's first scores (its O is not written before the softmax warps have read this
-          // item's: their P of the new item follows their reads).
-          tc_commit(bar(C::B_QE));
-          has_nxt = advance(uses_n);
-          mbar_wait(bar(C::B_F + vs), (u / C::NP) & 1, wc);
+        // the TMA barrier first (V of this tile and K of the next): the data has normally landed long ago, and
+        // checking here keeps it out of the gap between a stream's P arriving and its MMAs being issued
+        if (!mbar_wait(bar(C::B_F + vs), (u / C::NP) & 1, wc)) break;   // abandoned: the record may never come
+        const uint32_t nxt = records[vs];
+        if (cur & kLast) {
+          // An item ends.  Both P V go first, then the next item's first scores (its O is not written before the softmax
+          // warps have read this item's: their P of the new item follows their reads).
 #pragma unroll 1
           for (int j = 0; j < 2; ++j) {
-            if (uses_c & (1 << j)) {
+            if (cur & (1 << j)) {
               mbar_wait(bar(C::B_PF + j), (pv_par >> j) & 1, wc);
               tc_fence_after();
               issue_pv(j, vs, (acc >> j) & 1);
@@ -422,12 +466,12 @@ __global__ void __launch_bounds__(kThreads, 1) rf_attn_kernel(const __grid_const
             }
           }
           acc = 0;
-          if (has_nxt) {
+          if (nxt & kMore) {
             mbar_wait(bar(C::B_Q), nq & 1, wc);
             ++nq;
 #pragma unroll 1
             for (int j = 0; j < 2; ++j) {
-              if (uses_n & (1 << j)) {
+              if (nxt & (1 << j)) {
                 if (C::S_EARLY) mbar_wait(bar(C::B_SE + j), (s_par >> j) & 1, wc);
                 tc_fence_after();
                 issue_s(j, ksn);
@@ -435,28 +479,20 @@ __global__ void __launch_bounds__(kThreads, 1) rf_attn_kernel(const __grid_const
               }
             }
           }
-          tc_commit(bar(C::B_E + vs));
-          has_cur = has_nxt;
-          uses_c = uses_n;
-          continue;
-        }
-        // the TMA barrier first (V of this tile and K of the next): the data has normally landed long ago, and
-        // checking here keeps it out of the gap between a stream's P arriving and its MMAs being issued
-        mbar_wait(bar(C::B_F + vs), (u / C::NP) & 1, wc);
-        if constexpr (C::S_EARLY) {
+        } else if constexpr (C::S_EARLY) {
           // Per stream: the next tile's scores (S is free as soon as the softmax warps have read the current
           // one), then O += P V of the current tile.  Stream 1's next scores are thus only issued once stream 0
           // has delivered its P: the two streams settle half a tile apart and take turns at the MUFU unit
           // instead of sitting in their exponentials at the same time.
 #pragma unroll
           for (int j = 0; j < 2; ++j) {
-            if (uses_n & (1 << j)) {
+            if (nxt & (1 << j)) {
               mbar_wait(bar(C::B_SE + j), (s_par >> j) & 1, wc);
               tc_fence_after();
               issue_s(j, ksn);
               s_par ^= 1u << j;
             }
-            if (uses_c & (1 << j)) {
+            if (cur & (1 << j)) {
               mbar_wait(bar(C::B_PF + j), (pv_par >> j) & 1, wc);
               tc_fence_after();
               issue_pv(j, vs, (acc >> j) & 1);
@@ -467,19 +503,19 @@ __global__ void __launch_bounds__(kThreads, 1) rf_attn_kernel(const __grid_const
         } else {
 #pragma unroll
           for (int j = 0; j < 2; ++j) {
-            if (uses_c & (1 << j)) {
+            if (cur & (1 << j)) {
               mbar_wait(bar(C::B_PF + j), (pv_par >> j) & 1, wc);
               tc_fence_after();
               issue_pv(j, vs, (acc >> j) & 1);
               acc |= 1u << j;
               pv_par ^= 1u << j;
             }
-            if (uses_n & (1 << j)) issue_s(j, ksn);
+            if (nxt & (1 << j)) issue_s(j, ksn);
           }
         }
+        if ((nxt & (kMore | kLast)) == (kMore | kLast)) tc_commit(bar(C::B_QE));   // the item's last scores are under way
         tc_commit(bar(C::B_E + vs));
-        has_cur = has_nxt;
-        uses_c = uses_n;
+        cur = nxt;
       }
     }
   }
@@ -498,13 +534,9 @@ __global__ void __launch_bounds__(kThreads, 1) rf_attn_kernel(const __grid_const
     im.n0 = im.n1 = 0;
     // (a warp leaves as a whole: after an abandoned wait its lanes may differ in what they saw)
     for (int item = 0; __all_sync(0xffffffffu, take(item, im, im.n0 + im.n1)); ++item) {
-    if (lane == 0) mbar_arrive(bar(C::B_IE + item % kItemSlots));
-    const int bh = im.bh, cls = im.cls;
-    const int r = (im.qt0 + j) * BM + row_in_tile;    // query slot in the head's coordinate space
     const int n = j == 0 ? im.n0 : im.n1;
-    const int32_t* list = a.head_class != nullptr ? a.kv_tile + ((size_t)bh * g.nQ + min(im.qt0 + j, g.nQ - 1)) * g.nKmax : nullptr;
-    const bool perm = cls == RF_TEMPORAL && g.permute;
-    const RowMask rmask = make_row_mask(g, cls, im.window, min(r, g.N - 1));
+    const int32_t* list = a.head_class != nullptr ? a.kv_tile + ((size_t)im.bh * g.nQ + min(im.qt0 + j, g.nQ - 1)) * g.nKmax : nullptr;
+    const RowMask rmask = make_row_mask(g, im.cls, im.window, min((im.qt0 + j) * BM + row_in_tile, g.N - 1));
     float m_run = -INFINITY;   // running maximum, log2 domain (score * sc)
     float l_run = 0.f;         // sum of the weights as rounded to bf16, the ones P V multiplies: normalises O
     float l_exact = 0.f;       // sum of the unrounded weights: the log-sum-exp (LSE only)
@@ -524,29 +556,13 @@ __global__ void __launch_bounds__(kThreads, 1) rf_attn_kernel(const __grid_const
       mbar_wait(bar(C::B_SF + j), (done + it) & 1, wc);
       tc_fence_after();
       uint32_t s[128];
-      {
-        uint32_t(&s0)[32] = *reinterpret_cast<uint32_t(*)[32]>(&s[0]);
-        uint32_t(&s1)[32] = *reinterpret_cast<uint32_t(*)[32]>(&s[32]);
-        uint32_t(&s2)[32] = *reinterpret_cast<uint32_t(*)[32]>(&s[64]);
-        uint32_t(&s3)[32] = *reinterpret_cast<uint32_t(*)[32]>(&s[96]);
-        tmem_ld32(t_s, s0);
-        tmem_ld32(t_s + 32, s1);
-        tmem_ld32(t_s + 64, s2);
-        tmem_ld32(t_s + 96, s3);
-        tc_wait_ld();
-      }
+      load_scores(t_s, s);
       if constexpr (C::S_EARLY) {   // the accumulator is handed back at once; P goes to TMEM columns of its own
         tc_fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive(bar(C::B_SE + j));
       }
-      if (partial) {
-        const uint4 kw = *keep;
-        const uint32_t w[4] = {kw.x, kw.y, kw.z, kw.w};
-#pragma unroll
-        for (int c = 0; c < 128; ++c)
-          if (!((w[c >> 5] >> (c & 31)) & 1u)) s[c] = 0xff800000u;  // -inf
-      }
+      if (partial) mask_scores(keep, s);
       if constexpr (C::S_EARLY) {
         // The scores are gone from TMEM, so the exact row maximum comes first and the exponentials are
         // taken once; the running maximum is raised only when the tile exceeds it by kLazyRaise.
@@ -637,6 +653,8 @@ __global__ void __launch_bounds__(kThreads, 1) rf_attn_kernel(const __grid_const
         }
         m_use = m_run == -INFINITY ? 0.f : m_run;
         la = make_float2(0.f, 0.f);
+        load_scores(t_s, s);   // again: they need not survive the rescaling in registers (or on the stack)
+        if (partial) mask_scores(keep, s);
         take_weights<0, kSpec, LSE>(s, pk, la, sc2, make_float2(-m_use, -m_use));
       }
       const uint32_t t_p = tmem_base + lane_sel + (j ? C::P_COL1 : C::P_COL0);
@@ -662,33 +680,26 @@ __global__ void __launch_bounds__(kThreads, 1) rf_attn_kernel(const __grid_const
     if (n > 0) {
       mbar_wait(bar(C::B_OF + j), (done + n - 1) & 1, wc);
       tc_fence_after();
-      int tok = r;
-      if (perm && r < g.Nv) tok = (r % g.T) * g.S + r / g.T;
+      done += n;
+      // the item's words are read again here: kept in registers they would be in the way of the scores
+      const Row row = output_row(a, items + (item % kItemSlots) * kItemWords, j, row_in_tile);
       const float inv = l_run > 0.f ? 1.f / l_run : 0.f;
-      // a thread writes its row alone, so a warp's store touches 32 rows: whole 32-byte sectors where O allows it
-      const bool o32 = (reinterpret_cast<uintptr_t>(a.o) & 31u) == 0;
-      uint4* dst = reinterpret_cast<uint4*>(a.o + ((size_t)bh * g.N + min(tok, g.N - 1)) * D);
 #pragma unroll
       for (int c = 0; c < D / 32; ++c) {
         uint32_t v[32];
         tmem_ld32(t_o + c * 32, v);   // warp-collective: rows past N take part, they just do not store
         tc_wait_ld();
-        if (r < g.N && rf_in_bounds(tok, g.N, a.dev_status)) {
+        if (row.inside) {
 #pragma unroll
           for (int i = 0; i < 16; ++i) v[i] = pack_bf16(__uint_as_float(v[2 * i]) * inv, __uint_as_float(v[2 * i + 1]) * inv);
-          if (o32) {
-            st_global_v8(dst + c * 4, v);
-            st_global_v8(dst + c * 4 + 2, v + 8);
-          } else {
-#pragma unroll
-            for (int i = 0; i < 4; ++i) dst[c * 4 + i] = make_uint4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
-          }
+          store_columns(row.o + c * 4, v, row.o32);
         }
       }
-      if (LSE && r < g.N && rf_in_bounds(tok, g.N, a.dev_status)) a.lse[(size_t)bh * g.N + tok] = (m_run + log2f(l_exact)) * 0.6931471805599453f;
+      if (LSE && row.inside) a.lse[row.at] = (m_run + log2f(l_exact)) * 0.6931471805599453f;
       tc_fence_before();   // O has been read: the next P hand-over lets it be overwritten
-      done += n;
     }
+    __syncwarp();
+    if (lane == 0) mbar_arrive(bar(C::B_IE + item % kItemSlots));
     }
   }
 

@@ -124,6 +124,7 @@ inline bool rf_regs_ok(K kernel) {
 }
 
 // True in one lane of a converged warp.  (Unlike `lane == 0` this tells the compiler that a single thread runs the branch.)
+// True in one lane of a converged warp.
 __device__ __forceinline__ bool elect_one() {
   uint32_t ok;
   asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(ok));
