@@ -20,7 +20,7 @@ _LIB_PATH = os.environ.get("RAINFUSION_LIBRARY") or os.path.join(os.path.dirname
 _lib = None
 
 EXPORTS = ["rf_status_string", "rf_schedule_dims", "rf_workspace_bytes", "rf_arm_classify",
-           "rf_build_block_mask", "rf_reorder_tokens", "rf_sparse_attn_fwd", "rf_dense_attn_fwd",
+           "rf_build_block_mask", "rf_reorder_tokens", "rf_sparse_attn_fwd", "rf_dense_attn_fwd", "rf_dense_workspace_bytes",
            "rf_arm_classify_noalloc", "rf_selftest_wait_timeout", "rf_arm_classify_plus", "rf_build_block_mask_plus", "rf_sparse_attn_fwd_plus",
            "rf_sparse_attn_reordered", "rf_selftest_arm_abandoned", "rf_bounds_checked", "rf_host_pipeline_staging_bytes",
            "rf_host_pipeline_create", "rf_host_pipeline_run", "rf_host_pipeline_status", "rf_host_pipeline_destroy",
@@ -107,6 +107,8 @@ def load():
     lib.rf_selftest_wait_timeout.argtypes = [V, C.c_int32, V, V]
     lib.rf_reorder_tokens.restype = I
     lib.rf_reorder_tokens.argtypes = [P(rf_shape), P(rf_params), V, V, V, V, V, Z, V]
+    lib.rf_dense_workspace_bytes.restype = Z
+    lib.rf_dense_workspace_bytes.argtypes = [P(rf_shape)]
     lib.rf_dense_attn_fwd.restype = I
     lib.rf_dense_attn_fwd.argtypes = [P(rf_shape), V, V, V, V, V, V, Z, V, V]
     _lib = lib
@@ -318,5 +320,10 @@ def rf_reorder_tokens(shape, params, q, k, v, head_class, ws):
 
 
 def rf_dense_attn_fwd(shape, q, k, v, o, lse, dev_status=None):
-    _check(load().rf_dense_attn_fwd(C.byref(shape), q.data_ptr(), k.data_ptr(), v.data_ptr(), o.data_ptr(), _ptr(lse),
-                                    None, 0, _ptr(dev_status), _stream()), "rf_dense_attn_fwd")
+    """Takes the scratch that split items need (shapes of few items only) from torch's allocator for the call."""
+    import torch
+    lib = load()
+    n = lib.rf_dense_workspace_bytes(C.byref(shape))
+    ws = torch.empty(n, dtype=torch.uint8, device=q.device) if n else None
+    _check(lib.rf_dense_attn_fwd(C.byref(shape), q.data_ptr(), k.data_ptr(), v.data_ptr(), o.data_ptr(), _ptr(lse),
+                                 _ptr(ws), n, _ptr(dev_status), _stream()), "rf_dense_attn_fwd")

@@ -1,4 +1,5 @@
 // C ABI of the RainFusion CUDA path: argument validation, workspace layout, tensor-map encoding.
+#include <algorithm>
 #include <math.h>
 #include <string.h>
 
@@ -109,6 +110,16 @@ bool encode_map(CUtensorMap* m, const void* ptr, int D, int rows, int head_rows,
   return rf_encode_rows_map(m, ptr, D, rows, (size_t)D * 2, (size_t)head_rows * D * 2, heads);
 }
 
+// Where the pieces of split items live: behind ARM's scratch.
+size_t split_offset(const RfGeom& g, const rf_params* p) {
+  return 3 * tensor_bytes(g) + align_up(rf_arm_scratch_floats(g, p->sample_stride, RF_MAX_BANDWIDTHS) * sizeof(float));
+}
+void set_split(RfAttnArgs* a, const RfSplit& sp, uint8_t* at) {
+  a->sp = sp;
+  a->tickets = sp.on ? reinterpret_cast<int32_t*>(at) : nullptr;
+  a->pieces = sp.on ? reinterpret_cast<float*>(at + rf_split_ticket_bytes(sp)) : nullptr;
+}
+
 rf_status check_attn_shape(const rf_shape* s) {
   rf_status st = check_shape(s);
   if (st != RF_OK) return st;
@@ -147,7 +158,8 @@ namespace {
 // reads the reordered copies a preceding rf_reorder_tokens call left in the workspace.
 rf_status sparse_attn_impl(const rf_shape* shape, const rf_params* params, const void* q, const void* k, const void* v,
                            const int32_t* head_class, const int32_t* head_window, const rf_schedule* sched, void* o,
-                           float* lse, void* ws, size_t ws_bytes, int32_t* dev_status, void* cuda_stream, bool gather) {
+                           float* lse, void* ws, size_t ws_bytes, int32_t* dev_status, void* cuda_stream, bool gather,
+                           int heads_total, int head0) {
   rf_status st = check_attn_shape(shape);
   if (st != RF_OK) return st;
   st = check_params(params);
@@ -162,7 +174,7 @@ rf_status sparse_attn_impl(const rf_shape* shape, const rf_params* params, const
       (reinterpret_cast<uintptr_t>(ws) & (kAlign - 1)) != 0)
     return RF_ERR_INVALID_ARG;
   if (head_window != nullptr && params->temporal_window_2d) return RF_ERR_UNSUPPORTED;
-  if (ws_bytes < rf_workspace_bytes(shape, params)) return RF_ERR_WORKSPACE_TOO_SMALL;
+  if (ws_bytes < rf_group_workspace_bytes(shape, params, heads_total, head0)) return RF_ERR_WORKSPACE_TOO_SMALL;
   const RfGeom g = make_geom(shape, params);
   if (sched->nQ != g.nQ || sched->nKmax != g.nKmax) return RF_ERR_INVALID_ARG;
   cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
@@ -180,14 +192,15 @@ rf_status sparse_attn_impl(const rf_shape* shape, const rf_params* params, const
             encode_map(&maps[6], wk, g.D, g.LkvTex, g.N, heads) && encode_map(&maps[7], wv, g.D, g.LkvTex, g.N, heads);
   if (!ok) return RF_ERR_CUDA;
 
+  RfAttnArgs a;
+  set_split(&a, rf_split_plan(g, true, heads_total, head0), w + split_offset(g, params));
   if (gather) {
     cudaError_t e = rf_launch_gather(g, head_class, static_cast<const __nv_bfloat16*>(q),
                                      static_cast<const __nv_bfloat16*>(k), static_cast<const __nv_bfloat16*>(v), wq, wk, wv,
-                                     dev_status, stream);
+                                     a.tickets, (int)a.sp.n_tickets, dev_status, stream);
     if (e != cudaSuccess) return RF_ERR_CUDA;
   }
 
-  RfAttnArgs a;
   a.g = g;
   a.head_class = head_class;
   a.head_window = head_window;
@@ -200,6 +213,75 @@ rf_status sparse_attn_impl(const rf_shape* shape, const rf_params* params, const
   return rf_launch_attention(a, maps, stream);
 }
 }  // namespace
+
+// ------------------------------------------------------------------------------------------------
+// The plan of split items (see RfSplit).  Costs are counted in tiles of an item (about 2 us): a unit of work costs its
+// tiles and kUnit more, joining pieces kJoin, and a piece kPiece (its O through the L2 twice, over all SMs).  Leaving a
+// piece takes 5 to 7 us against 2 to 3 for writing O out, so a piece needs tiles enough to pay for it: four where SMs
+// would otherwise stay idle, more in a call of more items than SMs, whose last wave is not empty to begin with (masked
+// calls most, as their items' lengths differ and fill each other's gaps).  Measured, whole calls: 27 items of 9 tiles (3
+// heads, 2146 tokens, D = 96) 56.8 -> 48.0 us; 42 items of 14 230 -> 203; 205 items of 41 321 -> 273; 360 dense items of 30
+// 183 -> 173; with pieces of 4 tiles 192 items of 12 became slower (83 -> 91), with text rows' pairs alone split 84 items
+// of 7 too (99 -> 102).
+// ------------------------------------------------------------------------------------------------
+RfSplit rf_split_plan(const RfGeom& g, bool sparse, int heads_total, int head0) {
+  constexpr int W = 148;                                // SMs, one CTA each
+  constexpr long long kMostWaves = 32, kMostSlots = 384;
+  constexpr double kUnit = 2.5, kJoin = 2.0, kPiece = 0.02;
+  RfSplit sp = {};
+  const int heads = g.B * g.H;
+  const int nK = rf_cdiv(g.N, 128), pairs = rf_cdiv(rf_cdiv(g.N, 128), 2);
+  const long long items = (long long)heads_total * pairs;
+  if (items > kMostWaves * W) return sp;
+  const int least = items < W ? 4 : (sparse ? 16 : 8);  // tiles a piece has at least
+  const int usual = sparse ? (nK + 1) / 2 : nK;         // tiles an item lists: the patterns keep about half
+  sp.text_pairs = sparse ? pairs - g.Nv / 256 : 0;
+  const long long tail = std::min(items % W, (long long)heads_total * (pairs - sp.text_pairs));
+  sp.kr = 1;
+  double best = 1e30;
+  for (int k = 1; k <= 8 && tail > 0; ++k) {
+    if (k > 1 && (usual < least * k || tail * k > kMostSlots)) break;
+    const double cost = (double)((tail * k + W - 1) / W) * ((double)usual / k + kUnit) + (k > 1 ? kJoin + kPiece * tail * k : 0.0);
+    if (cost < best) { best = cost; sp.kr = k; }
+  }
+  sp.lr = rf_cdiv(usual, sp.kr);
+  sp.kt = 1;
+  sp.lt = items < W ? sp.lr : usual;
+  const long long text = (long long)heads_total * sp.text_pairs;
+  if (sp.kr == 1) return RfSplit{};
+  if (text > 0 && items < 3 * W && text * rf_cdiv(nK, sp.lt) + tail * sp.kr <= kMostSlots) sp.kt = rf_cdiv(nK, sp.lt);
+  sp.on = 1;
+  if (sp.kt == 1) sp.text_pairs = 0;
+  // the items of this group of heads
+  const long long t0 = (long long)heads_total * (pairs - sp.text_pairs) - tail;
+  sp.row0 = (int)(t0 / heads_total);
+  sp.head_row0 = (int)std::min<long long>(std::max<long long>(t0 % heads_total - head0, 0), heads);
+  sp.n_text = (uint32_t)(heads * sp.text_pairs * sp.kt);
+  sp.first_tail = (uint32_t)(sp.row0 * heads + sp.head_row0);
+  const uint32_t n_tail = (uint32_t)(heads * (pairs - sp.text_pairs)) - sp.first_tail;
+  sp.n_units = sp.n_text + sp.first_tail + n_tail * sp.kr;
+  sp.n_slots = (sp.kt > 1 ? sp.n_text : 0) + n_tail * sp.kr;
+  sp.n_tickets = 8 * ((sp.kt > 1 ? heads * sp.text_pairs : 0) + n_tail);
+  return sp;
+}
+size_t rf_split_ticket_bytes(const RfSplit& sp) { return align_up(sp.n_tickets * sizeof(int32_t)); }
+size_t rf_split_bytes(const RfSplit& sp, int D) {
+  return sp.on ? rf_split_ticket_bytes(sp) + align_up((size_t)sp.n_slots * 2 * 128 * (D + 4) * sizeof(float)) : 0;
+}
+
+size_t rf_group_workspace_bytes(const rf_shape* shape, const rf_params* params, int heads_total, int head0) {
+  if (check_shape(shape) != RF_OK || check_params(params) != RF_OK) return 0;
+  const RfGeom g = make_geom(shape, params);
+  return split_offset(g, params) + rf_split_bytes(rf_split_plan(g, true, heads_total, head0), g.D);
+}
+
+rf_status rf_sparse_attn_group(const rf_shape* shape, const rf_params* params, const void* q, const void* k, const void* v,
+                               const int32_t* head_class, const int32_t* head_window, const rf_schedule* sched, void* o,
+                               float* lse, void* ws, size_t ws_bytes, int32_t* dev_status, void* cuda_stream, int heads_total,
+                               int head0) {
+  return sparse_attn_impl(shape, params, q, k, v, head_class, head_window, sched, o, lse, ws, ws_bytes, dev_status, cuda_stream,
+                          true, heads_total, head0);
+}
 
 extern "C" {
 
@@ -240,9 +322,7 @@ rf_status rf_schedule_dims(const rf_shape* shape, const rf_params* params, int32
 }
 
 size_t rf_workspace_bytes(const rf_shape* shape, const rf_params* params) {
-  if (check_shape(shape) != RF_OK || check_params(params) != RF_OK) return 0;
-  const RfGeom g = make_geom(shape, params);
-  return 3 * tensor_bytes(g) + align_up(rf_arm_scratch_floats(g, params->sample_stride, RF_MAX_BANDWIDTHS) * sizeof(float));
+  return check_shape(shape) == RF_OK ? rf_group_workspace_bytes(shape, params, shape->B * shape->H, 0) : 0;
 }
 
 rf_status rf_arm_classify(const rf_shape* shape, const rf_params* params, const void* q, const void* k,
@@ -353,7 +433,7 @@ rf_status rf_sparse_attn_fwd_plus(const rf_shape* shape, const rf_params* params
                                   const rf_schedule* sched, void* o, float* lse, void* ws, size_t ws_bytes,
                                   int32_t* dev_status, void* cuda_stream) {
   return sparse_attn_impl(shape, params, q, k, v, head_class, head_window, sched, o, lse, ws, ws_bytes, dev_status,
-                          cuda_stream, true);
+                          cuda_stream, true, shape != nullptr ? shape->B * shape->H : 0, 0);
 }
 
 rf_status rf_sparse_attn_reordered(const rf_shape* shape, const rf_params* params, const void* q, const void* k,
@@ -361,7 +441,7 @@ rf_status rf_sparse_attn_reordered(const rf_shape* shape, const rf_params* param
                                    const rf_schedule* sched, void* o, float* lse, void* ws, size_t ws_bytes,
                                    int32_t* dev_status, void* cuda_stream) {
   return sparse_attn_impl(shape, params, q, k, v, head_class, head_window, sched, o, lse, ws, ws_bytes, dev_status,
-                          cuda_stream, false);
+                          cuda_stream, false, shape != nullptr ? shape->B * shape->H : 0, 0);
 }
 
 rf_status rf_selftest_wait_timeout(int32_t* dev_status, int32_t limit_ms, int32_t* waits_returned, void* cuda_stream) {
@@ -384,18 +464,23 @@ rf_status rf_reorder_tokens(const rf_shape* shape, const rf_params* params, cons
   if (ws_bytes < rf_workspace_bytes(shape, params)) return RF_ERR_WORKSPACE_TOO_SMALL;
   const RfGeom g = make_geom(shape, params);
   uint8_t* w = static_cast<uint8_t*>(ws);
+  RfAttnArgs a;   // a following rf_sparse_attn_reordered finds its tickets at zero
+  set_split(&a, rf_split_plan(g, true, g.B * g.H, 0), w + split_offset(g, params));
   cudaError_t e = rf_launch_gather(g, head_class, static_cast<const __nv_bfloat16*>(q), static_cast<const __nv_bfloat16*>(k),
                                    static_cast<const __nv_bfloat16*>(v), reinterpret_cast<__nv_bfloat16*>(w),
                                    reinterpret_cast<__nv_bfloat16*>(w + tensor_bytes(g)),
-                                   reinterpret_cast<__nv_bfloat16*>(w + 2 * tensor_bytes(g)), nullptr,
+                                   reinterpret_cast<__nv_bfloat16*>(w + 2 * tensor_bytes(g)), a.tickets, (int)a.sp.n_tickets, nullptr,
                                    static_cast<cudaStream_t>(cuda_stream));
   return e == cudaSuccess ? RF_OK : RF_ERR_CUDA;
 }
 
+size_t rf_dense_workspace_bytes(const rf_shape* shape) {
+  if (check_attn_shape(shape) != RF_OK) return 0;
+  return rf_split_bytes(rf_split_plan(make_geom(shape, 0, 0, 1, 128, 128, 0), false, shape->B * shape->H, 0), shape->D);
+}
+
 rf_status rf_dense_attn_fwd(const rf_shape* shape, const void* q, const void* k, const void* v, void* o, float* lse,
                             void* ws, size_t ws_bytes, int32_t* dev_status, void* cuda_stream) {
-  (void)ws;
-  (void)ws_bytes;
   rf_status st = check_attn_shape(shape);
   if (st != RF_OK) return st;
   if (q == nullptr || k == nullptr || v == nullptr || o == nullptr) return RF_ERR_INVALID_ARG;
@@ -408,6 +493,10 @@ rf_status rf_dense_attn_fwd(const rf_shape* shape, const void* q, const void* k,
   if (!ok) return RF_ERR_CUDA;
   for (int i = 3; i < 8; ++i) maps[i] = maps[i % 3];
   RfAttnArgs a;
+  const RfSplit sp = rf_split_plan(g, false, heads, 0);
+  const bool split = sp.on && ws != nullptr && (reinterpret_cast<uintptr_t>(ws) & (kAlign - 1)) == 0 && ws_bytes >= rf_split_bytes(sp, g.D);
+  set_split(&a, split ? sp : RfSplit{}, static_cast<uint8_t*>(ws));
+  if (split && rf_launch_zero(a.tickets, (int)sp.n_tickets, static_cast<cudaStream_t>(cuda_stream)) != cudaSuccess) return RF_ERR_CUDA;
   a.g = g;
   a.head_class = nullptr;
   a.head_window = nullptr;

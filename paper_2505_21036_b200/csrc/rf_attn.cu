@@ -32,7 +32,7 @@ using namespace rf_attn;
 
 constexpr int kThreads = kWsThreads;        // 3 warpgroups: softmax 0, softmax 1, {TMA, MMA, 2 idle warps}
 constexpr int kTmaWarp = 8, kMmaWarp = 9, kItemWarp = 10;
-constexpr int kItemSlots = 2, kItemWords = 8, kItemReaders = 9;   // readers: eight softmax warps and the TMA thread
+constexpr int kItemSlots = 2, kItemWords = 12, kItemReaders = 9;   // readers: eight softmax warps and the TMA thread
 constexpr uint32_t kMore = 4, kLast = 8;   // of a tile record, see the TMA producer
 constexpr int kAskAhead = 4;   // tiles an item has left when the next one is asked for: about 8 us, an answer takes about one
 // What bounds the loop: a stream is the chain scores -> softmax -> P V -> Q K^T, so what counts is how few dependent
@@ -101,7 +101,8 @@ struct Cfg {
 };
 
 // One item of work: two adjacent query tiles of one head.
-struct Item { int bh, qt0, cls, n0, n1, window; };
+// (or, of a split one, a piece: n0 and n1 entries of the two lists from b0 and b1 on)
+struct Item { int bh, qt0, cls, n0, n1, window, b0, b1; };
 
 // Which item the CTA of index `lin` of the grid stands for.  Heads are taken in groups whose K and V fit the L2 cache
 // together (one head at a time where they are long); inside a group the last pair of query tiles of every head comes
@@ -115,15 +116,59 @@ __device__ __forceinline__ void place_item(uint64_t lin, int group, int heads, i
   pair = pairs - 1 - (int)(r / in);
 }
 
-// 32 bf16 columns of an output row.
-__device__ __forceinline__ void store_columns(uint4* dst, const uint32_t* v, bool o32) {
+// What a unit of the grid is: an item, or one piece of an item that may be split.
+struct Unit { int bh, pair, piece, most, tiles, slot, split; };
+__device__ __forceinline__ void place_unit(uint64_t lin, const RfAttnArgs& a, Unit& un) {
+  const RfSplit& sp = a.sp;
+  const int heads = a.g.B * a.g.H, pairs = rf_cdiv(a.g.nQ, 2);
+  un.piece = 0;
+  un.most = 1;
+  un.tiles = un.slot = un.split = 0;
+  if (!sp.on) {
+    place_item(lin, a.heads_l2, heads, pairs, un.bh, un.pair);
+    return;
+  }
+  const uint32_t u = (uint32_t)lin;
+  if (u < sp.n_text) {                                  // pairs with text rows
+    const int item = (int)(u / sp.kt);
+    un.most = sp.kt; un.tiles = sp.lt; un.piece = (int)(u % sp.kt); un.slot = (int)u; un.split = item;
+    un.bh = item % heads;
+    un.pair = pairs - 1 - item / heads;
+    return;
+  }
+  int item = (int)(u - sp.n_text), row;
+  if (item >= (int)sp.first_tail) {                     // the tail: from row0 on, row by row
+    const int t = item - (int)sp.first_tail, i = t / sp.kr, head = sp.head_row0 + i;
+    un.most = sp.kr; un.tiles = sp.lr; un.piece = t % sp.kr;
+    un.slot = (int)(sp.kt > 1 ? sp.n_text : 0) + t;
+    un.split = (sp.kt > 1 ? heads * sp.text_pairs : 0) + i;
+    row = sp.row0 + head / heads;
+    un.bh = head % heads;
+  } else {                                              // whole items: in groups of heads as in place_item
+    int g0 = 0, in, n;
+    for (;; g0 += a.heads_l2, item -= n) {
+      in = min(a.heads_l2, heads - g0);
+      n = in * sp.row0 + min(max(sp.head_row0 - g0, 0), in);
+      if (item < n) break;
+    }
+    row = item / in;
+    un.bh = g0 + item % in;
+  }
+  un.pair = pairs - sp.text_pairs - 1 - row;
+}
+
+// 16 and 32 bf16 columns of an output row.
+__device__ __forceinline__ void store_sector(uint4* dst, const uint32_t* v, bool o32) {
   if (o32) {
     st_global_v8(dst, v);
-    st_global_v8(dst + 2, v + 8);
   } else {
-#pragma unroll
-    for (int i = 0; i < 4; ++i) dst[i] = make_uint4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
+    dst[0] = make_uint4(v[0], v[1], v[2], v[3]);
+    dst[1] = make_uint4(v[4], v[5], v[6], v[7]);
   }
+}
+__device__ __forceinline__ void store_columns(uint4* dst, const uint32_t* v, bool o32) {
+  store_sector(dst, v, o32);
+  store_sector(dst + 2, v + 8, o32);
 }
 
 // Where this thread's row of an item goes.
@@ -144,6 +189,89 @@ __device__ __forceinline__ Row output_row(const RfAttnArgs& a, const int* iw, in
   row.o = reinterpret_cast<uint4*>(a.o + row.at * g.D);
   row.o32 = (reinterpret_cast<uintptr_t>(a.o) & 31u) == 0;
   return row;
+}
+
+// One warp's 32 rows of a piece of a split item: O and the sums go to the workspace as they are, and the last warp to
+// arrive at these rows joins the pieces.  They are taken in order, so the bits do not depend on who does it.  Out of
+// line: the loop over the tiles has no register to spare.
+template <int D, bool LSE>
+__device__ __noinline__ void leave_piece(const RfAttnArgs& a, const int* iw, uint32_t t_o, int warp, int lane, float m_run, float l_run,
+                                         float l_exact, bool has_o) {
+  constexpr size_t kRows = (size_t)(D / 4 + 1) * BM;          // float4 of one piece of one stream
+  const int j = warp >> 2, row_in_tile = (warp & 3) * 32 + lane, pieces = iw[8];
+  if (iw[1] + j >= a.g.nQ || !rf_in_bounds(iw[9], a.sp.n_slots, a.dev_status)) return;   // (the warp as a whole)
+  float4* first = reinterpret_cast<float4*>(a.pieces) + ((size_t)(iw[9] - iw[11]) * 2 + j) * kRows + row_in_tile;
+  float4* mine = first + (size_t)iw[11] * 2 * kRows;
+  if (has_o) {
+#pragma unroll 1
+    for (int c = 0; c < D / 32; ++c) {
+      uint32_t v[32];
+      tmem_ld32(t_o + c * 32, v);
+      tc_wait_ld();
+#pragma unroll
+      for (int i = 0; i < 8; ++i)
+        __stcg(mine + (c * 8 + i) * BM, make_float4(__uint_as_float(v[4 * i]), __uint_as_float(v[4 * i + 1]),
+                                                    __uint_as_float(v[4 * i + 2]), __uint_as_float(v[4 * i + 3])));
+    }
+  }
+  __stcg(mine + (D / 4) * BM, make_float4(m_run, l_run, l_exact, has_o ? 1.f : 0.f));
+  __threadfence();
+  __syncwarp();
+  int32_t* ticket = a.tickets + iw[10] * 8 + warp;
+  int before = 0;
+  if (lane == 0) before = atomicAdd(ticket, 1);
+  if (__shfl_sync(0xffffffffu, before, 0) != pieces - 1) return;
+  __threadfence();
+  if (lane == 0) *ticket = 0;                                  // the next call on this workspace finds it as this one did
+  const Row row = output_row(a, iw, j, row_in_tile);
+  // half a row at a time, so that all loads of a piece are under way together
+  constexpr int kCols = D == 64 ? 64 : D / 2;
+#pragma unroll 1
+  for (int c0 = 0; c0 < D; c0 += kCols) {
+    float m = -INFINITY, l = 0.f, l_all = 0.f;
+    float4 acc[kCols / 4];
+#pragma unroll
+    for (int i = 0; i < kCols / 4; ++i) acc[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 1
+    for (int p = 0; p < pieces; ++p) {
+      const float4* at = first + p * 2 * kRows;
+      const float4 st = __ldcg(at + (D / 4) * BM);
+      float4 o[kCols / 4];
+#pragma unroll
+      for (int i = 0; i < kCols / 4; ++i) o[i] = __ldcg(at + (c0 / 4 + i) * BM);
+      if (st.w == 0.f) continue;                               // listed no tile: its O was never written
+      // where one side has no maximum its O and sums are zero (or not numbers): they are added as they are
+      float keep = 1.f, w = 1.f;
+      if (st.x > m) {
+        if (m > -INFINITY) keep = ex2(m - st.x);
+        m = st.x;
+      } else if (st.x > -INFINITY) {
+        w = ex2(st.x - m);
+      }
+      l = l * keep + st.y * w;
+      l_all = l_all * keep + st.z * w;
+#pragma unroll
+      for (int i = 0; i < kCols / 4; ++i) {
+        acc[i].x = acc[i].x * keep + o[i].x * w;
+        acc[i].y = acc[i].y * keep + o[i].y * w;
+        acc[i].z = acc[i].z * keep + o[i].z * w;
+        acc[i].w = acc[i].w * keep + o[i].w * w;
+      }
+    }
+    if (!row.inside) continue;
+    const float inv = l > 0.f ? 1.f / l : 0.f;
+#pragma unroll
+    for (int q = 0; q < kCols / 16; ++q) {
+      uint32_t v[8];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        v[2 * i] = pack_bf16(acc[q * 4 + i].x * inv, acc[q * 4 + i].y * inv);
+        v[2 * i + 1] = pack_bf16(acc[q * 4 + i].z * inv, acc[q * 4 + i].w * inv);
+      }
+      store_sector(row.o + c0 / 8 + q * 2, v, row.o32);
+    }
+    if (LSE && c0 == 0) a.lse[row.at] = (m + log2f(l_all)) * 0.6931471805599453f;
+  }
 }
 
 // This thread's row of O times alpha (warp-collective).
@@ -248,7 +376,7 @@ __global__ void __launch_bounds__(kThreads, 1) rf_attn_kernel(const __grid_const
     const int slot = i % kItemSlots;
     if (!mbar_wait_long(bar(C::B_IF + slot), (i / kItemSlots) & 1, wc, waited)) return false;
     const int* w = items + slot * kItemWords;
-    im.bh = w[0]; im.qt0 = w[1]; im.cls = w[2]; im.n0 = w[3]; im.n1 = w[4]; im.window = w[5];
+    im.bh = w[0]; im.qt0 = w[1]; im.cls = w[2]; im.n0 = w[3]; im.n1 = w[4]; im.window = w[5]; im.b0 = w[6]; im.b1 = w[7];
     return im.bh >= 0;
   };
   auto lists = [&](const Item& im) -> Lists {
@@ -257,8 +385,9 @@ __global__ void __launch_bounds__(kThreads, 1) rf_attn_kernel(const __grid_const
     L.listed = a.head_class != nullptr;
     L.n0 = im.n0;
     L.n1 = im.n1;
-    L.l0 = L.listed ? a.kv_tile + ((size_t)im.bh * g.nQ + im.qt0) * g.nKmax : nullptr;
-    L.l1 = L.listed ? a.kv_tile + ((size_t)im.bh * g.nQ + min(im.qt0 + 1, g.nQ - 1)) * g.nKmax : nullptr;
+    L.first = im.b0;
+    L.l0 = L.listed ? a.kv_tile + ((size_t)im.bh * g.nQ + im.qt0) * g.nKmax + im.b0 : nullptr;
+    L.l1 = L.listed ? a.kv_tile + ((size_t)im.bh * g.nQ + min(im.qt0 + 1, g.nQ - 1)) * g.nKmax + im.b1 : nullptr;
     return L;
   };
 
@@ -267,17 +396,26 @@ __global__ void __launch_bounds__(kThreads, 1) rf_attn_kernel(const __grid_const
   if (warp == kItemWarp) {
     // ------------------------------------------------------------ items: the own one, then those of CTAs not started yet
     if (lane == 0) {
-      uint32_t x = blockIdx.x, y = blockIdx.y;
+      uint32_t x = blockIdx.x, y = blockIdx.y, asked = 0;
       bool more = true;
+      // asks for another unit of work; false: there is none
+      auto ask = [&]() -> bool {
+        fence_proxy_async_smem();
+        mbar_expect_tx(bar(C::B_CLC), 16);
+        clc_request(base + C::ANSWER, bar(C::B_CLC));
+        const bool ok = mbar_wait(bar(C::B_CLC), asked & 1, wc) && clc_answer(base + C::ANSWER, x, y);
+        ++asked;
+        return ok;
+      };
       for (int i = 0;; ++i) {
         const int slot = i % kItemSlots;
         int* w = items + slot * kItemWords;
         if (i >= kItemSlots) mbar_wait(bar(C::B_IE + slot), ((i / kItemSlots) - 1) & 1, wc);
         int n0 = 0, n1 = 0;
-        if (more) {
-          int bh, pair;
-          place_item((uint64_t)y * gridDim.x + x, a.heads_l2, g.B * g.H, gridDim.x, bh, pair);
-          const int qt0 = 2 * pair, qt1 = qt0 + 1;
+        for (; more; more = ask()) {
+          Unit un;
+          place_unit((uint64_t)y * gridDim.x + x, a, un);
+          const int bh = un.bh, qt0 = 2 * un.pair, qt1 = qt0 + 1;
           int cls = RF_DENSE, window = -1;
           if (a.head_class != nullptr) {
             cls = a.head_class[bh];
@@ -295,21 +433,28 @@ __global__ void __launch_bounds__(kThreads, 1) rf_attn_kernel(const __grid_const
             n0 = rf_cdiv(rf_kv_len(g, cls), BN);
             n1 = qt1 < g.nQ ? n0 : 0;
           }
-          w[0] = bh; w[1] = qt0; w[2] = cls; w[3] = n0; w[4] = n1; w[5] = window;
-        } else {
+          int b0 = 0, b1 = 0, k = 1;
+          if (un.most > 1) {
+            const int u = max(n0, n1);
+            k = 4 * u > 5 * un.tiles ? min(rf_cdiv(u, un.tiles), un.most) : 1;   // up to a quarter more stays in one piece
+            if (un.piece >= k) continue;
+            b0 = n0 * un.piece / k;                                              // (at most 32 waves: the products are small)
+            b1 = n1 * un.piece / k;
+            n0 = n0 * (un.piece + 1) / k - b0;
+            n1 = n1 * (un.piece + 1) / k - b1;
+          }
+          w[0] = bh; w[1] = qt0; w[2] = cls; w[3] = n0; w[4] = n1; w[5] = window; w[6] = b0; w[7] = b1;
+          w[8] = k; w[9] = un.slot; w[10] = un.split; w[11] = un.piece;
+          break;
+        }
+        if (!more) {
           w[0] = -1;
+          rf_grid_trigger();
         }
         mbar_arrive(bar(C::B_IF + slot));
         if (!more) break;
-        more = false;
         // not before the TMA warp has nearly worked the item off: an item taken early would wait here while other SMs idle
-        if (mbar_wait_long(bar(C::B_REQ), i & 1, wc, n0 + n1)) {
-          fence_proxy_async_smem();
-          mbar_expect_tx(bar(C::B_CLC), 16);
-          clc_request(base + C::ANSWER, bar(C::B_CLC));
-          if (mbar_wait(bar(C::B_CLC), i & 1, wc)) more = clc_answer(base + C::ANSWER, x, y);
-        }
-        if (!more) rf_grid_trigger();
+        more = mbar_wait_long(bar(C::B_REQ), i & 1, wc, n0 + n1) && ask();
       }
     }
   } else if (warp == kTmaWarp) {
@@ -541,8 +686,10 @@ __global__ void __launch_bounds__(kThreads, 1) rf_attn_kernel(const __grid_const
     float l_run = 0.f;         // sum of the weights as rounded to bf16, the ones P V multiplies: normalises O
     float l_exact = 0.f;       // sum of the unrounded weights: the log-sum-exp (LSE only)
 
-    for (int it = 0; it < n; ++it) {
-      const uint32_t entry = list != nullptr ? (uint32_t)list[it] : dense_entry(it, g.N);
+    const int begin = j == 0 ? im.b0 : im.b1, end = begin + n;
+    bool opens = true;         // the stream's first tile of the item (or piece)
+    for (int t = begin; t < end; ++t, ++done, opens = false) {
+      const uint32_t entry = list != nullptr ? (uint32_t)list[t] : dense_entry(t, g.N);
       // The keep words of a PARTIAL tile do not depend on its scores: they are worked out before the wait for the
       // scores, where a stream spends a third of its time anyway, and wait in shared memory (four registers live
       // through the exponentials cost every tile 3 %).
@@ -553,7 +700,7 @@ __global__ void __launch_bounds__(kThreads, 1) rf_attn_kernel(const __grid_const
         partial = __any_sync(0xffffffffu, (w[0] & w[1] & w[2] & w[3]) != 0xffffffffu);   // a warp's rows may keep it whole
         *keep = make_uint4(w[0], w[1], w[2], w[3]);
       }
-      mbar_wait(bar(C::B_SF + j), (done + it) & 1, wc);
+      mbar_wait(bar(C::B_SF + j), done & 1, wc);
       tc_fence_after();
       uint32_t s[128];
       load_scores(t_s, s);
@@ -586,9 +733,9 @@ __global__ void __launch_bounds__(kThreads, 1) rf_attn_kernel(const __grid_const
         // rescaled once everything issued into it has landed.  The wait sits in front of the P store (the
         // exponentials of this tile run under the previous tile's P V); it also keeps this stream at most
         // one tile ahead of the MMA warp, which tracks the P barrier by phase parity.
-        bool o_landed = it == 0;
-        if (it > 0 && any_raise) {
-          mbar_wait(bar(C::B_OF + j), (done + it - 1) & 1, wc);
+        bool o_landed = opens;
+        if (!opens && any_raise) {
+          mbar_wait(bar(C::B_OF + j), (done - 1) & 1, wc);
           o_landed = true;
           rescale_o<D>(t_o, alpha);
         }
@@ -609,7 +756,7 @@ __global__ void __launch_bounds__(kThreads, 1) rf_attn_kernel(const __grid_const
         }
         if (LSE) l_exact += la.x + la.y;
         l_run += lb.x + lb.y;
-        if (!o_landed) mbar_wait(bar(C::B_OF + j), (done + it - 1) & 1, wc);
+        if (!o_landed) mbar_wait(bar(C::B_OF + j), (done - 1) & 1, wc);
         {
           const uint32_t t_p = tmem_base + lane_sel + (j ? C::P_COL1 : C::P_COL0);
           uint32_t(&p0)[32] = *reinterpret_cast<uint32_t(*)[32]>(&pk[0]);
@@ -646,9 +793,9 @@ __global__ void __launch_bounds__(kThreads, 1) rf_attn_kernel(const __grid_const
           l_run *= alpha;
           if (LSE) l_exact *= alpha;
         }
-        if (it > 0) {
+        if (!opens) {
           // O of the previous tiles must be complete before it is rescaled
-          mbar_wait(bar(C::B_OF + j), (done + it - 1) & 1, wc);
+          mbar_wait(bar(C::B_OF + j), (done - 1) & 1, wc);
           rescale_o<D>(t_o, alpha);
         }
         m_use = m_run == -INFINITY ? 0.f : m_run;
@@ -678,11 +825,15 @@ __global__ void __launch_bounds__(kThreads, 1) rf_attn_kernel(const __grid_const
     }
 
     if (n > 0) {
-      mbar_wait(bar(C::B_OF + j), (done + n - 1) & 1, wc);
+      mbar_wait(bar(C::B_OF + j), (done - 1) & 1, wc);
       tc_fence_after();
-      done += n;
-      // the item's words are read again here: kept in registers they would be in the way of the scores
-      const Row row = output_row(a, items + (item % kItemSlots) * kItemWords, j, row_in_tile);
+    }
+    // the item's words are read again here: kept in registers they would be in the way of the scores
+    const int* iw = items + (item % kItemSlots) * kItemWords;
+    if (iw[8] > 1) {
+      leave_piece<D, LSE>(a, iw, t_o, warp, lane, m_run, l_run, l_exact, n > 0);
+    } else if (n > 0) {
+      const Row row = output_row(a, iw, j, row_in_tile);
       const float inv = l_run > 0.f ? 1.f / l_run : 0.f;
 #pragma unroll
       for (int c = 0; c < D / 32; ++c) {
@@ -696,8 +847,8 @@ __global__ void __launch_bounds__(kThreads, 1) rf_attn_kernel(const __grid_const
         }
       }
       if (LSE && row.inside) a.lse[row.at] = (m_run + log2f(l_exact)) * 0.6931471805599453f;
-      tc_fence_before();   // O has been read: the next P hand-over lets it be overwritten
     }
+    tc_fence_before();   // O has been read: the next P hand-over lets it be overwritten
     __syncwarp();
     if (lane == 0) mbar_arrive(bar(C::B_IE + item % kItemSlots));
     }
@@ -727,7 +878,8 @@ rf_status launch(RfAttnArgs a, const CUtensorMap* maps, cudaStream_t st) {
   for (int i = 0; i < 8; ++i) m.m[i] = maps[i];
   const size_t kv_bytes = (size_t)a.g.N * D * 2 * sizeof(__nv_bfloat16);
   a.heads_l2 = (int)std::min<size_t>(std::max<size_t>(kL2Bytes / kv_bytes, 1), (size_t)a.g.B * a.g.H);
-  dim3 grid(rf_cdiv(a.g.nQ, 2), a.g.B * a.g.H);   // one CTA an item; running CTAs take over what has not started
+  // one CTA a unit of work; running CTAs take over what has not started
+  const dim3 grid = a.sp.on ? dim3(a.sp.n_units) : dim3(rf_cdiv(a.g.nQ, 2), a.g.B * a.g.H);
   return rf_launch(rf_attn_kernel<D, LSE>, grid, kThreads, Cfg<D>::ALLOC, st, m, a) == cudaSuccess ? RF_OK : RF_ERR_CUDA;
 }
 template <int D>

@@ -131,11 +131,12 @@ struct Lists {
   const int32_t* l0;
   const int32_t* l1;
   int n0, n1;
+  int first;      // dense: the first tile of the piece
   int lkv;
   bool listed;
   __device__ __forceinline__ uint32_t entry(int j, int i) const {
     if (listed) return (uint32_t)(j == 0 ? l0[i] : l1[i]);
-    return dense_entry(i, lkv);
+    return dense_entry(first + i, lkv);
   }
 };
 struct Merge {

@@ -76,7 +76,7 @@ cudaError_t rf_launch_build_tiles(const RfGeom& g, const int32_t* head_class, co
                                   int32_t* kv_tile, uint32_t* bitmap, int32_t* kv_len, int32_t* dev_status, cudaStream_t st);
 cudaError_t rf_launch_gather(const RfGeom& g, const int32_t* head_class, const __nv_bfloat16* q,
                              const __nv_bfloat16* k, const __nv_bfloat16* v, __nv_bfloat16* wq, __nv_bfloat16* wk,
-                             __nv_bfloat16* wv, int32_t* dev_status, cudaStream_t st);
+                             __nv_bfloat16* wv, int32_t* tickets, int n_tickets, int32_t* dev_status, cudaStream_t st);
 // nb candidate windows per pattern (ws_list for Temporal, wf_list for Spatial, ascending).  head_window == nullptr:
 // plain Algorithm 1 on the first candidate (recall: [B,H,3] or null).  Otherwise dynamic bandwidth: head_window
 // receives each head's chosen window, recall_plus ([B,H,2,nb] or null) the candidates' recalls.
@@ -97,6 +97,30 @@ bool rf_encode_rows_map(CUtensorMap* m, const void* ptr, int D, int rows, size_t
 // Validates shape and parameters as the entry points do and fills the kernel-side geometry.
 rf_status rf_checked_geom(const rf_shape* shape, const rf_params* params, RfGeom* out);
 
+// Split items.  An item of the attention kernel is a pair of query tiles of one head; one CTA per SM works items off, so a
+// call of a few hundred items ends with most SMs idle, and one of fewer items than SMs never fills them.  The items of
+// the last, partial wave (all of them when there are fewer items than SMs) are therefore cut into pieces of their tile
+// lists, and so are the pairs with text rows, whose lists are twice as long as the others', when there are at most three
+// waves.  A piece leaves its unnormalised O and its sums in the workspace; whoever finishes last joins them.  The plan
+// depends on the whole call's shape alone (and on the item's own list), so that a call made in groups of heads gives
+// the same bits as the call made at once.
+struct RfSplit {
+  int on;                    // 0: one unit of work per item, in the order of place_item
+  int text_pairs;            // pairs of query tiles that may hold text rows (the last ones of a head): the first units
+  int kt, lt;                // pieces such an item has at most, tiles of a piece
+  int kr, lr;                // the same for the tail items
+  uint32_t n_text;           // units of the pairs with text rows
+  int row0, head_row0;       // the other items lie in rows (one item per head), last pairs first: the tail is the rows from
+                             // row0 on, of row0 itself the heads from head_row0 on
+  uint32_t first_tail;       // the items that stay whole come before the tail
+  uint32_t n_units, n_slots, n_tickets;
+};
+RfSplit rf_split_plan(const RfGeom& g, bool sparse, int heads_total, int head0);
+// Bytes of the split region: the tickets (one word per piece-joining warp, zero when a call begins), then the pieces.
+size_t rf_split_ticket_bytes(const RfSplit& sp);
+size_t rf_split_bytes(const RfSplit& sp, int D);
+cudaError_t rf_launch_zero(int32_t* words, int n, cudaStream_t st);
+
 struct RfAttnArgs {
   RfGeom g;
   const int32_t* head_class;  // nullptr: every head Dense, implicit full tile list
@@ -107,10 +131,20 @@ struct RfAttnArgs {
   float* lse;
   int32_t* dev_status;
   float scale_log2;           // log2(e) / sqrt(D)
+  RfSplit sp;
+  int32_t* tickets;           // [n_tickets], zero
+  float* pieces;              // [n_slots][2 streams][D/4 + 1][128 rows] float4: O, then {m, l, l exact, has O}
   int heads_l2 = 1;           // heads whose items are interleaved (filled by the launcher)
 };
 // Tensor maps: [0..2] Q/K/V in original order, [3..5] the workspace copies with N rows per head
 // (position-major Q/K/V of Temporal heads), [6..7] workspace K/V with LkvTex rows per head (Textural).
 constexpr int RF_ATTN_MAPS = 8;
 rf_status rf_launch_attention(const RfAttnArgs& a, const CUtensorMap* maps, cudaStream_t st);
+// rf_sparse_attn_fwd_plus for heads [head0, head0 + B*H) of a call of heads_total heads made in groups; the workspace needs
+// rf_group_workspace_bytes.
+size_t rf_group_workspace_bytes(const rf_shape* shape, const rf_params* params, int heads_total, int head0);
+rf_status rf_sparse_attn_group(const rf_shape* shape, const rf_params* params, const void* q, const void* k, const void* v,
+                               const int32_t* head_class, const int32_t* head_window, const rf_schedule* sched, void* o,
+                               float* lse, void* ws, size_t ws_bytes, int32_t* dev_status, void* cuda_stream, int heads_total,
+                               int head0);
 rf_status rf_launch_selftest_timeout(int32_t* dev_status, uint64_t limit_ns, int32_t* waits_returned, cudaStream_t st);

@@ -10,6 +10,7 @@
 // (a CTA runs for about a millisecond at the large shapes) then leave their SMs to the next group's kernels instead
 // of to nobody.
 // The pipeline object holds streams and events only; device memory comes from the caller in one block.
+#include <algorithm>
 #include <new>
 #include <vector>
 
@@ -53,8 +54,10 @@ bool layout_of(const rf_shape* shape, const rf_params* params, int groups, rf_sh
   gshape->B = 1;
   gshape->H = (int32_t)(heads / groups);
   if (rf_schedule_dims(gshape, params, nQ, nK) != RF_OK) return false;
-  const size_t ws = rf_workspace_bytes(gshape, params);
+  size_t ws = rf_workspace_bytes(gshape, params);
   if (ws == 0) return false;
+  // the groups share their compute stream's workspace
+  for (int g = 0; g < groups; ++g) ws = std::max(ws, rf_group_workspace_bytes(gshape, params, (int)heads, g * gshape->H));
   const size_t N = (size_t)shape->T * shape->frame_h * shape->frame_w + shape->L_text;
   L->tensor = align_up((size_t)heads * N * shape->D * sizeof(__nv_bfloat16));
   L->ws = align_up(ws);
@@ -184,6 +187,7 @@ rf_status rf_host_pipeline_set_bandwidths(rf_host_pipeline* p, const float* band
 rf_status rf_host_pipeline_run(rf_host_pipeline* p, const void* q_host, const void* k_host, const void* v_host, void* o_host,
                                void* wait_stream) {
   if (p == nullptr || q_host == nullptr || k_host == nullptr || v_host == nullptr || o_host == nullptr) return RF_ERR_INVALID_ARG;
+  const int heads = p->groups * p->heads_per_group;
   const size_t gelems = (size_t)p->heads_per_group * p->head_elems, gbytes = gelems * sizeof(__nv_bfloat16);
   auto at = [&](const void* base, int g) { return static_cast<const uint8_t*>(base) + (size_t)g * gbytes; };
 #define RF_TRY(call) do { if ((call) != cudaSuccess) return RF_ERR_CUDA; } while (0)
@@ -210,14 +214,14 @@ rf_status rf_host_pipeline_run(rf_host_pipeline* p, const void* q_host, const vo
                                 run);
       if (st == RF_OK) st = rf_build_block_mask_plus(&p->gshape, &p->params, hc, hw, &p->sched[r], p->status, run);
       if (st == RF_OK)
-        st = rf_sparse_attn_fwd_plus(&p->gshape, &p->params, q, k, v, hc, hw, &p->sched[r], p->o + g * gelems, nullptr, p->ws[r],
-                                     p->ws_bytes, p->status, run);
+        st = rf_sparse_attn_group(&p->gshape, &p->params, q, k, v, hc, hw, &p->sched[r], p->o + g * gelems, nullptr, p->ws[r],
+                                  p->ws_bytes, p->status, run, heads, g * p->heads_per_group);
     } else {
       st = rf_arm_classify(&p->gshape, &p->params, q, k, hc, nullptr, p->ws[r], p->ws_bytes, p->status, run);
       if (st == RF_OK) st = rf_build_block_mask(&p->gshape, &p->params, hc, &p->sched[r], p->status, run);
       if (st == RF_OK)
-        st = rf_sparse_attn_fwd(&p->gshape, &p->params, q, k, v, hc, &p->sched[r], p->o + g * gelems, nullptr, p->ws[r],
-                                p->ws_bytes, p->status, run);
+        st = rf_sparse_attn_group(&p->gshape, &p->params, q, k, v, hc, nullptr, &p->sched[r], p->o + g * gelems, nullptr, p->ws[r],
+                                  p->ws_bytes, p->status, run, heads, g * p->heads_per_group);
     }
     if (st != RF_OK) return st;
     RF_TRY(cudaEventRecord(p->run_done[g], run));

@@ -163,9 +163,12 @@ constexpr int kGatherRows = 4;
 __global__ void __launch_bounds__(256) rf_gather_kernel(RfGeom g, const int32_t* __restrict__ head_class,
                                                          const uint4* __restrict__ q, const uint4* __restrict__ k,
                                                          const uint4* __restrict__ v, uint4* __restrict__ wq,
-                                                         uint4* __restrict__ wk, uint4* __restrict__ wv, int32_t* dev_status) {
+                                                         uint4* __restrict__ wk, uint4* __restrict__ wv, int32_t* tickets,
+                                                         int n_tickets, int32_t* dev_status) {
   rf_grid_trigger();
   rf_grid_wait();
+  if (blockIdx.y == 0)   // the attention kernel's tickets start at zero
+    for (int i = blockIdx.x * 256 + threadIdx.x; i < n_tickets; i += gridDim.x * 256) tickets[i] = 0;
   const int bh = blockIdx.y;
   const int cls = head_class[bh];
   const bool perm = cls == RF_TEMPORAL && g.permute;
@@ -221,7 +224,17 @@ __global__ void __launch_bounds__(256) rf_gather_kernel(RfGeom g, const int32_t*
   }
 }
 
+__global__ void __launch_bounds__(256) rf_zero_kernel(int32_t* words, int n) {
+  rf_grid_trigger();
+  rf_grid_wait();
+  for (int i = blockIdx.x * 256 + threadIdx.x; i < n; i += gridDim.x * 256) words[i] = 0;
+}
+
 }  // namespace
+
+cudaError_t rf_launch_zero(int32_t* words, int n, cudaStream_t st) {
+  return rf_launch(rf_zero_kernel, dim3(rf_cdiv(n, 1024)), 256, 0, st, words, n);
+}
 
 cudaError_t rf_launch_build_tiles(const RfGeom& g, const int32_t* head_class, const int32_t* head_window, int32_t* count,
                                   int32_t* kv_tile, uint32_t* bitmap, int32_t* kv_len, int32_t* dev_status, cudaStream_t st) {
@@ -231,8 +244,8 @@ cudaError_t rf_launch_build_tiles(const RfGeom& g, const int32_t* head_class, co
 
 cudaError_t rf_launch_gather(const RfGeom& g, const int32_t* head_class, const __nv_bfloat16* q,
                              const __nv_bfloat16* k, const __nv_bfloat16* v, __nv_bfloat16* wq, __nv_bfloat16* wk,
-                             __nv_bfloat16* wv, int32_t* dev_status, cudaStream_t st) {
+                             __nv_bfloat16* wv, int32_t* tickets, int n_tickets, int32_t* dev_status, cudaStream_t st) {
   const int rows_per_cta = 256 / (g.D / 8) * kGatherRows;
   return rf_launch(rf_gather_kernel, dim3(rf_cdiv(g.N, rows_per_cta), g.B * g.H), 256, 0, st, g, head_class, (const uint4*)q,
-                   (const uint4*)k, (const uint4*)v, (uint4*)wq, (uint4*)wk, (uint4*)wv, dev_status);
+                   (const uint4*)k, (const uint4*)v, (uint4*)wq, (uint4*)wk, (uint4*)wv, tickets, n_tickets, dev_status);
 }
