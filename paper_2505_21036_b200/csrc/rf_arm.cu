@@ -1,20 +1,27 @@
 // ARM: Adaptive Recognition Module (Sec. 3.3, Eq. 6, Algorithm 1).
 //
 // The sampled score matrix S' = Q' K'^T / sqrt(d) is a dense contraction, so it runs on tcgen05 like the
-// attention kernel, minus everything that concerns V: one CTA takes two 128-row tiles of sampled queries
-// ("streams") of one head and walks all 128-key tiles of the sample.  Sampled rows are fetched straight
-// from Q and K by TMA through tensor maps whose row stride is omega tokens (no gather pass).  Warp roles:
-//   warps 0-3 / 4-7  softmax statistics of stream 0 / 1 (one thread per sampled query row)
-//   warp 8           TMA producer: both Q tiles once, then K tiles into a shared-memory ring
-//   warp 9           MMA issuer; each stream's S accumulator is double-buffered in TMEM (4 x 128 columns),
-//                    so the next tile's scores are computed while the current ones are being reduced
-// Per tile a softmax thread reads its row of S (tcgen05.ld), hands the buffer back, and updates an
-// online softmax (running maximum, total mass) plus the masked masses Algorithm 1 needs: the share of
-// the row kept by the sampled Temporal / Spatial (/ Textural, when recalls are requested) mask.
+// attention kernel, minus everything that concerns V: one CTA takes one 128-row tile of sampled queries of one
+// head and walks all 128-key tiles of the sample.  Sampled rows are fetched straight from Q and K by TMA through
+// tensor maps whose row stride is omega tokens (no gather pass).  Warp roles:
+//   warps 0-3 / 4-7  softmax statistics of the even / odd key tiles (one thread per sampled query row)
+//   warp 8           TMA producer: the Q tile once, then K tiles into a shared-memory ring
+//   warp 9           MMA issuer; S is double-buffered in TMEM (2 x 128 columns), a buffer per warpgroup
+// The kernel is bound by its exponentials (one per score; 1024 cycles of the exponential pipe per warp and tile) once
+// enough warps hide the chain load -> maximum -> exponentials -> sums of each other's tiles: two CTAs share an SM
+// (half of its TMEM, shared memory and registers each), so a sub-partition holds four softmax warps and one CTA's start
+// runs beside the other's tiles.  A thread holds 64 scores at a time and takes the first half from TMEM twice (maximum,
+// then exponentials).  Measured against one CTA per SM with two warps a sub-partition, 128 scores a thread and two
+// query tiles a CTA (rf_arm_classify alone, us): 24 heads, samples of 1024 39.1 -> 29.4; 48 heads, 1170 and 1350, D = 64
+// 94.7 -> 71.5; 24 heads, 3300 and 3600 258 -> 217; with four candidate windows, 1920 and 2040 169 -> 125; with the
+// per-key table (both recalls on the stride sample, 867 of 86 400 tokens) 38.4 -> 31.2.
+// Per tile a softmax thread updates an online softmax (running maximum, total mass) plus the masked masses
+// Algorithm 1 needs: the share of the row kept by the sampled Temporal / Spatial (/ Textural, when recalls are
+// requested) mask; the two warpgroups' statistics of a row are joined at the end.
 // On the first-frame sample positions equal sample indices, and on the stride sample frames grow
-// with the sample index, so a row's kept keys form one index interval: tiles wholly inside or outside
-// it for all 32 rows of a warp cost nothing extra, tiles an edge crosses use a 128-bit keep word per
-// row.  Only the Temporal mask on the stride sample (RF_SAMPLE_GLOBAL) and the Textural diagnostic
+// with the sample index, so a row's kept keys form one index interval: half tiles wholly inside or outside
+// it for all 32 rows of a warp cost nothing extra (which they are is worked out before the scores arrive), those
+// an edge crosses use a 64-bit keep word per row.  Only the Temporal mask on the stride sample (RF_SAMPLE_GLOBAL) and the Textural diagnostic
 // need per-key attributes, computed cooperatively per tile.
 // With the first frame as a key frame of Spatial heads (Sec. 3.2: adjacent or key frames) the Spatial masks keep,
 // in addition, the sampled keys of frame 0, a prefix of the stride sample.
@@ -32,7 +39,8 @@ namespace {
 using namespace sm100;
 
 constexpr int ARM_TILE = 128;
-constexpr int ARM_THREADS = kWsThreads;    // softmax 0, softmax 1, {TMA, MMA, 2 idle warps}
+constexpr int ARM_HALF = 64;               // scores a thread holds at a time
+constexpr int ARM_THREADS = 320;           // softmax of even tiles, of odd tiles, TMA, MMA
 constexpr int ARM_TMA_WARP = 8, ARM_MMA_WARP = 9;
 
 struct ArmMaps { CUtensorMap q[2], k[2]; };   // per sample: 0 = stride sample, 1 = first-frame sample
@@ -42,7 +50,7 @@ constexpr int ARM_MAX_NB = RF_MAX_BANDWIDTHS;   // candidate windows per pattern
 struct ArmSample {
   int n;          // sampled tokens
   int stride;     // token index of sample m is m * stride
-  int pairs;      // CTAs per head: ceil(ceil(n/128) / 2)
+  int tiles;      // CTAs per head: ceil(n / 128)
   int want_t;     // accumulate the Temporal masses on this sample
   int want_s;     // accumulate the Spatial masses on this sample
   float* out;     // [B*H][2*NB+1][n_pad]: Temporal per window, Spatial per window, Textural
@@ -55,16 +63,17 @@ struct ArmCfg {
   static constexpr int COL1 = 64;   // D = 96: the second 64-column box reaches past the tensor and is zero-filled
   static constexpr uint32_t BLK = 128 * 128;
   static constexpr uint32_t TILE = KB * BLK;
-  static constexpr int NK = D == 64 ? 6 : 4;
+  static constexpr int NK = D == 64 ? 4 : 2;
   static constexpr uint32_t Q = 0;
-  static constexpr uint32_t K0 = Q + 2 * TILE;
+  static constexpr uint32_t K0 = Q + TILE;
   static constexpr uint32_t BAR = K0 + NK * TILE;
-  static constexpr int B_Q = 0, B_KF = 1, B_KE = B_KF + NK, B_SF = B_KE + NK, B_SE = B_SF + 4, B_COUNT = B_SE + 4;
+  static constexpr int B_Q = 0, B_KF = 1, B_KE = B_KF + NK, B_SF = B_KE + NK, B_SE = B_SF + 2, B_COUNT = B_SE + 2;
   static constexpr uint32_t MISC = BAR + 8 * ((B_COUNT + 7) / 8 * 8);
   static constexpr uint32_t ATTR = MISC + 64;                    // int [8 warps][2][128]: key position / checkerboard flag
-  static constexpr uint32_t TOTAL = ATTR + 8 * 2 * 128 * 4;
+  static constexpr uint32_t JOIN = ATTR + 8 * 2 * 128 * 4;       // float [masks + 2][128]: the odd tiles' statistics
+  static constexpr uint32_t TOTAL = JOIN + (2 * ARM_MAX_NB + 3) * 128 * 4;
   static constexpr uint32_t ALLOC = TOTAL + 1024;
-  static_assert(ALLOC <= 227 * 1024, "exceeds the shared memory a CTA can opt in to");
+  static_assert(2 * (ALLOC + 1024) <= 228 * 1024, "two CTAs exceed the shared memory of an SM");
   static __host__ __device__ constexpr uint32_t koff(int ks) {
     return ks < 4 ? (uint32_t)ks * 32u : BLK + (uint32_t)(ks - 4) * 32u;
   }
@@ -76,19 +85,72 @@ __device__ __forceinline__ float ex2f(float x) {
   return y;
 }
 __device__ __forceinline__ uint32_t bits_below(int n) { return n >= 32 ? 0xffffffffu : ((1u << n) - 1u); }
-// Bits of the tile starting at key u0 that fall in the key interval [a, b).
-__device__ __forceinline__ void interval_bits(uint32_t (&w)[4], int u0, int a, int b) {
+// Bits of the half tile starting at key u0 that fall in the key interval [a, b).
+__device__ __forceinline__ void interval_bits(uint32_t (&w)[2], int u0, int a, int b) {
   a = max(a - u0, 0);
-  b = min(b - u0, ARM_TILE);
+  b = min(b - u0, ARM_HALF);
 #pragma unroll
-  for (int k = 0; k < 4; ++k) {
+  for (int k = 0; k < 2; ++k) {
     const int lo = min(max(a - 32 * k, 0), 32), hi = min(max(b - 32 * k, 0), 32);
-    w[k] = hi > lo ? (bits_below(hi) & ~bits_below(lo)) : 0u;
+    w[k] |= hi > lo ? (bits_below(hi) & ~bits_below(lo)) : 0u;
   }
+}
+__device__ __forceinline__ void load_half(uint32_t t_s, uint32_t (&s)[ARM_HALF]) {
+  tmem_ld32(t_s, *reinterpret_cast<uint32_t(*)[32]>(&s[0]));
+  tmem_ld32(t_s + 32, *reinterpret_cast<uint32_t(*)[32]>(&s[32]));
+  tc_wait_ld();
+}
+// Keys past the sample score -inf; returns the largest of the others (or mx).
+__device__ __forceinline__ float half_max(uint32_t (&s)[ARM_HALF], int u0, int n, float mx) {
+  if (u0 + ARM_HALF > n) {
+#pragma unroll
+    for (int c = 0; c < ARM_HALF; ++c)
+      if (u0 + c >= n) s[c] = 0xff800000u;
+  }
+  float m0 = mx, m1 = -INFINITY;
+#pragma unroll
+  for (int c = 0; c < ARM_HALF; c += 4) {
+    m0 = fmaxf(m0, fmaxf(__uint_as_float(s[c]), __uint_as_float(s[c + 1])));
+    m1 = fmaxf(m1, fmaxf(__uint_as_float(s[c + 2]), __uint_as_float(s[c + 3])));
+  }
+  return fmaxf(m0, m1);
+}
+// Exponentials in place, 2^(score * sc - m); returns their sum.
+__device__ __forceinline__ float half_exp(uint32_t (&s)[ARM_HALF], float sc, float m) {
+  const float2 sc2 = make_float2(sc, sc), mneg = make_float2(-m, -m);
+  float2 la = make_float2(0.f, 0.f), lb = make_float2(0.f, 0.f);
+#pragma unroll
+  for (int c = 0; c < ARM_HALF; c += 4) {
+    float2 e0 = __ffma2_rn(make_float2(__uint_as_float(s[c]), __uint_as_float(s[c + 1])), sc2, mneg);
+    float2 e1 = __ffma2_rn(make_float2(__uint_as_float(s[c + 2]), __uint_as_float(s[c + 3])), sc2, mneg);
+    e0.x = ex2f(e0.x); e0.y = ex2f(e0.y);
+    e1.x = ex2f(e1.x); e1.y = ex2f(e1.y);
+    la = __fadd2_rn(la, e0);
+    lb = __fadd2_rn(lb, e1);
+    s[c] = __float_as_uint(e0.x); s[c + 1] = __float_as_uint(e0.y);
+    s[c + 2] = __float_as_uint(e1.x); s[c + 3] = __float_as_uint(e1.y);
+  }
+  return (la.x + la.y) + (lb.x + lb.y);
+}
+
+// Sum of the weights whose key's attribute (table in shared memory, 16-byte aligned) is kept; four chains of additions.
+template <typename F>
+__device__ __forceinline__ float table_sum(const uint32_t (&s)[ARM_HALF], const int* table, F kept) {
+  const int4* t = reinterpret_cast<const int4*>(table);
+  float p0 = 0.f, p1 = 0.f, p2 = 0.f, p3 = 0.f;
+#pragma unroll
+  for (int c = 0; c < ARM_HALF; c += 4) {
+    const int4 a = t[c / 4];
+    p0 += kept(a.x) ? __uint_as_float(s[c]) : 0.f;
+    p1 += kept(a.y) ? __uint_as_float(s[c + 1]) : 0.f;
+    p2 += kept(a.z) ? __uint_as_float(s[c + 2]) : 0.f;
+    p3 += kept(a.w) ? __uint_as_float(s[c + 3]) : 0.f;
+  }
+  return (p0 + p1) + (p2 + p3);
 }
 
 template <int D, int NB, bool TEX>
-__global__ void __launch_bounds__(ARM_THREADS, 1) rf_arm_kernel(const __grid_constant__ ArmMaps maps, const RfGeom g,
+__global__ void __launch_bounds__(ARM_THREADS, 2) rf_arm_kernel(const __grid_constant__ ArmMaps maps, const RfGeom g,
                                                                 const ArmSample sm0, const ArmSample sm1,
                                                                 const ArmWindows win, int n_pad, float scale_log2,
                                                                 int32_t* arm_flag) {
@@ -104,14 +166,12 @@ __global__ void __launch_bounds__(ARM_THREADS, 1) rf_arm_kernel(const __grid_con
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int bh = blockIdx.y;
   // blockIdx.x enumerates the CTAs of the stride sample first, then those of the first-frame sample
-  const bool second = (int)blockIdx.x >= sm0.pairs;
+  const bool second = (int)blockIdx.x >= sm0.tiles;
   const ArmSample& sm = second ? sm1 : sm0;
   const int which = second ? 1 : 0;
-  const int pair = second ? blockIdx.x - sm0.pairs : blockIdx.x;
+  const int qt = second ? blockIdx.x - sm0.tiles : blockIdx.x;
   const int n = sm.n, stride = sm.stride;
   const int nt = rf_cdiv(n, ARM_TILE);
-  const int qt0 = 2 * pair;
-  const bool stream1 = qt0 + 1 < nt;
   const CUtensorMap* map_q = &maps.q[which];
   const CUtensorMap* map_k = &maps.k[which];
   // positions equal sample indices only while the sample is contiguous and stays inside the first frame
@@ -121,14 +181,14 @@ __global__ void __launch_bounds__(ARM_THREADS, 1) rf_arm_kernel(const __grid_con
   if (tid == 0) {
     mbar_init(bar(C::B_Q), 1);
     for (int s = 0; s < C::NK; ++s) { mbar_init(bar(C::B_KF + s), 1); mbar_init(bar(C::B_KE + s), 1); }
-    for (int s = 0; s < 4; ++s) { mbar_init(bar(C::B_SF + s), 1); mbar_init(bar(C::B_SE + s), 4); }
+    for (int s = 0; s < 2; ++s) { mbar_init(bar(C::B_SF + s), 1); mbar_init(bar(C::B_SE + s), 4); }
     *abort_flag = 0;
     mbar_init_fence();
   }
   if (warp == ARM_TMA_WARP) {
     if (lane == 0) { prefetch_tmap(map_q); prefetch_tmap(map_k); }
     __syncwarp();
-    tmem_alloc(smem_u32(const_cast<uint32_t*>(tmem_slot)), 512);
+    tmem_alloc(smem_u32(const_cast<uint32_t*>(tmem_slot)), 2 * ARM_TILE);
   }
   tc_fence_before();
   __syncthreads();
@@ -143,208 +203,172 @@ __global__ void __launch_bounds__(ARM_THREADS, 1) rf_arm_kernel(const __grid_con
   if (blockIdx.x == 0 && blockIdx.y == 0 && tid == 0) *arm_flag = 0;
 #endif
 
-  if (warp >= 8) {
-    RF_SETMAXNREG_DEC();
-    if (warp == ARM_TMA_WARP) {
-      if (lane == 0) {
-        mbar_expect_tx(bar(C::B_Q), 2 * C::TILE);
+  // Masks k = 0..NB-1: Temporal with window win.ws[k]; k = NB..2NB-1: Spatial with win.wf[k-NB];
+  // k = 2NB: Textural.  Band masks keep one key interval per row in sample-index space.
+  constexpr int NM = 2 * NB + 1;
+  float mx = -INFINITY, l_all = 0.f;
+  float l_m[NM];
 #pragma unroll
-        for (int j = 0; j < 2; ++j)
+  for (int k = 0; k < NM; ++k) l_m[k] = 0.f;
+  float* join = reinterpret_cast<float*>(base_ptr + C::JOIN) + (tid & 127);
+  const int m = qt * ARM_TILE + (tid & 127);                   // sampled row of a softmax thread
+
+  if (warp == ARM_TMA_WARP) {
+    if (lane == 0) {
+      mbar_expect_tx(bar(C::B_Q), C::TILE);
 #pragma unroll
-          for (int kb = 0; kb < C::KB; ++kb)
-            tma_load_3d(base + C::Q + j * C::TILE + kb * C::BLK, map_q, kb * C::COL1, (qt0 + j) * ARM_TILE, bh, bar(C::B_Q));
-        for (int u = 0; u < nt; ++u) {
-          const int ks = u % C::NK;
-          if (u >= C::NK) mbar_wait(bar(C::B_KE + ks), ((u / C::NK) - 1) & 1, wc);
-          mbar_expect_tx(bar(C::B_KF + ks), C::TILE);
+      for (int kb = 0; kb < C::KB; ++kb)
+        tma_load_3d(base + C::Q + kb * C::BLK, map_q, kb * C::COL1, qt * ARM_TILE, bh, bar(C::B_Q));
+      for (int u = 0; u < nt; ++u) {
+        const int ks = u % C::NK;
+        if (u >= C::NK) mbar_wait(bar(C::B_KE + ks), ((u / C::NK) - 1) & 1, wc);
+        mbar_expect_tx(bar(C::B_KF + ks), C::TILE);
 #pragma unroll
-          for (int kb = 0; kb < C::KB; ++kb)
-            tma_load_3d(base + C::K0 + ks * C::TILE + kb * C::BLK, map_k, kb * C::COL1, u * ARM_TILE, bh, bar(C::B_KF + ks));
-        }
+        for (int kb = 0; kb < C::KB; ++kb)
+          tma_load_3d(base + C::K0 + ks * C::TILE + kb * C::BLK, map_k, kb * C::COL1, u * ARM_TILE, bh, bar(C::B_KF + ks));
       }
-    } else if (warp == ARM_MMA_WARP) {
-      if (lane == 0) {
-        constexpr uint32_t DESC_HI = (1024u >> 4) | (1u << 14) | (2u << 29);
-        auto desc = [](uint32_t lo) -> uint64_t { return ((uint64_t)DESC_HI << 32) | lo; };
-        const uint32_t q_lo = ((base + C::Q) >> 4) | (1u << 16), k_lo = ((base + C::K0) >> 4) | (1u << 16);
-        mbar_wait(bar(C::B_Q), 0, wc);
-        for (int u = 0; u < nt; ++u) {
-          const int ks = u % C::NK, b = u & 1;
-          mbar_wait(bar(C::B_KF + ks), (u / C::NK) & 1, wc);
+    }
+  } else if (warp == ARM_MMA_WARP) {
+    if (lane == 0) {
+      constexpr uint32_t DESC_HI = (1024u >> 4) | (1u << 14) | (2u << 29);
+      auto desc = [](uint32_t lo) -> uint64_t { return ((uint64_t)DESC_HI << 32) | lo; };
+      const uint32_t q_lo = ((base + C::Q) >> 4) | (1u << 16), k_lo = ((base + C::K0) >> 4) | (1u << 16);
+      mbar_wait(bar(C::B_Q), 0, wc);
+      for (int u = 0; u < nt; ++u) {
+        const int ks = u % C::NK, b = u & 1;
+        mbar_wait(bar(C::B_KF + ks), (u / C::NK) & 1, wc);
+        if (u >= 2) mbar_wait(bar(C::B_SE + b), ((u >> 1) - 1) & 1, wc);
+        tc_fence_after();
+        const uint32_t b0 = k_lo + ks * (C::TILE >> 4);
 #pragma unroll
-          for (int j = 0; j < 2; ++j) {
-            if (j == 1 && !stream1) continue;
-            if (u >= 2) mbar_wait(bar(C::B_SE + j * 2 + b), ((u >> 1) - 1) & 1, wc);
-            tc_fence_after();
-            const uint32_t a0 = q_lo + j * (C::TILE >> 4), b0 = k_lo + ks * (C::TILE >> 4);
-#pragma unroll
-            for (int k = 0; k < D / 16; ++k)
-              mma_ss(tmem_base + (j * 2 + b) * 128, desc(a0 + (C::koff(k) >> 4)), desc(b0 + (C::koff(k) >> 4)), IDESC_S, k > 0);
-            tc_commit(bar(C::B_SF + j * 2 + b));
-          }
-          tc_commit(bar(C::B_KE + ks));
-        }
+        for (int k = 0; k < D / 16; ++k)
+          mma_ss(tmem_base + b * ARM_TILE, desc(q_lo + (C::koff(k) >> 4)), desc(b0 + (C::koff(k) >> 4)), IDESC_S, k > 0);
+        tc_commit(bar(C::B_SF + b));
+        tc_commit(bar(C::B_KE + ks));
       }
     }
   } else {
-    RF_SETMAXNREG_INC();
-    const int j = warp >> 2;
-    if (j == 0 || stream1) {
-      const int m = (qt0 + j) * ARM_TILE + (tid & 127);          // sampled row of this thread
-      const int mc = min(m, n - 1);
-      const int tok = mc * stride;
-      const int rf = tok / g.S, rp = tok - rf * g.S;
-      const int ry = rp / g.Wf, rx = rp - ry * g.Wf;
-      // Masks k = 0..NB-1: Temporal with window win.ws[k]; k = NB..2NB-1: Spatial with win.wf[k-NB];
-      // k = 2NB: Textural.  Band masks keep one key interval [lo, hi) per row in sample-index space.
-      constexpr int NM = 2 * NB + 1;
-      int lo[2 * NB], hi[2 * NB];
+    const int grp = warp >> 2;                                 // even or odd key tiles
+    const int tok = min(m, n - 1) * stride;
+    const int rf = tok / g.S, rp = tok - rf * g.S;
+    const int ry = rp / g.Wf, rx = rp - ry * g.Wf;
+    int slo[NB], shi[NB];                                      // Spatial: stride sample, frames grow with the index
 #pragma unroll
-      for (int i = 0; i < NB; ++i) {
-        lo[i] = rp - win.ws[i];                                     // first-frame sample: position = index
-        hi[i] = rp + win.ws[i] + 1;
-        lo[NB + i] = rf_cdiv(max(rf - win.wf[i], 0) * g.S, stride);  // stride sample: frames grow with the index
-        hi[NB + i] = rf_cdiv((rf + win.wf[i] + 1) * g.S, stride);
-      }
-      const uint32_t t_s = tmem_base + ((uint32_t)((warp & 3) * 32) << 16) + j * 256;
-      int* attr_p = reinterpret_cast<int*>(base_ptr + C::ATTR) + warp * 256;           // per-warp tables
-      int* attr_c = attr_p + 128;
-      float mx = -INFINITY, l_all = 0.f;
-      float l_m[NM];
-#pragma unroll
-      for (int k = 0; k < NM; ++k) l_m[k] = 0.f;
+    for (int i = 0; i < NB; ++i) {
+      slo[i] = rf_cdiv(max(rf - win.wf[i], 0) * g.S, stride);
+      shi[i] = rf_cdiv((rf + win.wf[i] + 1) * g.S, stride);
+    }
+    // Spatial masks with the first frame as key frame also keep the sampled keys of frame 0: a prefix
+    // [0, pre) of the stride sample, the same for every row
+    const int pre = g.key_first ? rf_cdiv(g.S, stride) : 0;
+    const uint32_t t_s = tmem_base + ((uint32_t)((warp & 3) * 32) << 16) + grp * ARM_TILE;
+    int* attr_p = reinterpret_cast<int*>(base_ptr + C::ATTR) + warp * 256;           // per-warp tables
+    int* attr_c = attr_p + 128;
+    const bool by_table_t = sm.want_t && t_generic;
 
-      for (int u = 0; u < nt; ++u) {
-        const int b = u & 1, u0 = u * ARM_TILE;
-        mbar_wait(bar(C::B_SF + j * 2 + b), (u >> 1) & 1, wc);
-        tc_fence_after();
-        uint32_t s[128];
-        {
-          uint32_t(&s0)[32] = *reinterpret_cast<uint32_t(*)[32]>(&s[0]);
-          uint32_t(&s1)[32] = *reinterpret_cast<uint32_t(*)[32]>(&s[32]);
-          uint32_t(&s2)[32] = *reinterpret_cast<uint32_t(*)[32]>(&s[64]);
-          uint32_t(&s3)[32] = *reinterpret_cast<uint32_t(*)[32]>(&s[96]);
-          tmem_ld32(t_s + b * 128, s0);
-          tmem_ld32(t_s + b * 128 + 32, s1);
-          tmem_ld32(t_s + b * 128 + 64, s2);
-          tmem_ld32(t_s + b * 128 + 96, s3);
-          tc_wait_ld();
-        }
-        tc_fence_before();
+    for (int u = grp; u < nt; u += 2) {
+      const int u0 = u * ARM_TILE;
+      if (by_table_t || TEX) {
+        // per-key attributes of the tile, four keys per lane, into this warp's table
         __syncwarp();
-        if (lane == 0) mbar_arrive(bar(C::B_SE + j * 2 + b));   // the buffer may be refilled
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const int c = lane * 4 + i;
+          const int ktok = min(u0 + c, n - 1) * stride;
+          const int kp = ktok % g.S;
+          const int y = kp / g.Wf, x = kp - y * g.Wf;
+          attr_p[c] = g.t2d ? ((y << 16) | x) : kp;    // frame dimensions stay below 2^15 with the 2-D window
+          attr_c[c] = (y % g.tau) == (x % g.tau);
+        }
+        __syncwarp();
+      }
+      // Per mask and half tile, two bits: 2 - the half lies inside the row's kept interval for the whole warp (its sum
+      // is added), 0 - outside it (nothing), 1 - an edge crosses it, or the mask goes by the table.
+      uint32_t cls[2];
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int c0 = u0 + h * ARM_HALF, c1 = min(c0 + ARM_HALF, n);
+        uint32_t bits = 0;
+        if (c0 < n) {
+#pragma unroll
+          for (int i = 0; i < NB; ++i) {
+            if (sm.want_t) {
+              const bool in = rp - win.ws[i] <= c0 && c1 <= rp + win.ws[i] + 1;
+              const bool out = c1 <= rp - win.ws[i] || rp + win.ws[i] + 1 <= c0;
+              bits |= (t_generic ? 1u : (__all_sync(0xffffffffu, in) ? 2u : (__all_sync(0xffffffffu, out) ? 0u : 1u))) << (2 * i);
+            }
+            if (sm.want_s) {
+              const bool in = (slo[i] <= c0 && c1 <= shi[i]) || c1 <= pre, out = (c1 <= slo[i] || shi[i] <= c0) && c0 >= pre;
+              bits |= (__all_sync(0xffffffffu, in) ? 2u : (__all_sync(0xffffffffu, out) ? 0u : 1u)) << (2 * (NB + i));
+            }
+          }
+          if (TEX) bits |= 1u << (4 * NB);
+        }
+        cls[h] = bits;
+      }
 
-        if (u0 + ARM_TILE > n) {                                 // keys past the sample
+      mbar_wait(bar(C::B_SF + grp), (u >> 1) & 1, wc);
+      tc_fence_after();
+      uint32_t s[ARM_HALF];
+      load_half(t_s, s);
+      float top = half_max(s, u0, n, -INFINITY);
+      load_half(t_s + ARM_HALF, s);
+      top = half_max(s, u0 + ARM_HALF, n, top);
+      const float m_new = fmaxf(mx, top * scale_log2);   // finite: every tile holds a real key
+      const float corr = ex2f(mx - m_new);
+      l_all *= corr;
 #pragma unroll
-          for (int c = 0; c < 128; ++c)
-            if (u0 + c >= n) s[c] = 0xff800000u;
+      for (int k = 0; k < NM; ++k) l_m[k] *= corr;
+      mx = m_new;
+#pragma unroll 1
+      for (int h = 1; h >= 0; --h) {
+        const int c0 = u0 + h * ARM_HALF;
+        if (h == 0) {
+          load_half(t_s, s);
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(bar(C::B_SE + grp));   // the buffer may be refilled
+          half_max(s, c0, n, -INFINITY);                    // (for the keys past the sample)
         }
-        float m0 = -INFINITY, m1 = -INFINITY;
-#pragma unroll
-        for (int c = 0; c < 128; c += 4) {
-          m0 = fmaxf(m0, fmaxf(__uint_as_float(s[c]), __uint_as_float(s[c + 1])));
-          m1 = fmaxf(m1, fmaxf(__uint_as_float(s[c + 2]), __uint_as_float(s[c + 3])));
-        }
-        const float m_new = fmaxf(mx, fmaxf(m0, m1) * scale_log2);   // finite: every tile holds a real key
-        const float corr = ex2f(mx - m_new);
-        l_all *= corr;
-#pragma unroll
-        for (int k = 0; k < NM; ++k) l_m[k] *= corr;
-        mx = m_new;
-
-        // exponentials once, in place; their sum serves every mask the tile lies wholly inside
-        const float2 sc2 = make_float2(scale_log2, scale_log2), mneg = make_float2(-m_new, -m_new);
-        float2 la = make_float2(0.f, 0.f), lb = make_float2(0.f, 0.f);
-#pragma unroll
-        for (int c = 0; c < 128; c += 4) {
-          float2 e0 = __ffma2_rn(make_float2(__uint_as_float(s[c]), __uint_as_float(s[c + 1])), sc2, mneg);
-          float2 e1 = __ffma2_rn(make_float2(__uint_as_float(s[c + 2]), __uint_as_float(s[c + 3])), sc2, mneg);
-          e0.x = ex2f(e0.x); e0.y = ex2f(e0.y);
-          e1.x = ex2f(e1.x); e1.y = ex2f(e1.y);
-          la = __fadd2_rn(la, e0);
-          lb = __fadd2_rn(lb, e1);
-          s[c] = __float_as_uint(e0.x); s[c + 1] = __float_as_uint(e0.y);
-          s[c + 2] = __float_as_uint(e1.x); s[c + 3] = __float_as_uint(e1.y);
-        }
-        const float bs = (la.x + la.y) + (lb.x + lb.y);
+        const float bs = half_exp(s, scale_log2, mx);
         l_all += bs;
-
-        // per mask: the tile lies inside the row's kept interval for the whole warp (add the tile sum),
-        // outside it (nothing), or an edge crosses it (masked sum with a 128-bit keep word)
-        const int u1 = min(u0 + ARM_TILE, n);
-        bool table_ready = false;
+        const uint32_t bits = h ? cls[1] : cls[0];
+#pragma unroll
+        for (int k = 0; k < NM; ++k)
+          if (((bits >> (2 * k)) & 3u) == 2u) l_m[k] += bs;
+        if ((bits & 0x55555555u) == 0) continue;
 #pragma unroll 1
         for (int k = 0; k < NM; ++k) {
+          if (((bits >> (2 * k)) & 3u) != 1u) continue;
           const bool is_t = k < NB, is_x = k == 2 * NB;
-          if (is_x ? !TEX : (is_t ? !sm.want_t : !sm.want_s)) continue;
-          const bool by_table = is_x || (is_t && t_generic);
-          int cls = 1;
-          int klo = 0, khi = 0, pre = 0;
-          if (!by_table) {
-#pragma unroll
-            for (int i = 0; i < 2 * NB; ++i)
-              if (i == k) { klo = lo[i]; khi = hi[i]; }
-            // Spatial masks with the first frame as key frame also keep the sampled keys of frame 0: a prefix
-            // [0, pre) of the stride sample, the same for every row
-            pre = (!is_t && g.key_first) ? rf_cdiv(g.S, stride) : 0;
-            const bool in = (klo <= u0 && u1 <= khi) || u1 <= pre, out = (u1 <= klo || khi <= u0) && u0 >= pre;
-            cls = __all_sync(0xffffffffu, in) ? 2 : (__all_sync(0xffffffffu, out) ? 0 : 1);
-          }
           float add = 0.f;
-          if (cls == 2) {
-            add = bs;
-          } else if (cls == 1) {
-            uint32_t w[4] = {0, 0, 0, 0};
-            if (!by_table) {
-              interval_bits(w, u0, klo, khi);
-              if (pre > u0) {
-                uint32_t wp[4];
-                interval_bits(wp, u0, 0, pre);
+          if (is_x) {
+            add = table_sum(s, attr_c + h * ARM_HALF, [](int a) { return a != 0; });
+          } else if (is_t && t_generic) {
+            int wk = 0;
 #pragma unroll
-                for (int q4 = 0; q4 < 4; ++q4) w[q4] |= wp[q4];
-              }
+            for (int i = 0; i < NB; ++i)
+              if (i == k) wk = win.ws[i];
+            if (g.t2d) {
+              const int wy = g.wy, wx = g.wx;
+              add = table_sum(s, attr_p + h * ARM_HALF, [=](int a) { return abs((a >> 16) - ry) <= wy && abs((a & 0xffff) - rx) <= wx; });
             } else {
-              if (!table_ready) {
-                // per-key attributes of the tile, four keys per lane, into this warp's table
-                __syncwarp();
-#pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                  const int c = lane * 4 + i;
-                  const int ktok = min(u0 + c, n - 1) * stride;
-                  const int kp = ktok % g.S;
-                  const int y = kp / g.Wf, x = kp - y * g.Wf;
-                  attr_p[c] = g.t2d ? ((y << 16) | x) : kp;    // frame dimensions stay below 2^15 with the 2-D window
-                  attr_c[c] = (y % g.tau) == (x % g.tau);
-                }
-                __syncwarp();
-                table_ready = true;
-              }
-              int wk = 0;
-#pragma unroll
-              for (int i = 0; i < NB; ++i)
-                if (i == k) wk = win.ws[i];
-#pragma unroll
-              for (int q4 = 0; q4 < 4; ++q4) {
-                uint32_t bits = 0;
-#pragma unroll 8
-                for (int c = 0; c < 32; ++c) {
-                  bool keep;
-                  if (is_x) {
-                    keep = attr_c[q4 * 32 + c] != 0;
-                  } else if (g.t2d) {
-                    const int yx = attr_p[q4 * 32 + c];
-                    keep = abs((yx >> 16) - ry) <= g.wy && abs((yx & 0xffff) - rx) <= g.wx;
-                  } else {
-                    const int dp = attr_p[q4 * 32 + c] - rp;
-                    keep = (dp < 0 ? -dp : dp) <= wk;
-                  }
-                  bits |= (keep ? 1u : 0u) << c;
-                }
-                w[q4] = bits;
-              }
+              const int off = wk - rp;                           // |position - rp| <= wk
+              const uint32_t span = 2u * (uint32_t)wk;
+              add = table_sum(s, attr_p + h * ARM_HALF, [=](int a) { return (uint32_t)(a + off) <= span; });
             }
+          } else {
+            int klo = 0, khi = 0;
 #pragma unroll
-            for (int c = 0; c < 128; ++c)
+            for (int i = 0; i < NB; ++i) {
+              if (i == k) { klo = rp - win.ws[i]; khi = rp + win.ws[i] + 1; }
+              if (NB + i == k) { klo = slo[i]; khi = shi[i]; }
+            }
+            uint32_t w[2] = {0, 0};
+            interval_bits(w, c0, klo, khi);
+            if (!is_t && pre > c0) interval_bits(w, c0, 0, pre);
+#pragma unroll
+            for (int c = 0; c < ARM_HALF; ++c)
               if ((w[c >> 5] >> (c & 31)) & 1u) add += __uint_as_float(s[c]);
           }
 #pragma unroll
@@ -352,16 +376,26 @@ __global__ void __launch_bounds__(ARM_THREADS, 1) rf_arm_kernel(const __grid_con
             if (i == k) l_m[i] += add;
         }
       }
-      if (m < n) {
-        float* out = sm.out + (size_t)bh * NM * n_pad;
-        const float inv = 1.f / l_all;
+    }
+    if (grp == 1) {
+      join[0] = mx;
+      join[128] = l_all;
 #pragma unroll
-        for (int k = 0; k < NM; ++k) {
-          const bool is_t = k < NB, is_x = k == 2 * NB;
-          if ((is_x ? TEX : (is_t ? sm.want_t != 0 : sm.want_s != 0)) && rf_in_bounds(m, n_pad, arm_flag))
-            out[(size_t)k * n_pad + m] = l_m[k] * inv;
-        }
-      }
+      for (int k = 0; k < NM; ++k) join[(2 + k) * 128] = l_m[k];
+    }
+  }
+
+  __syncthreads();
+  if (warp < 4 && m < n) {
+    const float m1 = join[0], top = fmaxf(mx, m1);
+    const float f0 = ex2f(mx - top), f1 = ex2f(m1 - top);        // no odd tile: m1 = -inf, factor 0
+    const float inv = 1.f / (l_all * f0 + join[128] * f1);
+    float* out = sm.out + (size_t)bh * NM * n_pad;
+#pragma unroll
+    for (int k = 0; k < NM; ++k) {
+      const bool is_t = k < NB, is_x = k == 2 * NB;
+      if ((is_x ? TEX : (is_t ? sm.want_t != 0 : sm.want_s != 0)) && rf_in_bounds(m, n_pad, arm_flag))
+        out[(size_t)k * n_pad + m] = (l_m[k] * f0 + join[(2 + k) * 128] * f1) * inv;
     }
   }
 
@@ -370,7 +404,7 @@ __global__ void __launch_bounds__(ARM_THREADS, 1) rf_arm_kernel(const __grid_con
   if (warp == ARM_TMA_WARP) {
     if (*abort_flag) __nanosleep(20000);
     __syncwarp();
-    tmem_dealloc(tmem_base, 512);
+    tmem_dealloc(tmem_base, 2 * ARM_TILE);
   }
 }
 
@@ -465,12 +499,13 @@ cudaError_t launch_arm_t(const ArmMaps& maps, const RfGeom& g, const ArmSample& 
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
   if (dev >= 0 && dev < 64 && !configured[dev]) {
-    if (!rf_regs_ok(rf_arm_kernel<D, NB, TEX>)) return cudaErrorLaunchOutOfResources;   // setmaxnreg.inc could never be granted
     e = cudaFuncSetAttribute(rf_arm_kernel<D, NB, TEX>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ArmCfg<D>::ALLOC);
+    if (e != cudaSuccess) return e;
+    e = cudaFuncSetAttribute(rf_arm_kernel<D, NB, TEX>, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
     if (e != cudaSuccess) return e;
     configured[dev] = true;
   }
-  dim3 grid(s0.pairs + s1.pairs, g.B * g.H);
+  dim3 grid(s0.tiles + s1.tiles, g.B * g.H);
   const float scale_log2 = 1.4426950408889634f / sqrtf((float)D);
   return rf_launch(rf_arm_kernel<D, NB, TEX>, grid, ARM_THREADS, ArmCfg<D>::ALLOC, st, maps, g, s0, s1, win, n_pad, scale_log2, arm_flag);
 }
@@ -524,9 +559,9 @@ cudaError_t rf_launch_arm(const RfGeom& g, int sample_mode, int omega, float alp
             rf_encode_rows_map(&maps.k[1], k, g.D, n_loc, row_bytes, head_bytes, heads);
   if (!ok) return cudaErrorUnknown;
   ArmSample s0, s1;
-  s0.n = n_glb; s0.stride = omega; s0.pairs = rf_cdiv(rf_cdiv(n_glb, ARM_TILE), 2);
+  s0.n = n_glb; s0.stride = omega; s0.tiles = rf_cdiv(n_glb, ARM_TILE);
   s0.want_t = alg1 ? 0 : 1; s0.want_s = 1; s0.out = rows_glb;
-  s1.n = n_loc; s1.stride = 1; s1.pairs = alg1 ? rf_cdiv(rf_cdiv(n_loc, ARM_TILE), 2) : 0;
+  s1.n = n_loc; s1.stride = 1; s1.tiles = alg1 ? rf_cdiv(n_loc, ARM_TILE) : 0;
   s1.want_t = 1; s1.want_s = 0; s1.out = rows_loc;
   cudaError_t e = cudaSuccess;
 #ifdef RF_BOUNDS_CHECK
