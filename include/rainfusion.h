@@ -235,6 +235,17 @@ rf_status rf_sparse_attn_fwd_plus(const rf_shape *shape, const rf_params *params
                                   int32_t *dev_status, void *cuda_stream);
 
 /*
+ * One sparse call as a sampler makes it (Fig. 2a): rf_arm_classify, rf_build_block_mask and rf_sparse_attn_fwd one after the
+ * other on the stream, or their _plus forms when n_bandwidths > 0 (head_window is then written, else it may be NULL).  The
+ * same launches and the same results; a caller at the end of a foreign-function interface crosses it once instead of three times.
+ * Returns the first status that is not RF_OK.  Arguments as for the three calls.
+ */
+rf_status rf_sparse_call(const rf_shape *shape, const rf_params *params, const float *bandwidths, int32_t n_bandwidths,
+                         const void *q, const void *k, const void *v, int32_t *head_class, int32_t *head_window,
+                         rf_schedule *sched, void *o, float *lse, void *ws, size_t ws_bytes, int32_t *dev_status,
+                         void *cuda_stream);
+
+/*
  * The whole path of Fig. 2a (ARM of Sec. 3.3 -> masks of Sec. 3.2 -> masked attention, Eq. 1-2) for callers whose
  * Q, K, V and O live in HOST memory.  Heads are independent at every stage (Algorithm 1 outputs one category per
  * head), so a run is pipelined over `head_groups` groups of heads (head_groups must divide B*H) on streams of the

@@ -20,7 +20,7 @@ _LIB_PATH = os.environ.get("RAINFUSION_LIBRARY") or os.path.join(os.path.dirname
 _lib = None
 
 EXPORTS = ["rf_status_string", "rf_schedule_dims", "rf_workspace_bytes", "rf_arm_classify",
-           "rf_build_block_mask", "rf_reorder_tokens", "rf_sparse_attn_fwd", "rf_dense_attn_fwd", "rf_dense_workspace_bytes",
+           "rf_build_block_mask", "rf_reorder_tokens", "rf_sparse_attn_fwd", "rf_dense_attn_fwd", "rf_dense_workspace_bytes", "rf_sparse_call",
            "rf_arm_classify_noalloc", "rf_selftest_wait_timeout", "rf_arm_classify_plus", "rf_build_block_mask_plus", "rf_sparse_attn_fwd_plus",
            "rf_sparse_attn_reordered", "rf_selftest_arm_abandoned", "rf_bounds_checked", "rf_host_pipeline_staging_bytes",
            "rf_host_pipeline_create", "rf_host_pipeline_run", "rf_host_pipeline_status", "rf_host_pipeline_destroy",
@@ -107,6 +107,8 @@ def load():
     lib.rf_selftest_wait_timeout.argtypes = [V, C.c_int32, V, V]
     lib.rf_reorder_tokens.restype = I
     lib.rf_reorder_tokens.argtypes = [P(rf_shape), P(rf_params), V, V, V, V, V, Z, V]
+    lib.rf_sparse_call.restype = I
+    lib.rf_sparse_call.argtypes = [P(rf_shape), P(rf_params), P(C.c_float), C.c_int32, V, V, V, V, V, P(rf_schedule), V, V, V, Z, V, V]
     lib.rf_dense_workspace_bytes.restype = Z
     lib.rf_dense_workspace_bytes.argtypes = [P(rf_shape)]
     lib.rf_dense_attn_fwd.restype = I
@@ -251,6 +253,15 @@ def rf_selftest_arm_abandoned(shape, params, q, k, head_class, ws, dev_status):
     _check(load().rf_selftest_arm_abandoned(C.byref(shape), C.byref(params), q.data_ptr(), k.data_ptr(),
                                             head_class.data_ptr(), ws.data_ptr(), ws.numel(), _ptr(dev_status), _stream()),
            "rf_selftest_arm_abandoned")
+
+
+def rf_sparse_call(shape, params, bandwidths, q, k, v, head_class, head_window, sched: Schedule, o, lse, ws, dev_status=None):
+    """ARM -> schedule -> masked attention in one crossing into the library (bandwidths: None, or the candidates)."""
+    n = len(bandwidths) if bandwidths else 0
+    arr = (C.c_float * n)(*bandwidths) if n else None
+    _check(load().rf_sparse_call(C.byref(shape), C.byref(params), arr, n, q.data_ptr(), k.data_ptr(), v.data_ptr(),
+                                 head_class.data_ptr(), _ptr(head_window), C.byref(sched.c), o.data_ptr(), _ptr(lse),
+                                 ws.data_ptr(), ws.numel(), _ptr(dev_status), _stream()), "rf_sparse_call")
 
 
 class HostPipeline:

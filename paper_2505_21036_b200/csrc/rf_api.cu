@@ -444,6 +444,20 @@ rf_status rf_sparse_attn_reordered(const rf_shape* shape, const rf_params* param
                           cuda_stream, false, shape != nullptr ? shape->B * shape->H : 0, 0);
 }
 
+rf_status rf_sparse_call(const rf_shape* shape, const rf_params* params, const float* bandwidths, int32_t n_bandwidths, const void* q,
+                         const void* k, const void* v, int32_t* head_class, int32_t* head_window, rf_schedule* sched, void* o,
+                         float* lse, void* ws, size_t ws_bytes, int32_t* dev_status, void* cuda_stream) {
+  if (n_bandwidths < 0) return RF_ERR_INVALID_ARG;
+  if (n_bandwidths == 0) head_window = nullptr;
+  rf_status st = n_bandwidths > 0 ? rf_arm_classify_plus(shape, params, bandwidths, n_bandwidths, q, k, head_class, head_window,
+                                                         nullptr, ws, ws_bytes, dev_status, cuda_stream)
+                                  : rf_arm_classify(shape, params, q, k, head_class, nullptr, ws, ws_bytes, dev_status, cuda_stream);
+  if (st == RF_OK) st = rf_build_block_mask_plus(shape, params, head_class, head_window, sched, dev_status, cuda_stream);
+  if (st == RF_OK)
+    st = rf_sparse_attn_fwd_plus(shape, params, q, k, v, head_class, head_window, sched, o, lse, ws, ws_bytes, dev_status, cuda_stream);
+  return st;
+}
+
 rf_status rf_selftest_wait_timeout(int32_t* dev_status, int32_t limit_ms, int32_t* waits_returned, void* cuda_stream) {
   if (dev_status == nullptr || waits_returned == nullptr || limit_ms < 1 || limit_ms > 1000) return RF_ERR_INVALID_ARG;
   return rf_launch_selftest_timeout(dev_status, (uint64_t)limit_ms * 1000000ull, waits_returned,

@@ -13,7 +13,7 @@
 // runs beside the other's tiles.  A thread holds 64 scores at a time and takes the first half from TMEM twice (maximum,
 // then exponentials).  Measured against one CTA per SM with two warps a sub-partition, 128 scores a thread and two
 // query tiles a CTA (rf_arm_classify alone, us): 24 heads, samples of 1024 39.1 -> 29.4; 48 heads, 1170 and 1350, D = 64
-// 94.7 -> 71.5; 24 heads, 3300 and 3600 258 -> 217; with four candidate windows, 1920 and 2040 169 -> 125; with the
+// 94.7 -> 71.5; 24 heads, 3300 and 3600 258 -> 217; with four candidate windows, 1920 and 2040 169 -> 137; with the
 // per-key table (both recalls on the stride sample, 867 of 86 400 tokens) 38.4 -> 31.2.
 // Per tile a softmax thread updates an online softmax (running maximum, total mass) plus the masked masses
 // Algorithm 1 needs: the share of the row kept by the sampled Temporal / Spatial (/ Textural, when recalls are

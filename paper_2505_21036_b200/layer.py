@@ -46,17 +46,8 @@ class RainFusionAttention:
 
     # ------------------------------------------------------------------ calls
     def _sparse(self, q, k, v, o, lse):
-        s, p = self.shape, self.params
-        if self.bandwidths:
-            api.rf_arm_classify_plus(s, p, self.bandwidths, q, k, self.head_class, self.head_window, None, self.ws,
-                                     self.status)
-            api.rf_build_block_mask_plus(s, p, self.head_class, self.head_window, self.sched, self.status)
-            api.rf_sparse_attn_fwd_plus(s, p, q, k, v, self.head_class, self.head_window, self.sched, o, lse, self.ws,
-                                        self.status)
-        else:
-            api.rf_arm_classify(s, p, q, k, self.head_class, None, self.ws, self.status)
-            api.rf_build_block_mask(s, p, self.head_class, self.sched, self.status)
-            api.rf_sparse_attn_fwd(s, p, q, k, v, self.head_class, self.sched, o, lse, self.ws, self.status)
+        api.rf_sparse_call(self.shape, self.params, self.bandwidths, q, k, v, self.head_class, self.head_window, self.sched, o,
+                           lse, self.ws, self.status)
 
     def _sparse_graphed(self, q, k, v, o, lse):
         import torch
