@@ -55,6 +55,12 @@ __host__ __device__ __forceinline__ int rf_kv_len(const RfGeom& g, int cls) {
 // rf_grid_trigger lets the next kernel's CTAs come in as soon as every CTA of this one has called it or ended.
 __device__ __forceinline__ void rf_grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void rf_grid_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+// While an RfPlainLaunches is alive, its thread launches without the attribute: see rf_host_pipeline_run.
+inline thread_local int rf_plain_launches = 0;
+struct RfPlainLaunches {
+  RfPlainLaunches() { ++rf_plain_launches; }
+  ~RfPlainLaunches() { --rf_plain_launches; }
+};
 template <typename... P, typename... A>
 inline cudaError_t rf_launch(void (*kernel)(P...), dim3 grid, unsigned block, size_t smem, cudaStream_t st, const A&... args) {
   cudaLaunchConfig_t c = {};
@@ -66,7 +72,7 @@ inline cudaError_t rf_launch(void (*kernel)(P...), dim3 grid, unsigned block, si
   at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at.val.programmaticStreamSerializationAllowed = 1;
   c.attrs = &at;
-  c.numAttrs = 1;
+  c.numAttrs = rf_plain_launches > 0 ? 0 : 1;
   return cudaLaunchKernelEx(&c, kernel, static_cast<P>(args)...);
 }
 
