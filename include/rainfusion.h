@@ -303,8 +303,8 @@ void rf_host_pipeline_destroy(rf_host_pipeline *p);
  *   - The first call on each device looks up the array's device address (cudaGetSymbolAddress, with
  *     that device current).  Make that first call outside any stream capture.
  *   - All calls share the one array and it keeps the previous call's contents.  The one word of it that
- *     has to start at zero (the flag that records a wait that ran out) is cleared by every call on its
- *     stream before its kernels run; every other element that is read was written earlier in the same
+ *     has to start at zero (the flag that records a wait that ran out) is cleared by every call at the start of its
+ *     first kernel; every other element that is read was written earlier in the same
  *     call.  But two calls that overlap on the GPU - different streams, or different host threads -
  *     race on the array.  Serialise them, or use rf_arm_classify with separate workspaces.
  *   - dev_status: as for rf_arm_classify.

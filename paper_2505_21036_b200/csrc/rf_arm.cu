@@ -27,8 +27,8 @@
 // in addition, the sampled keys of frame 0, a prefix of the stride sample.
 // Per-row recalls go to scratch; a second kernel averages them in a fixed order (deterministic) and
 // takes Algorithm 1's decision.  The n x n score matrix is never written.
-// A bounded wait that runs out is recorded in a flag word at the end of the scratch (cleared at the start of
-// every call); the decision kernel then writes class -1 for every head instead of a class computed from
+// A bounded wait that runs out is recorded in a flag word at the end of the scratch (cleared by the score
+// kernel as it starts); the decision kernel then writes class -1 for every head instead of a class computed from
 // unwritten rows, and passes the code on to the caller's status word.  The tile builder and the attention
 // kernel report a class outside 0..3 through their own status, so the failure cannot go unnoticed even by a
 // caller that gave ARM no status pointer.

@@ -93,7 +93,7 @@ cudaError_t rf_launch_arm(const RfGeom& g, int sample_mode, int omega, float alp
                           int32_t* head_window, float* recall, float* recall_plus, float* row_scratch, int32_t* dev_status,
                           cudaStream_t st, bool selftest_abandon = false);
 // Floats of ARM scratch: the per-row recalls plus RF_ARM_FLAG_FLOATS at the end whose first word records a
-// wait that ran out inside the score kernel (cleared by every call before its kernels run).
+// wait that ran out inside the score kernel (cleared by every call at the start of its first kernel).
 #define RF_ARM_FLAG_FLOATS 64
 size_t rf_arm_scratch_floats(const RfGeom& g, int omega, int nb);
 // Tensor map over bf16 rows: [heads][rows][D] with the given row and head strides in bytes (multiples of 16),
