@@ -13,7 +13,7 @@
 // runs beside the other's tiles.  A thread holds 64 scores at a time and takes the first half from TMEM twice (maximum,
 // then exponentials).  Measured against one CTA per SM with two warps a sub-partition, 128 scores a thread and two
 // query tiles a CTA (rf_arm_classify alone, us): 24 heads, samples of 1024 39.1 -> 29.4; 48 heads, 1170 and 1350, D = 64
-// 94.7 -> 71.5; 24 heads, 3300 and 3600 258 -> 217; with four candidate windows, 1920 and 2040 169 -> 137; with the
+// 94.7 -> 71.5; 24 heads, 3300 and 3600 258 -> 217; with three candidate windows, 1920 and 2040 169 -> 121; with the
 // per-key table (both recalls on the stride sample, 867 of 86 400 tokens) 38.4 -> 31.2.
 // Per tile a softmax thread updates an online softmax (running maximum, total mass) plus the masked masses
 // Algorithm 1 needs: the share of the row kept by the sampled Temporal / Spatial (/ Textural, when recalls are
@@ -55,7 +55,7 @@ struct ArmSample {
   int want_s;     // accumulate the Spatial masses on this sample
   float* out;     // [B*H][2*NB+1][n_pad]: Temporal per window, Spatial per window, Textural
 };
-struct ArmWindows { int ws[ARM_MAX_NB], wf[ARM_MAX_NB]; };   // candidate spatial (Temporal) / frame (Spatial) windows
+struct ArmWindows { int ws[ARM_MAX_NB], wf[ARM_MAX_NB], n; };   // candidate spatial (Temporal) / frame (Spatial) windows
 
 template <int D>
 struct ArmCfg {
@@ -292,6 +292,7 @@ __global__ void __launch_bounds__(ARM_THREADS, 2) rf_arm_kernel(const __grid_con
         if (c0 < n) {
 #pragma unroll
           for (int i = 0; i < NB; ++i) {
+            if (i >= win.n) break;                   // slots past the caller's candidates stay empty
             if (sm.want_t) {
               const bool in = rp - win.ws[i] <= c0 && c1 <= rp + win.ws[i] + 1;
               const bool out = c1 <= rp - win.ws[i] || rp + win.ws[i] + 1 <= c0;
@@ -420,7 +421,7 @@ __global__ void __launch_bounds__(256) rf_arm_decide_kernel(int nb, int nb_user,
                                                              int32_t* __restrict__ head_window, float* __restrict__ recall,
                                                              float* __restrict__ recall_plus,
                                                              const int32_t* __restrict__ arm_flag, int32_t* dev_status) {
-  __shared__ double red[2 * ARM_MAX_NB + 1][256];
+  __shared__ double red[2 * ARM_MAX_NB + 1][8];
   rf_grid_trigger();
   rf_grid_wait();
   const int bh = blockIdx.x, tid = threadIdx.x;
@@ -445,17 +446,17 @@ __global__ void __launch_bounds__(256) rf_arm_decide_kernel(int nb, int nb_user,
     double acc = 0.0;
     if (!is_x || with_tex)
       for (int i = tid; i < cnt; i += 256) acc += (double)src[i];
-    red[k][tid] = acc;
+    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    if ((tid & 31) == 0) red[k][tid >> 5] = acc;
   }
   __syncthreads();
-  for (int o = 128; o > 0; o >>= 1) {
-    if (tid < o)
-      for (int k = 0; k < nm; ++k) red[k][tid] += red[k][tid + o];
-    __syncthreads();
-  }
   if (tid == 0) {
     float R[2 * ARM_MAX_NB + 1];
-    for (int k = 0; k < nm; ++k) R[k] = (float)(red[k][0] / ((k < nb && local_t) ? n_loc : n_glb));
+    for (int k = 0; k < nm; ++k) {
+      double sum = 0.0;
+      for (int w = 0; w < 8; ++w) sum += red[k][w];
+      R[k] = (float)(sum / ((k < nb && local_t) ? n_loc : n_glb));
+    }
     if (head_window == nullptr) {
       const float Rt = R[0], Rs = R[nb], Rc = R[2 * nb];
       if (recall) { recall[bh * 3] = Rt; recall[bh * 3 + 1] = Rs; recall[bh * 3 + 2] = Rc; }
@@ -539,6 +540,7 @@ cudaError_t rf_launch_arm(const RfGeom& g, int sample_mode, int omega, float alp
   const int NB = plus ? ARM_MAX_NB : 1;           // windows the kernel evaluates (candidate list padded by repetition)
   if (nb < 1 || nb > NB) return cudaErrorInvalidValue;
   ArmWindows win;
+  win.n = nb;
   for (int i = 0; i < ARM_MAX_NB; ++i) {
     win.ws[i] = ws_list[i < nb ? i : nb - 1];
     win.wf[i] = wf_list[i < nb ? i : nb - 1];
