@@ -30,7 +30,7 @@ namespace {
 using namespace sm100;
 using namespace rf_attn;
 
-constexpr int kThreads = kWsThreads;        // 3 warpgroups: softmax 0, softmax 1, {TMA, MMA, 2 idle warps}
+constexpr int kThreads = kWsThreads;        // 3 warpgroups: softmax 0, softmax 1, {TMA, MMA, items, 1 idle warp}
 constexpr int kTmaWarp = 8, kMmaWarp = 9, kItemWarp = 10;
 constexpr int kItemSlots = 2, kItemWords = 12, kItemReaders = 9;   // readers: eight softmax warps and the TMA thread
 constexpr uint32_t kMore = 4, kLast = 8;   // of a tile record, see the TMA producer

@@ -144,7 +144,7 @@ struct Merge {
   // tiles the union has left at most
   __device__ __forceinline__ int left(const Lists& L) const { return max(L.n0 - i0, L.n1 - i1); }
   // Raw list entries at i0 / i1, loaded by the previous call and not touched until the next one, so
-  // that the load latency never sits between two MMA bursts of the (in-order) issuing thread.
+  // that the load latency never sits between two tiles' copies of the (in-order) TMA thread.
   uint32_t raw0 = 0, raw1 = 0;
   __device__ __forceinline__ void start(const Lists& L) {
     i0 = i1 = 0;

@@ -102,8 +102,8 @@ __device__ __forceinline__ bool clc_answer(uint32_t response, uint32_t& x, uint3
 }
 
 // ---------------------------------------------------------------- register budget of warp-specialised CTAs
-// The attention and ARM kernels run 384 threads: two softmax warpgroups that raise their register count with
-// setmaxnreg.inc and one warpgroup (TMA, MMA, two filler warps) that lowers its own first.  setmaxnreg.inc waits,
+// The attention kernel runs 384 threads: two softmax warpgroups that raise their register count with
+// setmaxnreg.inc and one warpgroup (TMA, MMA, items, a filler warp) that lowers its own first.  setmaxnreg.inc waits,
 // without any bound, until the CTA's register pool can grant the request, and the pool is what the CTA got at
 // launch: registers per thread (as allocated by ptxas) x 384.  The split is therefore checked twice: at compile
 // time against the 64 K registers of an SM, and on the host before the first launch against the kernel's actual
