@@ -433,6 +433,11 @@ __global__ void __launch_bounds__(kThreads, 1) rf_attn_kernel(const __grid_const
             n0 = rf_cdiv(rf_kv_len(g, cls), BN);
             n1 = qt1 < g.nQ ? n0 : 0;
           }
+          // Nothing is written for a pair whose lists are both empty (a schedule that the tile builder did not write).  It is
+          // not published either: the TMA thread holds back the last V of the item before while it looks for the next tile,
+          // so with two slots an empty item in between would wait for that V and keep it waiting.  (Below, a piece has at
+          // least one entry of the longer list, so no published item is empty.)
+          if (n0 == 0 && n1 == 0) continue;
           int b0 = 0, b1 = 0, k = 1;
           if (un.most > 1) {
             const int u = max(n0, n1);
@@ -464,25 +469,23 @@ __global__ void __launch_bounds__(kThreads, 1) rf_attn_kernel(const __grid_const
       Item im;
       Lists L;
       Merge mg;
-      int item = -1, tile = 0, ntile = 0, uses, left = 0;
+      int item = -1, tile = 0, ntile = 0, uses, listed = 0;   // listed: tiles of the item at most
       bool asked = true;
       const CUtensorMap *map_k = nullptr, *map_v = nullptr;
-      // moves on to the next item that lists a tile; Q is fetched by the caller
+      // moves on to the next item; Q is fetched by the caller
       auto advance = [&](int& t) -> bool {
-        for (;;) {
-          if (!asked) mbar_arrive(bar(C::B_REQ));
-          ++item;
-          if (!take(item, im, left)) return false;
-          mbar_arrive(bar(C::B_IE + item % kItemSlots));
-          asked = false;
-          L = lists(im);
-          mg.start(L);
-          left = mg.left(L);
-          const bool perm = im.cls == RF_TEMPORAL && g.permute, tex = im.cls == RF_TEXTURAL;
-          map_k = &maps.m[perm ? 4 : (tex ? 6 : 1)];
-          map_v = &maps.m[perm ? 5 : (tex ? 7 : 2)];
-          if (mg.next(L, t, uses)) return true;
-        }
+        if (!asked) mbar_arrive(bar(C::B_REQ));
+        ++item;
+        if (!take(item, im, listed)) return false;
+        mbar_arrive(bar(C::B_IE + item % kItemSlots));
+        asked = false;
+        L = lists(im);
+        mg.start(L);
+        listed = im.n0 + im.n1;
+        const bool perm = im.cls == RF_TEMPORAL && g.permute, tex = im.cls == RF_TEXTURAL;
+        map_k = &maps.m[perm ? 4 : (tex ? 6 : 1)];
+        map_v = &maps.m[perm ? 5 : (tex ? 7 : 2)];
+        return mg.next(L, t, uses);      // (an item lists a tile)
       };
       auto load_q = [&]() {
         const CUtensorMap* map_q = &maps.m[im.cls == RF_TEMPORAL && g.permute ? 3 : 0];

@@ -3,10 +3,11 @@ off and one joins.  Sizes at the edges of the plan: fewer items than SMs, an odd
 partial last wave whose tail begins inside a row of heads."""
 import numpy as np
 import pytest
+import torch
 
 import gpu_util as gu
 from oracle import rainfusion_oracle as orc
-from paper_2505_21036_b200 import synth
+from paper_2505_21036_b200 import api, synth
 
 pytestmark = pytest.mark.gpu
 
@@ -34,3 +35,35 @@ def test_split_items_match_the_oracle(B, H, D, T, fh, fw, L, omega):
                                                  gu.geom(wl), gu.pparams(wl), rows=rows)
                 gu.check_attention(o[b, h][rows], lse[b, h][rows], ref, lref, f"head {b},{h}", strict=False)
         assert np.isfinite(o).all() and np.isfinite(lse).all()
+
+
+def test_pairs_that_list_no_tile_between_others():
+    """A caller's schedule may leave query tiles without any key tile: their rows are not written, and the items before and
+    after such a pair on the same CTA (more pairs than SMs, so a CTA works off several) give the bits they give without it."""
+    wl = synth.small_workload("empty", H=64, D=64, T=6, fh=12, fw=11, L=37, wf=1, ws=20, tau=2, mode=0, omega=6)
+    run = gu.Run(wl)
+    run.force_classes([h % 4 for h in range(wl.H)])
+    run.build()
+    o, lse = run.sparse()
+    none = np.zeros((wl.H, run.sched.nQ), dtype=bool)
+    rng = np.random.default_rng(3)
+    for h in range(wl.H):
+        for pair in range(-(-run.sched.nQ // 2)):
+            kind = rng.integers(4)                     # both tiles, one of them, or neither keeps its list
+            none[h, 2 * pair:2 * pair + 2] = {0: True, 1: [True, False][:run.sched.nQ - 2 * pair], 2: False, 3: False}[int(kind)]
+    run.sched.count[0, torch.from_numpy(none).cuda()] = 0
+    o2, lse2 = run.outputs()
+    api.rf_sparse_attn_fwd(run.shape, run.params, run.q, run.k, run.v, run.head_class, run.sched, o2, lse2, run.ws, run.status)
+    torch.cuda.synchronize()
+    assert int(run.status.item()) == 0
+    run.mem.check("attention with empty lists")
+    slot = np.arange(wl.N)
+    for h in range(wl.H):
+        tok = slot.copy()
+        if h % 4 == orc.TEMPORAL:                      # position-major slots
+            tok[:wl.Nv] = (slot[:wl.Nv] % wl.T) * wl.S + slot[:wl.Nv] // wl.T
+        written = np.empty(wl.N, dtype=bool)
+        written[tok] = ~none[h, slot // 128]
+        got_o, got_l = o2[0, h].float().cpu().numpy(), lse2[0, h].cpu().numpy()
+        assert np.isnan(got_o[~written]).all() and np.isnan(got_l[~written]).all(), h
+        assert np.array_equal(got_o[written], o[0, h][written]) and np.array_equal(got_l[written], lse[0, h][written]), h
