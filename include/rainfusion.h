@@ -116,8 +116,10 @@ int32_t rf_bounds_checked(void);
 /* Host, pure: nQ = ceil(N/block_m), nKmax = ceil(N/block_n). */
 rf_status rf_schedule_dims(const rf_shape *shape, const rf_params *params, int32_t *nQ, int32_t *nKmax);
 
-/* Host, pure: bytes of device workspace that rf_arm_classify / rf_sparse_attn_fwd need
- * (reordered Q/K/V copies for Temporal and Textural heads, ARM per-row recalls).  0 on bad arguments. */
+/* Host, pure: bytes of device workspace that rf_arm_classify / rf_sparse_attn_fwd need (reordered Q/K/V copies for
+ * Temporal and Textural heads, ARM per-row recalls and, for shapes of few query tiles, up to 52 MB for the partial results
+ * of query tiles that several SMs share).  0 on bad arguments.  Every call that takes a workspace writes to it, so calls
+ * that may overlap on the GPU need one each. */
 size_t rf_workspace_bytes(const rf_shape *shape, const rf_params *params);
 
 /*
@@ -172,7 +174,8 @@ rf_status rf_reorder_tokens(const rf_shape *shape, const rf_params *params, cons
  * arguments as rf_sparse_attn_fwd_plus (head_window may be NULL), but no reordering pass is launched.  ws must
  * hold what rf_reorder_tokens wrote for the same q, k, v and head_class, earlier on the same stream.
  * rf_reorder_tokens followed by this call is rf_sparse_attn_fwd, bit for bit; the split lets a caller reuse
- * one reordering for several calls and lets each of the two kernels be timed by itself.
+ * one reordering for several calls, one after the other, and lets each of the two kernels be timed by itself.  The copies in
+ * ws are only read; of the params, those of the sampling may differ from the reordering's.
  */
 rf_status rf_sparse_attn_reordered(const rf_shape *shape, const rf_params *params, const void *q, const void *k,
                                    const void *v, const int32_t *head_class, const int32_t *head_window,

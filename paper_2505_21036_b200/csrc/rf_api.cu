@@ -110,9 +110,12 @@ bool encode_map(CUtensorMap* m, const void* ptr, int D, int rows, int head_rows,
   return rf_encode_rows_map(m, ptr, D, rows, (size_t)D * 2, (size_t)head_rows * D * 2, heads);
 }
 
-// Where the pieces of split items live: behind ARM's scratch.
-size_t split_offset(const RfGeom& g, const rf_params* p) {
-  return 3 * tensor_bytes(g) + align_up(rf_arm_scratch_floats(g, p->sample_stride, RF_MAX_BANDWIDTHS) * sizeof(float));
+// The workspace: the reordered copies of Q, K and V, the pieces of split items, ARM's scratch.  The offsets depend on the
+// shape alone, so that calls whose other parameters differ find the same things in the same places.
+size_t split_offset(const RfGeom& g) { return 3 * tensor_bytes(g); }
+size_t arm_offset(const RfGeom& g) { return split_offset(g) + rf_split_bytes(rf_split_plan(g, true, g.B * g.H, 0), g.D); }
+size_t arm_bytes(const RfGeom& g, const rf_params* p) {
+  return align_up(rf_arm_scratch_floats(g, p->sample_stride, RF_MAX_BANDWIDTHS) * sizeof(float));
 }
 void set_split(RfAttnArgs* a, const RfSplit& sp, uint8_t* at) {
   a->sp = sp;
@@ -193,12 +196,14 @@ rf_status sparse_attn_impl(const rf_shape* shape, const rf_params* params, const
   if (!ok) return RF_ERR_CUDA;
 
   RfAttnArgs a;
-  set_split(&a, rf_split_plan(g, true, heads_total, head0), w + split_offset(g, params));
+  set_split(&a, rf_split_plan(g, true, heads_total, head0), w + split_offset(g));
   if (gather) {
     cudaError_t e = rf_launch_gather(g, head_class, static_cast<const __nv_bfloat16*>(q),
                                      static_cast<const __nv_bfloat16*>(k), static_cast<const __nv_bfloat16*>(v), wq, wk, wv,
                                      a.tickets, (int)a.sp.n_tickets, dev_status, stream);
     if (e != cudaSuccess) return RF_ERR_CUDA;
+  } else if (a.sp.on && rf_launch_zero(a.tickets, (int)a.sp.n_tickets, stream) != cudaSuccess) {
+    return RF_ERR_CUDA;   // whatever ran on this workspace since the reordering, the tickets begin at zero
   }
 
   a.g = g;
@@ -272,7 +277,8 @@ size_t rf_split_bytes(const RfSplit& sp, int D) {
 size_t rf_group_workspace_bytes(const rf_shape* shape, const rf_params* params, int heads_total, int head0) {
   if (check_shape(shape) != RF_OK || check_params(params) != RF_OK) return 0;
   const RfGeom g = make_geom(shape, params);
-  return split_offset(g, params) + rf_split_bytes(rf_split_plan(g, true, heads_total, head0), g.D);
+  // (a group's pieces may reach into ARM's scratch, which is done with by then)
+  return std::max(arm_offset(g) + arm_bytes(g, params), split_offset(g) + rf_split_bytes(rf_split_plan(g, true, heads_total, head0), g.D));
 }
 
 rf_status rf_sparse_attn_group(const rf_shape* shape, const rf_params* params, const void* q, const void* k, const void* v,
@@ -339,7 +345,7 @@ rf_status rf_arm_classify(const rf_shape* shape, const rf_params* params, const 
   if (!aligned16(q) || !aligned16(k) || (reinterpret_cast<uintptr_t>(ws) & (kAlign - 1)) != 0) return RF_ERR_INVALID_ARG;
   if (ws_bytes < rf_workspace_bytes(shape, params)) return RF_ERR_WORKSPACE_TOO_SMALL;
   const RfGeom g = make_geom(shape, params);
-  float* scratch = reinterpret_cast<float*>(static_cast<uint8_t*>(ws) + 3 * tensor_bytes(g));
+  float* scratch = reinterpret_cast<float*>(static_cast<uint8_t*>(ws) + arm_offset(g));
   cudaError_t e = rf_launch_arm(g, params->sample_mode, params->sample_stride, params->alpha, 1, &g.ws, &g.wf,
                                 static_cast<const __nv_bfloat16*>(q), static_cast<const __nv_bfloat16*>(k), head_class,
                                 nullptr, recall, nullptr, scratch, dev_status, static_cast<cudaStream_t>(cuda_stream));
@@ -359,7 +365,7 @@ rf_status rf_selftest_arm_abandoned(const rf_shape* shape, const rf_params* para
   if (!aligned16(q) || !aligned16(k) || (reinterpret_cast<uintptr_t>(ws) & (kAlign - 1)) != 0) return RF_ERR_INVALID_ARG;
   if (ws_bytes < rf_workspace_bytes(shape, params)) return RF_ERR_WORKSPACE_TOO_SMALL;
   const RfGeom g = make_geom(shape, params);
-  float* scratch = reinterpret_cast<float*>(static_cast<uint8_t*>(ws) + 3 * tensor_bytes(g));
+  float* scratch = reinterpret_cast<float*>(static_cast<uint8_t*>(ws) + arm_offset(g));
   cudaError_t e = rf_launch_arm(g, params->sample_mode, params->sample_stride, params->alpha, 1, &g.ws, &g.wf,
                                 static_cast<const __nv_bfloat16*>(q), static_cast<const __nv_bfloat16*>(k), head_class,
                                 nullptr, nullptr, nullptr, scratch, dev_status, static_cast<cudaStream_t>(cuda_stream), true);
@@ -390,7 +396,7 @@ rf_status rf_arm_classify_plus(const rf_shape* shape, const rf_params* params, c
     wf_list[i] = (int)floor((double)b * g.T);
     ws_list[i] = (int)floor((double)b * g.S);
   }
-  float* scratch = reinterpret_cast<float*>(static_cast<uint8_t*>(ws) + 3 * tensor_bytes(g));
+  float* scratch = reinterpret_cast<float*>(static_cast<uint8_t*>(ws) + arm_offset(g));
   cudaError_t e = rf_launch_arm(g, params->sample_mode, params->sample_stride, params->alpha, n_bandwidths, ws_list,
                                 wf_list, static_cast<const __nv_bfloat16*>(q), static_cast<const __nv_bfloat16*>(k),
                                 head_class, head_window, nullptr, recall, scratch, dev_status,
@@ -478,12 +484,10 @@ rf_status rf_reorder_tokens(const rf_shape* shape, const rf_params* params, cons
   if (ws_bytes < rf_workspace_bytes(shape, params)) return RF_ERR_WORKSPACE_TOO_SMALL;
   const RfGeom g = make_geom(shape, params);
   uint8_t* w = static_cast<uint8_t*>(ws);
-  RfAttnArgs a;   // a following rf_sparse_attn_reordered finds its tickets at zero
-  set_split(&a, rf_split_plan(g, true, g.B * g.H, 0), w + split_offset(g, params));
   cudaError_t e = rf_launch_gather(g, head_class, static_cast<const __nv_bfloat16*>(q), static_cast<const __nv_bfloat16*>(k),
                                    static_cast<const __nv_bfloat16*>(v), reinterpret_cast<__nv_bfloat16*>(w),
                                    reinterpret_cast<__nv_bfloat16*>(w + tensor_bytes(g)),
-                                   reinterpret_cast<__nv_bfloat16*>(w + 2 * tensor_bytes(g)), a.tickets, (int)a.sp.n_tickets, nullptr,
+                                   reinterpret_cast<__nv_bfloat16*>(w + 2 * tensor_bytes(g)), nullptr, 0, nullptr,
                                    static_cast<cudaStream_t>(cuda_stream));
   return e == cudaSuccess ? RF_OK : RF_ERR_CUDA;
 }

@@ -222,7 +222,6 @@ __device__ __noinline__ void leave_piece(const RfAttnArgs& a, const int* iw, uin
   if (lane == 0) before = atomicAdd(ticket, 1);
   if (__shfl_sync(0xffffffffu, before, 0) != pieces - 1) return;
   __threadfence();
-  if (lane == 0) *ticket = 0;                                  // the next call on this workspace finds it as this one did
   const Row row = output_row(a, iw, j, row_in_tile);
   // half a row at a time, so that all loads of a piece are under way together
   constexpr int kCols = D == 64 ? 64 : D / 2;

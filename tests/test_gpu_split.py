@@ -67,3 +67,39 @@ def test_pairs_that_list_no_tile_between_others():
         got_o, got_l = o2[0, h].float().cpu().numpy(), lse2[0, h].cpu().numpy()
         assert np.isnan(got_o[~written]).all() and np.isnan(got_l[~written]).all(), h
         assert np.array_equal(got_o[written], o[0, h][written]) and np.array_equal(got_l[written], lse[0, h][written]), h
+
+
+def small_split(**kw):
+    """The first shape above: 27 items of 9 tiles, every one of them in two pieces."""
+    base = dict(name="split", B=1, H=3, D=96, T=10, frame_h=12, frame_w=16, L_text=226, frame_window=2, spatial_window=48,
+                textural_stride=2, sample_mode=0, sample_stride=10, alpha=0.9, amp=2.0, config_id=9)
+    base.update(kw)
+    return synth.Workload(**base)
+
+
+def attention(run, call, params=None, windows=None):
+    """One call of an entry point that takes the sparse arguments; (o, lse) as the bits they hold."""
+    o, lse = run.outputs()
+    call(run.shape, params or run.params, run.q, run.k, run.v, run.head_class, windows, run.sched, o, lse, run.ws, run.status)
+    torch.cuda.synchronize()
+    assert int(run.status.item()) == 0
+    return gu.bits_of(o).copy(), lse.cpu().numpy().view(np.uint32).copy()
+
+
+def same_bits(a, b):
+    return all(np.array_equal(x, y) for x, y in zip(a, b))
+
+
+def test_one_reordering_serves_calls_of_other_sampling_parameters():
+    """rf_sparse_attn_reordered depends on the copies alone: neither the sampling stride of the reordering nor what the rest
+    of the workspace holds may matter, and a second call finds what the first one found."""
+    run = gu.Run(small_split())
+    run.force_classes([0, 1, 2])
+    run.build()
+    ref = attention(run, api.rf_sparse_attn_fwd_plus)
+    other = api.params_of(small_split(sample_stride=5))
+    run.ws = run.mem.alloc((max(api.rf_workspace_bytes(run.shape, p) for p in (run.params, other)),), torch.uint8, 0x5A, "ws")
+    api.rf_reorder_tokens(run.shape, run.params, run.q, run.k, run.v, run.head_class, run.ws)
+    for _ in range(2):
+        assert same_bits(attention(run, api.rf_sparse_attn_reordered, other), ref)
+    run.mem.check("rf_sparse_attn_reordered")
