@@ -203,14 +203,19 @@ rf_status rf_selftest_arm_abandoned(const rf_shape *shape, const rf_params *para
                                     int32_t *head_class, void *ws, size_t ws_bytes, int32_t *dev_status,
                                     void *cuda_stream);
 
-/*
- * Full 3D attention (Eq. 1-2, all-zero mask): the same kernel walking every tile.  ws may be NULL.  With a workspace of
- * rf_dense_workspace_bytes(shape) bytes (256-byte aligned; 0: none is of use) the items of the last wave are cut into
- * pieces that more SMs share; without it every item is worked off by one CTA.
- */
-size_t rf_dense_workspace_bytes(const rf_shape *shape);
+/* Full 3D attention (Eq. 1-2, all-zero mask): the same kernel walking every tile.  ws may be NULL; it is not touched. */
 rf_status rf_dense_attn_fwd(const rf_shape *shape, const void *q, const void *k, const void *v, void *o,
                             float *lse, void *ws, size_t ws_bytes, int32_t *dev_status, void *cuda_stream);
+
+/*
+ * The same with a scratch block for shapes of few query tiles: the tiles that would be left for the last, partial wave are
+ * cut into pieces that more SMs share.  scratch: device memory of rf_dense_workspace_bytes(shape) bytes, 256-byte aligned,
+ * overwritten; calls that may overlap on the GPU need one each.  Where that size is 0, the block smaller or misaligned, or
+ * scratch NULL, the call is rf_dense_attn_fwd.
+ */
+size_t rf_dense_workspace_bytes(const rf_shape *shape);
+rf_status rf_dense_attn_fwd_split(const rf_shape *shape, const void *q, const void *k, const void *v, void *o,
+                                  float *lse, void *scratch, size_t scratch_bytes, int32_t *dev_status, void *cuda_stream);
 
 /*
  * RainFusion+ (Sec. 4.3, last paragraph): per-head dynamic bandwidth.  ARM evaluates every candidate bandwidth

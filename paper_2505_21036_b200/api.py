@@ -20,7 +20,7 @@ _LIB_PATH = os.environ.get("RAINFUSION_LIBRARY") or os.path.join(os.path.dirname
 _lib = None
 
 EXPORTS = ["rf_status_string", "rf_schedule_dims", "rf_workspace_bytes", "rf_arm_classify",
-           "rf_build_block_mask", "rf_reorder_tokens", "rf_sparse_attn_fwd", "rf_dense_attn_fwd", "rf_dense_workspace_bytes", "rf_sparse_call",
+           "rf_build_block_mask", "rf_reorder_tokens", "rf_sparse_attn_fwd", "rf_dense_attn_fwd", "rf_dense_attn_fwd_split", "rf_dense_workspace_bytes", "rf_sparse_call",
            "rf_arm_classify_noalloc", "rf_selftest_wait_timeout", "rf_arm_classify_plus", "rf_build_block_mask_plus", "rf_sparse_attn_fwd_plus",
            "rf_sparse_attn_reordered", "rf_selftest_arm_abandoned", "rf_bounds_checked", "rf_host_pipeline_staging_bytes",
            "rf_host_pipeline_create", "rf_host_pipeline_run", "rf_host_pipeline_status", "rf_host_pipeline_destroy",
@@ -113,6 +113,8 @@ def load():
     lib.rf_dense_workspace_bytes.argtypes = [P(rf_shape)]
     lib.rf_dense_attn_fwd.restype = I
     lib.rf_dense_attn_fwd.argtypes = [P(rf_shape), V, V, V, V, V, V, Z, V, V]
+    lib.rf_dense_attn_fwd_split.restype = I
+    lib.rf_dense_attn_fwd_split.argtypes = lib.rf_dense_attn_fwd.argtypes
     _lib = lib
     return lib
 
@@ -336,5 +338,5 @@ def rf_dense_attn_fwd(shape, q, k, v, o, lse, dev_status=None):
     lib = load()
     n = lib.rf_dense_workspace_bytes(C.byref(shape))
     ws = torch.empty(n, dtype=torch.uint8, device=q.device) if n else None
-    _check(lib.rf_dense_attn_fwd(C.byref(shape), q.data_ptr(), k.data_ptr(), v.data_ptr(), o.data_ptr(), _ptr(lse),
-                                 _ptr(ws), n, _ptr(dev_status), _stream()), "rf_dense_attn_fwd")
+    _check(lib.rf_dense_attn_fwd_split(C.byref(shape), q.data_ptr(), k.data_ptr(), v.data_ptr(), o.data_ptr(), _ptr(lse),
+                                       _ptr(ws), n, _ptr(dev_status), _stream()), "rf_dense_attn_fwd")

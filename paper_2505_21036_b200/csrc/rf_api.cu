@@ -497,8 +497,8 @@ size_t rf_dense_workspace_bytes(const rf_shape* shape) {
   return rf_split_bytes(rf_split_plan(make_geom(shape, 0, 0, 1, 128, 128, 0), false, shape->B * shape->H, 0), shape->D);
 }
 
-rf_status rf_dense_attn_fwd(const rf_shape* shape, const void* q, const void* k, const void* v, void* o, float* lse,
-                            void* ws, size_t ws_bytes, int32_t* dev_status, void* cuda_stream) {
+rf_status rf_dense_attn_fwd_split(const rf_shape* shape, const void* q, const void* k, const void* v, void* o, float* lse,
+                                  void* scratch, size_t scratch_bytes, int32_t* dev_status, void* cuda_stream) {
   rf_status st = check_attn_shape(shape);
   if (st != RF_OK) return st;
   if (q == nullptr || k == nullptr || v == nullptr || o == nullptr) return RF_ERR_INVALID_ARG;
@@ -512,8 +512,9 @@ rf_status rf_dense_attn_fwd(const rf_shape* shape, const void* q, const void* k,
   for (int i = 3; i < 8; ++i) maps[i] = maps[i % 3];
   RfAttnArgs a;
   const RfSplit sp = rf_split_plan(g, false, heads, 0);
-  const bool split = sp.on && ws != nullptr && (reinterpret_cast<uintptr_t>(ws) & (kAlign - 1)) == 0 && ws_bytes >= rf_split_bytes(sp, g.D);
-  set_split(&a, split ? sp : RfSplit{}, static_cast<uint8_t*>(ws));
+  const bool split = sp.on && scratch != nullptr && (reinterpret_cast<uintptr_t>(scratch) & (kAlign - 1)) == 0 &&
+                     scratch_bytes >= rf_split_bytes(sp, g.D);
+  set_split(&a, split ? sp : RfSplit{}, static_cast<uint8_t*>(scratch));
   if (split && rf_launch_zero(a.tickets, (int)sp.n_tickets, static_cast<cudaStream_t>(cuda_stream)) != cudaSuccess) return RF_ERR_CUDA;
   a.g = g;
   a.head_class = nullptr;
@@ -525,6 +526,13 @@ rf_status rf_dense_attn_fwd(const rf_shape* shape, const void* q, const void* k,
   a.dev_status = dev_status;
   a.scale_log2 = 1.4426950408889634f / sqrtf((float)g.D);
   return rf_launch_attention(a, maps, static_cast<cudaStream_t>(cuda_stream));
+}
+
+rf_status rf_dense_attn_fwd(const rf_shape* shape, const void* q, const void* k, const void* v, void* o, float* lse,
+                            void* ws, size_t ws_bytes, int32_t* dev_status, void* cuda_stream) {
+  (void)ws;
+  (void)ws_bytes;
+  return rf_dense_attn_fwd_split(shape, q, k, v, o, lse, nullptr, 0, dev_status, cuda_stream);
 }
 
 }  // extern "C"

@@ -1,6 +1,8 @@
 """Split items of the attention kernel: shapes of few items, whose tile lists are cut into pieces that several CTAs work
 off and one joins.  Sizes at the edges of the plan: fewer items than SMs, an odd number of query tiles, no text rows, a
 partial last wave whose tail begins inside a row of heads."""
+import ctypes as C
+
 import numpy as np
 import pytest
 import torch
@@ -103,3 +105,33 @@ def test_one_reordering_serves_calls_of_other_sampling_parameters():
     for _ in range(2):
         assert same_bits(attention(run, api.rf_sparse_attn_reordered, other), ref)
     run.mem.check("rf_sparse_attn_reordered")
+
+
+def test_a_dense_call_leaves_the_workspace_it_is_given_alone():
+    """rf_dense_attn_fwd takes a workspace for the sake of one calling form and uses none of it: copies that
+    rf_reorder_tokens left there survive.  The form with a scratch block of its own gives the same attention."""
+    run = gu.Run(small_split())
+    run.force_classes([0, 1, 2])
+    run.build()
+    ref = attention(run, api.rf_sparse_attn_fwd_plus)
+    lib, n = api.load(), api.load().rf_dense_workspace_bytes(C.byref(run.shape))
+    assert n > 0
+    run.ws = run.mem.alloc((run.ws.numel() + n,), torch.uint8, name="ws")
+    scratch = run.mem.alloc((n,), torch.uint8, 0x5A, "scratch")
+
+    def dense(call, block):
+        o, lse = run.outputs()
+        code = call(C.byref(run.shape), run.q.data_ptr(), run.k.data_ptr(), run.v.data_ptr(), o.data_ptr(), lse.data_ptr(),
+                    block.data_ptr(), block.numel(), run.status.data_ptr(), None)
+        torch.cuda.synchronize()
+        assert code == 0 and int(run.status.item()) == 0
+        return o.float().cpu().numpy().astype(np.float64), lse.cpu().numpy().astype(np.float64)
+
+    api.rf_reorder_tokens(run.shape, run.params, run.q, run.k, run.v, run.head_class, run.ws)
+    before = run.ws.clone()
+    plain, split = dense(lib.rf_dense_attn_fwd, run.ws), dense(lib.rf_dense_attn_fwd_split, scratch)
+    assert torch.equal(run.ws, before)
+    assert same_bits(attention(run, api.rf_sparse_attn_reordered), ref)
+    for h in range(run.wl.H):
+        gu.check_attention(split[0][0, h], split[1][0, h], plain[0][0, h], plain[1][0, h], f"head {h}", strict=False)
+    run.mem.check("dense calls")
