@@ -118,8 +118,10 @@ rf_status rf_schedule_dims(const rf_shape *shape, const rf_params *params, int32
 
 /* Host, pure: bytes of device workspace that rf_arm_classify / rf_sparse_attn_fwd need (reordered Q/K/V copies for
  * Temporal and Textural heads, ARM per-row recalls and, for shapes of few query tiles, up to 52 MB for the partial results
- * of query tiles that several SMs share).  0 on bad arguments.  Every call that takes a workspace writes to it, so calls
- * that may overlap on the GPU need one each. */
+ * of query tiles that several SMs share).  0 on bad arguments.  A block that has room for all but those partial results
+ * (one sized for a shape of more query tiles, which may need less) is taken as well: no query tile is shared then, which costs
+ * time and changes the rounding.  Every call that takes a workspace writes to it, so calls that may overlap on the GPU need
+ * one each. */
 size_t rf_workspace_bytes(const rf_shape *shape, const rf_params *params);
 
 /*
@@ -263,7 +265,8 @@ rf_status rf_sparse_call(const rf_shape *shape, const rf_params *params, const f
  * to back.
  *   rf_host_pipeline_staging_bytes  host, pure: device bytes the pipeline needs (staged Q, K, V, O for all heads,
  *                                   workspace and schedule of one group per compute stream, classes, status).
- *                                   0 on bad arguments.
+ *                                   0 on bad arguments.  As with rf_workspace_bytes, a block that lacks room for partial
+ *                                   results only is taken as well.
  *   rf_host_pipeline_create         staging: device memory of at least that size, 256-byte aligned, owned by the caller
  *                                   and handed to the pipeline until it is destroyed.  Creates streams and events only.
  *   rf_host_pipeline_run            q/k/v/o_host: host bf16 [B,H,N,D], pinned for the copies to overlap; the inputs

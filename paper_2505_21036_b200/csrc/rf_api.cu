@@ -117,6 +117,13 @@ size_t arm_offset(const RfGeom& g) { return split_offset(g) + rf_split_bytes(rf_
 size_t arm_bytes(const RfGeom& g, const rf_params* p) {
   return align_up(rf_arm_scratch_floats(g, p->sample_stride, RF_MAX_BANDWIDTHS) * sizeof(float));
 }
+// The pieces are no necessity: a block that lacks the room for them (one sized for a larger shape that needs none, say) does
+// for the copies and ARM's scratch, and the items stay whole.
+size_t least_bytes(const RfGeom& g, const rf_params* p) { return 3 * tensor_bytes(g) + arm_bytes(g, p); }
+float* arm_scratch(const RfGeom& g, const rf_params* p, void* ws, size_t ws_bytes) {
+  const size_t at = ws_bytes >= arm_offset(g) + arm_bytes(g, p) ? arm_offset(g) : split_offset(g);
+  return reinterpret_cast<float*>(static_cast<uint8_t*>(ws) + at);
+}
 void set_split(RfAttnArgs* a, const RfSplit& sp, uint8_t* at) {
   a->sp = sp;
   a->tickets = sp.on ? reinterpret_cast<int32_t*>(at) : nullptr;
@@ -177,8 +184,8 @@ rf_status sparse_attn_impl(const rf_shape* shape, const rf_params* params, const
       (reinterpret_cast<uintptr_t>(ws) & (kAlign - 1)) != 0)
     return RF_ERR_INVALID_ARG;
   if (head_window != nullptr && params->temporal_window_2d) return RF_ERR_UNSUPPORTED;
-  if (ws_bytes < rf_group_workspace_bytes(shape, params, heads_total, head0)) return RF_ERR_WORKSPACE_TOO_SMALL;
   const RfGeom g = make_geom(shape, params);
+  if (ws_bytes < least_bytes(g, params)) return RF_ERR_WORKSPACE_TOO_SMALL;
   if (sched->nQ != g.nQ || sched->nKmax != g.nKmax) return RF_ERR_INVALID_ARG;
   cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
 
@@ -196,7 +203,8 @@ rf_status sparse_attn_impl(const rf_shape* shape, const rf_params* params, const
   if (!ok) return RF_ERR_CUDA;
 
   RfAttnArgs a;
-  set_split(&a, rf_split_plan(g, true, heads_total, head0), w + split_offset(g));
+  const bool room = ws_bytes >= rf_group_workspace_bytes(shape, params, heads_total, head0);
+  set_split(&a, room ? rf_split_plan(g, true, heads_total, head0) : RfSplit{}, w + split_offset(g));
   if (gather) {
     cudaError_t e = rf_launch_gather(g, head_class, static_cast<const __nv_bfloat16*>(q),
                                      static_cast<const __nv_bfloat16*>(k), static_cast<const __nv_bfloat16*>(v), wq, wk, wv,
@@ -281,6 +289,10 @@ size_t rf_group_workspace_bytes(const rf_shape* shape, const rf_params* params, 
   return std::max(arm_offset(g) + arm_bytes(g, params), split_offset(g) + rf_split_bytes(rf_split_plan(g, true, heads_total, head0), g.D));
 }
 
+size_t rf_least_workspace_bytes(const rf_shape* shape, const rf_params* params) {
+  return check_shape(shape) == RF_OK && check_params(params) == RF_OK ? least_bytes(make_geom(shape, params), params) : 0;
+}
+
 rf_status rf_sparse_attn_group(const rf_shape* shape, const rf_params* params, const void* q, const void* k, const void* v,
                                const int32_t* head_class, const int32_t* head_window, const rf_schedule* sched, void* o,
                                float* lse, void* ws, size_t ws_bytes, int32_t* dev_status, void* cuda_stream, int heads_total,
@@ -343,9 +355,9 @@ rf_status rf_arm_classify(const rf_shape* shape, const rf_params* params, const 
   if (shape->D != 64 && shape->D != 96 && shape->D != 128) return RF_ERR_UNSUPPORTED;
   if (q == nullptr || k == nullptr || head_class == nullptr || ws == nullptr) return RF_ERR_INVALID_ARG;
   if (!aligned16(q) || !aligned16(k) || (reinterpret_cast<uintptr_t>(ws) & (kAlign - 1)) != 0) return RF_ERR_INVALID_ARG;
-  if (ws_bytes < rf_workspace_bytes(shape, params)) return RF_ERR_WORKSPACE_TOO_SMALL;
   const RfGeom g = make_geom(shape, params);
-  float* scratch = reinterpret_cast<float*>(static_cast<uint8_t*>(ws) + arm_offset(g));
+  if (ws_bytes < least_bytes(g, params)) return RF_ERR_WORKSPACE_TOO_SMALL;
+  float* scratch = arm_scratch(g, params, ws, ws_bytes);
   cudaError_t e = rf_launch_arm(g, params->sample_mode, params->sample_stride, params->alpha, 1, &g.ws, &g.wf,
                                 static_cast<const __nv_bfloat16*>(q), static_cast<const __nv_bfloat16*>(k), head_class,
                                 nullptr, recall, nullptr, scratch, dev_status, static_cast<cudaStream_t>(cuda_stream));
@@ -363,9 +375,9 @@ rf_status rf_selftest_arm_abandoned(const rf_shape* shape, const rf_params* para
   if (shape->D != 64 && shape->D != 96 && shape->D != 128) return RF_ERR_UNSUPPORTED;
   if (q == nullptr || k == nullptr || head_class == nullptr || ws == nullptr) return RF_ERR_INVALID_ARG;
   if (!aligned16(q) || !aligned16(k) || (reinterpret_cast<uintptr_t>(ws) & (kAlign - 1)) != 0) return RF_ERR_INVALID_ARG;
-  if (ws_bytes < rf_workspace_bytes(shape, params)) return RF_ERR_WORKSPACE_TOO_SMALL;
   const RfGeom g = make_geom(shape, params);
-  float* scratch = reinterpret_cast<float*>(static_cast<uint8_t*>(ws) + arm_offset(g));
+  if (ws_bytes < least_bytes(g, params)) return RF_ERR_WORKSPACE_TOO_SMALL;
+  float* scratch = arm_scratch(g, params, ws, ws_bytes);
   cudaError_t e = rf_launch_arm(g, params->sample_mode, params->sample_stride, params->alpha, 1, &g.ws, &g.wf,
                                 static_cast<const __nv_bfloat16*>(q), static_cast<const __nv_bfloat16*>(k), head_class,
                                 nullptr, nullptr, nullptr, scratch, dev_status, static_cast<cudaStream_t>(cuda_stream), true);
@@ -387,8 +399,8 @@ rf_status rf_arm_classify_plus(const rf_shape* shape, const rf_params* params, c
   if (bandwidths == nullptr || n_bandwidths < 1 || n_bandwidths > RF_MAX_BANDWIDTHS) return RF_ERR_INVALID_ARG;
   if (q == nullptr || k == nullptr || head_class == nullptr || head_window == nullptr || ws == nullptr) return RF_ERR_INVALID_ARG;
   if (!aligned16(q) || !aligned16(k) || (reinterpret_cast<uintptr_t>(ws) & (kAlign - 1)) != 0) return RF_ERR_INVALID_ARG;
-  if (ws_bytes < rf_workspace_bytes(shape, params)) return RF_ERR_WORKSPACE_TOO_SMALL;
   const RfGeom g = make_geom(shape, params);
+  if (ws_bytes < least_bytes(g, params)) return RF_ERR_WORKSPACE_TOO_SMALL;
   int ws_list[RF_MAX_BANDWIDTHS], wf_list[RF_MAX_BANDWIDTHS];
   for (int i = 0; i < n_bandwidths; ++i) {
     const float b = bandwidths[i];
@@ -396,7 +408,7 @@ rf_status rf_arm_classify_plus(const rf_shape* shape, const rf_params* params, c
     wf_list[i] = (int)floor((double)b * g.T);
     ws_list[i] = (int)floor((double)b * g.S);
   }
-  float* scratch = reinterpret_cast<float*>(static_cast<uint8_t*>(ws) + arm_offset(g));
+  float* scratch = arm_scratch(g, params, ws, ws_bytes);
   cudaError_t e = rf_launch_arm(g, params->sample_mode, params->sample_stride, params->alpha, n_bandwidths, ws_list,
                                 wf_list, static_cast<const __nv_bfloat16*>(q), static_cast<const __nv_bfloat16*>(k),
                                 head_class, head_window, nullptr, recall, scratch, dev_status,
@@ -481,8 +493,8 @@ rf_status rf_reorder_tokens(const rf_shape* shape, const rf_params* params, cons
   if (q == nullptr || k == nullptr || v == nullptr || head_class == nullptr || ws == nullptr) return RF_ERR_INVALID_ARG;
   if (!aligned16(q) || !aligned16(k) || !aligned16(v) || (reinterpret_cast<uintptr_t>(ws) & (kAlign - 1)) != 0)
     return RF_ERR_INVALID_ARG;
-  if (ws_bytes < rf_workspace_bytes(shape, params)) return RF_ERR_WORKSPACE_TOO_SMALL;
   const RfGeom g = make_geom(shape, params);
+  if (ws_bytes < least_bytes(g, params)) return RF_ERR_WORKSPACE_TOO_SMALL;
   uint8_t* w = static_cast<uint8_t*>(ws);
   cudaError_t e = rf_launch_gather(g, head_class, static_cast<const __nv_bfloat16*>(q), static_cast<const __nv_bfloat16*>(k),
                                    static_cast<const __nv_bfloat16*>(v), reinterpret_cast<__nv_bfloat16*>(w),

@@ -147,7 +147,8 @@ struct RfAttnArgs {
 constexpr int RF_ATTN_MAPS = 8;
 rf_status rf_launch_attention(const RfAttnArgs& a, const CUtensorMap* maps, cudaStream_t st);
 // rf_sparse_attn_fwd_plus for heads [head0, head0 + B*H) of a call of heads_total heads made in groups; the workspace needs
-// rf_group_workspace_bytes.
+// rf_group_workspace_bytes, or rf_least_workspace_bytes if no item is to be split.
+size_t rf_least_workspace_bytes(const rf_shape* shape, const rf_params* params);
 size_t rf_group_workspace_bytes(const rf_shape* shape, const rf_params* params, int heads_total, int head0);
 rf_status rf_sparse_attn_group(const rf_shape* shape, const rf_params* params, const void* q, const void* k, const void* v,
                                const int32_t* head_class, const int32_t* head_window, const rf_schedule* sched, void* o,

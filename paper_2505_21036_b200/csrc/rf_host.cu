@@ -46,7 +46,9 @@ struct Layout {
   size_t tensor, ws, count, kv_tile, kv_len, head_class, status, total;
 };
 
-bool layout_of(const rf_shape* shape, const rf_params* params, int groups, rf_shape* gshape, Layout* L, int32_t* nQ, int32_t* nK) {
+// pieces: with room for the pieces of split items (see rf_workspace_bytes).
+bool layout_of(const rf_shape* shape, const rf_params* params, int groups, bool pieces, rf_shape* gshape, Layout* L, int32_t* nQ,
+               int32_t* nK) {
   if (shape == nullptr || params == nullptr || groups < 1) return false;
   const long long heads = (long long)shape->B * shape->H;
   if (heads < 1 || heads % groups != 0) return false;
@@ -54,10 +56,10 @@ bool layout_of(const rf_shape* shape, const rf_params* params, int groups, rf_sh
   gshape->B = 1;
   gshape->H = (int32_t)(heads / groups);
   if (rf_schedule_dims(gshape, params, nQ, nK) != RF_OK) return false;
-  size_t ws = rf_workspace_bytes(gshape, params);
+  size_t ws = rf_least_workspace_bytes(gshape, params);
   if (ws == 0) return false;
   // the groups share their compute stream's workspace
-  for (int g = 0; g < groups; ++g) ws = std::max(ws, rf_group_workspace_bytes(gshape, params, (int)heads, g * gshape->H));
+  for (int g = 0; pieces && g < groups; ++g) ws = std::max(ws, rf_group_workspace_bytes(gshape, params, (int)heads, g * gshape->H));
   const size_t N = (size_t)shape->T * shape->frame_h * shape->frame_w + shape->L_text;
   L->tensor = align_up((size_t)heads * N * shape->D * sizeof(__nv_bfloat16));
   L->ws = align_up(ws);
@@ -92,7 +94,7 @@ size_t rf_host_pipeline_staging_bytes(const rf_shape* shape, const rf_params* pa
   rf_shape gs;
   Layout L;
   int32_t nQ, nK;
-  return layout_of(shape, params, head_groups, &gs, &L, &nQ, &nK) ? L.total : 0;
+  return layout_of(shape, params, head_groups, true, &gs, &L, &nQ, &nK) ? L.total : 0;
 }
 
 rf_status rf_host_pipeline_create(const rf_shape* shape, const rf_params* params, int32_t head_groups, void* staging,
@@ -102,10 +104,11 @@ rf_status rf_host_pipeline_create(const rf_shape* shape, const rf_params* params
   rf_shape gs;
   Layout L;
   int32_t nQ, nK;
-  if (!layout_of(shape, params, head_groups, &gs, &L, &nQ, &nK)) return RF_ERR_INVALID_ARG;
+  if (!layout_of(shape, params, head_groups, true, &gs, &L, &nQ, &nK)) return RF_ERR_INVALID_ARG;
   if (shape->D != 64 && shape->D != 96 && shape->D != 128) return RF_ERR_UNSUPPORTED;
   if (params->block_m != 128 || params->block_n != 128) return RF_ERR_UNSUPPORTED;
   if (staging == nullptr || (reinterpret_cast<uintptr_t>(staging) & (kAlign - 1)) != 0) return RF_ERR_INVALID_ARG;
+  if (staging_bytes < L.total) layout_of(shape, params, head_groups, false, &gs, &L, &nQ, &nK);
   if (staging_bytes < L.total) return RF_ERR_WORKSPACE_TOO_SMALL;
   rf_host_pipeline* p = new (std::nothrow) rf_host_pipeline();
   if (p == nullptr) return RF_ERR_CUDA;

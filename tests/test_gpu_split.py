@@ -135,3 +135,38 @@ def test_a_dense_call_leaves_the_workspace_it_is_given_alone():
     for h in range(run.wl.H):
         gu.check_attention(split[0][0, h], split[1][0, h], plain[0][0, h], plain[1][0, h], f"head {h}", strict=False)
     run.mem.check("dense calls")
+
+
+def test_a_workspace_without_room_for_pieces_still_serves():
+    """A block sized for seven heads (224 items: none is split) serves six (192 items, the last 44 in pieces), although six
+    need more for themselves: the copies and ARM's scratch fit."""
+    shapes = [small_split(H=h, D=64, T=16, frame_h=16, frame_w=32, L_text=0, sample_stride=16, frame_window=4, spatial_window=128)
+              for h in (7, 6)]
+    seven, six = (api.rf_workspace_bytes(api.shape_of(w), api.params_of(w)) for w in shapes)
+    assert seven < six
+    run = gu.Run(shapes[1])
+    ref_cls, ref_rec = run.arm()
+    run.build()
+    ref = run.sparse()
+    run.ws = run.mem.alloc((seven,), torch.uint8, 0x5A, "ws")
+    cls, rec = run.arm()
+    assert np.array_equal(cls, ref_cls) and np.array_equal(rec, ref_rec)
+    whole = run.sparse()
+    for h in range(run.wl.H):
+        gu.check_attention(whole[0][0, h], whole[1][0, h], ref[0][0, h], ref[1][0, h], f"head {h}", strict=False)
+    bits = attention(run, api.rf_sparse_attn_fwd_plus)
+    api.rf_reorder_tokens(run.shape, run.params, run.q, run.k, run.v, run.head_class, run.ws)
+    assert same_bits(attention(run, api.rf_sparse_attn_reordered), bits)
+    run.mem.check("workspace without pieces")
+    # the host pipeline's block: without the room the groups' pieces would take, the call's bits are those of whole items
+    lib, pipe = api.load(), C.c_void_p()
+    full = lib.rf_host_pipeline_staging_bytes(C.byref(run.shape), C.byref(run.params), 2)
+    staging = torch.empty(full, dtype=torch.uint8, device="cuda")
+    assert lib.rf_host_pipeline_create(C.byref(run.shape), C.byref(run.params), 2, staging.data_ptr(), full - (1 << 20), C.byref(pipe)) == 0
+    q, k, v, o = (t.cpu().pin_memory() for t in (run.q, run.k, run.v, torch.zeros_like(run.q)))
+    assert lib.rf_host_pipeline_run(pipe, q.data_ptr(), k.data_ptr(), v.data_ptr(), o.data_ptr(), None) == 0
+    lib.rf_host_pipeline_destroy(pipe)                 # waits
+    assert np.array_equal(gu.bits_of(o), bits[0])
+    run.ws = run.ws[:3 * run.q.numel() * 2]            # no room for ARM's scratch either: refused as ever
+    with pytest.raises(api.RainFusionError, match="workspace"):
+        run.arm()
