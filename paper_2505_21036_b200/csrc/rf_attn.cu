@@ -228,6 +228,7 @@ __device__ __noinline__ void leave_piece(const RfAttnArgs& a, const int* iw, uin
 #pragma unroll 1
   for (int c0 = 0; c0 < D; c0 += kCols) {
     float m = -INFINITY, l = 0.f, l_all = 0.f;
+    bool any = false;                                          // some piece lists a tile for these rows
     float4 acc[kCols / 4];
 #pragma unroll
     for (int i = 0; i < kCols / 4; ++i) acc[i] = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -239,6 +240,7 @@ __device__ __noinline__ void leave_piece(const RfAttnArgs& a, const int* iw, uin
 #pragma unroll
       for (int i = 0; i < kCols / 4; ++i) o[i] = __ldcg(at + (c0 / 4 + i) * BM);
       if (st.w == 0.f) continue;                               // listed no tile: its O was never written
+      any = true;
       // where one side has no maximum its O and sums are zero (or not numbers): they are added as they are
       float keep = 1.f, w = 1.f;
       if (st.x > m) {
@@ -257,7 +259,7 @@ __device__ __noinline__ void leave_piece(const RfAttnArgs& a, const int* iw, uin
         acc[i].w = acc[i].w * keep + o[i].w * w;
       }
     }
-    if (!row.inside) continue;
+    if (!row.inside || !any) continue;
     const float inv = l > 0.f ? 1.f / l : 0.f;
 #pragma unroll
     for (int q = 0; q < kCols / 16; ++q) {

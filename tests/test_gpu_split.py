@@ -170,3 +170,21 @@ def test_a_workspace_without_room_for_pieces_still_serves():
     run.ws = run.ws[:3 * run.q.numel() * 2]            # no room for ARM's scratch either: refused as ever
     with pytest.raises(api.RainFusionError, match="workspace"):
         run.arm()
+
+
+def test_rows_that_list_no_tile_are_not_written_in_a_split_item_either():
+    """One query tile of a split pair without an entry: its rows stay as they are, the other tile's are what they were."""
+    run = gu.Run(small_split())
+    run.force_classes([orc.SPATIAL, orc.SPATIAL, orc.TEXTURAL])   # original order: a tile's rows are its tokens
+    run.build()
+    o, lse = run.sparse()
+    run.sched.count[0, :, 3] = 0
+    o2, lse2 = run.outputs()
+    api.rf_sparse_attn_fwd(run.shape, run.params, run.q, run.k, run.v, run.head_class, run.sched, o2, lse2, run.ws, run.status)
+    torch.cuda.synchronize()
+    assert int(run.status.item()) == 0
+    got_o, got_l = o2.float().cpu().numpy(), lse2.cpu().numpy()
+    none = np.zeros(run.wl.N, dtype=bool)
+    none[3 * 128:4 * 128] = True
+    assert np.isnan(got_o[:, :, none]).all() and np.isnan(got_l[:, :, none]).all()
+    assert np.array_equal(got_o[:, :, ~none], o[:, :, ~none]) and np.array_equal(got_l[:, :, ~none], lse[:, :, ~none])
