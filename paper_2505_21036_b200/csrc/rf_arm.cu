@@ -42,6 +42,7 @@ constexpr int ARM_TILE = 128;
 constexpr int ARM_HALF = 64;               // scores a thread holds at a time
 constexpr int ARM_THREADS = 320;           // softmax of even tiles, of odd tiles, TMA, MMA
 constexpr int ARM_TMA_WARP = 8, ARM_MMA_WARP = 9;
+constexpr float kLeast = -1e38f;           // scores times log2(e) / sqrt(D), at most 0.18, stay above -6.2e37
 
 struct ArmMaps { CUtensorMap q[2], k[2]; };   // per sample: 0 = stride sample, 1 = first-frame sample
 
@@ -206,7 +207,9 @@ __global__ void __launch_bounds__(ARM_THREADS, 2) rf_arm_kernel(const __grid_con
   // Masks k = 0..NB-1: Temporal with window win.ws[k]; k = NB..2NB-1: Spatial with win.wf[k-NB];
   // k = 2NB: Textural.  Band masks keep one key interval per row in sample-index space.
   constexpr int NM = 2 * NB + 1;
-  float mx = -INFINITY, l_all = 0.f;
+  // The running maximum starts at a finite value below any finite score: a tile whose scores are all -inf (a key that is -inf
+  // where the query is not zero) then adds nothing, instead of -inf - -inf.
+  float mx = kLeast, l_all = 0.f;
   float l_m[NM];
 #pragma unroll
   for (int k = 0; k < NM; ++k) l_m[k] = 0.f;
@@ -315,7 +318,7 @@ __global__ void __launch_bounds__(ARM_THREADS, 2) rf_arm_kernel(const __grid_con
       float top = half_max(s, u0, n, -INFINITY);
       load_half(t_s + ARM_HALF, s);
       top = half_max(s, u0 + ARM_HALF, n, top);
-      const float m_new = fmaxf(mx, top * scale_log2);   // finite: every tile holds a real key
+      const float m_new = fmaxf(mx, top * scale_log2);
       const float corr = ex2f(mx - m_new);
       l_all *= corr;
 #pragma unroll
@@ -389,7 +392,7 @@ __global__ void __launch_bounds__(ARM_THREADS, 2) rf_arm_kernel(const __grid_con
   __syncthreads();
   if (warp < 4 && m < n) {
     const float m1 = join[0], top = fmaxf(mx, m1);
-    const float f0 = ex2f(mx - top), f1 = ex2f(m1 - top);        // no odd tile: m1 = -inf, factor 0
+    const float f0 = ex2f(mx - top), f1 = ex2f(m1 - top);        // no odd tile: m1 = kLeast, factor 0
     const float inv = 1.f / (l_all * f0 + join[128] * f1);
     float* out = sm.out + (size_t)bh * NM * n_pad;
 #pragma unroll

@@ -272,6 +272,20 @@ def test_arm_edge_shapes():
             check_arm(wl)
 
 
+@pytest.mark.parametrize("mode", [0, 1])
+def test_arm_with_a_key_tile_of_minus_infinity(mode):
+    """Sampled keys 128..255, the second tile of the sample, score -inf with every query: they weigh nothing, and the other
+    tiles' masses are what they are."""
+    wl = synth.small_workload("inf", H=3, D=64, T=4, fh=15, fw=20, L=9, wf=1, ws=75, tau=2, mode=mode, omega=4, amp=2.0)
+    q, k, v = (x.copy() for x in synth.make_qkv(wl))
+    q[..., 0] = synth.f32_to_bf16_bits(np.float32(4.0))
+    k[..., 0] = 0
+    second = np.arange(128, 256)
+    for stride in (1, 4) if mode == 0 else (4,):          # the first frame, the stride sample
+        k[:, :, second * stride, 0] = 0xFF80
+    check_arm(wl, gu.Run(wl, qkv=(q, k, v)))
+
+
 def test_windows_and_stride_far_past_the_extent():
     """frame_window, spatial_window and textural_stride at INT_MAX: the masks are those of the extent itself
     (everything kept; the diagonal y == x), recalls 1, and nothing in the index arithmetic overflows."""
