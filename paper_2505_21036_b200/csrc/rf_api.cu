@@ -164,12 +164,10 @@ rf_status rf_checked_geom(const rf_shape* shape, const rf_params* params, RfGeom
 }
 
 namespace {
-// Shared by rf_sparse_attn_fwd(_plus) and rf_sparse_attn_reordered: the second skips the gather pass and
-// reads the reordered copies a preceding rf_reorder_tokens call left in the workspace.
-rf_status sparse_attn_impl(const rf_shape* shape, const rf_params* params, const void* q, const void* k, const void* v,
-                           const int32_t* head_class, const int32_t* head_window, const rf_schedule* sched, void* o,
-                           float* lse, void* ws, size_t ws_bytes, int32_t* dev_status, void* cuda_stream, bool gather,
-                           int heads_total, int head0) {
+// What the host can see wrong with the arguments of a sparse attention call.
+rf_status check_sparse_attn(const rf_shape* shape, const rf_params* params, const void* q, const void* k, const void* v,
+                            const int32_t* head_class, const int32_t* head_window, const rf_schedule* sched, const void* o,
+                            const void* ws, size_t ws_bytes) {
   rf_status st = check_attn_shape(shape);
   if (st != RF_OK) return st;
   st = check_params(params);
@@ -186,7 +184,18 @@ rf_status sparse_attn_impl(const rf_shape* shape, const rf_params* params, const
   if (head_window != nullptr && params->temporal_window_2d) return RF_ERR_UNSUPPORTED;
   const RfGeom g = make_geom(shape, params);
   if (ws_bytes < least_bytes(g, params)) return RF_ERR_WORKSPACE_TOO_SMALL;
-  if (sched->nQ != g.nQ || sched->nKmax != g.nKmax) return RF_ERR_INVALID_ARG;
+  return sched->nQ == g.nQ && sched->nKmax == g.nKmax ? RF_OK : RF_ERR_INVALID_ARG;
+}
+
+// Shared by rf_sparse_attn_fwd(_plus) and rf_sparse_attn_reordered: the second skips the gather pass and
+// reads the reordered copies a preceding rf_reorder_tokens call left in the workspace.
+rf_status sparse_attn_impl(const rf_shape* shape, const rf_params* params, const void* q, const void* k, const void* v,
+                           const int32_t* head_class, const int32_t* head_window, const rf_schedule* sched, void* o,
+                           float* lse, void* ws, size_t ws_bytes, int32_t* dev_status, void* cuda_stream, bool gather,
+                           int heads_total, int head0) {
+  const rf_status st = check_sparse_attn(shape, params, q, k, v, head_class, head_window, sched, o, ws, ws_bytes);
+  if (st != RF_OK) return st;
+  const RfGeom g = make_geom(shape, params);
   cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
 
   uint8_t* w = static_cast<uint8_t*>(ws);
@@ -467,9 +476,13 @@ rf_status rf_sparse_call(const rf_shape* shape, const rf_params* params, const f
                          float* lse, void* ws, size_t ws_bytes, int32_t* dev_status, void* cuda_stream) {
   if (n_bandwidths < 0) return RF_ERR_INVALID_ARG;
   if (n_bandwidths == 0) head_window = nullptr;
-  rf_status st = n_bandwidths > 0 ? rf_arm_classify_plus(shape, params, bandwidths, n_bandwidths, q, k, head_class, head_window,
-                                                         nullptr, ws, ws_bytes, dev_status, cuda_stream)
-                                  : rf_arm_classify(shape, params, q, k, head_class, nullptr, ws, ws_bytes, dev_status, cuda_stream);
+  // ARM checks its own arguments before it launches; what the two calls after it would refuse is refused here
+  rf_status st = check_sparse_attn(shape, params, q, k, v, head_class, head_window, sched, o, ws, ws_bytes);
+  if (st == RF_OK && sched->kv_len == nullptr) st = RF_ERR_INVALID_ARG;
+  if (st != RF_OK) return st;
+  st = n_bandwidths > 0 ? rf_arm_classify_plus(shape, params, bandwidths, n_bandwidths, q, k, head_class, head_window, nullptr, ws,
+                                               ws_bytes, dev_status, cuda_stream)
+                        : rf_arm_classify(shape, params, q, k, head_class, nullptr, ws, ws_bytes, dev_status, cuda_stream);
   if (st == RF_OK) st = rf_build_block_mask_plus(shape, params, head_class, head_window, sched, dev_status, cuda_stream);
   if (st == RF_OK)
     st = rf_sparse_attn_fwd_plus(shape, params, q, k, v, head_class, head_window, sched, o, lse, ws, ws_bytes, dev_status, cuda_stream);

@@ -90,6 +90,26 @@ def test_bad_shapes_and_pointers_are_rejected_before_cuda(lib):
                                   1 << 30, None, None) == 2            # attention needs 128 x 128 tiles
 
 
+def test_a_sparse_call_is_refused_before_its_first_launch(lib):
+    """rf_sparse_call: what the last of its three calls would refuse is refused before the first one launches anything
+    (which here, without a device, would be RF_ERR_CUDA)."""
+    wl = synth.WORKLOADS["tiny"]
+    s, p = api.shape_of(wl), api.params_of(wl)
+    nq, nk = api.rf_schedule_dims(s, p)
+    good = dict(params=p, n=0, v=256, hw=None, sched=api.rf_schedule(256, 256, None, 256, nq, nk), o=256, ws=1 << 30)
+
+    def call(**kw):
+        a = dict(good, **kw)
+        bw = (C.c_float * 4)(0.125, 0.25, 0.5, 1.0)
+        return lib.rf_sparse_call(C.byref(s), C.byref(a["params"]), bw, a["n"], 256, 256, a["v"], 256, a["hw"], C.byref(a["sched"]),
+                                  a["o"], None, 256, a["ws"], None, None)
+    assert call(o=None) == call(v=None) == call(o=264) == call(n=-1) == call(n=3) == call(n=5, hw=256) == 1
+    assert call(sched=api.rf_schedule(256, 256, None, None, nq, nk)) == call(sched=api.rf_schedule(256, 256, None, 256, nq, 1)) == 1
+    assert call(params=api.params_of(wl, 64, 64)) == 2
+    assert call(params=api.params_of(wl, temporal_window_2d=(1, 1)), n=3, hw=256) == 2
+    assert call(ws=16) == 3
+
+
 def test_oversized_windows_and_strides_are_accepted_and_bounded(lib):
     """A window past the extent or a checkerboard stride past the frame means what the extent means; the host
     side must neither reject it nor loop over it (textural_stride = INT_MAX used to cost 2^31 iterations)."""
