@@ -503,6 +503,7 @@ rf_status rf_reorder_tokens(const rf_shape* shape, const rf_params* params, cons
   if (st != RF_OK) return st;
   st = check_2d(shape, params);
   if (st != RF_OK) return st;
+  if (shape->D > 2048) return RF_ERR_UNSUPPORTED;   // a row is at most one CTA's 256 vectors of 16 bytes
   if (q == nullptr || k == nullptr || v == nullptr || head_class == nullptr || ws == nullptr) return RF_ERR_INVALID_ARG;
   if (!aligned16(q) || !aligned16(k) || !aligned16(v) || (reinterpret_cast<uintptr_t>(ws) & (kAlign - 1)) != 0)
     return RF_ERR_INVALID_ARG;

@@ -3,6 +3,8 @@ declares, and rejects bad arguments before anything touches CUDA."""
 import ctypes as C
 import os
 import re
+import subprocess
+import sys
 
 import pytest
 
@@ -108,6 +110,18 @@ def test_a_sparse_call_is_refused_before_its_first_launch(lib):
     assert call(params=api.params_of(wl, 64, 64)) == 2
     assert call(params=api.params_of(wl, temporal_window_2d=(1, 1)), n=3, hw=256) == 2
     assert call(ws=16) == 3
+
+
+def test_reordering_of_rows_wider_than_a_cta_is_refused():
+    """In a process of its own: a division by zero on the host would end it."""
+    code = """if True:
+        import ctypes as C
+        from paper_2505_21036_b200 import api
+        for D in (2056, 4096):
+            s, p = api.make_shape(1, 1, D, 2, 4, 4, 0), api.make_params(1, 1)
+            assert api.load().rf_reorder_tokens(C.byref(s), C.byref(p), 256, 256, 256, 256, 256, 1 << 40, None) == 2"""
+    res = subprocess.run([sys.executable, "-c", code], cwd=ROOT, capture_output=True, text=True)
+    assert res.returncode == 0, (res.returncode, res.stderr)
 
 
 def test_oversized_windows_and_strides_are_accepted_and_bounded(lib):
