@@ -418,12 +418,11 @@ __global__ void __launch_bounds__(ARM_THREADS, 2) rf_arm_kernel(const __grid_con
 //   the head takes the smallest qualifying window (candidates ascend); Textural heads get window -1.
 __global__ void __launch_bounds__(256) rf_arm_decide_kernel(int nb, int nb_user, int n_loc, int n_glb, int n_pad, int sample_mode,
                                                              float alpha, int two_mask, ArmWindows win, int with_tex,
-                                                             const float* __restrict__ rows_loc,
-                                                             const float* __restrict__ rows_glb,
+                                                             const float* rows_loc, const float* rows_glb,
                                                              int32_t* __restrict__ head_class,
                                                              int32_t* __restrict__ head_window, float* __restrict__ recall,
                                                              float* __restrict__ recall_plus,
-                                                             const int32_t* __restrict__ arm_flag, int32_t* dev_status) {
+                                                             const int32_t* arm_flag, int32_t* dev_status) {
   __shared__ double red[2 * ARM_MAX_NB + 1][8];
   rf_grid_trigger();
   rf_grid_wait();

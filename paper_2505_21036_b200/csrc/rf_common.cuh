@@ -52,6 +52,8 @@ __host__ __device__ __forceinline__ int rf_kv_len(const RfGeom& g, int cls) {
 // Programmatic dependent launch.  Every kernel of the path is launched so that its CTAs may become resident, and set up
 // what depends on no global memory, while the kernel before it in the stream drains; rf_grid_wait then waits until all of
 // that kernel's writes are visible.  All threads of a kernel call it before their first access to global memory.
+// Inputs are plain pointers: const __restrict__ or __ldg would promise that they do not change while the kernel runs, and it
+// runs from before the wait, so such a load need not stay behind it.
 // rf_grid_trigger lets the next kernel's CTAs come in as soon as every CTA of this one has called it or ended.
 __device__ __forceinline__ void rf_grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void rf_grid_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }

@@ -109,8 +109,7 @@ __device__ int tile_flag(const RfGeom& g, int cls, int a, int b) {
 
 // One warp per (query tile, head): flags for 32 key tiles at a time, ordered compaction by ballot.
 // No block-level synchronisation; eight rows per CTA.
-__global__ void __launch_bounds__(256) rf_build_tiles_kernel(RfGeom g, const int32_t* __restrict__ head_class,
-                                                              const int32_t* __restrict__ head_window,
+__global__ void __launch_bounds__(256) rf_build_tiles_kernel(RfGeom g, const int32_t* head_class, const int32_t* head_window,
                                                               int32_t* __restrict__ count, int32_t* __restrict__ kv_tile,
                                                               uint32_t* __restrict__ bitmap, int32_t* __restrict__ kv_len,
                                                               int32_t* dev_status) {
@@ -160,9 +159,8 @@ __global__ void __launch_bounds__(256) rf_build_tiles_kernel(RfGeom g, const int
 // row that is not copied and no table has to be built first.  48 heads, 17 776 tokens, D = 64, all Textural: 133 -> 44 us
 // (221 MB); 24 heads, 8448 tokens, D = 128, 8/8/8: 41 -> 25 us (139 MB).
 constexpr int kGatherRows = 4;
-__global__ void __launch_bounds__(256) rf_gather_kernel(RfGeom g, const int32_t* __restrict__ head_class,
-                                                         const uint4* __restrict__ q, const uint4* __restrict__ k,
-                                                         const uint4* __restrict__ v, uint4* __restrict__ wq,
+__global__ void __launch_bounds__(256) rf_gather_kernel(RfGeom g, const int32_t* head_class, const uint4* q, const uint4* k,
+                                                         const uint4* v, uint4* __restrict__ wq,
                                                          uint4* __restrict__ wk, uint4* __restrict__ wv, int32_t* tickets,
                                                          int n_tickets, int32_t* dev_status) {
   rf_grid_trigger();
@@ -209,9 +207,9 @@ __global__ void __launch_bounds__(256) rf_gather_kernel(RfGeom g, const int32_t*
     for (int r = 0; r < kGatherRows; ++r) {
       if (!on[r]) continue;
       const size_t s = head_off + (size_t)src[r] * vec;
-      if (perm) tq[r] = __ldg(q + s);
-      tk[r] = __ldg(k + s);
-      tv[r] = __ldg(v + s);
+      if (perm) tq[r] = q[s];
+      tk[r] = k[s];
+      tv[r] = v[s];
     }
 #pragma unroll
     for (int r = 0; r < kGatherRows; ++r) {
