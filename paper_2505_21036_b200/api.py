@@ -332,11 +332,19 @@ def rf_reorder_tokens(shape, params, q, k, v, head_class, ws):
                                     head_class.data_ptr(), ws.data_ptr(), ws.numel(), _stream()), "rf_reorder_tokens")
 
 
-def rf_dense_attn_fwd(shape, q, k, v, o, lse, dev_status=None):
-    """Takes the scratch that split items need (shapes of few items only) from torch's allocator for the call."""
+def rf_dense_attn_fwd(shape, q, k, v, o, lse, dev_status=None, scratch=None):
+    """Shapes of few query tiles share the last ones between SMs and need scratch for that (rf_dense_workspace_bytes): the
+    caller's uint8 tensor (one that is too small, an empty one say, does without), or by default a block from torch's
+    allocator for the time of the call, so that calls on several streams stay independent; where it has none left the call does
+    without."""
     import torch
     lib = load()
-    n = lib.rf_dense_workspace_bytes(C.byref(shape))
-    ws = torch.empty(n, dtype=torch.uint8, device=q.device) if n else None
+    if scratch is None:
+        n = lib.rf_dense_workspace_bytes(C.byref(shape))
+        try:
+            scratch = torch.empty(n, dtype=torch.uint8, device=q.device) if n else None
+        except torch.OutOfMemoryError:
+            pass
     _check(lib.rf_dense_attn_fwd_split(C.byref(shape), q.data_ptr(), k.data_ptr(), v.data_ptr(), o.data_ptr(), _ptr(lse),
-                                       _ptr(ws), n, _ptr(dev_status), _stream()), "rf_dense_attn_fwd")
+                                       _ptr(scratch), 0 if scratch is None else scratch.numel(), _ptr(dev_status), _stream()),
+           "rf_dense_attn_fwd")

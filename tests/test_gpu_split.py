@@ -188,3 +188,27 @@ def test_rows_that_list_no_tile_are_not_written_in_a_split_item_either():
     none[3 * 128:4 * 128] = True
     assert np.isnan(got_o[:, :, none]).all() and np.isnan(got_l[:, :, none]).all()
     assert np.array_equal(got_o[:, :, ~none], o[:, :, ~none]) and np.array_equal(got_l[:, :, ~none], lse[:, :, ~none])
+
+
+def test_a_dense_call_does_without_scratch(monkeypatch):
+    """The scratch of a dense call is no necessity: with none left in torch's allocator, or with a tensor of the caller's
+    that is too small, the items stay whole; a tensor that is large enough gives the bits of the default."""
+    run = gu.Run(small_split())
+    n = api.load().rf_dense_workspace_bytes(C.byref(run.shape))
+    own, none = run.mem.alloc((n,), torch.uint8, 0x5A, "scratch"), run.mem.alloc((0,), torch.uint8, name="none")
+
+    def dense(**kw):
+        o, lse = run.outputs()
+        api.rf_dense_attn_fwd(run.shape, run.q, run.k, run.v, o, lse, run.status, **kw)
+        torch.cuda.synchronize()
+        assert int(run.status.item()) == 0
+        run.mem.check("rf_dense_attn_fwd")
+        return gu.bits_of(o).copy(), lse.cpu().numpy().view(np.uint32).copy()
+
+    split = dense()
+
+    def exhausted(*args, **kw):
+        raise torch.OutOfMemoryError("none left")
+    monkeypatch.setattr(torch, "empty", exhausted)
+    without = dense()
+    assert same_bits(dense(scratch=own), split) and same_bits(dense(scratch=none), without) and not same_bits(split, without)
