@@ -199,7 +199,10 @@ __device__ __noinline__ void leave_piece(const RfAttnArgs& a, const int* iw, uin
                                          float l_exact, bool has_o) {
   constexpr size_t kRows = (size_t)(D / 4 + 1) * BM;          // float4 of one piece of one stream
   const int j = warp >> 2, row_in_tile = (warp & 3) * 32 + lane, pieces = iw[8];
-  if (iw[1] + j >= a.g.nQ || !rf_in_bounds(iw[9], a.sp.n_slots, a.dev_status)) return;   // (the warp as a whole)
+  // (the warp as a whole)
+  if (iw[1] + j >= a.g.nQ || !rf_in_bounds(iw[9], a.sp.n_slots, a.dev_status) ||
+      !rf_in_bounds(iw[10] * 8 + warp, a.sp.n_tickets, a.dev_status))
+    return;
   float4* first = reinterpret_cast<float4*>(a.pieces) + ((size_t)(iw[9] - iw[11]) * 2 + j) * kRows + row_in_tile;
   float4* mine = first + (size_t)iw[11] * 2 * kRows;
   if (has_o) {

@@ -52,7 +52,8 @@ def run_child(args, lib, timeout=1200):
 
 def test_small_parity_tests_pass_on_the_checked_build(checked_lib):
     r = run_child([sys.executable, "-m", "pytest", "-q", "-x", "-m", "gpu", "-p", "no:cacheprovider",
-                   "tests/test_gpu_parity.py", "tests/test_gpu_plus.py", "tests/test_golden.py", "tests/test_zz_no_alloc.py"], checked_lib)
+                   "tests/test_gpu_parity.py", "tests/test_gpu_plus.py", "tests/test_gpu_split.py", "tests/test_golden.py",
+                   "tests/test_zz_no_alloc.py"], checked_lib)
     assert r.returncode == 0, r.stdout[-3000:] + r.stderr[-2000:]
 
 
