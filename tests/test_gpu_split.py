@@ -10,6 +10,7 @@ import torch
 import gpu_util as gu
 from oracle import rainfusion_oracle as orc
 from paper_2505_21036_b200 import api, synth
+from paper_2505_21036_b200.layer import RainFusionAttention
 
 pytestmark = pytest.mark.gpu
 
@@ -212,3 +213,106 @@ def test_a_dense_call_does_without_scratch(monkeypatch):
     monkeypatch.setattr(torch, "empty", exhausted)
     without = dense()
     assert same_bits(dense(scratch=own), split) and same_bits(dense(scratch=none), without) and not same_bits(split, without)
+
+
+def check_rows(run, out, classes, windows=None, key_first=False, t2d=None):
+    """96 rows of every head and the last one against the oracle."""
+    wl = run.wl
+    rows = np.unique(np.concatenate([np.random.default_rng(5).choice(wl.N, 96, replace=False), [wl.N - 1]]))
+    for h in range(wl.H):
+        pp = gu.pparams(wl, key_first, t2d)
+        if windows is not None:
+            w = int(windows[h])
+            pp = orc.PatternParams(w if classes[h] == orc.SPATIAL else wl.frame_window,
+                                   w if classes[h] == orc.TEMPORAL else wl.spatial_window, wl.textural_stride)
+        ref, lref = orc.masked_attention(run.q_bits[0, h], run.k_bits[0, h], run.v_bits[0, h], int(classes[h]), gu.geom(wl), pp,
+                                         rows=rows)
+        gu.check_attention(out[0][0, h][rows], out[1][0, h][rows], ref, lref, f"head {h} class {classes[h]}", strict=False)
+
+
+@pytest.mark.parametrize("permute", [0, 1])
+@pytest.mark.parametrize("D", [64, 128])
+def test_split_items_with_the_other_readings_of_the_patterns(D, permute):
+    run = gu.Run(small_split(D=D), temporal_permute=permute, t2d=(3, 4), key_first=1)
+    classes = [orc.SPATIAL, orc.TEMPORAL, orc.TEXTURAL]
+    run.force_classes(classes)
+    run.build()
+    check_rows(run, run.sparse(), classes, key_first=True, t2d=(3, 4))
+
+
+def test_split_items_with_a_window_per_head():
+    run = gu.Run(small_split())
+    classes, windows, _ = run.arm_plus([0.125, 0.25, 0.5])
+    run.build_plus()
+    check_rows(run, run.sparse_plus(), classes[0], windows[0])
+
+
+@pytest.mark.parametrize("shape", [dict(), dict(T=4, L_text=37)])      # in pieces, whole
+@pytest.mark.parametrize("D", [64, 96, 128])
+def test_output_without_lse_is_the_output_with_it(D, shape):
+    run = gu.Run(small_split(D=D, **shape))
+    run.force_classes([0, 1, 2])
+    run.build()
+    o, lse = run.outputs()
+
+    def both(call):
+        bits = []
+        for wanted in (lse, None):
+            o.fill_(float("nan"))
+            call(wanted)
+            torch.cuda.synchronize()
+            assert int(run.status.item()) == 0
+            bits.append(gu.bits_of(o).copy())
+        assert np.array_equal(*bits) and np.isfinite(o.float().cpu().numpy()).all()
+    both(lambda l: api.rf_sparse_attn_fwd(run.shape, run.params, run.q, run.k, run.v, run.head_class, run.sched, o, l, run.ws, run.status))
+    both(lambda l: api.rf_dense_attn_fwd(run.shape, run.q, run.k, run.v, o, l, run.status))
+
+
+# four heads: every item in pieces; six: the last 44 of 192, which begin inside the second of two groups
+FOUR = small_split(H=4)
+SIX = small_split(H=6, D=64, T=16, frame_h=16, frame_w=32, L_text=0, sample_stride=16, frame_window=4, spatial_window=128)
+
+
+def test_the_shapes_here_have_items_in_pieces():
+    """Their workspaces hold more than the reordered copies and ARM's rows, else the tests around this one show little."""
+    for wl in (small_split(), FOUR, SIX):
+        rows = -(-max(wl.S, -(-wl.Nv // wl.sample_stride)) // 64) * 64
+        others = 3 * wl.H * wl.N * wl.D * 2 + 2 * wl.H * 9 * rows * 4
+        piece = 2 * 128 * (wl.D + 4) * 4
+        assert api.rf_workspace_bytes(api.shape_of(wl), api.params_of(wl)) > others + 2 * piece
+
+
+@pytest.mark.parametrize("bandwidths", [None, [0.125, 0.25, 0.5]])
+@pytest.mark.parametrize("wl,groups", [(FOUR, 1), (FOUR, 2), (FOUR, 4), (SIX, 2), (SIX, 3), (SIX, 6)])
+def test_split_items_of_a_call_in_groups_of_heads(wl, groups, bandwidths):
+    """The plan is the whole call's, whichever heads a group holds: the output's bits are the resident call's."""
+    shape, params = api.shape_of(wl), api.params_of(wl)
+    host = [torch.from_numpy(x.view(np.int16)).view(torch.bfloat16).pin_memory() for x in synth.make_qkv(wl)]
+    oh = torch.full(host[0].shape, float("nan"), dtype=torch.bfloat16).pin_memory()
+    pipe = api.HostPipeline(shape, params, "cuda", groups)
+    pipe.set_bandwidths(bandwidths or [])
+    for _ in range(2):
+        pipe.run(*host, oh)
+    assert pipe.status() == 0
+    resident = RainFusionAttention(shape, params, "cuda", dense_fraction=0.0, bandwidths=bandwidths)
+    q, k, v = (t.cuda() for t in host)
+    o = torch.empty_like(q)
+    resident(q, k, v, o)
+    resident.check()
+    assert torch.equal(oh.view(torch.int16), o.cpu().view(torch.int16))
+    pipe.close()
+
+
+def test_split_items_in_a_replayed_graph():
+    shape, params = api.shape_of(FOUR), api.params_of(FOUR)
+    eager, graphed = (RainFusionAttention(shape, params, "cuda", dense_fraction=0.0, graph=g) for g in (False, True))
+    q, k, v = (gu.to_dev(x) for x in synth.make_qkv(FOUR))
+    og, oe = torch.empty_like(q), torch.empty_like(q)
+    for _ in range(3):
+        graphed(q, k, v, og)
+        eager(q, k, v, oe)
+        torch.cuda.synchronize()
+        assert torch.equal(og.view(torch.int16), oe.view(torch.int16))
+        q.copy_(torch.roll(q.clone(), 1, dims=1))          # other classes, other lists, other pieces
+    eager.check()
+    graphed.check()
