@@ -472,7 +472,7 @@ __global__ void __launch_bounds__(256) rf_arm_decide_kernel(int nb, int nb_user,
         cls = t ? RF_TEMPORAL : RF_SPATIAL;
         window = t ? win.ws[nb_user - 1] : win.wf[nb_user - 1];
       }
-      // nb slots were evaluated (the caller's nb_user candidates, padded by repeating the last one)
+      // of the kernel's nb slots the caller's nb_user candidates are the first; the others stay empty
       for (int i = nb_user - 1; i >= 0; --i)
         if (R[nb + i] >= alpha) { cls = RF_SPATIAL; window = win.wf[i]; }
       for (int i = nb_user - 1; i >= 0; --i)
@@ -539,7 +539,7 @@ cudaError_t rf_launch_arm(const RfGeom& g, int sample_mode, int omega, float alp
                           int32_t* head_window, float* recall, float* recall_plus, float* row_scratch, int32_t* dev_status,
                           cudaStream_t st, bool selftest_abandon) {
   const bool plus = head_window != nullptr;
-  const int NB = plus ? ARM_MAX_NB : 1;           // windows the kernel evaluates (candidate list padded by repetition)
+  const int NB = plus ? ARM_MAX_NB : 1;           // windows the kernel has room for; it evaluates the first nb
   if (nb < 1 || nb > NB) return cudaErrorInvalidValue;
   ArmWindows win;
   win.n = nb;

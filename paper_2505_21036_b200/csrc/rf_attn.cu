@@ -10,7 +10,7 @@
 // thread's shorter code).  Warp roles:
 //   warps 0-3  softmax of stream 0   (one thread per query row, TMEM lane = row)
 //   warps 4-7  softmax of stream 1
-//   warp  8    TMA producer: Q once, then K and V tiles into two shared-memory rings (V of tile u and K of
+//   warp  8    TMA producer: Q once per item, K and V tiles into two shared-memory rings (V of tile u and K of
 //              tile u + 1 as a pair under one full / one empty mbarrier)
 //   warp  9    MMA issuer: tcgen05.mma, accumulators in TMEM (S0, S1, O0, O1)
 //   warp  10   one thread fetches items and publishes them in shared memory
@@ -34,7 +34,7 @@ constexpr int kThreads = kWsThreads;        // 3 warpgroups: softmax 0, softmax 
 constexpr int kTmaWarp = 8, kMmaWarp = 9, kItemWarp = 10;
 constexpr int kItemSlots = 2, kItemWords = 12, kItemReaders = 9;   // readers: eight softmax warps and the TMA thread
 constexpr uint32_t kMore = 4, kLast = 8;   // of a tile record, see the TMA producer
-constexpr int kAskAhead = 4;   // tiles an item has left when the next one is asked for: about 8 us, an answer takes about one
+constexpr int kAskAhead = 4;   // tiles an item's longer list has left when the next item is asked for: 8 us or more, an answer takes about one
 // What bounds the loop: a stream is the chain scores -> softmax -> P V -> Q K^T, so what counts is how few dependent
 // operations stand between the scores' arrival and the hand-over of P.  At D = 96 / 128 the first kSpec weights are taken
 // while the tile's maximum is being found, the first half of P is stored under the second half's exponentials, and the

@@ -141,7 +141,7 @@ struct Lists {
 };
 struct Merge {
   int i0 = 0, i1 = 0;
-  // tiles the union has left at most
+  // entries the longer list has left, so tiles the union has left at least; 0 when both lists are through
   __device__ __forceinline__ int left(const Lists& L) const { return max(L.n0 - i0, L.n1 - i1); }
   // Raw list entries at i0 / i1, loaded by the previous call and not touched until the next one, so
   // that the load latency never sits between two tiles' copies of the (in-order) TMA thread.

@@ -1,7 +1,7 @@
 // Thin inline-PTX layer for sm_100a: mbarrier, TMA tile loads, tcgen05 (TMEM alloc, MMA, ld/st, fences).
 // Every wait is bounded: when the limit runs out the CTA-wide abort flag is raised, the error is
-// reported to the host-visible status word, and every later wait returns at once, so all roles run
-// their fixed-trip-count loops to the end and the kernel terminates normally.
+// reported to the host-visible status word, and every later wait returns at once, so every role comes to the end of
+// its finite work, or leaves where the next step would need what it no longer gets, and the kernel terminates normally.
 #pragma once
 
 #include "rf_common.cuh"
@@ -124,7 +124,6 @@ inline bool rf_regs_ok(K kernel) {
 }
 
 // True in one lane of a converged warp.  (Unlike `lane == 0` this tells the compiler that a single thread runs the branch.)
-// True in one lane of a converged warp.
 __device__ __forceinline__ bool elect_one() {
   uint32_t ok;
   asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(ok));
@@ -160,16 +159,6 @@ __device__ __forceinline__ void tc_commit(uint32_t bar) {
 __device__ __forceinline__ void tc_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 __device__ __forceinline__ void tc_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 
-// Shared-memory matrix descriptor, 128-byte swizzle (layout type 2), descriptor version 1.
-__device__ __forceinline__ uint64_t smem_desc_sw128(uint32_t saddr, uint32_t lbo_bytes, uint32_t sbo_bytes) {
-  uint64_t d = 0;
-  d |= (uint64_t)((saddr & 0x3FFFFu) >> 4);
-  d |= (uint64_t)((lbo_bytes >> 4) & 0x3FFFu) << 16;
-  d |= (uint64_t)((sbo_bytes >> 4) & 0x3FFFu) << 32;
-  d |= 1ull << 46;
-  d |= 2ull << 61;
-  return d;
-}
 // Instruction descriptor, kind::f16: bf16 x bf16 -> fp32, A K-major, B K-major (0) or MN-major (1).
 __host__ __device__ constexpr uint32_t idesc_bf16(int M, int N, int b_mn_major) {
   return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)b_mn_major << 16) | ((uint32_t)(N >> 3) << 17) |
