@@ -109,6 +109,10 @@ EncodeTiledFn encode_fn() {
 bool encode_map(CUtensorMap* m, const void* ptr, int D, int rows, int head_rows, int heads) {
   return rf_encode_rows_map(m, ptr, D, rows, (size_t)D * 2, (size_t)head_rows * D * 2, heads);
 }
+// The same for V: at D = 96 in boxes of 32 columns.
+bool encode_v_map(CUtensorMap* m, const void* ptr, int D, int rows, int head_rows, int heads) {
+  return rf_encode_rows_map(m, ptr, D, rows, (size_t)D * 2, (size_t)head_rows * D * 2, heads, D == 96 ? 32 : 64);
+}
 
 // The workspace: the reordered copies of Q, K and V, the pieces of split items, ARM's scratch.  The offsets depend on the
 // shape alone, so that calls whose other parameters differ find the same things in the same places.
@@ -140,15 +144,15 @@ rf_status check_attn_shape(const rf_shape* s) {
 }  // namespace
 
 bool rf_encode_rows_map(CUtensorMap* m, const void* ptr, int D, int rows, size_t row_stride_bytes,
-                        size_t head_stride_bytes, int heads) {
+                        size_t head_stride_bytes, int heads, int box_columns) {
   EncodeTiledFn fn = encode_fn();
   if (fn == nullptr) return false;
   cuuint64_t dims[3] = {(cuuint64_t)D, (cuuint64_t)rows, (cuuint64_t)heads};
   cuuint64_t strides[2] = {(cuuint64_t)row_stride_bytes, (cuuint64_t)head_stride_bytes};
-  cuuint32_t box[3] = {64, 128, 1};
+  cuuint32_t box[3] = {(cuuint32_t)box_columns, 128, 1};
   cuuint32_t estr[3] = {1, 1, 1};
   return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(ptr), dims, strides, box, estr,
-            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+            CU_TENSOR_MAP_INTERLEAVE_NONE, box_columns == 64 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
@@ -206,9 +210,9 @@ rf_status sparse_attn_impl(const rf_shape* shape, const rf_params* params, const
   CUtensorMap maps[RF_ATTN_MAPS];
   const int heads = g.B * g.H;
   bool ok = encode_map(&maps[0], q, g.D, g.N, g.N, heads) && encode_map(&maps[1], k, g.D, g.N, g.N, heads) &&
-            encode_map(&maps[2], v, g.D, g.N, g.N, heads) && encode_map(&maps[3], wq, g.D, g.N, g.N, heads) &&
-            encode_map(&maps[4], wk, g.D, g.N, g.N, heads) && encode_map(&maps[5], wv, g.D, g.N, g.N, heads) &&
-            encode_map(&maps[6], wk, g.D, g.LkvTex, g.N, heads) && encode_map(&maps[7], wv, g.D, g.LkvTex, g.N, heads);
+            encode_v_map(&maps[2], v, g.D, g.N, g.N, heads) && encode_map(&maps[3], wq, g.D, g.N, g.N, heads) &&
+            encode_map(&maps[4], wk, g.D, g.N, g.N, heads) && encode_v_map(&maps[5], wv, g.D, g.N, g.N, heads) &&
+            encode_map(&maps[6], wk, g.D, g.LkvTex, g.N, heads) && encode_v_map(&maps[7], wv, g.D, g.LkvTex, g.N, heads);
   if (!ok) return RF_ERR_CUDA;
 
   RfAttnArgs a;
@@ -533,7 +537,7 @@ rf_status rf_dense_attn_fwd_split(const rf_shape* shape, const void* q, const vo
   CUtensorMap maps[RF_ATTN_MAPS];
   const int heads = g.B * g.H;
   bool ok = encode_map(&maps[0], q, g.D, g.N, g.N, heads) && encode_map(&maps[1], k, g.D, g.N, g.N, heads) &&
-            encode_map(&maps[2], v, g.D, g.N, g.N, heads);
+            encode_v_map(&maps[2], v, g.D, g.N, g.N, heads);
   if (!ok) return RF_ERR_CUDA;
   for (int i = 3; i < 8; ++i) maps[i] = maps[i % 3];
   RfAttnArgs a;

@@ -16,9 +16,11 @@
 //   warp  10   one thread fetches items and publishes them in shared memory
 //   (warp 11 only fills the third warpgroup, which hands its registers to the softmax warpgroups)
 // Per listed tile and stream: S lands in TMEM, the softmax warps read their rows (tcgen05.ld), keep a
-// running maximum and sum in fp32, write P as packed bf16 back into TMEM (tcgen05.st: on top of the S
+// running maximum in fp32, write P as packed bf16 back into TMEM (tcgen05.st: on top of the S
 // columns at D = 96 / 128, into spare columns at D = 64) and the MMA warp multiplies it with V straight
-// from TMEM.  The running maximum is raised lazily (see kRaise), in which case the softmax warp itself
+// from TMEM.  V carries one column more, of ones: O's column D is the row sum of the weights as rounded to bf16, the ones that
+// are multiplied with V, and normalises O (which makes O an exact convex combination of V rows with slightly perturbed
+// weights: the rounding of a dominant weight cancels instead of scaling the output row).  The running maximum is raised lazily (see kRaise), in which case the softmax warp itself
 // rescales its rows of O in TMEM; the final O / l and the log-sum-exp do not depend on it.
 // PARTIAL tiles apply the exact element mask of the head's pattern; FULL tiles skip it.
 #include <algorithm>
@@ -36,13 +38,15 @@ constexpr int kItemSlots = 2, kItemWords = 12, kItemReaders = 9;   // readers: e
 constexpr uint32_t kMore = 4, kLast = 8;   // of a tile record, see the TMA producer
 constexpr int kAskAhead = 4;   // tiles an item's longer list has left when the next item is asked for: 8 us or more, an answer takes about one
 // What bounds the loop: a stream is the chain scores -> softmax -> P V -> Q K^T, so what counts is how few dependent
-// operations stand between the scores' arrival and the hand-over of P.  At D = 96 / 128 the first kSpec weights are taken
-// while the tile's maximum is being found, the first half of P is stored under the second half's exponentials, and the
-// row sums (192 of 512 instructions) follow the hand-over.  24 heads, 8448 tokens, D = 128 (B200, one box): masked
-// 513 -> 490 us, dense 945 -> 928 us against checking the row sum before the store; without lse the exact sum is left out
-// (a template: dense D = 64, 17776 tokens, 48 heads 5.74 -> 5.59 ms).
-// At D = 64 the maximum comes first and the sums stay in the exponential loop: taking them after the hand-over made the
-// masked case slower (2.94 -> 3.14 ms), the two streams then meet at the exponential pipe.
+// operations stand between the scores' arrival and the hand-over of P, and, once the board is at its power limit (every long
+// call), the energy of a tile, a sixth of which are the softmax warps' instructions.  At D = 96 / 128 the first kSpec weights
+// are taken while the tile's maximum is being found and the first half of P is stored under the second half's exponentials;
+// at D = 64 the maximum comes first.  The row sums of the rounded weights were 192 of a row's 512 instructions a tile
+// (two to widen a pair, one to add it); the tensor pipe takes them in 16 columns more of P V (64 cycles of its 2048 a pair of
+// tiles at D = 128).  Repeated calls at the power limit, before and after: dense 24 heads, 8448 tokens, D = 128 870 -> 841 us;
+// 24 heads, 119 056 tokens 73.8 -> 71.7 ms; 48 heads, 5082 tokens, D = 96 2530 -> 2415 us; 48 heads, 17 776 tokens,
+// D = 64 2900 -> 2763 us masked, 5340 -> 4990 dense.  Error against 64 bits the same to 1e-7 on rel 1.7e-3.
+// Without lse the sum of the unrounded weights is left out (a template: dense D = 64 5.74 -> 5.59 ms).
 // Lazy rescaling of the running maximum: it is raised once a tile's maximum exceeds it by kRaise (log2 units; all rows
 // of the warp more than kRaiseMargin above theirs then raise it together).  A tile's weights thus sum to 2^32 at most;
 // bf16 P and the fp32 sums carry the same relative precision at every exponent and 2^32 times the longest row is far
@@ -75,10 +79,18 @@ struct Cfg {
   static __host__ __device__ constexpr uint32_t koff(int ks) {
     return ks < 4 ? (uint32_t)ks * 32u : BLK + (uint32_t)(ks - 4) * 32u;
   }
+  // V, the MN-major operand of P V, lies in blocks of VBOX columns; behind its D columns stands a block whose first column
+  // is one and whose others are zero, so that O's column D is the row sum of the weights (see the softmax).  At D = 96
+  // blocks of 32 columns (64-byte swizzle) put that block next to column 95.
+  static constexpr int VBOX = D == 96 ? 32 : 64;
+  static constexpr uint32_t VROW = VBOX * 2, VBLK = 128 * VROW, VLOAD = D / VBOX * VBLK, VTILE = VLOAD + VBLK;
+  static constexpr int NPV = D + 16;                  // columns of O += P V
+  // Byte offset of the 16-byte chunk c of a row of such a block; chunks 0 and 1 are the 16 columns P V takes.
+  static __host__ __device__ constexpr uint32_t vchunk(int row, int c) { return row * VROW + ((VBOX == 64 ? c ^ (row & 7) : c ^ ((row >> 1) & 3)) << 4); }
   static constexpr uint32_t Q = 0;
   static constexpr uint32_t K0 = Q + 2 * TILE;
   static constexpr uint32_t V0 = K0 + NK * TILE;
-  static constexpr uint32_t BAR = V0 + NV * TILE;
+  static constexpr uint32_t BAR = V0 + NV * VTILE;
   // barrier slots (8 bytes each)
   // V of tile u and K of tile u + 1 travel as a pair: they are wanted in the same iteration of the MMA warp and
   // released by it together, so one full and one empty barrier per pair (B_F, B_E) serve both; K of the first
@@ -86,18 +98,22 @@ struct Cfg {
   static_assert(NK == NV, "K and V rings advance together");
   static constexpr int NP = NV;
   static constexpr int B_Q = 0, B_K0 = 1, B_K0E = 2, B_F = 3, B_E = B_F + NP, B_SF = B_E + NP,
-                       B_PF = B_SF + 2, B_OF = B_PF + 2, B_SE = B_OF + 2 /* S read, S_EARLY only */, B_QE = B_SE + 2 /* Q consumed */,
+                       B_PF = B_SF + 2, B_OF = B_PF + 2, B_SE = B_OF + 2 /* S read, not at D = 96 */, B_QE = B_SE + 2 /* Q consumed */,
                        B_REQ = B_QE + 1, B_CLC = B_REQ + 1, B_IF = B_CLC + 1, B_IE = B_IF + kItemSlots, B_COUNT = B_IE + kItemSlots;
   static constexpr uint32_t MISC = BAR + 8 * ((B_COUNT + 7) / 8 * 8);
-  static constexpr uint32_t KEEP = MISC + 64;         // 128-bit keep word per softmax thread
-  static constexpr uint32_t ITEM = KEEP + 256 * 16;   // kItemSlots items of kItemWords words, then the launch-control answer
+  static constexpr uint32_t ITEM = MISC + 64;         // kItemSlots items of kItemWords words, then the launch-control answer
   static constexpr uint32_t ANSWER = ITEM + kItemSlots * kItemWords * 4;
   static constexpr uint32_t RECORD = ANSWER + 16;     // tile records: one per ring slot, then the first tile's
   static constexpr uint32_t TOTAL = RECORD + 4 * (NP + 1);
   static constexpr uint32_t ALLOC = TOTAL + 1024;     // slack for manual 1024-byte alignment
-  // TMEM columns
-  static constexpr uint32_t S_COL0 = 0, S_COL1 = 128, O_COL0 = 256, O_COL1 = S_EARLY ? 320 : 384, TMEM_COLS = 512;
-  static constexpr uint32_t P_COL0 = S_EARLY ? 384 : S_COL0, P_COL1 = S_EARLY ? 448 : S_COL1;   // packed bf16, 64 columns
+  static_assert(ALLOC <= 227 * 1024, "shared memory of a CTA");
+  // TMEM columns.  The row sums' 16 columns a stream do not fit beside two whole S at D = 64 and 128, so S0 and S1 share 32
+  // columns there (P lies outside them): a stream's scores are computed once the other stream has read its own.
+  static constexpr bool S_SHARED = D != 96;
+  static constexpr uint32_t S_COL0 = 0, S_COL1 = S_SHARED ? 96 : 128, S_END = S_COL1 + 128, TMEM_COLS = 512;
+  static constexpr uint32_t P_COL0 = S_EARLY ? S_END : S_COL0, P_COL1 = S_EARLY ? S_END + 64 : S_COL1 + 64;   // packed bf16, 64 columns
+  static constexpr uint32_t O_COL0 = S_EARLY ? S_END + 128 : S_END, O_COL1 = O_COL0 + NPV;
+  static_assert(O_COL1 + NPV <= TMEM_COLS, "TMEM columns");
 };
 
 // One item of work: two adjacent query tiles of one head.
@@ -278,7 +294,7 @@ __device__ __noinline__ void leave_piece(const RfAttnArgs& a, const int* iw, uin
   }
 }
 
-// This thread's row of O times alpha (warp-collective).
+// This thread's row of O, and its sum of weights, times alpha (warp-collective).
 template <int D>
 __device__ __forceinline__ void rescale_o(uint32_t t_o, float alpha) {
   tc_fence_after();
@@ -291,6 +307,9 @@ __device__ __forceinline__ void rescale_o(uint32_t t_o, float alpha) {
     for (int i = 0; i < 32; ++i) v[i] = __float_as_uint(__uint_as_float(v[i]) * alpha);
     tmem_st32(t_o + c * 32, v);
   }
+  uint32_t l = tmem_ld1(t_o + D);
+  tc_wait_ld();
+  tmem_st1(t_o + D, __float_as_uint(__uint_as_float(l) * alpha));
   tc_wait_st();
   tc_fence_before();
 }
@@ -331,7 +350,7 @@ __global__ void __launch_bounds__(kThreads, 1) rf_attn_kernel(const __grid_const
   using C = Cfg<D>;
   constexpr int KB = C::KB;
   constexpr uint32_t IDESC_S = idesc_bf16(BM, BN, 0);
-  constexpr uint32_t IDESC_PV = idesc_bf16(BM, D, 1);
+  constexpr uint32_t IDESC_PV = idesc_bf16(BM, C::NPV, 1);
 
   extern __shared__ uint8_t smem_raw[];
   const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
@@ -363,6 +382,11 @@ __global__ void __launch_bounds__(kThreads, 1) rf_attn_kernel(const __grid_const
     *abort_flag = 0;
     mbar_init_fence();
   }
+  for (int i = tid; i < C::NV * BN * 2; i += kThreads) {   // the 16 columns behind V's: one, then zeros
+    const int v = i / (BN * 2), row = i / 2 % BN, c = i % 2;
+    *reinterpret_cast<uint4*>(base_ptr + C::V0 + v * C::VTILE + C::VLOAD + C::vchunk(row, c)) = make_uint4(c == 0 ? 0x3f80u : 0u, 0u, 0u, 0u);
+  }
+  fence_proxy_async_smem();
   if (warp == kTmaWarp) {
     if (lane < 8) prefetch_tmap(&maps.m[lane]);
     __syncwarp();
@@ -529,10 +553,10 @@ __global__ void __launch_bounds__(kThreads, 1) rf_attn_kernel(const __grid_const
         if (u >= C::NP) mbar_wait(bar(C::B_E + ps), ((u / C::NP) - 1) & 1, wc);
         else if (has_nxt && ksn == 0) mbar_wait(bar(C::B_K0E), 0, wc);
         records[ps] = record(has_nxt);
-        mbar_expect_tx(bar(C::B_F + ps), has_nxt ? 2 * C::TILE : C::TILE);
+        mbar_expect_tx(bar(C::B_F + ps), has_nxt ? C::VLOAD + C::TILE : C::VLOAD);
 #pragma unroll
-        for (int kb = 0; kb < KB; ++kb)
-          tma_load_3d(base + C::V0 + ps * C::TILE + kb * C::BLK, cur_v, kb * C::COL1, tile * BN, cur_bh, bar(C::B_F + ps));
+        for (int vb = 0; vb < D / C::VBOX; ++vb)
+          tma_load_3d(base + C::V0 + ps * C::VTILE + vb * C::VBLK, cur_v, vb * C::VBOX, tile * BN, cur_bh, bar(C::B_F + ps));
         if (has_nxt) {
 #pragma unroll
           for (int kb = 0; kb < KB; ++kb)
@@ -557,9 +581,11 @@ __global__ void __launch_bounds__(kThreads, 1) rf_attn_kernel(const __grid_const
       // Descriptors differ only in their 14-bit start-address field: keep the constant words in
       // registers and add the byte offset (>> 4) per k-step.
       constexpr uint32_t DESC_HI = (1024u >> 4) | (1u << 14) | (2u << 29);      // SBO 1024 B, version 1, 128B swizzle
+      constexpr uint32_t DESC_HI_V = C::VBOX == 64 ? DESC_HI : (512u >> 4) | (1u << 14) | (4u << 29);   // SBO 512 B, 64B swizzle
       constexpr uint32_t LO_KMAJOR = 1u << 16;                                    // LBO field unused for K-major
-      constexpr uint32_t LO_VMAJOR = (C::BLK >> 4) << 16;                         // LBO = one 64-column block
+      constexpr uint32_t LO_VMAJOR = (C::VBLK >> 4) << 16;                        // LBO = one block of columns
       auto desc = [](uint32_t lo) -> uint64_t { return ((uint64_t)DESC_HI << 32) | lo; };
+      auto desc_v = [](uint32_t lo) -> uint64_t { return ((uint64_t)DESC_HI_V << 32) | lo; };
       const uint32_t q_lo = ((base + C::Q) >> 4) | LO_KMAJOR, k_lo = ((base + C::K0) >> 4) | LO_KMAJOR;
       const uint32_t v_lo = ((base + C::V0) >> 4) | LO_VMAJOR;
       auto issue_s = [&](int j, int ks) {
@@ -576,17 +602,25 @@ __global__ void __launch_bounds__(kThreads, 1) rf_attn_kernel(const __grid_const
         tc_commit(bar(C::B_SF + j));
       };
       auto issue_pv = [&](int j, int vs, uint32_t acc) {
-        const uint32_t b0 = v_lo + vs * (C::TILE >> 4);
+        const uint32_t b0 = v_lo + vs * (C::VTILE >> 4);
         const uint32_t t_p = tmem_base + (j ? C::P_COL1 : C::P_COL0), t_o = tmem_base + (j ? C::O_COL1 : C::O_COL0);
-        mma_ts(t_o, t_p, desc(b0), IDESC_PV, acc);
+        mma_ts(t_o, t_p, desc_v(b0), IDESC_PV, acc);
 #pragma unroll
         for (int k = 1; k < BN / 16; ++k)
-          mma_ts_c<true>(t_o, t_p + k * 8, desc(b0 + k * (2048 >> 4)), IDESC_PV);
+          mma_ts_c<true>(t_o, t_p + k * 8, desc_v(b0 + k * (16 * C::VROW >> 4)), IDESC_PV);
         tc_commit(bar(C::B_OF + j));
       };
       // one bit per stream
       uint32_t pv_par = 0;               // parity of the P V bursts issued
-      uint32_t s_par = 3;                // S_EARLY: parity of the S tiles issued, less one
+      uint32_t s_par = 3;                // parity of the S tiles issued, less one
+      // Until the columns of S_j may be written: where P lies elsewhere the stream has read its last scores (else its last P V,
+      // issued before, says so), where S0 and S1 share columns the other stream has too.
+      auto s_free = [&](int j) {
+        if (C::S_EARLY) mbar_wait(bar(C::B_SE + j), (s_par >> j) & 1, wc);
+        if (C::S_SHARED) mbar_wait(bar(C::B_SE + (j ^ 1)), (s_par >> (j ^ 1)) & 1, wc);
+        if (C::S_EARLY || C::S_SHARED) tc_fence_after();
+        s_par ^= 1u << j;
+      };
       uint32_t acc = 0;                  // the stream's next P V adds to O (clear: it opens an item)
       uint32_t cur = 0, nq = 0;          // the current tile's record; Q tiles taken
       if (mbar_wait(bar(C::B_K0), 0, wc)) cur = records[C::NP];
@@ -594,8 +628,8 @@ __global__ void __launch_bounds__(kThreads, 1) rf_attn_kernel(const __grid_const
         mbar_wait(bar(C::B_Q), 0, wc);
         ++nq;
         tc_fence_after();
-        if (cur & 1) { issue_s(0, 0); s_par ^= 1; }
-        if (cur & 2) { issue_s(1, 0); s_par ^= 2; }
+        if (cur & 1) { s_free(0); issue_s(0, 0); }
+        if (cur & 2) { s_free(1); issue_s(1, 0); }
         tc_commit(bar(C::B_K0E));
         if (cur & kLast) tc_commit(bar(C::B_QE));
       }
@@ -624,10 +658,9 @@ __global__ void __launch_bounds__(kThreads, 1) rf_attn_kernel(const __grid_const
 #pragma unroll 1
             for (int j = 0; j < 2; ++j) {
               if (nxt & (1 << j)) {
-                if (C::S_EARLY) mbar_wait(bar(C::B_SE + j), (s_par >> j) & 1, wc);
+                s_free(j);
                 tc_fence_after();
                 issue_s(j, ksn);
-                s_par ^= 1u << j;
               }
             }
           }
@@ -639,10 +672,8 @@ __global__ void __launch_bounds__(kThreads, 1) rf_attn_kernel(const __grid_const
 #pragma unroll
           for (int j = 0; j < 2; ++j) {
             if (nxt & (1 << j)) {
-              mbar_wait(bar(C::B_SE + j), (s_par >> j) & 1, wc);
-              tc_fence_after();
+              s_free(j);
               issue_s(j, ksn);
-              s_par ^= 1u << j;
             }
             if (cur & (1 << j)) {
               mbar_wait(bar(C::B_PF + j), (pv_par >> j) & 1, wc);
@@ -662,7 +693,10 @@ __global__ void __launch_bounds__(kThreads, 1) rf_attn_kernel(const __grid_const
               acc |= 1u << j;
               pv_par ^= 1u << j;
             }
-            if (nxt & (1 << j)) issue_s(j, ksn);
+            if (nxt & (1 << j)) {
+              s_free(j);
+              issue_s(j, ksn);
+            }
           }
         }
         if ((nxt & (kMore | kLast)) == (kMore | kLast)) tc_commit(bar(C::B_QE));   // the item's last scores are under way
@@ -680,7 +714,8 @@ __global__ void __launch_bounds__(kThreads, 1) rf_attn_kernel(const __grid_const
     const uint32_t t_s = tmem_base + lane_sel + (j ? C::S_COL1 : C::S_COL0);
     const uint32_t t_o = tmem_base + lane_sel + (j ? C::O_COL1 : C::O_COL0);
     const float sc = a.scale_log2;
-    uint4* keep = reinterpret_cast<uint4*>(base_ptr + C::KEEP) + tid;   // this row's keep words of a PARTIAL tile
+    // this row's keep words of a PARTIAL tile, in the part of V's first block of ones that nothing reads
+    uint4* keep = reinterpret_cast<uint4*>(base_ptr + C::V0 + C::VLOAD + C::vchunk(row_in_tile, 2 + j));
     uint32_t done = 0;         // tiles of this stream in the items before: the barriers' phases run on
     Item im;
     im.n0 = im.n1 = 0;
@@ -690,7 +725,6 @@ __global__ void __launch_bounds__(kThreads, 1) rf_attn_kernel(const __grid_const
     const int32_t* list = a.head_class != nullptr ? a.kv_tile + ((size_t)im.bh * g.nQ + min(im.qt0 + j, g.nQ - 1)) * g.nKmax : nullptr;
     const RowMask rmask = make_row_mask(g, im.cls, im.window, min((im.qt0 + j) * BM + row_in_tile, g.N - 1));
     float m_run = -INFINITY;   // running maximum, log2 domain (score * sc)
-    float l_run = 0.f;         // sum of the weights as rounded to bf16, the ones P V multiplies: normalises O
     float l_exact = 0.f;       // sum of the unrounded weights: the log-sum-exp (LSE only)
 
     const int begin = j == 0 ? im.b0 : im.b1, end = begin + n;
@@ -733,7 +767,6 @@ __global__ void __launch_bounds__(kThreads, 1) rf_attn_kernel(const __grid_const
         if (raise) {
           alpha = ex2(m_run - m_tile);   // 0 when m_run = -inf
           m_run = m_tile;
-          l_run *= alpha;
           if (LSE) l_exact *= alpha;
         }
         // P V of the previous tile reads the P columns this tile is about to overwrite, and O may only be
@@ -748,7 +781,7 @@ __global__ void __launch_bounds__(kThreads, 1) rf_attn_kernel(const __grid_const
         }
         const float m_use = m_run == -INFINITY ? 0.f : m_run;
         const float2 sc2 = make_float2(sc, sc), mneg = make_float2(-m_use, -m_use);
-        float2 la = make_float2(0.f, 0.f), lb = make_float2(0.f, 0.f);
+        float2 la = make_float2(0.f, 0.f);
         uint32_t pk[64];
 #pragma unroll
         for (int c = 0; c < 128; c += 4) {
@@ -759,10 +792,8 @@ __global__ void __launch_bounds__(kThreads, 1) rf_attn_kernel(const __grid_const
           pk[c / 2] = pack_bf16(e0.x, e0.y);
           pk[c / 2 + 1] = pack_bf16(e1.x, e1.y);
           if (LSE) la = __fadd2_rn(la, __fadd2_rn(e0, e1));
-          lb = __fadd2_rn(lb, __fadd2_rn(unpack_bf16(pk[c / 2]), unpack_bf16(pk[c / 2 + 1])));
         }
         if (LSE) l_exact += la.x + la.y;
-        l_run += lb.x + lb.y;
         if (!o_landed) mbar_wait(bar(C::B_OF + j), (done - 1) & 1, wc);
         {
           const uint32_t t_p = tmem_base + lane_sel + (j ? C::P_COL1 : C::P_COL0);
@@ -797,7 +828,6 @@ __global__ void __launch_bounds__(kThreads, 1) rf_attn_kernel(const __grid_const
         if (m_tile > m_run + kRaiseMargin) {
           alpha = ex2(m_run - m_tile);   // 0 when m_run = -inf
           m_run = m_tile;
-          l_run *= alpha;
           if (LSE) l_exact *= alpha;
         }
         if (!opens) {
@@ -811,6 +841,11 @@ __global__ void __launch_bounds__(kThreads, 1) rf_attn_kernel(const __grid_const
         if (partial) mask_scores(keep, s);
         take_weights<0, kSpec, LSE>(s, pk, la, sc2, make_float2(-m_use, -m_use));
       }
+      if constexpr (C::S_SHARED) {
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(bar(C::B_SE + j));
+      }
       const uint32_t t_p = tmem_base + lane_sel + (j ? C::P_COL1 : C::P_COL0);
       take_weights<kSpec, 64, LSE>(s, pk, la, sc2, make_float2(-m_use, -m_use));
       tmem_st32(t_p, *reinterpret_cast<uint32_t(*)[32]>(&pk[0]));
@@ -820,20 +855,18 @@ __global__ void __launch_bounds__(kThreads, 1) rf_attn_kernel(const __grid_const
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(bar(C::B_PF + j));
-      // The row sums gate nothing: they are taken after P has been handed over, under the wait for the next scores.
-      float2 lb[4];
-      lb[0] = lb[1] = lb[2] = lb[3] = make_float2(0.f, 0.f);
-#pragma unroll
-      for (int c = 0; c < 64; c += 2)
-        lb[(c >> 1) & 3] = __fadd2_rn(lb[(c >> 1) & 3], __fadd2_rn(unpack_bf16(pk[c]), unpack_bf16(pk[c + 1])));
-      lb[0] = __fadd2_rn(__fadd2_rn(lb[0], lb[1]), __fadd2_rn(lb[2], lb[3]));
-      l_run += lb[0].x + lb[0].y;
       if (LSE) l_exact += la.x + la.y;
     }
 
     if (n > 0) {
       mbar_wait(bar(C::B_OF + j), (done - 1) & 1, wc);
       tc_fence_after();
+    }
+    // the sum of the weights as rounded to bf16, the ones P V multiplied: normalises O
+    float l_run = 0.f;
+    if (n > 0) {
+      l_run = __uint_as_float(tmem_ld1(t_o + D));
+      tc_wait_ld();
     }
     // the item's words are read again here: kept in registers they would be in the way of the scores
     const int* iw = items + (item % kItemSlots) * kItemWords;

@@ -10,13 +10,6 @@ using namespace sm100;
 
 constexpr int BM = 128, BN = 128;
 
-// The two bf16 values of a packed word, widened exactly.  The row sum is taken over these rounded weights, the
-// ones the tensor core multiplies with V: O / l is then an exact convex combination of V rows with slightly
-// perturbed weights, and the rounding of a dominant weight cancels instead of scaling the whole output row.
-__device__ __forceinline__ float2 unpack_bf16(uint32_t w) {
-  return make_float2(__uint_as_float(w << 16), __uint_as_float(w & 0xffff0000u));
-}
-
 __device__ __forceinline__ float ex2(float x) {
   float y;
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));

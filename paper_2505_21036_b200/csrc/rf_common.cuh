@@ -99,9 +99,9 @@ cudaError_t rf_launch_arm(const RfGeom& g, int sample_mode, int omega, float alp
 #define RF_ARM_FLAG_FLOATS 64
 size_t rf_arm_scratch_floats(const RfGeom& g, int omega, int nb);
 // Tensor map over bf16 rows: [heads][rows][D] with the given row and head strides in bytes (multiples of 16),
-// box = 64 columns x 128 rows, 128-byte swizzle, zero fill past `rows`.
+// box = 64 (or 32) columns x 128 rows, swizzled by the box's row of 128 (64) bytes, zero fill past `rows`.
 bool rf_encode_rows_map(CUtensorMap* m, const void* ptr, int D, int rows, size_t row_stride_bytes,
-                        size_t head_stride_bytes, int heads);
+                        size_t head_stride_bytes, int heads, int box_columns = 64);
 // Validates shape and parameters as the entry points do and fills the kernel-side geometry.
 rf_status rf_checked_geom(const rf_shape* shape, const rf_params* params, RfGeom* out);
 
