@@ -40,8 +40,8 @@ constexpr int kAskAhead = 4;   // tiles an item's longer list has left when the 
 // What bounds the loop: a stream is the chain scores -> softmax -> P V -> Q K^T, so what counts is how few dependent
 // operations stand between the scores' arrival and the hand-over of P, and, once the board is at its power limit (every long
 // call), the energy of a tile, a sixth of which are the softmax warps' instructions.  At D = 96 / 128 the first kSpec weights
-// are taken while the tile's maximum is being found and the first half of P is stored under the second half's exponentials;
-// at D = 64 the maximum comes first.  The row sums of the rounded weights were 192 of a row's 512 instructions a tile
+// are taken while the tile's maximum is being found and the first half of P is stored and multiplied under the second half's
+// exponentials; at D = 64 the maximum comes first.  The row sums of the rounded weights were 192 of a row's 512 instructions a tile
 // (two to widen a pair, one to add it); the tensor pipe takes them in 16 columns more of P V (64 cycles of its 2048 a pair of
 // tiles at D = 128).  Repeated calls at the power limit, before and after: dense 24 heads, 8448 tokens, D = 128 870 -> 841 us;
 // 24 heads, 119 056 tokens 73.8 -> 71.7 ms; 48 heads, 5082 tokens, D = 96 2530 -> 2415 us; 48 heads, 17 776 tokens,
@@ -85,6 +85,11 @@ struct Cfg {
   static constexpr int VBOX = D == 96 ? 32 : 64;
   static constexpr uint32_t VROW = VBOX * 2, VBLK = 128 * VROW, VLOAD = D / VBOX * VBLK, VTILE = VLOAD + VBLK;
   static constexpr int NPV = D + 16;                  // columns of O += P V
+  // P is handed over in parts, part p the keys [cut(p), cut(p + 1)): P V of the first half runs under the exponentials of the
+  // second.  (At D = 64 P V is not on a stream's chain, and half as a part of its own costs more than it hides: dense 8500 ->
+  // 9010 kcycles a call; parts of 96 + 32 or 64 + 32 + 32 keys at D = 96 / 128 are up to 4 % behind the halves.)
+  static constexpr int PARTS = D == 64 ? 1 : 2;
+  static __host__ __device__ constexpr int cut(int p) { return p * (BN / PARTS); }
   // Byte offset of the 16-byte chunk c of a row of such a block; chunks 0 and 1 are the 16 columns P V takes.
   static __host__ __device__ constexpr uint32_t vchunk(int row, int c) { return row * VROW + ((VBOX == 64 ? c ^ (row & 7) : c ^ ((row >> 1) & 3)) << 4); }
   static constexpr uint32_t Q = 0;
@@ -98,7 +103,7 @@ struct Cfg {
   static_assert(NK == NV, "K and V rings advance together");
   static constexpr int NP = NV;
   static constexpr int B_Q = 0, B_K0 = 1, B_K0E = 2, B_F = 3, B_E = B_F + NP, B_SF = B_E + NP,
-                       B_PF = B_SF + 2, B_OF = B_PF + 2, B_SE = B_OF + 2 /* S read, not at D = 96 */, B_QE = B_SE + 2 /* Q consumed */,
+                       B_PF = B_SF + 2, B_OF = B_PF + 2 * PARTS, B_SE = B_OF + 2 /* S read, not at D = 96 */, B_QE = B_SE + 2 /* Q consumed */,
                        B_REQ = B_QE + 1, B_CLC = B_REQ + 1, B_IF = B_CLC + 1, B_IE = B_IF + kItemSlots, B_COUNT = B_IE + kItemSlots;
   static constexpr uint32_t MISC = BAR + 8 * ((B_COUNT + 7) / 8 * 8);
   static constexpr uint32_t ITEM = MISC + 64;         // kItemSlots items of kItemWords words, then the launch-control answer
@@ -295,23 +300,36 @@ __device__ __noinline__ void leave_piece(const RfAttnArgs& a, const int* iw, uin
 }
 
 // This thread's row of O, and its sum of weights, times alpha (warp-collective).
+__device__ __forceinline__ void rescale_columns(uint32_t t_o, float alpha) {
+  uint32_t v[32];
+  tmem_ld32(t_o, v);
+  tc_wait_ld();
+#pragma unroll
+  for (int i = 0; i < 32; ++i) v[i] = __float_as_uint(__uint_as_float(v[i]) * alpha);
+  tmem_st32(t_o, v);
+}
+__device__ __forceinline__ void rescale_sum(uint32_t t_l, float alpha) {
+  const uint32_t l = tmem_ld1(t_l);
+  tc_wait_ld();
+  tmem_st1(t_l, __float_as_uint(__uint_as_float(l) * alpha));
+  tc_wait_st();
+  tc_fence_before();
+}
 template <int D>
 __device__ __forceinline__ void rescale_o(uint32_t t_o, float alpha) {
   tc_fence_after();
 #pragma unroll
-  for (int c = 0; c < D / 32; ++c) {
-    uint32_t v[32];
-    tmem_ld32(t_o + c * 32, v);
-    tc_wait_ld();
-#pragma unroll
-    for (int i = 0; i < 32; ++i) v[i] = __float_as_uint(__uint_as_float(v[i]) * alpha);
-    tmem_st32(t_o + c * 32, v);
-  }
-  uint32_t l = tmem_ld1(t_o + D);
-  tc_wait_ld();
-  tmem_st1(t_o + D, __float_as_uint(__uint_as_float(l) * alpha));
-  tc_wait_st();
-  tc_fence_before();
+  for (int c = 0; c < D; c += 32) rescale_columns(t_o + c, alpha);
+  rescale_sum(t_o + D, alpha);
+}
+// The same out of line, for D = 96 / 128: rare as it is, the scores then stay in registers around it and the loop over the
+// tiles is free of spills.
+template <int D>
+__device__ __noinline__ void rescale_o_call(uint32_t t_o, float alpha) {
+  tc_fence_after();
+#pragma unroll 1
+  for (int c = 0; c < D; c += 32) rescale_columns(t_o + c, alpha);
+  rescale_sum(t_o + D, alpha);
 }
 
 // This thread's row of scores, and the masked ones of a PARTIAL tile set to -inf.
@@ -345,6 +363,14 @@ __device__ __forceinline__ void take_weights(const uint32_t (&s)[BN], uint32_t (
   }
 }
 
+// The packed weights of the key columns [C0, C1) into P.  Eight registers at a time: longer stores want that many consecutive
+// registers, which costs moves (24 heads, 8448 tokens, dense, D = 128: 1153 kcycles a call with 32, 1112 with 16, 1108 with 8).
+template <int C0, int C1>
+__device__ __forceinline__ void store_weights(uint32_t t_p, const uint32_t (&pk)[BN / 2]) {
+#pragma unroll
+  for (int c = C0 / 2; c < C1 / 2; c += 8) tmem_st8(t_p + c, *reinterpret_cast<const uint32_t(*)[8]>(&pk[c]));
+}
+
 template <int D, bool LSE>
 __global__ void __launch_bounds__(kThreads, 1) rf_attn_kernel(const __grid_constant__ Maps maps, const __grid_constant__ RfAttnArgs a) {
   using C = Cfg<D>;
@@ -371,7 +397,7 @@ __global__ void __launch_bounds__(kThreads, 1) rf_attn_kernel(const __grid_const
     for (int s = 0; s < C::NP; ++s) { mbar_init(bar(C::B_F + s), 1); mbar_init(bar(C::B_E + s), 1); }
     for (int j = 0; j < 2; ++j) {
       mbar_init(bar(C::B_SF + j), 1);
-      mbar_init(bar(C::B_PF + j), 4);   // one arrival per softmax warp
+      for (int p = 0; p < C::PARTS; ++p) mbar_init(bar(C::B_PF + j * C::PARTS + p), 4);   // one arrival per softmax warp
       mbar_init(bar(C::B_OF + j), 1);
       mbar_init(bar(C::B_SE + j), 4);
     }
@@ -601,13 +627,20 @@ __global__ void __launch_bounds__(kThreads, 1) rf_attn_kernel(const __grid_const
           mma_ss_c<true>(t_d, desc(a0 + (C::koff(k) >> 4)), desc(b0 + (C::koff(k) >> 4)), IDESC_S);
         tc_commit(bar(C::B_SF + j));
       };
-      auto issue_pv = [&](int j, int vs, uint32_t acc) {
+      // waits for the parts of P (par: the parity they are handed over with) and issues their share of O += P V
+      auto issue_pv = [&](int j, int vs, uint32_t acc, uint32_t par) {
         const uint32_t b0 = v_lo + vs * (C::VTILE >> 4);
         const uint32_t t_p = tmem_base + (j ? C::P_COL1 : C::P_COL0), t_o = tmem_base + (j ? C::O_COL1 : C::O_COL0);
-        mma_ts(t_o, t_p, desc_v(b0), IDESC_PV, acc);
 #pragma unroll
-        for (int k = 1; k < BN / 16; ++k)
-          mma_ts_c<true>(t_o, t_p + k * 8, desc_v(b0 + k * (16 * C::VROW >> 4)), IDESC_PV);
+        for (int p = 0; p < C::PARTS; ++p) {
+          mbar_wait(bar(C::B_PF + j * C::PARTS + p), par, wc);
+          tc_fence_after();
+#pragma unroll
+          for (int k = C::cut(p) / 16; k < C::cut(p + 1) / 16; ++k) {
+            if (k == 0) mma_ts(t_o, t_p, desc_v(b0), IDESC_PV, acc);
+            else mma_ts_c<true>(t_o, t_p + k * 8, desc_v(b0 + k * (16 * C::VROW >> 4)), IDESC_PV);
+          }
+        }
         tc_commit(bar(C::B_OF + j));
       };
       // one bit per stream
@@ -645,9 +678,7 @@ __global__ void __launch_bounds__(kThreads, 1) rf_attn_kernel(const __grid_const
 #pragma unroll 1
           for (int j = 0; j < 2; ++j) {
             if (cur & (1 << j)) {
-              mbar_wait(bar(C::B_PF + j), (pv_par >> j) & 1, wc);
-              tc_fence_after();
-              issue_pv(j, vs, (acc >> j) & 1);
+              issue_pv(j, vs, (acc >> j) & 1, (pv_par >> j) & 1);
               pv_par ^= 1u << j;
             }
           }
@@ -676,9 +707,7 @@ __global__ void __launch_bounds__(kThreads, 1) rf_attn_kernel(const __grid_const
               issue_s(j, ksn);
             }
             if (cur & (1 << j)) {
-              mbar_wait(bar(C::B_PF + j), (pv_par >> j) & 1, wc);
-              tc_fence_after();
-              issue_pv(j, vs, (acc >> j) & 1);
+              issue_pv(j, vs, (acc >> j) & 1, (pv_par >> j) & 1);
               acc |= 1u << j;
               pv_par ^= 1u << j;
             }
@@ -687,9 +716,7 @@ __global__ void __launch_bounds__(kThreads, 1) rf_attn_kernel(const __grid_const
 #pragma unroll
           for (int j = 0; j < 2; ++j) {
             if (cur & (1 << j)) {
-              mbar_wait(bar(C::B_PF + j), (pv_par >> j) & 1, wc);
-              tc_fence_after();
-              issue_pv(j, vs, (acc >> j) & 1);
+              issue_pv(j, vs, (acc >> j) & 1, (pv_par >> j) & 1);
               acc |= 1u << j;
               pv_par ^= 1u << j;
             }
@@ -745,7 +772,7 @@ __global__ void __launch_bounds__(kThreads, 1) rf_attn_kernel(const __grid_const
       tc_fence_after();
       uint32_t s[128];
       load_scores(t_s, s);
-      if constexpr (C::S_EARLY) {   // the accumulator is handed back at once; P goes to TMEM columns of its own
+      if constexpr (C::S_SHARED) {   // S is handed back at once: its columns are the other stream's too, or (D = 64) its own next scores'
         tc_fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive(bar(C::B_SE + j));
@@ -833,28 +860,28 @@ __global__ void __launch_bounds__(kThreads, 1) rf_attn_kernel(const __grid_const
         if (!opens) {
           // O of the previous tiles must be complete before it is rescaled
           mbar_wait(bar(C::B_OF + j), (done - 1) & 1, wc);
-          rescale_o<D>(t_o, alpha);
+          rescale_o_call<D>(t_o, alpha);
         }
         m_use = m_run == -INFINITY ? 0.f : m_run;
         la = make_float2(0.f, 0.f);
-        load_scores(t_s, s);   // again: they need not survive the rescaling in registers (or on the stack)
-        if (partial) mask_scores(keep, s);
         take_weights<0, kSpec, LSE>(s, pk, la, sc2, make_float2(-m_use, -m_use));
       }
-      if constexpr (C::S_SHARED) {
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(bar(C::B_SE + j));
-      }
       const uint32_t t_p = tmem_base + lane_sel + (j ? C::P_COL1 : C::P_COL0);
-      take_weights<kSpec, 64, LSE>(s, pk, la, sc2, make_float2(-m_use, -m_use));
-      tmem_st32(t_p, *reinterpret_cast<uint32_t(*)[32]>(&pk[0]));
-      take_weights<64, BN, LSE>(s, pk, la, sc2, make_float2(-m_use, -m_use));
-      tmem_st32(t_p + 32, *reinterpret_cast<uint32_t(*)[32]>(&pk[32]));
+      const float2 mneg = make_float2(-m_use, -m_use);
+      static_assert(C::S_EARLY || C::PARTS == 2, "the first half is handed over under the exponentials of the second");
+      take_weights<kSpec, 64, LSE>(s, pk, la, sc2, mneg);
+      store_weights<0, 64>(t_p, pk);
+      take_weights<64, 80, LSE>(s, pk, la, sc2, mneg);
+      tc_wait_st();              // the store has had these exponentials' time
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(bar(C::B_PF + j * C::PARTS));
+      take_weights<80, BN, LSE>(s, pk, la, sc2, mneg);
+      store_weights<64, BN>(t_p, pk);
       tc_wait_st();
       tc_fence_before();
       __syncwarp();
-      if (lane == 0) mbar_arrive(bar(C::B_PF + j));
+      if (lane == 0) mbar_arrive(bar(C::B_PF + j * C::PARTS + 1));
       if (LSE) l_exact += la.x + la.y;
     }
 
