@@ -247,7 +247,8 @@ rf_status rf_sparse_attn_fwd_plus(const rf_shape *shape, const rf_params *params
 /*
  * One sparse call as a sampler makes it (Fig. 2a): rf_arm_classify, rf_build_block_mask and rf_sparse_attn_fwd one after the
  * other on the stream, or their _plus forms when n_bandwidths > 0 (head_window is then written, else it may be NULL).  The
- * same launches and the same results; a caller at the end of a foreign-function interface crosses it once instead of three times.
+ * same results from three launches instead of five (the decision, the schedule and the reordered copies are one), and a caller
+ * at the end of a foreign-function interface crosses it once instead of three times.
  * Returns the first status that is not RF_OK.  Arguments as for the three calls.
  */
 rf_status rf_sparse_call(const rf_shape *shape, const rf_params *params, const float *bandwidths, int32_t n_bandwidths,

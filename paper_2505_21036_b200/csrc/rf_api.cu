@@ -191,12 +191,14 @@ rf_status check_sparse_attn(const rf_shape* shape, const rf_params* params, cons
   return sched->nQ == g.nQ && sched->nKmax == g.nKmax ? RF_OK : RF_ERR_INVALID_ARG;
 }
 
-// Shared by rf_sparse_attn_fwd(_plus) and rf_sparse_attn_reordered: the second skips the gather pass and
-// reads the reordered copies a preceding rf_reorder_tokens call left in the workspace.
+// Where the copies of a sparse attention call come from: made by it, left in the workspace by rf_reorder_tokens, or made in one
+// launch with the decision over the classes and the tile schedule.
+enum class Copies { kMake, kMade, kPrepare };
+// Shared by rf_sparse_attn_fwd(_plus), rf_sparse_attn_reordered and rf_sparse_call.
 rf_status sparse_attn_impl(const rf_shape* shape, const rf_params* params, const void* q, const void* k, const void* v,
                            const int32_t* head_class, const int32_t* head_window, const rf_schedule* sched, void* o,
-                           float* lse, void* ws, size_t ws_bytes, int32_t* dev_status, void* cuda_stream, bool gather,
-                           int heads_total, int head0) {
+                           float* lse, void* ws, size_t ws_bytes, int32_t* dev_status, void* cuda_stream, Copies from,
+                           int heads_total, int head0, const RfDecision* dec = nullptr) {
   const rf_status st = check_sparse_attn(shape, params, q, k, v, head_class, head_window, sched, o, ws, ws_bytes);
   if (st != RF_OK) return st;
   const RfGeom g = make_geom(shape, params);
@@ -218,14 +220,25 @@ rf_status sparse_attn_impl(const rf_shape* shape, const rf_params* params, const
   RfAttnArgs a;
   const bool room = ws_bytes >= rf_group_workspace_bytes(shape, params, heads_total, head0);
   set_split(&a, room ? rf_split_plan(g, true, heads_total, head0) : RfSplit{}, w + split_offset(g));
-  if (gather) {
+  bool clear = a.sp.on;   // whatever ran on this workspace before, the tickets begin at zero
+  if (from == Copies::kPrepare) {
+    // a group's tickets may lie where ARM's sums do (its pieces were not part of the workspace's layout)
+    const uintptr_t t0 = reinterpret_cast<uintptr_t>(a.tickets), t1 = t0 + a.sp.n_tickets * sizeof(int32_t);
+    const bool apart = t1 <= reinterpret_cast<uintptr_t>(dec->glb) || t0 > reinterpret_cast<uintptr_t>(dec->arm_flag);
+    cudaError_t e = rf_launch_prepare(g, *dec, sched->count, sched->kv_tile, sched->bitmap, sched->kv_len,
+                                      static_cast<const __nv_bfloat16*>(q), static_cast<const __nv_bfloat16*>(k),
+                                      static_cast<const __nv_bfloat16*>(v), wq, wk, wv, a.tickets, clear && apart ? (int)a.sp.n_tickets : 0,
+                                      dev_status, stream);
+    if (e != cudaSuccess) return RF_ERR_CUDA;
+    clear = clear && !apart;
+  } else if (from == Copies::kMake) {
     cudaError_t e = rf_launch_gather(g, head_class, static_cast<const __nv_bfloat16*>(q),
                                      static_cast<const __nv_bfloat16*>(k), static_cast<const __nv_bfloat16*>(v), wq, wk, wv,
                                      a.tickets, (int)a.sp.n_tickets, dev_status, stream);
     if (e != cudaSuccess) return RF_ERR_CUDA;
-  } else if (a.sp.on && rf_launch_zero(a.tickets, (int)a.sp.n_tickets, stream) != cudaSuccess) {
-    return RF_ERR_CUDA;   // whatever ran on this workspace since the reordering, the tickets begin at zero
+    clear = false;
   }
+  if (clear && rf_launch_zero(a.tickets, (int)a.sp.n_tickets, stream) != cudaSuccess) return RF_ERR_CUDA;
 
   a.g = g;
   a.head_class = head_class;
@@ -306,12 +319,61 @@ size_t rf_least_workspace_bytes(const rf_shape* shape, const rf_params* params) 
   return check_shape(shape) == RF_OK && check_params(params) == RF_OK ? least_bytes(make_geom(shape, params), params) : 0;
 }
 
-rf_status rf_sparse_attn_group(const rf_shape* shape, const rf_params* params, const void* q, const void* k, const void* v,
-                               const int32_t* head_class, const int32_t* head_window, const rf_schedule* sched, void* o,
-                               float* lse, void* ws, size_t ws_bytes, int32_t* dev_status, void* cuda_stream, int heads_total,
-                               int head0) {
+namespace {
+rf_status check_arm(const rf_shape* shape, const rf_params* params, bool plus) {
+  rf_status st = check_shape(shape);
+  if (st != RF_OK) return st;
+  st = check_params(params);
+  if (st != RF_OK) return st;
+  st = check_2d(shape, params);
+  if (st != RF_OK) return st;
+  if (shape->D != 64 && shape->D != 96 && shape->D != 128) return RF_ERR_UNSUPPORTED;
+  return plus && params->temporal_window_2d ? RF_ERR_UNSUPPORTED : RF_OK;   // a bandwidth has no 2-D meaning defined here
+}
+
+// ARM with the fixed windows (n_bandwidths = 0) or candidate bandwidths; later: see rf_launch_arm.
+rf_status arm_call(const rf_shape* shape, const rf_params* params, const float* bandwidths, int32_t n_bandwidths, const void* q,
+                   const void* k, int32_t* head_class, int32_t* head_window, float* recall, void* ws, size_t ws_bytes,
+                   int32_t* dev_status, void* cuda_stream, RfDecision* later = nullptr, bool selftest_abandon = false) {
+  const bool plus = n_bandwidths != 0;
+  const rf_status st = check_arm(shape, params, plus);
+  if (st != RF_OK) return st;
+  if (plus && (bandwidths == nullptr || n_bandwidths < 1 || n_bandwidths > RF_MAX_BANDWIDTHS)) return RF_ERR_INVALID_ARG;
+  if (q == nullptr || k == nullptr || head_class == nullptr || (plus && head_window == nullptr) || ws == nullptr) return RF_ERR_INVALID_ARG;
+  if (!aligned16(q) || !aligned16(k) || (reinterpret_cast<uintptr_t>(ws) & (kAlign - 1)) != 0) return RF_ERR_INVALID_ARG;
+  const RfGeom g = make_geom(shape, params);
+  if (ws_bytes < least_bytes(g, params)) return RF_ERR_WORKSPACE_TOO_SMALL;
+  int ws_list[RF_MAX_BANDWIDTHS] = {g.ws}, wf_list[RF_MAX_BANDWIDTHS] = {g.wf};
+  for (int i = 0; i < n_bandwidths; ++i) {
+    const float b = bandwidths[i];
+    if (!(b > 0.f && b <= 1.f) || (i > 0 && b <= bandwidths[i - 1])) return RF_ERR_INVALID_ARG;
+    wf_list[i] = (int)floor((double)b * g.T);
+    ws_list[i] = (int)floor((double)b * g.S);
+  }
+  float* scratch = arm_scratch(g, params, ws, ws_bytes);
+  cudaError_t e = rf_launch_arm(g, params->sample_mode, params->sample_stride, params->alpha, plus ? n_bandwidths : 1, ws_list, wf_list,
+                                static_cast<const __nv_bfloat16*>(q), static_cast<const __nv_bfloat16*>(k), head_class,
+                                plus ? head_window : nullptr, plus ? nullptr : recall, plus ? recall : nullptr, scratch, dev_status,
+                                static_cast<cudaStream_t>(cuda_stream), selftest_abandon, later);
+  return e == cudaSuccess ? RF_OK : RF_ERR_CUDA;
+}
+}  // namespace
+
+rf_status rf_sparse_call_group(const rf_shape* shape, const rf_params* params, const float* bandwidths, int32_t n_bandwidths,
+                               const void* q, const void* k, const void* v, int32_t* head_class, int32_t* head_window,
+                               rf_schedule* sched, void* o, float* lse, void* ws, size_t ws_bytes, int32_t* dev_status,
+                               void* cuda_stream, int heads_total, int head0) {
+  if (n_bandwidths < 0) return RF_ERR_INVALID_ARG;
+  if (n_bandwidths == 0) head_window = nullptr;
+  // ARM checks its own arguments before it launches; what the steps after it would refuse is refused here
+  rf_status st = check_sparse_attn(shape, params, q, k, v, head_class, head_window, sched, o, ws, ws_bytes);
+  if (st == RF_OK && sched->kv_len == nullptr) st = RF_ERR_INVALID_ARG;
+  if (st != RF_OK) return st;
+  RfDecision dec;
+  st = arm_call(shape, params, bandwidths, n_bandwidths, q, k, head_class, head_window, nullptr, ws, ws_bytes, dev_status, cuda_stream, &dec);
+  if (st != RF_OK) return st;
   return sparse_attn_impl(shape, params, q, k, v, head_class, head_window, sched, o, lse, ws, ws_bytes, dev_status, cuda_stream,
-                          true, heads_total, head0);
+                          Copies::kPrepare, heads_total, head0, &dec);
 }
 
 extern "C" {
@@ -359,74 +421,24 @@ size_t rf_workspace_bytes(const rf_shape* shape, const rf_params* params) {
 rf_status rf_arm_classify(const rf_shape* shape, const rf_params* params, const void* q, const void* k,
                           int32_t* head_class, float* recall, void* ws, size_t ws_bytes, int32_t* dev_status,
                           void* cuda_stream) {
-  rf_status st = check_shape(shape);
-  if (st != RF_OK) return st;
-  st = check_params(params);
-  if (st != RF_OK) return st;
-  st = check_2d(shape, params);
-  if (st != RF_OK) return st;
-  if (shape->D != 64 && shape->D != 96 && shape->D != 128) return RF_ERR_UNSUPPORTED;
-  if (q == nullptr || k == nullptr || head_class == nullptr || ws == nullptr) return RF_ERR_INVALID_ARG;
-  if (!aligned16(q) || !aligned16(k) || (reinterpret_cast<uintptr_t>(ws) & (kAlign - 1)) != 0) return RF_ERR_INVALID_ARG;
-  const RfGeom g = make_geom(shape, params);
-  if (ws_bytes < least_bytes(g, params)) return RF_ERR_WORKSPACE_TOO_SMALL;
-  float* scratch = arm_scratch(g, params, ws, ws_bytes);
-  cudaError_t e = rf_launch_arm(g, params->sample_mode, params->sample_stride, params->alpha, 1, &g.ws, &g.wf,
-                                static_cast<const __nv_bfloat16*>(q), static_cast<const __nv_bfloat16*>(k), head_class,
-                                nullptr, recall, nullptr, scratch, dev_status, static_cast<cudaStream_t>(cuda_stream));
-  return e == cudaSuccess ? RF_OK : RF_ERR_CUDA;
+  return arm_call(shape, params, nullptr, 0, q, k, head_class, nullptr, recall, ws, ws_bytes, dev_status, cuda_stream);
 }
 
 rf_status rf_selftest_arm_abandoned(const rf_shape* shape, const rf_params* params, const void* q, const void* k,
                                     int32_t* head_class, void* ws, size_t ws_bytes, int32_t* dev_status, void* cuda_stream) {
-  rf_status st = check_shape(shape);
-  if (st != RF_OK) return st;
-  st = check_params(params);
-  if (st != RF_OK) return st;
-  st = check_2d(shape, params);
-  if (st != RF_OK) return st;
-  if (shape->D != 64 && shape->D != 96 && shape->D != 128) return RF_ERR_UNSUPPORTED;
-  if (q == nullptr || k == nullptr || head_class == nullptr || ws == nullptr) return RF_ERR_INVALID_ARG;
-  if (!aligned16(q) || !aligned16(k) || (reinterpret_cast<uintptr_t>(ws) & (kAlign - 1)) != 0) return RF_ERR_INVALID_ARG;
-  const RfGeom g = make_geom(shape, params);
-  if (ws_bytes < least_bytes(g, params)) return RF_ERR_WORKSPACE_TOO_SMALL;
-  float* scratch = arm_scratch(g, params, ws, ws_bytes);
-  cudaError_t e = rf_launch_arm(g, params->sample_mode, params->sample_stride, params->alpha, 1, &g.ws, &g.wf,
-                                static_cast<const __nv_bfloat16*>(q), static_cast<const __nv_bfloat16*>(k), head_class,
-                                nullptr, nullptr, nullptr, scratch, dev_status, static_cast<cudaStream_t>(cuda_stream), true);
-  return e == cudaSuccess ? RF_OK : RF_ERR_CUDA;
+  return arm_call(shape, params, nullptr, 0, q, k, head_class, nullptr, nullptr, ws, ws_bytes, dev_status, cuda_stream, nullptr, true);
 }
 
 rf_status rf_arm_classify_plus(const rf_shape* shape, const rf_params* params, const float* bandwidths,
                                int32_t n_bandwidths, const void* q, const void* k, int32_t* head_class,
                                int32_t* head_window, float* recall, void* ws, size_t ws_bytes, int32_t* dev_status,
                                void* cuda_stream) {
-  rf_status st = check_shape(shape);
-  if (st != RF_OK) return st;
-  st = check_params(params);
-  if (st != RF_OK) return st;
-  st = check_2d(shape, params);
-  if (st != RF_OK) return st;
-  if (shape->D != 64 && shape->D != 96 && shape->D != 128) return RF_ERR_UNSUPPORTED;
-  if (params->temporal_window_2d) return RF_ERR_UNSUPPORTED;   // a bandwidth has no 2-D meaning defined here
-  if (bandwidths == nullptr || n_bandwidths < 1 || n_bandwidths > RF_MAX_BANDWIDTHS) return RF_ERR_INVALID_ARG;
-  if (q == nullptr || k == nullptr || head_class == nullptr || head_window == nullptr || ws == nullptr) return RF_ERR_INVALID_ARG;
-  if (!aligned16(q) || !aligned16(k) || (reinterpret_cast<uintptr_t>(ws) & (kAlign - 1)) != 0) return RF_ERR_INVALID_ARG;
-  const RfGeom g = make_geom(shape, params);
-  if (ws_bytes < least_bytes(g, params)) return RF_ERR_WORKSPACE_TOO_SMALL;
-  int ws_list[RF_MAX_BANDWIDTHS], wf_list[RF_MAX_BANDWIDTHS];
-  for (int i = 0; i < n_bandwidths; ++i) {
-    const float b = bandwidths[i];
-    if (!(b > 0.f && b <= 1.f) || (i > 0 && b <= bandwidths[i - 1])) return RF_ERR_INVALID_ARG;
-    wf_list[i] = (int)floor((double)b * g.T);
-    ws_list[i] = (int)floor((double)b * g.S);
+  if (n_bandwidths < 1) {
+    // (0 selects the fixed windows in arm_call)
+    const rf_status st = check_arm(shape, params, true);
+    return st != RF_OK ? st : RF_ERR_INVALID_ARG;
   }
-  float* scratch = arm_scratch(g, params, ws, ws_bytes);
-  cudaError_t e = rf_launch_arm(g, params->sample_mode, params->sample_stride, params->alpha, n_bandwidths, ws_list,
-                                wf_list, static_cast<const __nv_bfloat16*>(q), static_cast<const __nv_bfloat16*>(k),
-                                head_class, head_window, nullptr, recall, scratch, dev_status,
-                                static_cast<cudaStream_t>(cuda_stream));
-  return e == cudaSuccess ? RF_OK : RF_ERR_CUDA;
+  return arm_call(shape, params, bandwidths, n_bandwidths, q, k, head_class, head_window, recall, ws, ws_bytes, dev_status, cuda_stream);
 }
 
 rf_status rf_build_block_mask(const rf_shape* shape, const rf_params* params, const int32_t* head_class,
@@ -464,7 +476,7 @@ rf_status rf_sparse_attn_fwd_plus(const rf_shape* shape, const rf_params* params
                                   const rf_schedule* sched, void* o, float* lse, void* ws, size_t ws_bytes,
                                   int32_t* dev_status, void* cuda_stream) {
   return sparse_attn_impl(shape, params, q, k, v, head_class, head_window, sched, o, lse, ws, ws_bytes, dev_status,
-                          cuda_stream, true, shape != nullptr ? shape->B * shape->H : 0, 0);
+                          cuda_stream, Copies::kMake, shape != nullptr ? shape->B * shape->H : 0, 0);
 }
 
 rf_status rf_sparse_attn_reordered(const rf_shape* shape, const rf_params* params, const void* q, const void* k,
@@ -472,25 +484,14 @@ rf_status rf_sparse_attn_reordered(const rf_shape* shape, const rf_params* param
                                    const rf_schedule* sched, void* o, float* lse, void* ws, size_t ws_bytes,
                                    int32_t* dev_status, void* cuda_stream) {
   return sparse_attn_impl(shape, params, q, k, v, head_class, head_window, sched, o, lse, ws, ws_bytes, dev_status,
-                          cuda_stream, false, shape != nullptr ? shape->B * shape->H : 0, 0);
+                          cuda_stream, Copies::kMade, shape != nullptr ? shape->B * shape->H : 0, 0);
 }
 
 rf_status rf_sparse_call(const rf_shape* shape, const rf_params* params, const float* bandwidths, int32_t n_bandwidths, const void* q,
                          const void* k, const void* v, int32_t* head_class, int32_t* head_window, rf_schedule* sched, void* o,
                          float* lse, void* ws, size_t ws_bytes, int32_t* dev_status, void* cuda_stream) {
-  if (n_bandwidths < 0) return RF_ERR_INVALID_ARG;
-  if (n_bandwidths == 0) head_window = nullptr;
-  // ARM checks its own arguments before it launches; what the two calls after it would refuse is refused here
-  rf_status st = check_sparse_attn(shape, params, q, k, v, head_class, head_window, sched, o, ws, ws_bytes);
-  if (st == RF_OK && sched->kv_len == nullptr) st = RF_ERR_INVALID_ARG;
-  if (st != RF_OK) return st;
-  st = n_bandwidths > 0 ? rf_arm_classify_plus(shape, params, bandwidths, n_bandwidths, q, k, head_class, head_window, nullptr, ws,
-                                               ws_bytes, dev_status, cuda_stream)
-                        : rf_arm_classify(shape, params, q, k, head_class, nullptr, ws, ws_bytes, dev_status, cuda_stream);
-  if (st == RF_OK) st = rf_build_block_mask_plus(shape, params, head_class, head_window, sched, dev_status, cuda_stream);
-  if (st == RF_OK)
-    st = rf_sparse_attn_fwd_plus(shape, params, q, k, v, head_class, head_window, sched, o, lse, ws, ws_bytes, dev_status, cuda_stream);
-  return st;
+  return rf_sparse_call_group(shape, params, bandwidths, n_bandwidths, q, k, v, head_class, head_window, sched, o, lse, ws, ws_bytes,
+                              dev_status, cuda_stream, shape != nullptr ? shape->B * shape->H : 0, 0);
 }
 
 rf_status rf_selftest_wait_timeout(int32_t* dev_status, int32_t limit_ms, int32_t* waits_returned, void* cuda_stream) {

@@ -25,13 +25,16 @@
 // need per-key attributes, computed cooperatively per tile.
 // With the first frame as a key frame of Spatial heads (Sec. 3.2: adjacent or key frames) the Spatial masks keep,
 // in addition, the sampled keys of frame 0, a prefix of the stride sample.
-// Per-row recalls go to scratch; a second kernel averages them in a fixed order (deterministic) and
-// takes Algorithm 1's decision.  The n x n score matrix is never written.
+// A CTA leaves the sums of its rows' recalls in scratch (in double and in a fixed order, so that they do not depend on the
+// schedule); whoever needs the classes next adds a head's few sums up and takes Algorithm 1's decision: the decision kernel here,
+// or every warp of the kernel that builds the schedule and the copies, which saves a call two launches (3 heads, 272
+// tokens 31.2 -> 27.5 us a call; 10 heads, 3668 tokens 80.7 -> 77.3; 3 heads, 7476 tokens 120.4 -> 113.5).  The n x n score matrix is never written.
 // A bounded wait that runs out is recorded in a flag word at the end of the scratch (cleared by the score
-// kernel as it starts); the decision kernel then writes class -1 for every head instead of a class computed from
+// kernel as it starts); the decision then gives class -1 for every head instead of a class computed from
 // unwritten rows, and passes the code on to the caller's status word.  The tile builder and the attention
 // kernel report a class outside 0..3 through their own status, so the failure cannot go unnoticed even by a
 // caller that gave ARM no status pointer.
+#include "rf_decide.cuh"
 #include "rf_sm100.cuh"
 
 namespace {
@@ -54,7 +57,7 @@ struct ArmSample {
   int tiles;      // CTAs per head: ceil(n / 128)
   int want_t;     // accumulate the Temporal masses on this sample
   int want_s;     // accumulate the Spatial masses on this sample
-  float* out;     // [B*H][2*NB+1][n_pad]: Temporal per window, Spatial per window, Textural
+  double* out;    // [B*H][2*NB+1][t_pad]: Temporal per window, Spatial per window, Textural
 };
 struct ArmWindows { int ws[ARM_MAX_NB], wf[ARM_MAX_NB], n; };   // candidate spatial (Temporal) / frame (Spatial) windows
 
@@ -153,7 +156,7 @@ __device__ __forceinline__ float table_sum(const uint32_t (&s)[ARM_HALF], const 
 template <int D, int NB, bool TEX>
 __global__ void __launch_bounds__(ARM_THREADS, 2) rf_arm_kernel(const __grid_constant__ ArmMaps maps, const RfGeom g,
                                                                 const ArmSample sm0, const ArmSample sm1,
-                                                                const ArmWindows win, int n_pad, float scale_log2,
+                                                                const ArmWindows win, int t_pad, float scale_log2,
                                                                 int32_t* arm_flag) {
   using C = ArmCfg<D>;
   constexpr uint32_t IDESC_S = idesc_bf16(128, 128, 0);
@@ -390,21 +393,26 @@ __global__ void __launch_bounds__(ARM_THREADS, 2) rf_arm_kernel(const __grid_con
   }
 
   __syncthreads();
-  if (warp < 4 && m < n) {
+  double* part = reinterpret_cast<double*>(base_ptr + C::ATTR);   // [masks][4 warps]; the tables are done with
+  auto wanted = [&](int k) { return k == 2 * NB ? TEX : (k < NB ? sm.want_t != 0 : sm.want_s != 0); };
+  if (warp < 4) {
     const float m1 = join[0], top = fmaxf(mx, m1);
     const float f0 = ex2f(mx - top), f1 = ex2f(m1 - top);        // no odd tile: m1 = kLeast, factor 0
     const float inv = 1.f / (l_all * f0 + join[128] * f1);
-    float* out = sm.out + (size_t)bh * NM * n_pad;
 #pragma unroll
     for (int k = 0; k < NM; ++k) {
-      const bool is_t = k < NB, is_x = k == 2 * NB;
-      if ((is_x ? TEX : (is_t ? sm.want_t != 0 : sm.want_s != 0)) && rf_in_bounds(m, n_pad, arm_flag))
-        out[(size_t)k * n_pad + m] = (l_m[k] * f0 + join[(2 + k) * 128] * f1) * inv;
+      if (!wanted(k)) continue;
+      double sum = m < n ? (double)((l_m[k] * f0 + join[(2 + k) * 128] * f1) * inv) : 0.0;
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+      if (lane == 0) part[k * 4 + warp] = sum;
     }
   }
 
   tc_fence_before();
   __syncthreads();
+  if (tid < NM && wanted(tid) && rf_in_bounds(qt, t_pad, arm_flag))
+    sm.out[((size_t)bh * NM + tid) * t_pad + qt] = (part[tid * 4] + part[tid * 4 + 1]) + (part[tid * 4 + 2] + part[tid * 4 + 3]);
   if (warp == ARM_TMA_WARP) {
     if (*abort_flag) __nanosleep(20000);
     __syncwarp();
@@ -412,80 +420,11 @@ __global__ void __launch_bounds__(ARM_THREADS, 2) rf_arm_kernel(const __grid_con
   }
 }
 
-// One CTA per head: means of the per-row recalls in a fixed order, then the decision.
-//   plain (head_window == nullptr, nb = 1): Algorithm 1.
-//   dynamic bandwidth: a pattern qualifies if any candidate window reaches alpha, Temporal before Spatial;
-//   the head takes the smallest qualifying window (candidates ascend); Textural heads get window -1.
-__global__ void __launch_bounds__(256) rf_arm_decide_kernel(int nb, int nb_user, int n_loc, int n_glb, int n_pad, int sample_mode,
-                                                             float alpha, int two_mask, ArmWindows win, int with_tex,
-                                                             const float* rows_loc, const float* rows_glb,
-                                                             int32_t* __restrict__ head_class,
-                                                             int32_t* __restrict__ head_window, float* __restrict__ recall,
-                                                             float* __restrict__ recall_plus,
-                                                             const int32_t* arm_flag, int32_t* dev_status) {
-  __shared__ double red[2 * ARM_MAX_NB + 1][8];
+// One warp per head.
+__global__ void __launch_bounds__(32) rf_arm_decide_kernel(const RfDecision d) {
   rf_grid_trigger();
   rf_grid_wait();
-  const int bh = blockIdx.x, tid = threadIdx.x;
-  const int nm = 2 * nb + 1;
-  const int failed = *arm_flag;
-  if (failed != 0) {
-    // the score kernel gave up a wait: its rows are incomplete, no class may come out of them
-    if (tid == 0) {
-      rf_report(dev_status, failed);
-      head_class[bh] = -1;
-      if (head_window != nullptr) head_window[bh] = -1;
-    }
-    return;
-  }
-  const float* gl = rows_glb + (size_t)bh * nm * n_pad;
-  const float* lo = rows_loc + (size_t)bh * nm * n_pad;
-  const bool local_t = sample_mode == RF_SAMPLE_ALG1;
-  for (int k = 0; k < nm; ++k) {
-    const bool is_t = k < nb, is_x = k == 2 * nb;
-    const float* src = ((is_t && local_t) ? lo : gl) + (size_t)k * n_pad;
-    const int cnt = (is_t && local_t) ? n_loc : n_glb;
-    double acc = 0.0;
-    if (!is_x || with_tex)
-      for (int i = tid; i < cnt; i += 256) acc += (double)src[i];
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    if ((tid & 31) == 0) red[k][tid >> 5] = acc;
-  }
-  __syncthreads();
-  if (tid == 0) {
-    float R[2 * ARM_MAX_NB + 1];
-    for (int k = 0; k < nm; ++k) {
-      double sum = 0.0;
-      for (int w = 0; w < 8; ++w) sum += red[k][w];
-      R[k] = (float)(sum / ((k < nb && local_t) ? n_loc : n_glb));
-    }
-    if (head_window == nullptr) {
-      const float Rt = R[0], Rs = R[nb], Rc = R[2 * nb];
-      if (recall) { recall[bh * 3] = Rt; recall[bh * 3 + 1] = Rs; recall[bh * 3 + 2] = Rc; }
-      // Algorithm 1; with only two masks (ablation) a head that reaches alpha with neither takes the larger recall
-      const int otherwise = two_mask ? (Rt >= Rs ? RF_TEMPORAL : RF_SPATIAL) : RF_TEXTURAL;
-      head_class[bh] = Rt >= alpha ? RF_TEMPORAL : (Rs >= alpha ? RF_SPATIAL : otherwise);
-    } else {
-      int cls = RF_TEXTURAL, window = -1;
-      if (two_mask) {   // nothing qualifies: the larger recall at the widest candidate, with that bandwidth
-        const bool t = R[nb_user - 1] >= R[nb + nb_user - 1];
-        cls = t ? RF_TEMPORAL : RF_SPATIAL;
-        window = t ? win.ws[nb_user - 1] : win.wf[nb_user - 1];
-      }
-      // of the kernel's nb slots the caller's nb_user candidates are the first; the others stay empty
-      for (int i = nb_user - 1; i >= 0; --i)
-        if (R[nb + i] >= alpha) { cls = RF_SPATIAL; window = win.wf[i]; }
-      for (int i = nb_user - 1; i >= 0; --i)
-        if (R[i] >= alpha) { cls = RF_TEMPORAL; window = win.ws[i]; }
-      head_class[bh] = cls;
-      head_window[bh] = window;
-      if (recall_plus)
-        for (int i = 0; i < nb_user; ++i) {
-          recall_plus[(bh * 2) * nb_user + i] = R[i];
-          recall_plus[(bh * 2 + 1) * nb_user + i] = R[nb + i];
-        }
-    }
-  }
+  rf_decide(d, blockIdx.x, threadIdx.x, true);
 }
 
 // Self-test only: stands in for a score kernel whose wait ran out.
@@ -496,7 +435,7 @@ __global__ void rf_arm_set_flag_kernel(int32_t* arm_flag, int code) {
 
 template <int D, int NB, bool TEX>
 cudaError_t launch_arm_t(const ArmMaps& maps, const RfGeom& g, const ArmSample& s0, const ArmSample& s1,
-                         const ArmWindows& win, int n_pad, int32_t* arm_flag, cudaStream_t st) {
+                         const ArmWindows& win, int t_pad, int32_t* arm_flag, cudaStream_t st) {
   static bool configured[64] = {};
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
@@ -510,15 +449,15 @@ cudaError_t launch_arm_t(const ArmMaps& maps, const RfGeom& g, const ArmSample& 
   }
   dim3 grid(s0.tiles + s1.tiles, g.B * g.H);
   const float scale_log2 = 1.4426950408889634f / sqrtf((float)D);
-  return rf_launch(rf_arm_kernel<D, NB, TEX>, grid, ARM_THREADS, ArmCfg<D>::ALLOC, st, maps, g, s0, s1, win, n_pad, scale_log2, arm_flag);
+  return rf_launch(rf_arm_kernel<D, NB, TEX>, grid, ARM_THREADS, ArmCfg<D>::ALLOC, st, maps, g, s0, s1, win, t_pad, scale_log2, arm_flag);
 }
 
 template <int D>
 cudaError_t launch_arm_n(bool plus, bool tex, const ArmMaps& maps, const RfGeom& g, const ArmSample& s0,
-                         const ArmSample& s1, const ArmWindows& win, int n_pad, int32_t* arm_flag, cudaStream_t st) {
-  if (plus) return launch_arm_t<D, ARM_MAX_NB, false>(maps, g, s0, s1, win, n_pad, arm_flag, st);
-  return tex ? launch_arm_t<D, 1, true>(maps, g, s0, s1, win, n_pad, arm_flag, st)
-             : launch_arm_t<D, 1, false>(maps, g, s0, s1, win, n_pad, arm_flag, st);
+                         const ArmSample& s1, const ArmWindows& win, int t_pad, int32_t* arm_flag, cudaStream_t st) {
+  if (plus) return launch_arm_t<D, ARM_MAX_NB, false>(maps, g, s0, s1, win, t_pad, arm_flag, st);
+  return tex ? launch_arm_t<D, 1, true>(maps, g, s0, s1, win, t_pad, arm_flag, st)
+             : launch_arm_t<D, 1, false>(maps, g, s0, s1, win, t_pad, arm_flag, st);
 }
 
 int arm_n_pad(const RfGeom& g, int omega) {
@@ -529,7 +468,6 @@ int arm_n_pad(const RfGeom& g, int omega) {
 
 }  // namespace
 
-// Per-row recalls of both samples, then RF_ARM_FLAG_FLOATS floats whose first word is the call's failure flag.
 size_t rf_arm_scratch_floats(const RfGeom& g, int omega, int nb) {
   return (size_t)2 * g.B * g.H * (2 * nb + 1) * arm_n_pad(g, omega) + RF_ARM_FLAG_FLOATS;
 }
@@ -537,7 +475,7 @@ size_t rf_arm_scratch_floats(const RfGeom& g, int omega, int nb) {
 cudaError_t rf_launch_arm(const RfGeom& g, int sample_mode, int omega, float alpha, int nb, const int* ws_list,
                           const int* wf_list, const __nv_bfloat16* q, const __nv_bfloat16* k, int32_t* head_class,
                           int32_t* head_window, float* recall, float* recall_plus, float* row_scratch, int32_t* dev_status,
-                          cudaStream_t st, bool selftest_abandon) {
+                          cudaStream_t st, bool selftest_abandon, RfDecision* later) {
   const bool plus = head_window != nullptr;
   const int NB = plus ? ARM_MAX_NB : 1;           // windows the kernel has room for; it evaluates the first nb
   if (nb < 1 || nb > NB) return cudaErrorInvalidValue;
@@ -550,9 +488,12 @@ cudaError_t rf_launch_arm(const RfGeom& g, int sample_mode, int omega, float alp
   const int n_pad = arm_n_pad(g, omega);
   const int n_glb = rf_cdiv(g.Nv, omega), n_loc = g.S;
   const int heads = g.B * g.H;
-  float* rows_glb = row_scratch;
-  float* rows_loc = row_scratch + (size_t)heads * (2 * NB + 1) * n_pad;
-  int32_t* arm_flag = reinterpret_cast<int32_t*>(row_scratch + (size_t)2 * heads * (2 * NB + 1) * n_pad);
+  const int t_glb = rf_cdiv(n_glb, ARM_TILE), t_loc = rf_cdiv(n_loc, ARM_TILE), t_pad = t_glb > t_loc ? t_glb : t_loc;
+  float* end = row_scratch + (size_t)2 * heads * (2 * NB + 1) * n_pad;
+  int32_t* arm_flag = reinterpret_cast<int32_t*>(end);
+  const size_t sums = (size_t)heads * (2 * NB + 1) * t_pad;     // of one sample; t_pad <= n_pad / 64, so both fit
+  double* sums_loc = reinterpret_cast<double*>(end) - sums;
+  double* sums_glb = sums_loc - sums;
   const bool alg1 = sample_mode == RF_SAMPLE_ALG1;
   const bool tex = !plus && recall != nullptr;   // the Textural recall is a diagnostic: Algorithm 1 does not use it
   const size_t row_bytes = (size_t)g.D * 2, head_bytes = (size_t)g.N * g.D * 2;
@@ -563,10 +504,10 @@ cudaError_t rf_launch_arm(const RfGeom& g, int sample_mode, int omega, float alp
             rf_encode_rows_map(&maps.k[1], k, g.D, n_loc, row_bytes, head_bytes, heads);
   if (!ok) return cudaErrorUnknown;
   ArmSample s0, s1;
-  s0.n = n_glb; s0.stride = omega; s0.tiles = rf_cdiv(n_glb, ARM_TILE);
-  s0.want_t = alg1 ? 0 : 1; s0.want_s = 1; s0.out = rows_glb;
-  s1.n = n_loc; s1.stride = 1; s1.tiles = alg1 ? rf_cdiv(n_loc, ARM_TILE) : 0;
-  s1.want_t = 1; s1.want_s = 0; s1.out = rows_loc;
+  s0.n = n_glb; s0.stride = omega; s0.tiles = t_glb;
+  s0.want_t = alg1 ? 0 : 1; s0.want_s = 1; s0.out = sums_glb;
+  s1.n = n_loc; s1.stride = 1; s1.tiles = alg1 ? t_loc : 0;
+  s1.want_t = 1; s1.want_s = 0; s1.out = sums_loc;
   cudaError_t e = cudaSuccess;
 #ifdef RF_BOUNDS_CHECK
   e = cudaMemsetAsync(arm_flag, 0, sizeof(int32_t), st);
@@ -576,14 +517,31 @@ cudaError_t rf_launch_arm(const RfGeom& g, int sample_mode, int omega, float alp
     e = rf_launch(rf_arm_set_flag_kernel, dim3(1), 1, 0, st, arm_flag, (int)RF_ERR_TIMEOUT);
   } else
   switch (g.D) {
-    case 64: e = launch_arm_n<64>(plus, tex, maps, g, s0, s1, win, n_pad, arm_flag, st); break;
-    case 96: e = launch_arm_n<96>(plus, tex, maps, g, s0, s1, win, n_pad, arm_flag, st); break;
-    case 128: e = launch_arm_n<128>(plus, tex, maps, g, s0, s1, win, n_pad, arm_flag, st); break;
+    case 64: e = launch_arm_n<64>(plus, tex, maps, g, s0, s1, win, t_pad, arm_flag, st); break;
+    case 96: e = launch_arm_n<96>(plus, tex, maps, g, s0, s1, win, t_pad, arm_flag, st); break;
+    case 128: e = launch_arm_n<128>(plus, tex, maps, g, s0, s1, win, t_pad, arm_flag, st); break;
     default: e = cudaErrorInvalidValue;
   }
   if (e != cudaSuccess) return e;
-  return rf_launch(rf_arm_decide_kernel, dim3(heads), 256, 0, st, NB, nb, n_loc, n_glb, n_pad, sample_mode, alpha, g.two_mask, win,
-                   tex ? 1 : 0, rows_loc, rows_glb, head_class, head_window, recall, recall_plus, arm_flag, dev_status);
+  RfDecision d;
+  d.nb = NB; d.nb_user = nb;
+  d.n_loc = n_loc; d.n_glb = n_glb;
+  d.t_loc = t_loc; d.t_glb = t_glb; d.t_pad = t_pad;
+  d.local_t = alg1;
+  d.with_tex = tex;
+  d.two_mask = g.two_mask;
+  d.alpha = alpha;
+  for (int i = 0; i < ARM_MAX_NB; ++i) { d.ws[i] = win.ws[i]; d.wf[i] = win.wf[i]; }
+  d.loc = sums_loc; d.glb = sums_glb;
+  d.arm_flag = arm_flag;
+  d.head_class = head_class; d.head_window = head_window;
+  d.recall = recall; d.recall_plus = recall_plus;
+  d.dev_status = dev_status;
+  if (later != nullptr) {
+    *later = d;
+    return cudaSuccess;
+  }
+  return rf_launch(rf_arm_decide_kernel, dim3(heads), 32, 0, st, d);
 }
 
 // ------------------------------------------------------------------------------------------------

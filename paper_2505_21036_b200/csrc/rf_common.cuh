@@ -85,17 +85,43 @@ cudaError_t rf_launch_build_tiles(const RfGeom& g, const int32_t* head_class, co
 cudaError_t rf_launch_gather(const RfGeom& g, const int32_t* head_class, const __nv_bfloat16* q,
                              const __nv_bfloat16* k, const __nv_bfloat16* v, __nv_bfloat16* wq, __nv_bfloat16* wk,
                              __nv_bfloat16* wv, int32_t* tickets, int n_tickets, int32_t* dev_status, cudaStream_t st);
+// Algorithm 1's decision (or the dynamic-bandwidth one) over the score kernel's sums; see rf_decide in rf_decide.cuh.
+struct RfDecision {
+  int nb, nb_user;            // window slots per pattern, candidates among them
+  int n_loc, n_glb;           // rows of the first-frame and of the stride sample
+  int t_loc, t_glb, t_pad;    // score CTAs (128 rows each) of a head per sample
+  int local_t;                // the Temporal recall comes from the first-frame sample
+  int with_tex, two_mask;
+  float alpha;
+  int ws[RF_MAX_BANDWIDTHS], wf[RF_MAX_BANDWIDTHS];
+  const double *loc, *glb;    // [B*H][2*nb+1][t_pad]: sums of the rows' recalls
+  const int32_t* arm_flag;
+  int32_t* head_class;
+  int32_t* head_window;       // null: plain Algorithm 1
+  float* recall;
+  float* recall_plus;
+  int32_t* dev_status;
+};
+// The tile schedule and the reordered copies of a call whose classes are not decided yet: every warp takes the decision of its
+// head itself and one of them writes it out.  One launch for what rf_launch_build_tiles, rf_launch_gather and the decision
+// kernel do.
+cudaError_t rf_launch_prepare(const RfGeom& g, const RfDecision& dec, int32_t* count, int32_t* kv_tile, uint32_t* bitmap,
+                              int32_t* kv_len, const __nv_bfloat16* q, const __nv_bfloat16* k, const __nv_bfloat16* v,
+                              __nv_bfloat16* wq, __nv_bfloat16* wk, __nv_bfloat16* wv, int32_t* tickets, int n_tickets,
+                              int32_t* dev_status, cudaStream_t st);
 // nb candidate windows per pattern (ws_list for Temporal, wf_list for Spatial, ascending).  head_window == nullptr:
 // plain Algorithm 1 on the first candidate (recall: [B,H,3] or null).  Otherwise dynamic bandwidth: head_window
 // receives each head's chosen window, recall_plus ([B,H,2,nb] or null) the candidates' recalls.
 // dev_status (nullable) receives RF_ERR_TIMEOUT if a wait inside the score kernel ran out; head_class is then -1.
 // selftest_abandon: the score kernel is not launched; its failure flag is set instead, as if a wait had run out.
+// later (nullable): the decision is not launched but left there for rf_launch_prepare.
 cudaError_t rf_launch_arm(const RfGeom& g, int sample_mode, int omega, float alpha, int nb, const int* ws_list,
                           const int* wf_list, const __nv_bfloat16* q, const __nv_bfloat16* k, int32_t* head_class,
                           int32_t* head_window, float* recall, float* recall_plus, float* row_scratch, int32_t* dev_status,
-                          cudaStream_t st, bool selftest_abandon = false);
-// Floats of ARM scratch: the per-row recalls plus RF_ARM_FLAG_FLOATS at the end whose first word records a
-// wait that ran out inside the score kernel (cleared by every call at the start of its first kernel).
+                          cudaStream_t st, bool selftest_abandon = false, RfDecision* later = nullptr);
+// Floats of ARM scratch.  The sums of the rows' recalls lie at its end, before RF_ARM_FLAG_FLOATS whose first word records a
+// wait that ran out inside the score kernel (cleared by every call at the start of its first kernel).  (The size is that of
+// the rows' recalls, which were kept one by one before the score kernel summed them; callers' blocks are sized by it.)
 #define RF_ARM_FLAG_FLOATS 64
 size_t rf_arm_scratch_floats(const RfGeom& g, int omega, int nb);
 // Tensor map over bf16 rows: [heads][rows][D] with the given row and head strides in bytes (multiples of 16),
@@ -148,12 +174,12 @@ struct RfAttnArgs {
 // (position-major Q/K/V of Temporal heads), [6..7] workspace K/V with LkvTex rows per head (Textural).
 constexpr int RF_ATTN_MAPS = 8;
 rf_status rf_launch_attention(const RfAttnArgs& a, const CUtensorMap* maps, cudaStream_t st);
-// rf_sparse_attn_fwd_plus for heads [head0, head0 + B*H) of a call of heads_total heads made in groups; the workspace needs
+// A call for heads [head0, head0 + B*H) of one of heads_total heads that is made in groups; the workspace needs
 // rf_group_workspace_bytes, or rf_least_workspace_bytes if no item is to be split.
 size_t rf_least_workspace_bytes(const rf_shape* shape, const rf_params* params);
 size_t rf_group_workspace_bytes(const rf_shape* shape, const rf_params* params, int heads_total, int head0);
-rf_status rf_sparse_attn_group(const rf_shape* shape, const rf_params* params, const void* q, const void* k, const void* v,
-                               const int32_t* head_class, const int32_t* head_window, const rf_schedule* sched, void* o,
-                               float* lse, void* ws, size_t ws_bytes, int32_t* dev_status, void* cuda_stream, int heads_total,
-                               int head0);
+rf_status rf_sparse_call_group(const rf_shape* shape, const rf_params* params, const float* bandwidths, int32_t n_bandwidths,
+                               const void* q, const void* k, const void* v, int32_t* head_class, int32_t* head_window,
+                               rf_schedule* sched, void* o, float* lse, void* ws, size_t ws_bytes, int32_t* dev_status,
+                               void* cuda_stream, int heads_total, int head0);
 rf_status rf_launch_selftest_timeout(int32_t* dev_status, uint64_t limit_ns, int32_t* waits_returned, cudaStream_t st);

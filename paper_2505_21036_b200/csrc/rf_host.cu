@@ -213,22 +213,10 @@ rf_status rf_host_pipeline_run(rf_host_pipeline* p, const void* q_host, const vo
     if (p->ran) RF_TRY(cudaStreamWaitEvent(run, p->out_done[g], 0));
     int32_t* hc = p->head_class + (size_t)g * p->heads_per_group;
     const __nv_bfloat16 *q = p->q + g * gelems, *k = p->k + g * gelems, *v = p->v + g * gelems;
-    rf_status st;
-    if (p->n_bw > 0) {
-      int32_t* hw = p->head_window + (size_t)g * p->heads_per_group;
-      st = rf_arm_classify_plus(&p->gshape, &p->params, p->bw, p->n_bw, q, k, hc, hw, nullptr, p->ws[r], p->ws_bytes, p->status,
-                                run);
-      if (st == RF_OK) st = rf_build_block_mask_plus(&p->gshape, &p->params, hc, hw, &p->sched[r], p->status, run);
-      if (st == RF_OK)
-        st = rf_sparse_attn_group(&p->gshape, &p->params, q, k, v, hc, hw, &p->sched[r], p->o + g * gelems, nullptr, p->ws[r],
-                                  p->ws_bytes, p->status, run, heads, g * p->heads_per_group);
-    } else {
-      st = rf_arm_classify(&p->gshape, &p->params, q, k, hc, nullptr, p->ws[r], p->ws_bytes, p->status, run);
-      if (st == RF_OK) st = rf_build_block_mask(&p->gshape, &p->params, hc, &p->sched[r], p->status, run);
-      if (st == RF_OK)
-        st = rf_sparse_attn_group(&p->gshape, &p->params, q, k, v, hc, nullptr, &p->sched[r], p->o + g * gelems, nullptr, p->ws[r],
-                                  p->ws_bytes, p->status, run, heads, g * p->heads_per_group);
-    }
+    int32_t* hw = p->head_window + (size_t)g * p->heads_per_group;
+    const rf_status st = rf_sparse_call_group(&p->gshape, &p->params, p->bw, p->n_bw, q, k, v, hc, p->n_bw > 0 ? hw : nullptr, &p->sched[r],
+                                              p->o + g * gelems, nullptr, p->ws[r], p->ws_bytes, p->status, run, heads,
+                                              g * p->heads_per_group);
     if (st != RF_OK) return st;
     RF_TRY(cudaEventRecord(p->run_done[g], run));
     RF_TRY(cudaStreamWaitEvent(p->s_out, p->run_done[g], 0));

@@ -5,7 +5,9 @@
 // frames (Spatial), of in-frame positions (Temporal in position-major order) or a cyclic range
 // of positions (Temporal in original order), so "some pair kept" and "all pairs kept" reduce to
 // distances between at most two intervals per side.
-#include "rf_common.cuh"
+#include <algorithm>
+
+#include "rf_decide.cuh"
 
 namespace {
 
@@ -107,33 +109,23 @@ __device__ int tile_flag(const RfGeom& g, int cls, int a, int b) {
   return (all && full_width) ? 2 : 1;
 }
 
-// One warp per (query tile, head): flags for 32 key tiles at a time, ordered compaction by ballot.
+// One warp per (query tile a, head): flags for 32 key tiles at a time, ordered compaction by ballot.
 // No block-level synchronisation; eight rows per CTA.
-__global__ void __launch_bounds__(256) rf_build_tiles_kernel(RfGeom g, const int32_t* head_class, const int32_t* head_window,
-                                                              int32_t* __restrict__ count, int32_t* __restrict__ kv_tile,
-                                                              uint32_t* __restrict__ bitmap, int32_t* __restrict__ kv_len,
-                                                              int32_t* dev_status) {
-  const int lane = threadIdx.x & 31;
-  const int a = blockIdx.x * 8 + (threadIdx.x >> 5), bh = blockIdx.y;
-  rf_grid_trigger();
-  rf_grid_wait();
-  if (a >= g.nQ) return;   // whole warp
-  int cls = head_class[bh];
-  if (cls < 0 || cls > 3) {
-    if (lane == 0) rf_report(dev_status, RF_ERR_INVALID_ARG);
-    cls = RF_DENSE;
-  }
-  if (head_window != nullptr) {   // dynamic bandwidth: this head's own window
-    const int w = head_window[bh];
-    if (cls == RF_SPATIAL && w >= 0) g.wf = min(w, g.T);     // past the extent: same mask, no overflow
-    if (cls == RF_TEMPORAL && w >= 0) g.ws = min(w, g.S);
-  }
+struct TileArrays {
+  int32_t* count;
+  int32_t* kv_tile;
+  uint32_t* bitmap;
+  int32_t* kv_len;
+};
+__device__ __forceinline__ void build_row(RfGeom& g, int cls, int window, int a, int bh, int lane, const TileArrays& out, int32_t* dev_status) {
+  if (cls == RF_SPATIAL && window >= 0) g.wf = min(window, g.T);     // dynamic bandwidth: this head's own window; past the
+  if (cls == RF_TEMPORAL && window >= 0) g.ws = min(window, g.S);    // extent the mask is the same, and nothing overflows
   const int Lkv = rf_kv_len(g, cls);
   const int nK = rf_cdiv(Lkv, g.BN);
-  if (a == 0 && lane == 0 && rf_in_bounds(bh, (size_t)g.B * g.H, dev_status)) kv_len[bh] = Lkv;
-  int32_t* row = kv_tile + ((size_t)bh * g.nQ + a) * g.nKmax;
+  if (a == 0 && lane == 0 && rf_in_bounds(bh, (size_t)g.B * g.H, dev_status)) out.kv_len[bh] = Lkv;
+  int32_t* row = out.kv_tile + ((size_t)bh * g.nQ + a) * g.nKmax;
   const int words = rf_cdiv(g.nKmax, 32);
-  uint32_t* brow = bitmap ? bitmap + ((size_t)bh * g.nQ + a) * words : nullptr;
+  uint32_t* brow = out.bitmap ? out.bitmap + ((size_t)bh * g.nQ + a) * words : nullptr;
   int base = 0;
   for (int b0 = 0; b0 < words * 32; b0 += 32) {
     const int b = b0 + lane;
@@ -146,29 +138,46 @@ __global__ void __launch_bounds__(256) rf_build_tiles_kernel(RfGeom g, const int
     }
     base += __popc(m);
   }
-  if (lane == 0 && rf_in_bounds((size_t)bh * g.nQ + a, (size_t)g.B * g.H * g.nQ, dev_status)) count[(size_t)bh * g.nQ + a] = base;
+  if (lane == 0 && rf_in_bounds((size_t)bh * g.nQ + a, (size_t)g.B * g.H * g.nQ, dev_status)) out.count[(size_t)bh * g.nQ + a] = base;
+}
+__global__ void __launch_bounds__(256) rf_build_tiles_kernel(RfGeom g, const int32_t* head_class, const int32_t* head_window,
+                                                              const TileArrays out, int32_t* dev_status) {
+  const int lane = threadIdx.x & 31;
+  const int a = blockIdx.x * 8 + (threadIdx.x >> 5), bh = blockIdx.y;
+  rf_grid_trigger();
+  rf_grid_wait();
+  if (a >= g.nQ) return;   // whole warp
+  int cls = head_class[bh];
+  if (cls < 0 || cls > 3) {
+    if (lane == 0) rf_report(dev_status, RF_ERR_INVALID_ARG);
+    cls = RF_DENSE;
+  }
+  build_row(g, cls, head_window != nullptr ? head_window[bh] : -1, a, bh, lane, out, dev_status);
 }
 
 // Reordered copies for heads whose coordinate space is not the original one.
 //   Temporal + permute: Q, K, V  -> slot pos*T + frame (text rows keep their index)
 //   Textural:           K, V     -> frame*nC + rank(pos) for kept positions, text after T*nC
 // A byte mover: what bounds it is how many 16-byte vectors are under way.  A thread moves its column of kGatherRows rows
-// of two or three tensors, all loads before the first store; a CTA is done after one such step (grid.x walks rows, grid.y
-// heads).  Temporal heads are walked in source order, Textural heads in the order of the kept rows: the k-th kept position
-// of a frame follows in closed form (any tau consecutive frame rows keep W positions between them), so no thread visits a
-// row that is not copied and no table has to be built first.  48 heads, 17 776 tokens, D = 64, all Textural: 133 -> 44 us
-// (221 MB); 24 heads, 8448 tokens, D = 128, 8/8/8: 41 -> 25 us (139 MB).
+// of two or three tensors, all loads before the first store; the CTAs of a head (grid.y) share its rows.  Temporal heads are
+// walked in source order, Textural heads in the order of the kept rows: the k-th kept position of a frame follows in closed form
+// (any tau consecutive frame rows keep W positions between them), so no thread visits a row that is not copied and no table has
+// to be built first.  48 heads, 17 776 tokens, D = 64, all Textural: 133 -> 44 us (221 MB); 24 heads, 8448 tokens, D = 128,
+// 8/8/8: 41 -> 25 us (139 MB).
 constexpr int kGatherRows = 4;
-__global__ void __launch_bounds__(256) rf_gather_kernel(RfGeom g, const int32_t* head_class, const uint4* q, const uint4* k,
-                                                         const uint4* v, uint4* __restrict__ wq,
-                                                         uint4* __restrict__ wk, uint4* __restrict__ wv, int32_t* tickets,
-                                                         int n_tickets, int32_t* dev_status) {
-  rf_grid_trigger();
-  rf_grid_wait();
-  if (blockIdx.y == 0)   // the attention kernel's tickets start at zero
-    for (int i = blockIdx.x * 256 + threadIdx.x; i < n_tickets; i += gridDim.x * 256) tickets[i] = 0;
-  const int bh = blockIdx.y;
-  const int cls = head_class[bh];
+struct Copies {
+  const uint4 *q, *k, *v;
+  uint4 *wq, *wk, *wv;
+  int32_t* tickets;          // of the attention kernel: they start at zero
+  int n_tickets;
+};
+__device__ __forceinline__ void clear_tickets(const Copies& io, int block, int blocks) {
+  for (int i = block * 256 + threadIdx.x; i < io.n_tickets; i += blocks * 256) io.tickets[i] = 0;
+}
+// CTA `block` of the `blocks` that share head bh.
+__device__ __forceinline__ void gather_rows(const RfGeom& g, int cls, int bh, int block, int blocks, const Copies& io, int32_t* dev_status) {
+  const uint4 *q = io.q, *k = io.k, *v = io.v;
+  uint4 *wq = io.wq, *wk = io.wk, *wv = io.wv;
   const bool perm = cls == RF_TEMPORAL && g.permute;
   const bool tex = cls == RF_TEXTURAL;
   if (!perm && !tex) return;
@@ -178,8 +187,8 @@ __global__ void __launch_bounds__(256) rf_gather_kernel(RfGeom g, const int32_t*
   if (lr >= rows_per_step) return;
   const size_t head_off = (size_t)bh * g.N * vec + c;
   const int rows = perm ? g.N : g.LkvTex, video = perm ? g.Nv : g.T * g.nC;
-  for (long long i0 = (long long)blockIdx.x * rows_per_step * kGatherRows + lr; i0 < rows;
-       i0 += (long long)gridDim.x * rows_per_step * kGatherRows) {
+  for (long long i0 = (long long)block * rows_per_step * kGatherRows + lr; i0 < rows;
+       i0 += (long long)blocks * rows_per_step * kGatherRows) {
     int src[kGatherRows], dst[kGatherRows];
     bool on[kGatherRows];
 #pragma unroll
@@ -222,6 +231,30 @@ __global__ void __launch_bounds__(256) rf_gather_kernel(RfGeom g, const int32_t*
   }
 }
 
+__global__ void __launch_bounds__(256) rf_gather_kernel(RfGeom g, const int32_t* head_class, const Copies io, int32_t* dev_status) {
+  rf_grid_trigger();
+  rf_grid_wait();
+  if (blockIdx.y == 0) clear_tickets(io, blockIdx.x, gridDim.x);
+  gather_rows(g, head_class[blockIdx.y], blockIdx.y, blockIdx.x, gridDim.x, io, dev_status);
+}
+
+// Decision, schedule and copies in one launch: the first CTAs of a head build its tile lists, the others copy.  A warp's own
+// decision costs it one round of loads (a few sums per recall); what it saves is two launches' hand-over, and the lists are
+// built beside the copies, which wait for memory.
+__global__ void __launch_bounds__(256) rf_prepare_kernel(RfGeom g, const RfDecision dec, const TileArrays out, const Copies io, int tile_blocks,
+                                                          int32_t* dev_status) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, bh = blockIdx.y;
+  const bool lists = (int)blockIdx.x < tile_blocks;
+  rf_grid_trigger();
+  rf_grid_wait();
+  if (!lists && bh == 0) clear_tickets(io, blockIdx.x - tile_blocks, gridDim.x - tile_blocks);
+  const int a = blockIdx.x * 8 + warp;
+  if (lists && a >= g.nQ) return;   // whole warp
+  const RfHead h = rf_decide(dec, bh, lane, lists && a == 0);
+  if (lists) build_row(g, h.failed ? RF_DENSE : h.cls, h.window, a, bh, lane, out, dev_status);
+  else gather_rows(g, h.cls, bh, blockIdx.x - tile_blocks, gridDim.x - tile_blocks, io, dev_status);
+}
+
 __global__ void __launch_bounds__(256) rf_zero_kernel(int32_t* words, int n) {
   rf_grid_trigger();
   rf_grid_wait();
@@ -236,14 +269,33 @@ cudaError_t rf_launch_zero(int32_t* words, int n, cudaStream_t st) {
 
 cudaError_t rf_launch_build_tiles(const RfGeom& g, const int32_t* head_class, const int32_t* head_window, int32_t* count,
                                   int32_t* kv_tile, uint32_t* bitmap, int32_t* kv_len, int32_t* dev_status, cudaStream_t st) {
-  return rf_launch(rf_build_tiles_kernel, dim3(rf_cdiv(g.nQ, 8), g.B * g.H), 256, 0, st, g, head_class, head_window, count, kv_tile,
-                   bitmap, kv_len, dev_status);
+  return rf_launch(rf_build_tiles_kernel, dim3(rf_cdiv(g.nQ, 8), g.B * g.H), 256, 0, st, g, head_class, head_window,
+                   TileArrays{count, kv_tile, bitmap, kv_len}, dev_status);
 }
+
+namespace {
+int gather_blocks(const RfGeom& g) { return rf_cdiv(g.N, 256 / (g.D / 8) * kGatherRows); }
+Copies copies(const __nv_bfloat16* q, const __nv_bfloat16* k, const __nv_bfloat16* v, __nv_bfloat16* wq, __nv_bfloat16* wk,
+              __nv_bfloat16* wv, int32_t* tickets, int n_tickets) {
+  return Copies{(const uint4*)q, (const uint4*)k, (const uint4*)v, (uint4*)wq, (uint4*)wk, (uint4*)wv, tickets, n_tickets};
+}
+}  // namespace
 
 cudaError_t rf_launch_gather(const RfGeom& g, const int32_t* head_class, const __nv_bfloat16* q,
                              const __nv_bfloat16* k, const __nv_bfloat16* v, __nv_bfloat16* wq, __nv_bfloat16* wk,
                              __nv_bfloat16* wv, int32_t* tickets, int n_tickets, int32_t* dev_status, cudaStream_t st) {
-  const int rows_per_cta = 256 / (g.D / 8) * kGatherRows;
-  return rf_launch(rf_gather_kernel, dim3(rf_cdiv(g.N, rows_per_cta), g.B * g.H), 256, 0, st, g, head_class, (const uint4*)q,
-                   (const uint4*)k, (const uint4*)v, (uint4*)wq, (uint4*)wk, (uint4*)wv, tickets, n_tickets, dev_status);
+  return rf_launch(rf_gather_kernel, dim3(gather_blocks(g), g.B * g.H), 256, 0, st, g, head_class,
+                   copies(q, k, v, wq, wk, wv, tickets, n_tickets), dev_status);
+}
+
+cudaError_t rf_launch_prepare(const RfGeom& g, const RfDecision& dec, int32_t* count, int32_t* kv_tile, uint32_t* bitmap,
+                              int32_t* kv_len, const __nv_bfloat16* q, const __nv_bfloat16* k, const __nv_bfloat16* v,
+                              __nv_bfloat16* wq, __nv_bfloat16* wk, __nv_bfloat16* wv, int32_t* tickets, int n_tickets,
+                              int32_t* dev_status, cudaStream_t st) {
+  const int heads = g.B * g.H, tile_blocks = rf_cdiv(g.nQ, 8);
+  // One wave of copying CTAs (three to an SM): each pays for its decision once and then walks on (24 heads, 8448 tokens, D = 128:
+  // 508 us a call, 509 with four times as many, 517 with one CTA per step; small calls do not care).
+  const int blocks = std::min(gather_blocks(g), rf_cdiv(148 * 3, heads));
+  return rf_launch(rf_prepare_kernel, dim3(tile_blocks + blocks, heads), 256, 0, st, g, dec, TileArrays{count, kv_tile, bitmap, kv_len},
+                   copies(q, k, v, wq, wk, wv, tickets, n_tickets), tile_blocks, dev_status);
 }
