@@ -117,7 +117,7 @@ int32_t rf_bounds_checked(void);
 rf_status rf_schedule_dims(const rf_shape *shape, const rf_params *params, int32_t *nQ, int32_t *nKmax);
 
 /* Host, pure: bytes of device workspace that rf_arm_classify / rf_sparse_attn_fwd need (reordered Q/K/V copies for
- * Temporal and Textural heads, ARM per-row recalls and, for shapes of few query tiles, up to 52 MB for the partial results
+ * Temporal and Textural heads, room for ARM's recalls and, for shapes of few query tiles, up to 52 MB for the partial results
  * of query tiles that several SMs share).  0 on bad arguments.  A block that has room for all but those partial results
  * (one sized for a shape of more query tiles, which may need less) is taken as well: no query tile is shared then, which costs
  * time and changes the rounding.  Every call that takes a workspace writes to it, so calls that may overlap on the GPU need
