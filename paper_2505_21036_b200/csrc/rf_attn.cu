@@ -18,9 +18,10 @@
 // Per listed tile and stream: S lands in TMEM, the softmax warps read their rows (tcgen05.ld), keep a
 // running maximum in fp32, write P as packed bf16 back into TMEM (tcgen05.st: on top of the S
 // columns at D = 96 / 128, into spare columns at D = 64) and the MMA warp multiplies it with V straight
-// from TMEM.  V carries one column more, of ones: O's column D is the row sum of the weights as rounded to bf16, the ones that
-// are multiplied with V, and normalises O (which makes O an exact convex combination of V rows with slightly perturbed
-// weights: the rounding of a dominant weight cancels instead of scaling the output row).  The running maximum is raised lazily (see kRaise), in which case the softmax warp itself
+// from TMEM.  V carries one column more, of ones: O's column D is the sum of a row's weights of one tile as rounded to bf16, the
+// ones that are multiplied with V; the softmax warps take it out tile by tile, and the sum over the tiles normalises O (which makes
+// O an exact convex combination of V rows with slightly perturbed weights: the rounding of a dominant weight cancels instead of
+// scaling the output row).  The running maximum is raised lazily (see kRaise), in which case the softmax warp itself
 // rescales its rows of O in TMEM; the final O / l and the log-sum-exp do not depend on it.
 // PARTIAL tiles apply the exact element mask of the head's pattern; FULL tiles skip it.
 #include <algorithm>
@@ -42,10 +43,15 @@ constexpr int kAskAhead = 4;   // tiles an item's longer list has left when the 
 // call), the energy of a tile, a sixth of which are the softmax warps' instructions.  At D = 96 / 128 the first kSpec weights
 // are taken while the tile's maximum is being found and the first half of P is stored and multiplied under the second half's
 // exponentials; at D = 64 the maximum comes first.  The row sums of the rounded weights were 192 of a row's 512 instructions a tile
-// (two to widen a pair, one to add it); the tensor pipe takes them in 16 columns more of P V (64 cycles of its 2048 a pair of
+// (two to widen a pair, one to add it); the tensor pipe takes them in 16 columns more of P V (128 cycles beside 2048 a pair of
 // tiles at D = 128).  Repeated calls at the power limit, before and after: dense 24 heads, 8448 tokens, D = 128 870 -> 841 us;
 // 24 heads, 119 056 tokens 73.8 -> 71.7 ms; 48 heads, 5082 tokens, D = 96 2530 -> 2415 us; 48 heads, 17 776 tokens,
-// D = 64 2900 -> 2763 us masked, 5340 -> 4990 dense.  Error against 64 bits the same to 1e-7 on rel 1.7e-3.
+// D = 64 2900 -> 2763 us masked, 5340 -> 4990 dense.
+// Column D holds one tile's sum only: it is read and cleared before the next P is handed over, and the tiles are added up in fp32.
+// An accumulator of the whole row cuts every weight off at the last place of the sum so far: beside one key of weight 1, 2^18
+// keys of 2^-19 lost 2.1e-3 of the row's weight in it; with the sums by tile the error is what the outputs' rounding leaves, 5e-5, as it
+// is with all sums added up by the softmax warps, whose outputs are within rel 6e-5.  It costs a load and a store of one column a
+// tile: sixteen shapes, 0.997 to 1.010 times as fast as without.
 // Without lse the sum of the unrounded weights is left out (a template: dense D = 64 5.74 -> 5.59 ms).
 // Lazy rescaling of the running maximum: it is raised once a tile's maximum exceeds it by kRaise (log2 units; all rows
 // of the warp more than kRaiseMargin above theirs then raise it together).  A tile's weights thus sum to 2^32 at most;
@@ -80,7 +86,7 @@ struct Cfg {
     return ks < 4 ? (uint32_t)ks * 32u : BLK + (uint32_t)(ks - 4) * 32u;
   }
   // V, the MN-major operand of P V, lies in blocks of VBOX columns; behind its D columns stands a block whose first column
-  // is one and whose others are zero, so that O's column D is the row sum of the weights (see the softmax).  At D = 96
+  // is one and whose others are zero, so that O's column D is a tile's row sum of the weights (see the softmax).  At D = 96
   // blocks of 32 columns (64-byte swizzle) put that block next to column 95.
   static constexpr int VBOX = D == 96 ? 32 : 64;
   static constexpr uint32_t VROW = VBOX * 2, VBLK = 128 * VROW, VLOAD = D / VBOX * VBLK, VTILE = VLOAD + VBLK;
@@ -299,7 +305,7 @@ __device__ __noinline__ void leave_piece(const RfAttnArgs& a, const int* iw, uin
   }
 }
 
-// This thread's row of O, and its sum of weights, times alpha (warp-collective).
+// This thread's row of O times alpha (warp-collective).
 __device__ __forceinline__ void rescale_columns(uint32_t t_o, float alpha) {
   uint32_t v[32];
   tmem_ld32(t_o, v);
@@ -308,19 +314,13 @@ __device__ __forceinline__ void rescale_columns(uint32_t t_o, float alpha) {
   for (int i = 0; i < 32; ++i) v[i] = __float_as_uint(__uint_as_float(v[i]) * alpha);
   tmem_st32(t_o, v);
 }
-__device__ __forceinline__ void rescale_sum(uint32_t t_l, float alpha) {
-  const uint32_t l = tmem_ld1(t_l);
-  tc_wait_ld();
-  tmem_st1(t_l, __float_as_uint(__uint_as_float(l) * alpha));
-  tc_wait_st();
-  tc_fence_before();
-}
 template <int D>
 __device__ __forceinline__ void rescale_o(uint32_t t_o, float alpha) {
   tc_fence_after();
 #pragma unroll
   for (int c = 0; c < D; c += 32) rescale_columns(t_o + c, alpha);
-  rescale_sum(t_o + D, alpha);
+  tc_wait_st();
+  tc_fence_before();
 }
 // The same out of line, for D = 96 / 128: rare as it is, the scores then stay in registers around it and the loop over the
 // tiles is free of spills.
@@ -329,7 +329,8 @@ __device__ __noinline__ void rescale_o_call(uint32_t t_o, float alpha) {
   tc_fence_after();
 #pragma unroll 1
   for (int c = 0; c < D; c += 32) rescale_columns(t_o + c, alpha);
-  rescale_sum(t_o + D, alpha);
+  tc_wait_st();
+  tc_fence_before();
 }
 
 // This thread's row of scores, and the masked ones of a PARTIAL tile set to -inf.
@@ -752,6 +753,7 @@ __global__ void __launch_bounds__(kThreads, 1) rf_attn_kernel(const __grid_const
     const int32_t* list = a.head_class != nullptr ? a.kv_tile + ((size_t)im.bh * g.nQ + min(im.qt0 + j, g.nQ - 1)) * g.nKmax : nullptr;
     const RowMask rmask = make_row_mask(g, im.cls, im.window, min((im.qt0 + j) * BM + row_in_tile, g.N - 1));
     float m_run = -INFINITY;   // running maximum, log2 domain (score * sc)
+    float l_run = 0.f;         // sum of the weights as rounded to bf16, the ones P V multiplies: normalises O (the last tile's are in O's column D)
     float l_exact = 0.f;       // sum of the unrounded weights: the log-sum-exp (LSE only)
 
     const int begin = j == 0 ? im.b0 : im.b1, end = begin + n;
@@ -771,7 +773,11 @@ __global__ void __launch_bounds__(kThreads, 1) rf_attn_kernel(const __grid_const
       mbar_wait(bar(C::B_SF + j), done & 1, wc);
       tc_fence_after();
       uint32_t s[128];
+      // the sum of the last tile's weights, whose P V (D = 96 / 128) these scores were issued after
+      uint32_t l_tile;
+      if constexpr (!C::S_EARLY) l_tile = tmem_ld1(t_o + D);
       load_scores(t_s, s);
+      if constexpr (!C::S_EARLY) l_run = opens ? 0.f : l_run + __uint_as_float(l_tile);
       if constexpr (C::S_SHARED) {   // S is handed back at once: its columns are the other stream's too, or (D = 64) its own next scores'
         tc_fence_before();
         __syncwarp();
@@ -794,6 +800,7 @@ __global__ void __launch_bounds__(kThreads, 1) rf_attn_kernel(const __grid_const
         if (raise) {
           alpha = ex2(m_run - m_tile);   // 0 when m_run = -inf
           m_run = m_tile;
+          l_run *= alpha;
           if (LSE) l_exact *= alpha;
         }
         // P V of the previous tile reads the P columns this tile is about to overwrite, and O may only be
@@ -822,14 +829,19 @@ __global__ void __launch_bounds__(kThreads, 1) rf_attn_kernel(const __grid_const
         }
         if (LSE) l_exact += la.x + la.y;
         if (!o_landed) mbar_wait(bar(C::B_OF + j), (done - 1) & 1, wc);
+        tc_fence_after();
+        l_tile = tmem_ld1(t_o + D);   // the sum of the last tile's weights; cleared for this tile's
         {
           const uint32_t t_p = tmem_base + lane_sel + (j ? C::P_COL1 : C::P_COL0);
           uint32_t(&p0)[32] = *reinterpret_cast<uint32_t(*)[32]>(&pk[0]);
           uint32_t(&p1)[32] = *reinterpret_cast<uint32_t(*)[32]>(&pk[32]);
           tmem_st32(t_p, p0);
           tmem_st32(t_p + 32, p1);
+          tc_wait_ld();
+          tmem_st1(t_o + D, 0u);
           tc_wait_st();
         }
+        l_run = opens ? 0.f : l_run + __uint_as_float(l_tile) * alpha;
         tc_fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive(bar(C::B_PF + j));
@@ -855,6 +867,7 @@ __global__ void __launch_bounds__(kThreads, 1) rf_attn_kernel(const __grid_const
         if (m_tile > m_run + kRaiseMargin) {
           alpha = ex2(m_run - m_tile);   // 0 when m_run = -inf
           m_run = m_tile;
+          l_run *= alpha;
           if (LSE) l_exact *= alpha;
         }
         if (!opens) {
@@ -871,6 +884,7 @@ __global__ void __launch_bounds__(kThreads, 1) rf_attn_kernel(const __grid_const
       static_assert(C::S_EARLY || C::PARTS == 2, "the first half is handed over under the exponentials of the second");
       take_weights<kSpec, 64, LSE>(s, pk, la, sc2, mneg);
       store_weights<0, 64>(t_p, pk);
+      tmem_st1(t_o + D, 0u);     // the column of this tile's sum
       take_weights<64, 80, LSE>(s, pk, la, sc2, mneg);
       tc_wait_st();              // the store has had these exponentials' time
       tc_fence_before();
@@ -889,11 +903,10 @@ __global__ void __launch_bounds__(kThreads, 1) rf_attn_kernel(const __grid_const
       mbar_wait(bar(C::B_OF + j), (done - 1) & 1, wc);
       tc_fence_after();
     }
-    // the sum of the weights as rounded to bf16, the ones P V multiplied: normalises O
-    float l_run = 0.f;
     if (n > 0) {
-      l_run = __uint_as_float(tmem_ld1(t_o + D));
+      const uint32_t l_tile = tmem_ld1(t_o + D);
       tc_wait_ld();
+      l_run += __uint_as_float(l_tile);
     }
     // the item's words are read again here: kept in registers they would be in the way of the scores
     const int* iw = items + (item % kItemSlots) * kItemWords;
