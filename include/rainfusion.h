@@ -205,6 +205,16 @@ rf_status rf_selftest_arm_abandoned(const rf_shape *shape, const rf_params *para
                                     int32_t *head_class, void *ws, size_t ws_bytes, int32_t *dev_status,
                                     void *cuda_stream);
 
+/*
+ * The same for rf_sparse_call: its launches with the score kernel left out and the failure flag set.  Afterwards head_class
+ * (and head_window, with n_bandwidths > 0) is -1 for every head, *dev_status is RF_ERR_TIMEOUT if it was 0 before, no tokens
+ * were reordered and every query tile lists every key tile.  Arguments as for rf_sparse_call.
+ */
+rf_status rf_selftest_sparse_call_abandoned(const rf_shape *shape, const rf_params *params, const float *bandwidths,
+                                            int32_t n_bandwidths, const void *q, const void *k, const void *v,
+                                            int32_t *head_class, int32_t *head_window, rf_schedule *sched, void *o, float *lse,
+                                            void *ws, size_t ws_bytes, int32_t *dev_status, void *cuda_stream);
+
 /* Full 3D attention (Eq. 1-2, all-zero mask): the same kernel walking every tile.  ws may be NULL; it is not touched. */
 rf_status rf_dense_attn_fwd(const rf_shape *shape, const void *q, const void *k, const void *v, void *o,
                             float *lse, void *ws, size_t ws_bytes, int32_t *dev_status, void *cuda_stream);

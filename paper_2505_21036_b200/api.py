@@ -22,7 +22,7 @@ _lib = None
 EXPORTS = ["rf_status_string", "rf_schedule_dims", "rf_workspace_bytes", "rf_arm_classify",
            "rf_build_block_mask", "rf_reorder_tokens", "rf_sparse_attn_fwd", "rf_dense_attn_fwd", "rf_dense_attn_fwd_split", "rf_dense_workspace_bytes", "rf_sparse_call",
            "rf_arm_classify_noalloc", "rf_selftest_wait_timeout", "rf_arm_classify_plus", "rf_build_block_mask_plus", "rf_sparse_attn_fwd_plus",
-           "rf_sparse_attn_reordered", "rf_selftest_arm_abandoned", "rf_bounds_checked", "rf_host_pipeline_staging_bytes",
+           "rf_sparse_attn_reordered", "rf_selftest_arm_abandoned", "rf_selftest_sparse_call_abandoned", "rf_bounds_checked", "rf_host_pipeline_staging_bytes",
            "rf_host_pipeline_create", "rf_host_pipeline_run", "rf_host_pipeline_status", "rf_host_pipeline_destroy",
            "rf_host_pipeline_set_bandwidths", "rf_host_pipeline_head_class", "rf_host_pipeline_head_window"]
 
@@ -109,6 +109,8 @@ def load():
     lib.rf_reorder_tokens.argtypes = [P(rf_shape), P(rf_params), V, V, V, V, V, Z, V]
     lib.rf_sparse_call.restype = I
     lib.rf_sparse_call.argtypes = [P(rf_shape), P(rf_params), P(C.c_float), C.c_int32, V, V, V, V, V, P(rf_schedule), V, V, V, Z, V, V]
+    lib.rf_selftest_sparse_call_abandoned.restype = I
+    lib.rf_selftest_sparse_call_abandoned.argtypes = lib.rf_sparse_call.argtypes
     lib.rf_dense_workspace_bytes.restype = Z
     lib.rf_dense_workspace_bytes.argtypes = [P(rf_shape)]
     lib.rf_dense_attn_fwd.restype = I
@@ -259,11 +261,21 @@ def rf_selftest_arm_abandoned(shape, params, q, k, head_class, ws, dev_status):
 
 def rf_sparse_call(shape, params, bandwidths, q, k, v, head_class, head_window, sched: Schedule, o, lse, ws, dev_status=None):
     """ARM -> schedule -> masked attention in one crossing into the library (bandwidths: None, or the candidates)."""
+    _sparse_call("rf_sparse_call", shape, params, bandwidths, q, k, v, head_class, head_window, sched, o, lse, ws, dev_status)
+
+
+def rf_selftest_sparse_call_abandoned(shape, params, bandwidths, q, k, v, head_class, head_window, sched: Schedule, o, lse, ws,
+                                      dev_status=None):
+    _sparse_call("rf_selftest_sparse_call_abandoned", shape, params, bandwidths, q, k, v, head_class, head_window, sched, o, lse, ws,
+                 dev_status)
+
+
+def _sparse_call(name, shape, params, bandwidths, q, k, v, head_class, head_window, sched, o, lse, ws, dev_status):
     n = len(bandwidths) if bandwidths else 0
     arr = (C.c_float * n)(*bandwidths) if n else None
-    _check(load().rf_sparse_call(C.byref(shape), C.byref(params), arr, n, q.data_ptr(), k.data_ptr(), v.data_ptr(),
+    _check(getattr(load(), name)(C.byref(shape), C.byref(params), arr, n, q.data_ptr(), k.data_ptr(), v.data_ptr(),
                                  head_class.data_ptr(), _ptr(head_window), C.byref(sched.c), o.data_ptr(), _ptr(lse),
-                                 ws.data_ptr(), ws.numel(), _ptr(dev_status), _stream()), "rf_sparse_call")
+                                 ws.data_ptr(), ws.numel(), _ptr(dev_status), _stream()), name)
 
 
 class HostPipeline:

@@ -362,7 +362,7 @@ rf_status arm_call(const rf_shape* shape, const rf_params* params, const float* 
 rf_status rf_sparse_call_group(const rf_shape* shape, const rf_params* params, const float* bandwidths, int32_t n_bandwidths,
                                const void* q, const void* k, const void* v, int32_t* head_class, int32_t* head_window,
                                rf_schedule* sched, void* o, float* lse, void* ws, size_t ws_bytes, int32_t* dev_status,
-                               void* cuda_stream, int heads_total, int head0) {
+                               void* cuda_stream, int heads_total, int head0, bool selftest_abandon) {
   if (n_bandwidths < 0) return RF_ERR_INVALID_ARG;
   if (n_bandwidths == 0) head_window = nullptr;
   // ARM checks its own arguments before it launches; what the steps after it would refuse is refused here
@@ -370,7 +370,8 @@ rf_status rf_sparse_call_group(const rf_shape* shape, const rf_params* params, c
   if (st == RF_OK && sched->kv_len == nullptr) st = RF_ERR_INVALID_ARG;
   if (st != RF_OK) return st;
   RfDecision dec;
-  st = arm_call(shape, params, bandwidths, n_bandwidths, q, k, head_class, head_window, nullptr, ws, ws_bytes, dev_status, cuda_stream, &dec);
+  st = arm_call(shape, params, bandwidths, n_bandwidths, q, k, head_class, head_window, nullptr, ws, ws_bytes, dev_status, cuda_stream, &dec,
+                selftest_abandon);
   if (st != RF_OK) return st;
   return sparse_attn_impl(shape, params, q, k, v, head_class, head_window, sched, o, lse, ws, ws_bytes, dev_status, cuda_stream,
                           Copies::kPrepare, heads_total, head0, &dec);
@@ -492,6 +493,14 @@ rf_status rf_sparse_call(const rf_shape* shape, const rf_params* params, const f
                          float* lse, void* ws, size_t ws_bytes, int32_t* dev_status, void* cuda_stream) {
   return rf_sparse_call_group(shape, params, bandwidths, n_bandwidths, q, k, v, head_class, head_window, sched, o, lse, ws, ws_bytes,
                               dev_status, cuda_stream, shape != nullptr ? shape->B * shape->H : 0, 0);
+}
+
+rf_status rf_selftest_sparse_call_abandoned(const rf_shape* shape, const rf_params* params, const float* bandwidths, int32_t n_bandwidths,
+                                            const void* q, const void* k, const void* v, int32_t* head_class, int32_t* head_window,
+                                            rf_schedule* sched, void* o, float* lse, void* ws, size_t ws_bytes, int32_t* dev_status,
+                                            void* cuda_stream) {
+  return rf_sparse_call_group(shape, params, bandwidths, n_bandwidths, q, k, v, head_class, head_window, sched, o, lse, ws, ws_bytes,
+                              dev_status, cuda_stream, shape != nullptr ? shape->B * shape->H : 0, 0, true);
 }
 
 rf_status rf_selftest_wait_timeout(int32_t* dev_status, int32_t limit_ms, int32_t* waits_returned, void* cuda_stream) {

@@ -181,5 +181,5 @@ size_t rf_group_workspace_bytes(const rf_shape* shape, const rf_params* params, 
 rf_status rf_sparse_call_group(const rf_shape* shape, const rf_params* params, const float* bandwidths, int32_t n_bandwidths,
                                const void* q, const void* k, const void* v, int32_t* head_class, int32_t* head_window,
                                rf_schedule* sched, void* o, float* lse, void* ws, size_t ws_bytes, int32_t* dev_status,
-                               void* cuda_stream, int heads_total, int head0);
+                               void* cuda_stream, int heads_total, int head0, bool selftest_abandon = false);
 rf_status rf_launch_selftest_timeout(int32_t* dev_status, uint64_t limit_ns, int32_t* waits_returned, cudaStream_t st);

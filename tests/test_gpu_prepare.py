@@ -65,3 +65,40 @@ def test_one_call_gives_what_three_give(B, H, D, T, fh, fw, L, omega, opt, bw):
     for size in (full, full + 4096):
         for a, b in zip(first, call(shape, params, q, k, v, bw, size, True)):
             assert torch.equal(a, b) or (a.is_floating_point() and torch.equal(a.isnan(), b.isnan()) and torch.equal(a.nan_to_num(), b.nan_to_num()))
+
+
+@pytest.mark.parametrize("bw", [None, BW])
+@pytest.mark.parametrize("B,H,D,T,fh,fw,L,omega", [(1, 3, 64, 4, 8, 8, 16, 4), (2, 5, 96, 7, 19, 27, 77, 7)])
+def test_a_sparse_call_reports_a_score_kernel_that_gave_up(B, H, D, T, fh, fw, L, omega, bw):
+    """The call's launches with the score kernel's failure flag set in place of that kernel: the merged launch must hand the code on,
+    write class and window -1, list every tile, reorder nothing and leave a call that ends; the next call is a normal one."""
+    shape = api.make_shape(B, H, D, T, fh, fw, L)
+    params = api.make_params(max(T // 4, 1), fh * fw // 4, sample_stride=omega)
+    N = T * fh * fw + L
+    g = torch.Generator("cuda").manual_seed(N)
+    q, k, v = (torch.randn(B, H, N, D, device="cuda", generator=g).to(torch.bfloat16) for _ in range(3))
+    mem = gu.Guarded()
+    ws = mem.alloc((api.rf_workspace_bytes(shape, params),), torch.uint8, 0x5A, "ws")
+    sched = api.Schedule(shape, params, "cuda")
+    cls, win, status = (mem.alloc(s, torch.int32, f, n) for s, f, n in (((B, H), -9, "class"), ((B, H), -9, "window"), ((1,), 0, "status")))
+    o, lse = mem.alloc((B, H, N, D), torch.bfloat16, float("nan"), "o"), mem.alloc((B, H, N), torch.float32, float("nan"), "lse")
+    w = win if bw else None
+    api.rf_selftest_sparse_call_abandoned(shape, params, bw, q, k, v, cls, w, sched, o, lse, ws, status)
+    torch.cuda.synchronize()
+    mem.check("abandoned call")
+    assert int(status.item()) == 5                                     # RF_ERR_TIMEOUT
+    assert bool((cls == -1).all()) and bool((win == (-1 if bw else -9)).all())
+    assert bool((sched.count == sched.nKmax).all()) and bool((sched.kv_len == N).all())
+    assert torch.equal((sched.kv_tile & 0x7FFFFFFF).reshape(-1, sched.nKmax),
+                       torch.arange(sched.nKmax, device="cuda", dtype=torch.int32).expand(B * H * sched.nQ, -1))
+    copies = 3 * (-(-B * H * N * D * 2 // 256) * 256)
+    assert bool((ws[:copies] == 0x5A).all())
+    dense, dense_lse = torch.empty_like(q), torch.empty_like(lse)      # (its pieces may be cut elsewhere: equal but for rounding)
+    api.rf_dense_attn_fwd(shape, q, k, v, dense, dense_lse)
+    assert float((o.float() - dense.float()).abs().max()) < 2 * gu.O_MAX_ABS and float((lse - dense_lse).abs().max()) < 2 * gu.LSE_ABS
+    status.zero_()
+    full = ws.numel()
+    for a, b in zip(call(shape, params, q, k, v, bw, full, False), call(shape, params, q, k, v, bw, full, True)):
+        assert torch.equal(a, b) or (a.is_floating_point() and torch.equal(a.isnan(), b.isnan()) and torch.equal(a.nan_to_num(), b.nan_to_num()))
+    api.rf_sparse_call(shape, params, bw, q, k, v, cls, w, sched, o, lse, ws, status)
+    assert int(status.item()) == 0 and bool((cls >= 0).all())
