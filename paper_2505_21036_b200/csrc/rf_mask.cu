@@ -293,9 +293,16 @@ cudaError_t rf_launch_prepare(const RfGeom& g, const RfDecision& dec, int32_t* c
                               __nv_bfloat16* wq, __nv_bfloat16* wk, __nv_bfloat16* wv, int32_t* tickets, int n_tickets,
                               int32_t* dev_status, cudaStream_t st) {
   const int heads = g.B * g.H, tile_blocks = rf_cdiv(g.nQ, 8);
-  // One wave of copying CTAs (three to an SM): each pays for its decision once and then walks on (24 heads, 8448 tokens, D = 128:
-  // 508 us a call, 509 with four times as many, 517 with one CTA per step; small calls do not care).
-  const int blocks = std::min(gather_blocks(g), rf_cdiv(148 * 3, heads));
+  // A head's copying CTAs are fixed before its class is known; those of a head that copies nothing leave at once.  Two CTAs share an
+  // SM (registers).  Three CTAs an SM over all heads at least, so that each pays for its decision once and walks on (24 heads, 8448
+  // tokens, D = 128: 508 us a call, 517 with one CTA per step), and up to four times as many while each still has four steps,
+  // so that a few reordered heads of many spread over the SMs too.  us a call without and with the second half of the rule: 48 heads, 17 776
+  // tokens, D = 64, all reordered 1396 and 1378, one 1621 and 1615; 24 heads, 8448 tokens, D = 128, all 327 and 322, eight 368 and
+  // 363.  Calls of few steps keep their share: more CTAs cost them 1 to 3 % (24 heads, 2457 tokens, D = 96: 71.9, with twice as many 74.1).
+  // Three CTAs to an SM (80 registers) gained 1 % in some calls and lost as much in others (3 heads, 7476 tokens, D = 96: 113.5 and
+  // 115.6).
+  const int share = rf_cdiv(148 * 3, heads), steps = gather_blocks(g);
+  const int blocks = std::min(steps, std::max(share, std::min(rf_cdiv(steps, 4), 4 * share)));
   return rf_launch(rf_prepare_kernel, dim3(tile_blocks + blocks, heads), 256, 0, st, g, dec, TileArrays{count, kv_tile, bitmap, kv_len},
                    copies(q, k, v, wq, wk, wv, tickets, n_tickets), tile_blocks, dev_status);
 }

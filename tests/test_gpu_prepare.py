@@ -45,6 +45,7 @@ def call(shape, params, q, k, v, bw, ws_bytes, one):
     (1, 6, 64, 9, 45, 61, 0, 9, dict(spatial_key_first_frame=1)),
     (1, 3, 96, 6, 20, 21, 40, 5, dict(temporal_window_2d=(5, 6))),
     (2, 48, 64, 5, 20, 21, 9, 6, {}),                                  # a copying CTA takes several steps
+    (2, 48, 64, 9, 20, 21, 9, 6, {}),                                  # more copying CTAs than a head's share, four steps each
 ])
 def test_one_call_gives_what_three_give(B, H, D, T, fh, fw, L, omega, opt, bw):
     if bw and "temporal_window_2d" in opt:
