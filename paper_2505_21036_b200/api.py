@@ -131,9 +131,11 @@ def _ptr(t) -> Optional[int]:
 
 
 def _stream() -> Optional[int]:
-    # the current stream's handle without building a Stream object (3.4 -> 0.5 us of a call's host time)
+    # the current stream's handle without building a Stream object (3.4 -> 0.5 us of a call's host time), where torch has the
+    # function for that, which is not part of its public interface
     import torch
-    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device()) or None
+    raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+    return (raw(torch.cuda.current_device()) if raw is not None else torch.cuda.current_stream().cuda_stream) or None
 
 
 def make_shape(B, H, D, T, frame_h, frame_w, L_text) -> rf_shape:

@@ -222,3 +222,15 @@ def test_header_from_plain_c_matches_the_binding(lib, tmp_path):
     assert int(seen["bounds_checked"]) == lib.rf_bounds_checked()
     for c in range(8):
         assert seen[f"status_string.{c}"] == lib.rf_status_string(c).decode()
+
+
+def test_the_current_stream_is_found_without_torchs_private_function(monkeypatch):
+    """The binding's shortcut to the stream's handle is private to torch: a torch without it gives the handle by the public way."""
+    import torch
+    monkeypatch.delattr(torch._C, "_cuda_getCurrentRawStream", raising=False)
+    for handle, wanted in ((0x51, 0x51), (0, None)):
+        monkeypatch.setattr(torch.cuda, "current_device", lambda: 0)
+        monkeypatch.setattr(torch.cuda, "current_stream", lambda: type("Stream", (), {"cuda_stream": handle}))
+        assert api._stream() == wanted
+    monkeypatch.setattr(torch._C, "_cuda_getCurrentRawStream", lambda device: 0x52 + device, raising=False)
+    assert api._stream() == 0x52
