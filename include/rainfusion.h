@@ -314,12 +314,13 @@ void rf_host_pipeline_destroy(rf_host_pipeline *p);
  * Some callers of this library run where device allocation is off limits: inside a serving loop
  * whose memory pool was sized and frozen at start-up, or under a framework allocator that must not be
  * re-entered from a plug-in, so they have no buffer to hand over as `ws` and may not call cudaMalloc
- * to make one.  This entry point takes only inputs and outputs.  Its per-row recall scratch lives in
+ * to make one.  This entry point takes only inputs and outputs.  Its scratch lives in
  * a fixed array inside the library's device image: RF_ARM_STATIC_SCRATCH_FLOATS floats (4 MiB) that
  * every GPU which loads the library holds until the process exits.
  *
  *   - Limit: 2 * B * H * 3 * roundup64(max(frame_h*frame_w, ceil(T*frame_h*frame_w / sample_stride))) + 64
- *     floats must fit (the HunyuanVideo-720p layer needs 525 376).  Larger problems are rejected
+ *     floats must fit (525 376 for the HunyuanVideo-720p layer): room for a recall per sampled row, of which the sums
+ *     that are kept take a small part.  Larger problems are rejected
  *     with RF_ERR_STATIC_SCRATCH_TOO_SMALL before anything is launched.
  *   - Allocates nothing: no cudaMalloc / cudaFree, no allocating library call.
  *   - The first call on each device looks up the array's device address (cudaGetSymbolAddress, with

@@ -474,7 +474,7 @@ size_t rf_arm_scratch_floats(const RfGeom& g, int omega, int nb) {
 
 cudaError_t rf_launch_arm(const RfGeom& g, int sample_mode, int omega, float alpha, int nb, const int* ws_list,
                           const int* wf_list, const __nv_bfloat16* q, const __nv_bfloat16* k, int32_t* head_class,
-                          int32_t* head_window, float* recall, float* recall_plus, float* row_scratch, int32_t* dev_status,
+                          int32_t* head_window, float* recall, float* recall_plus, float* scratch, int32_t* dev_status,
                           cudaStream_t st, bool selftest_abandon, RfDecision* later) {
   const bool plus = head_window != nullptr;
   const int NB = plus ? ARM_MAX_NB : 1;           // windows the kernel has room for; it evaluates the first nb
@@ -489,7 +489,7 @@ cudaError_t rf_launch_arm(const RfGeom& g, int sample_mode, int omega, float alp
   const int n_glb = rf_cdiv(g.Nv, omega), n_loc = g.S;
   const int heads = g.B * g.H;
   const int t_glb = rf_cdiv(n_glb, ARM_TILE), t_loc = rf_cdiv(n_loc, ARM_TILE), t_pad = t_glb > t_loc ? t_glb : t_loc;
-  float* end = row_scratch + (size_t)2 * heads * (2 * NB + 1) * n_pad;
+  float* end = scratch + (size_t)2 * heads * (2 * NB + 1) * n_pad;
   int32_t* arm_flag = reinterpret_cast<int32_t*>(end);
   const size_t sums = (size_t)heads * (2 * NB + 1) * t_pad;     // of one sample; t_pad <= n_pad / 64, so both fit
   double* sums_loc = reinterpret_cast<double*>(end) - sums;
@@ -528,7 +528,6 @@ cudaError_t rf_launch_arm(const RfGeom& g, int sample_mode, int omega, float alp
   d.n_loc = n_loc; d.n_glb = n_glb;
   d.t_loc = t_loc; d.t_glb = t_glb; d.t_pad = t_pad;
   d.local_t = alg1;
-  d.with_tex = tex;
   d.two_mask = g.two_mask;
   d.alpha = alpha;
   for (int i = 0; i < ARM_MAX_NB; ++i) { d.ws[i] = win.ws[i]; d.wf[i] = win.wf[i]; }
@@ -545,8 +544,8 @@ cudaError_t rf_launch_arm(const RfGeom& g, int sample_mode, int omega, float alp
 }
 
 // ------------------------------------------------------------------------------------------------
-// Entry point for callers that can neither pass a workspace nor allocate one: the per-row recall
-// scratch is a fixed array in this library's device image.
+// Entry point for callers that can neither pass a workspace nor allocate one: ARM's scratch is a
+// fixed array in this library's device image.
 // ------------------------------------------------------------------------------------------------
 static __device__ __align__(256) float g_arm_static_scratch[RF_ARM_STATIC_SCRATCH_FLOATS];
 

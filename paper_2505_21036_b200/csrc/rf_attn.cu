@@ -51,7 +51,7 @@ constexpr int kAskAhead = 4;   // tiles an item's longer list has left when the 
 // An accumulator of the whole row cuts every weight off at the last place of the sum so far: beside one key of weight 1, 2^18
 // keys of 2^-19 lost 2.1e-3 of the row's weight in it; with the sums by tile the error is what the outputs' rounding leaves, 5e-5, as it
 // is with all sums added up by the softmax warps, whose outputs are within rel 6e-5.  It costs a load and a store of one column a
-// tile: sixteen shapes, 0.997 to 1.010 times as fast as without.
+// tile: sixteen shapes, 0.993 to 1.010 times as fast as without.
 // Without lse the sum of the unrounded weights is left out (a template: dense D = 64 5.74 -> 5.59 ms).
 // Lazy rescaling of the running maximum: it is raised once a tile's maximum exceeds it by kRaise (log2 units; all rows
 // of the warp more than kRaiseMargin above theirs then raise it together).  A tile's weights thus sum to 2^32 at most;
@@ -68,16 +68,15 @@ struct Maps { CUtensorMap m[8]; };
 template <int D>
 struct Cfg {
   static constexpr int KB = (D + 63) / 64;            // 64-column (128-byte) blocks per row
-  // first column of the second block.  D = 96 is fetched as columns [0,64) and [64,128): the TMA box
+  // first column of the second block.  Q and K of D = 96 are fetched as columns [0,64) and [64,128): the TMA box
   // reaches past the tensor's 96 columns and the missing ones arrive as zeros; they are never read
-  // (Q K^T runs 6 k-steps, P V is one N = 96 MMA per k-step over one and a half 64-column blocks)
+  // (Q K^T runs 6 k-steps).  V has blocks of its own, see VBOX.
   static constexpr int COL1 = 64;
   static constexpr uint32_t BLK = 128 * 128;          // bytes of one 128-row x 64-col bf16 block
   static constexpr uint32_t TILE = KB * BLK;          // bytes of one 128-row tile
-  // D = 64 leaves 128 TMEM columns unused (O is only 64 wide), room for P of both streams in columns of its
-  // own: the S accumulator is then free again as soon as the softmax warps have read it, and the next tile's
-  // scores are computed during the softmax of the current one.  At D = 96 / 128 TMEM is full and P lives on
-  // top of the S columns it was computed from.
+  // At D = 64 O is narrow enough for P of both streams to have TMEM columns of its own (with the row sums' columns that
+  // makes all 512): a stream's next scores are computed during the softmax of its current tile, once both streams
+  // have read theirs (S0 and S1 share columns).  At D = 96 / 128 P lives on top of the S columns it was computed from.
   static constexpr bool S_EARLY = D == 64;
   static constexpr int NK = D == 64 ? 3 : 2;          // K ring depth
   static constexpr int NV = D == 64 ? 3 : 2;          // V ring depth
@@ -323,7 +322,8 @@ __device__ __forceinline__ void rescale_o(uint32_t t_o, float alpha) {
   tc_fence_before();
 }
 // The same out of line, for D = 96 / 128: rare as it is, the scores then stay in registers around it and the loop over the
-// tiles is free of spills.
+// tiles is free of spills.  (At D = 64, inline, 16 bytes are spilt; out of line none, but 48 heads of 17 776 tokens took 5013 us
+// instead of 4932 dense and 2676 instead of 2639 all Textural.)
 template <int D>
 __device__ __noinline__ void rescale_o_call(uint32_t t_o, float alpha) {
   tc_fence_after();
@@ -817,16 +817,7 @@ __global__ void __launch_bounds__(kThreads, 1) rf_attn_kernel(const __grid_const
         const float2 sc2 = make_float2(sc, sc), mneg = make_float2(-m_use, -m_use);
         float2 la = make_float2(0.f, 0.f);
         uint32_t pk[64];
-#pragma unroll
-        for (int c = 0; c < 128; c += 4) {
-          float2 e0 = __ffma2_rn(make_float2(__uint_as_float(s[c]), __uint_as_float(s[c + 1])), sc2, mneg);
-          float2 e1 = __ffma2_rn(make_float2(__uint_as_float(s[c + 2]), __uint_as_float(s[c + 3])), sc2, mneg);
-          e0.x = ex2(e0.x); e0.y = ex2(e0.y);
-          e1.x = ex2(e1.x); e1.y = ex2(e1.y);
-          pk[c / 2] = pack_bf16(e0.x, e0.y);
-          pk[c / 2 + 1] = pack_bf16(e1.x, e1.y);
-          if (LSE) la = __fadd2_rn(la, __fadd2_rn(e0, e1));
-        }
+        take_weights<0, BN, LSE>(s, pk, la, sc2, mneg);
         if (LSE) l_exact += la.x + la.y;
         if (!o_landed) mbar_wait(bar(C::B_OF + j), (done - 1) & 1, wc);
         tc_fence_after();

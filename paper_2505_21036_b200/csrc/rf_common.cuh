@@ -91,7 +91,7 @@ struct RfDecision {
   int n_loc, n_glb;           // rows of the first-frame and of the stride sample
   int t_loc, t_glb, t_pad;    // score CTAs (128 rows each) of a head per sample
   int local_t;                // the Temporal recall comes from the first-frame sample
-  int with_tex, two_mask;
+  int two_mask;
   float alpha;
   int ws[RF_MAX_BANDWIDTHS], wf[RF_MAX_BANDWIDTHS];
   const double *loc, *glb;    // [B*H][2*nb+1][t_pad]: sums of the rows' recalls
@@ -117,11 +117,12 @@ cudaError_t rf_launch_prepare(const RfGeom& g, const RfDecision& dec, int32_t* c
 // later (nullable): the decision is not launched but left there for rf_launch_prepare.
 cudaError_t rf_launch_arm(const RfGeom& g, int sample_mode, int omega, float alpha, int nb, const int* ws_list,
                           const int* wf_list, const __nv_bfloat16* q, const __nv_bfloat16* k, int32_t* head_class,
-                          int32_t* head_window, float* recall, float* recall_plus, float* row_scratch, int32_t* dev_status,
+                          int32_t* head_window, float* recall, float* recall_plus, float* scratch, int32_t* dev_status,
                           cudaStream_t st, bool selftest_abandon = false, RfDecision* later = nullptr);
 // Floats of ARM scratch.  The sums of the rows' recalls lie at its end, before RF_ARM_FLAG_FLOATS whose first word records a
-// wait that ran out inside the score kernel (cleared by every call at the start of its first kernel).  (The size is that of
-// the rows' recalls, which were kept one by one before the score kernel summed them; callers' blocks are sized by it.)
+// wait that ran out inside the score kernel (cleared by every call at the start of its first kernel).  The size allows for a float
+// per sampled row and mask, of which a sum takes a 64th: the entry points accept and refuse callers' blocks, and
+// rf_arm_classify_noalloc shapes, by it.
 #define RF_ARM_FLAG_FLOATS 64
 size_t rf_arm_scratch_floats(const RfGeom& g, int omega, int nb);
 // Tensor map over bf16 rows: [heads][rows][D] with the given row and head strides in bytes (multiples of 16),

@@ -38,7 +38,7 @@ __device__ __forceinline__ RfHead rf_decide(const RfDecision& d, int bh, int lan
   if (d.head_window == nullptr) {
     const float rt = recall(0), rs = recall(d.nb);
     if (d.recall != nullptr) {
-      const float rc = d.with_tex ? recall(2 * d.nb) : 0.f;
+      const float rc = recall(2 * d.nb);   // (the score kernel sums it whenever recalls are asked for)
       if (write) { d.recall[bh * 3] = rt; d.recall[bh * 3 + 1] = rs; d.recall[bh * 3 + 2] = rc; }
     }
     // Algorithm 1; with only two masks (ablation) a head that reaches alpha with neither takes the larger recall
