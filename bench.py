@@ -33,10 +33,9 @@ UNIT = "TFLOP/s"
 # dram__bytes_read.sum + dram__bytes_write.sum of one rf_attn_kernel launch, from single-pass ncu captures; None
 # where no capture exists.  The figure is a recorded measurement, not taken in this run: TRAFFIC_SOURCE names the
 # summary it comes from and the state of the kernel source it was captured on; re-capture when rf_attn.cu changes.
-ATTN_DRAM_BYTES = {"hunyuan720p": 3.36e9, "sweep_33x3600": 3.36e9, "sweep_16x2040": 0.796e9}
+ATTN_DRAM_BYTES = {"hunyuan720p": 3.39e9, "sweep_33x3600": 3.39e9, "sweep_16x2040": 0.794e9}
 TRAFFIC_SOURCE = {"file": "profiles/rf_attn_kernel_hunyuan720p_dram_bytes.md",
-                  "captured_on": "the kernel whose running CTAs take over items (hunyuan720p, sweep_33x3600: commit a47c4f9; "
-                                 "sweep_16x2040: commit 537c860)"}
+                  "captured_on": "the kernel that takes row sums tile by tile out of P V (commit cd44374)"}
 NOMINAL_BF16_TFLOPS = 2250.0     # NVIDIA's dense bf16 figure for one B200 (the 4.5 PFLOP/s quoted per GPU is with 2:4 sparsity)
 
 
